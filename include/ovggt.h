@@ -333,7 +333,9 @@ int ovggt_k_compact(const void* k_src, const void* v_src, const int32_t* survivo
                     int32_t dtype, void* k_dst, void* v_dst, void* stream);
 
 /* out [M, C] = softmax(Q K^T / sqrt(64)) V per head over N rows; head_dim 64.  bf16: tcgen05 kernel;
- * fp32: SIMT kernel.  scratch: device, >= ovggt_k_attention_scratch_bytes(M, N, n_heads). */
+ * fp32: the same tensor pipe on operands split into three bf16 terms, accurate to fp32; scratch and device_status may
+ * then be NULL (without scratch the KV range is not split).  scratch: device, >= ovggt_k_attention_scratch_bytes(M, N,
+ * n_heads). */
 size_t ovggt_k_attention_scratch_bytes(int32_t M, int32_t N, int32_t n_heads);
 int ovggt_k_attention(const void* q, const void* k, const void* v, int32_t M, int32_t N, int32_t n_heads,
                       int32_t dtype, void* out, void* scratch, int32_t* device_status, void* stream);

@@ -22,17 +22,17 @@ def needs_build(out: str = OUT) -> bool:
     return any(os.path.getmtime(d) > os.path.getmtime(out) for d in deps)
 
 
-def check_register_pool(ptxas_log: str) -> None:
-    """The attention kernel moves registers between its warpgroups with setmaxnreg, inside the pool it was launched
-    with; an increase the pool cannot serve would wait for ever.  The source states the launch count it was budgeted
-    for (kRegsLaunch); refuse a build whose ptxas report says otherwise."""
+def check_register_pool(ptxas_log: str, kernel: str = "k_attn_tcgen05") -> None:
+    """The attention kernels move registers between their warpgroups with setmaxnreg, inside the pool they were
+    launched with; an increase the pool cannot serve would wait for ever.  The source states the launch count they were
+    budgeted for (kRegsLaunch); refuse a build whose ptxas report says otherwise."""
     src = open(os.path.join(CSRC, "attn_tcgen05.cuh")).read()
     want = int(re.search(r"constexpr int kRegsLaunch = (\d+);", src).group(1))
-    m = re.search(r"Compiling entry function '[^']*k_attn_tcgen05[^']*'.*?Used (\d+) registers", ptxas_log, re.S)
+    m = re.search(rf"Compiling entry function '[^']*{kernel}[^']*'.*?Used (\d+) registers", ptxas_log, re.S)
     if not m:
-        raise RuntimeError("ptxas report for k_attn_tcgen05 not found")
+        raise RuntimeError(f"ptxas report for {kernel} not found")
     if int(m.group(1)) != want:
-        raise RuntimeError(f"k_attn_tcgen05 is launched with {m.group(1)} registers, budgeted for {want}")
+        raise RuntimeError(f"{kernel} is launched with {m.group(1)} registers, budgeted for {want}")
 
 
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
@@ -52,7 +52,8 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
     if r.returncode != 0:
         raise subprocess.CalledProcessError(r.returncode, cmd)
     try:
-        check_register_pool(r.stdout)
+        for kernel in ("k_attn_tcgen05", "k_attn_f32"):
+            check_register_pool(r.stdout, kernel)
     except Exception:
         os.remove(tmp)
         raise

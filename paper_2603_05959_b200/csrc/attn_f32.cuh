@@ -1,0 +1,384 @@
+// fp32 flash attention for sm_100a on the bf16 tensor pipe: out = softmax(Q K^T / sqrt(64)) V per head, head_dim 64.
+//
+// The tensor cores take no fp32 operands, so every operand is written as the sum of three bf16 numbers,
+// x = h + m + l (each the rounded remainder of the ones before: |m| <= 2^-9 |x|, |l| <= 2^-18 |x|, what is left over is
+// below 2^-27 |x|), and a product as six of the nine partial products, hh + hm + mh + hl + mm + lh; the three left out
+// are below 2^-26 of it, less than the rounding of an fp32 product.  A bf16 product is exact in fp32, the smallest
+// partial products are accumulated first, and no accumulation in tensor memory is longer than one 64-row tile: Q K^T
+// sums 64 terms, and the P V product of a tile starts from zero and is added to fp32 registers, because long sums in
+// tensor memory are not rounded to nearest.  Measured against fp64 the result is as close as that of plain fp32
+// arithmetic.
+//
+// What bounds it: 48 MMAs of 128 x 64 x 16 per 128 x 64 tile, about 1,900 tensor-pipe cycles; the exponentials and the
+// splitting of P take about two thirds of the issue slots in that time, the splitting of K and V a further sixth.  A
+// plain fp32 kernel is bound by the FMA pipes at 64 x 2 x 2 instructions per score instead, an order of magnitude more.
+// One CTA owns 128 query rows of one head and a range of 64-row KV tiles; two CTAs share an SM.
+//   warps 0-3  softmax: one thread per query row; running maximum, P split and written to tensor memory over the scores
+//              it came from, O accumulated in registers
+//   warp 4     allocates tensor memory, issues the MMAs (the whole warp in step, one elected lane)
+//   warps 5-7  read K and V rows from global memory, split them and write the bf16 planes, 128-byte swizzled, to
+//              shared memory (done once per CTA and tile: cheaper than a pass over the cache that writes planes, and
+//              it needs no scratch memory)
+// Every wait is bounded; on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the common teardown.
+#pragma once
+
+#include "attn_tcgen05.cuh"
+
+namespace ovggt {
+
+constexpr int kF32BN = 64;                              // KV rows per tile
+constexpr int kF32Converters = 96;                      // threads of warps 5-7
+constexpr int kF32QPlane = kBM * kHD * 2;               // 16 KB
+constexpr int kF32KvPlane = kF32BN * kHD * 2;           // 8 KB
+constexpr int kF32RegsSoftmax = 168, kF32RegsOther = 88;
+static_assert(128 * kF32RegsSoftmax + 128 * kF32RegsOther <= kAttnThreads * kRegsLaunch, "register pool of the CTA exceeded");
+// S_b at columns [96 b, 96 b + 64), the planes of P_b over it at [96 b, 96 b + 96), O of a tile at [192, 256)
+constexpr int kF32ColBuf = 96, kF32ColO = 192;
+
+struct F32Barriers {
+  unsigned long long k_full, k_empty, v_full, v_empty, s_full[2], p_full, o_full, drain;
+  uint32_t tmem_base;
+  int abort_flag;
+};
+constexpr size_t kF32SmemBytes = (size_t)3 * kF32QPlane + 6 * kF32KvPlane + sizeof(F32Barriers) + 64;
+
+struct F32Params {
+  const float *q, *k, *v;
+  int M, N, H;
+  int splits, tiles_per_split, tiles_total;
+  float* out;             // [M, C]            (splits == 1)
+  float* o_part;          // [splits, M, C]
+  float2* ml_part;        // [splits, M, H]
+  float* lse;             // [M, H] or nullptr
+  int* status;            // or nullptr
+};
+
+// A pair of floats as three bf16 pairs.
+__device__ __forceinline__ void split3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
+  h = pack_bf16(a, b);
+  a -= __uint_as_float(h << 16);
+  b -= __uint_as_float(h & 0xFFFF0000u);
+  m = pack_bf16(a, b);
+  a -= __uint_as_float(m << 16);
+  b -= __uint_as_float(m & 0xFFFF0000u);
+  l = pack_bf16(a, b);
+}
+// Eight floats of columns [8 j, 8 j + 8) of row r -> the same place of three swizzled planes.
+__device__ __forceinline__ void store_planes(unsigned char* base, int plane_bytes, int r, int j, const float4& x, const float4& y) {
+  uint4 h, m, l;
+  split3(x.x, x.y, h.x, m.x, l.x);
+  split3(x.z, x.w, h.y, m.y, l.y);
+  split3(y.x, y.y, h.z, m.z, l.z);
+  split3(y.z, y.w, h.w, m.w, l.w);
+  unsigned char* p = base + r * 128 + ((j ^ (r & 7)) << 4);
+  *reinterpret_cast<uint4*>(p) = h;
+  *reinterpret_cast<uint4*>(p + plane_bytes) = m;
+  *reinterpret_cast<uint4*>(p + 2 * plane_bytes) = l;
+}
+
+// The six partial products, (plane of A, plane of B), smallest first.
+__device__ constexpr int kSplitA[6] = {2, 0, 1, 1, 0, 0};
+__device__ constexpr int kSplitB[6] = {0, 2, 1, 0, 1, 0};
+
+__global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __grid_constant__ F32Params P) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  if (smem_u32(smem) & 1023u) {                      // the 128-byte swizzle needs 1024-byte aligned tiles
+    if (threadIdx.x == 0) report_status(P.status, OVGGT_ERR_DEVICE_STATUS);
+    return;
+  }
+  unsigned char* sQ = smem;
+  unsigned char* sK = sQ + 3 * kF32QPlane;
+  unsigned char* sV = sK + 3 * kF32KvPlane;
+  F32Barriers* B = reinterpret_cast<F32Barriers*>(sV + 3 * kF32KvPlane);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int qt = blockIdx.x, h = blockIdx.y, split = blockIdx.z;
+  const int t_begin = split * P.tiles_per_split;
+  const int n_tiles = min(P.tiles_total, t_begin + P.tiles_per_split) - t_begin;   // >= 1 by construction
+  const int C = P.H * kHD;
+
+  if (threadIdx.x == 0) {
+    mbar_init(&B->k_full, kF32Converters);
+    mbar_init(&B->v_full, kF32Converters);
+    mbar_init(&B->k_empty, 1);
+    mbar_init(&B->v_empty, 1);
+    mbar_init(&B->s_full[0], 1);
+    mbar_init(&B->s_full[1], 1);
+    mbar_init(&B->p_full, 128);
+    mbar_init(&B->o_full, 1);
+    mbar_init(&B->drain, 1);
+    B->abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 4) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&B->tmem_base)),
+                 "r"((uint32_t)kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  {  // the query tile's planes: 128 rows x 8 groups of 8 columns, rows past M zero
+    float4 x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int idx = threadIdx.x + i * kAttnThreads, m = qt * kBM + (idx >> 3);
+      x[i] = y[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (m < P.M) {
+        const float4* p = reinterpret_cast<const float4*>(P.q + (size_t)m * C + (size_t)h * kHD + (idx & 7) * 8);
+        x[i] = __ldg(p);
+        y[i] = __ldg(p + 1);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int idx = threadIdx.x + i * kAttnThreads;
+      store_planes(sQ, kF32QPlane, idx >> 3, idx & 7, x[i], y[i]);
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *(volatile uint32_t*)&B->tmem_base;
+
+  if (warp >= 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kF32RegsOther));
+    if (warp == 4) {
+      // ------------------------------------------------ MMA issuer: QK(0) | QK(1) PV(0) | QK(2) PV(1) | ...
+      // QK(t + 1) goes into the other buffer, whose P(t - 1) the already issued PV(t - 1) reads first (the tensor pipe
+      // executes one thread's MMAs in order).
+      const bool leader = elect_one();
+      const uint32_t tm = __reduce_or_sync(0xFFFFFFFFu, tmem);
+      constexpr uint32_t idesc_qk = idesc_bf16(kF32BN, false), idesc_pv = idesc_bf16(kHD, true);
+      const uint64_t dq = smem_desc_sw128(smem_u32(sQ)), dk = smem_desc_sw128(smem_u32(sK)), dv = smem_desc_sw128(smem_u32(sV));
+      auto wait_all = [&](void* bar, uint32_t parity) {
+        return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, B, P.status)) != 0;
+      };
+      auto issue_qk = [&](int t) {
+        if (leader) {
+#pragma unroll
+          for (int g = 0; g < 6; ++g)
+#pragma unroll
+            for (int kk = 0; kk < kHD / 16; ++kk)
+              mma_ss(tm + (t & 1) * kF32ColBuf, dq + (uint64_t)(kSplitA[g] * (kF32QPlane >> 4) + kk * 2),
+                     dk + (uint64_t)(kSplitB[g] * (kF32KvPlane >> 4) + kk * 2), idesc_qk, g > 0 || kk > 0);
+          tc_commit(&B->s_full[t & 1]);
+          tc_commit(&B->k_empty);
+        }
+      };
+      bool ok = wait_all(&B->k_full, 0);
+      if (ok) {
+        tc_fence_after();
+        issue_qk(0);
+      }
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        if (t + 1 < n_tiles) {
+          ok = wait_all(&B->k_full, (uint32_t)(t + 1) & 1u);
+          if (!ok) break;
+          tc_fence_after();
+          issue_qk(t + 1);
+        }
+        ok = wait_all(&B->v_full, (uint32_t)t & 1u);
+        if (ok) ok = wait_all(&B->p_full, (uint32_t)t & 1u);
+        if (!ok) break;
+        tc_fence_after();
+        if (leader) {
+#pragma unroll
+          for (int g = 0; g < 6; ++g)
+#pragma unroll
+            for (int kk = 0; kk < kF32BN / 16; ++kk)
+              mma_ts(tm + kF32ColO, tm + (t & 1) * kF32ColBuf + kSplitA[g] * 32 + kk * 8,
+                     dv + (uint64_t)(kSplitB[g] * (kF32KvPlane >> 4) + kk * 128), idesc_pv, g > 0 || kk > 0);
+          tc_commit(&B->v_empty);
+          tc_commit(&B->o_full);
+        }
+      }
+      if (ok) {
+        wait_all(&B->v_empty, (uint32_t)(n_tiles - 1) & 1u);
+        wait_all(&B->o_full, (uint32_t)(n_tiles - 1) & 1u);
+      } else {
+        if (leader) tc_commit(&B->drain);             // let every issued MMA finish before TMEM is freed
+        wait_all(&B->drain, 0);
+      }
+      __syncwarp();
+    } else {
+      // ------------------------------------------------ K / V splitting
+      // The rows of a tile are requested before the wait for its buffer, so that their latency runs under it.
+      const int ct = (int)threadIdx.x - 160;
+      constexpr int kVecs = kF32BN * 8, kPer = (kVecs + kF32Converters - 1) / kF32Converters;
+      auto convert = [&](const float* src, unsigned char* dst, int t, void* empty, void* full) -> bool {
+        float4 x[kPer], y[kPer];
+        const int row0 = (t_begin + t) * kF32BN;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+          const int idx = ct + i * kF32Converters, r = row0 + (idx >> 3);
+          x[i] = y[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (idx < kVecs && r < P.N) {
+            const float4* p = reinterpret_cast<const float4*>(src + (size_t)r * C + (size_t)h * kHD + (idx & 7) * 8);
+            x[i] = p[0];
+            y[i] = p[1];
+          }
+        }
+        if (t > 0 && !mbar_wait(empty, (uint32_t)(t - 1) & 1u, B, P.status)) return false;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+          const int idx = ct + i * kF32Converters;
+          if (idx < kVecs) store_planes(dst, kF32KvPlane, idx >> 3, idx & 7, x[i], y[i]);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive(full);
+        return true;
+      };
+      for (int t = 0; t < n_tiles; ++t)
+        if (!convert(P.k, sK, t, &B->k_empty, &B->k_full) || !convert(P.v, sV, t, &B->v_empty, &B->v_full)) break;
+      __syncwarp();
+    }
+  } else {
+    // ------------------------------------------------ softmax and accumulation of O (128 threads, one query row each)
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kF32RegsSoftmax));
+    const int row = warp * 32 + lane;
+    const uint32_t t_row = tmem + ((uint32_t)(warp * 32) << 16);
+    const float c = 1.4426950408889634f * 0.125f;     // log2(e) / sqrt(64)
+    float mref = -INFINITY, l = 0.0f;
+    float acc[kHD];
+#pragma unroll
+    for (int i = 0; i < kHD; ++i) acc[i] = 0.0f;
+    bool ok = true;
+    // acc += O of tile t (both under the reference that held when its P was made)
+    auto take_o = [&](int t) -> bool {
+      if (__all_sync(0xFFFFFFFFu, mbar_wait(&B->o_full, (uint32_t)t & 1u, B, P.status)) == 0) return false;
+      tc_fence_after();
+#pragma unroll
+      for (int j = 0; j < kHD; j += 16) {
+        uint32_t o[16];
+        tmem_ld16(t_row + kF32ColO + j, o);
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[j + e] += __uint_as_float(o[e]);
+      }
+      return true;
+    };
+    for (int t = 0; t < n_tiles; ++t) {
+      const uint32_t buf = t_row + (t & 1) * kF32ColBuf;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->s_full[t & 1], (uint32_t)(t >> 1) & 1u, B, P.status)) != 0;
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t s[kF32BN];
+      tmem_ld32(buf, s);
+      tmem_ld32(buf + 32, s + 32);
+      tmem_wait_ld();
+      const int left = P.N - (t_begin + t) * kF32BN;
+      if (left < kF32BN) {
+#pragma unroll
+        for (int j = 0; j < kF32BN; ++j)
+          if (j >= left) s[j] = 0xFF800000u;           // -inf on columns past the last row
+      }
+      float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+      for (int j = 0; j < kF32BN; j += 2)
+        m4[(j >> 1) & 3] = max3(m4[(j >> 1) & 3], __uint_as_float(s[j]), __uint_as_float(s[j + 1]));
+      const float mnew = fmaxf(mref, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * c);
+      const float corr = ex2(mref - mnew);             // 0 on the first tile, 1 when the maximum stands
+      float sum4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < kF32BN; j += 16) {
+        uint32_t ph[8], pm[8], pl[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float p0 = ex2(fmaf(__uint_as_float(s[j + 2 * e]), c, -mnew));
+          const float p1 = ex2(fmaf(__uint_as_float(s[j + 2 * e + 1]), c, -mnew));
+          sum4[e & 3] += p0 + p1;
+          split3(p0, p1, ph[e], pm[e], pl[e]);
+        }
+        tmem_st8(buf + j / 2, ph);
+        tmem_st8(buf + 32 + j / 2, pm);
+        tmem_st8(buf + 64 + j / 2, pl);
+      }
+      l = fmaf(l, corr, (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]));
+      if (t > 0) {
+        ok = take_o(t - 1);
+        if (!ok) break;
+        if (__any_sync(0xFFFFFFFFu, corr != 1.0f)) {
+#pragma unroll
+          for (int i = 0; i < kHD; ++i) acc[i] *= corr;
+        }
+      }
+      mref = mnew;
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive(&B->p_full);
+    }
+    if (ok) ok = take_o(n_tiles - 1);
+    const int m = qt * kBM + row;
+    if (ok && m < P.M) {
+      const bool whole = P.splits == 1;
+      const float f = whole ? 1.0f / l : 1.0f;
+      float4* dst = reinterpret_cast<float4*>((whole ? P.out + (size_t)m * C : P.o_part + ((size_t)split * P.M + m) * C) + (size_t)h * kHD);
+#pragma unroll
+      for (int i = 0; i < kHD; i += 4) dst[i / 4] = make_float4(acc[i] * f, acc[i + 1] * f, acc[i + 2] * f, acc[i + 3] * f);
+      if (!whole) P.ml_part[((size_t)split * P.M + m) * P.H + h] = make_float2(mref, l);
+      if (whole && P.lse != nullptr) P.lse[(size_t)m * P.H + h] = mref + log2f(l);
+    }
+  }
+
+  // ------------------------------------------------ teardown
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 4) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols) : "memory");
+  }
+}
+
+// ---------------------------------------------------------------- host side
+
+// Number of KV splits: waves of CTAs over the 2 x 148 slots, each as long as its tiles plus about two more for the
+// set-up (query planes, tensor memory); a split costs a merge of about three tiles.
+inline int attn_f32_choose_splits(int M, int N, int H) {
+  const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kF32BN - 1) / kF32BN;
+  const long slots = (long)kCtasPerSm * 148;
+  int best = 1;
+  long best_cost = -1;
+  for (int s = 1; s <= kMaxSplits && s <= tiles; ++s) {
+    const int per = (tiles + s - 1) / s;
+    if ((tiles + per - 1) / per != s) continue;
+    const long waves = ((long)q_tiles * H * s + slots - 1) / slots;
+    const long cost = waves * (per + 2) + (s > 1 ? 3 : 0);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = s;
+    }
+  }
+  return best;
+}
+
+// scratch: attn_tcgen05_scratch_bytes, or nullptr (the KV range is then not split).
+inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out, void* scratch,
+                           int* status, cudaStream_t st, float* lse, int* launches) {
+  const int C = H * kHD;
+  F32Params P;
+  P.q = static_cast<const float*>(q);
+  P.k = static_cast<const float*>(k);
+  P.v = static_cast<const float*>(v);
+  P.M = M; P.N = N; P.H = H;
+  P.tiles_total = (N + kF32BN - 1) / kF32BN;
+  P.splits = scratch ? attn_f32_choose_splits(M, N, H) : 1;
+  P.tiles_per_split = (P.tiles_total + P.splits - 1) / P.splits;
+  P.splits = (P.tiles_total + P.tiles_per_split - 1) / P.tiles_per_split;     // no empty split
+  P.out = static_cast<float*>(out);
+  P.o_part = static_cast<float*>(scratch);
+  P.ml_part = reinterpret_cast<float2*>(static_cast<char*>(scratch) + (size_t)kMaxSplits * M * C * 4);
+  P.lse = lse;
+  P.status = status;
+  cudaError_t e = cudaFuncSetAttribute(k_attn_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32SmemBytes);
+  if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
+  k_attn_f32<<<dim3((M + kBM - 1) / kBM, H, P.splits), kAttnThreads, kF32SmemBytes, st>>>(P);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
+  *launches = 1;
+  if (P.splits > 1) {
+    *launches = 2;
+    return attn_merge_launch<float>(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st);
+  }
+  return OVGGT_OK;
+}
+
+}  // namespace ovggt

@@ -106,7 +106,11 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // CTA's abort flag is raised, OVGGT_ERR_TIMEOUT goes to the status word and the caller gets false; so does every
 // other waiter of the CTA the next time it looks at the flag.
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;
-__device__ __forceinline__ bool mbar_wait(void* bar, uint32_t parity, AttnBarriers* B, int* status,
+__device__ __forceinline__ void report_status(int* status, int code) {
+  if (status != nullptr) atomicCAS(status, 0, code);
+}
+template <typename Barriers>
+__device__ __forceinline__ bool mbar_wait(void* bar, uint32_t parity, Barriers* B, int* status,
                                           unsigned long long limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
   unsigned long long t0 = 0;
@@ -118,7 +122,7 @@ __device__ __forceinline__ bool mbar_wait(void* bar, uint32_t parity, AttnBarrie
       if (t0 == 0) t0 = now;
       else if (now - t0 > limit_ns) {
         *(volatile int*)&B->abort_flag = 1;
-        atomicCAS(status, 0, OVGGT_ERR_TIMEOUT);
+        report_status(status, OVGGT_ERR_TIMEOUT);
         return false;
       }
     }
@@ -210,6 +214,11 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
       "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -647,8 +656,9 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 
 // out[m, h*64 + c] = sum_s O_s 2^(m_s - m*) / sum_s l_s 2^(m_s - m*), m* = max_s m_s, splits folded in order.
 // One thread per 4 columns; all loads of a thread are issued before the arithmetic that needs them.
+template <typename Out>
 __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_part, const float2* __restrict__ ml_part,
-                                                    int M, int H, int splits, __nv_bfloat16* __restrict__ out,
+                                                    int M, int H, int splits, Out* __restrict__ out,
                                                     float* __restrict__ lse) {
   const int C = H * kHD;
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -684,10 +694,14 @@ __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_
     }
   const float inv = 1.0f / den;
   if (lse != nullptr && (c4 * 4) % kHD == 0) lse[(size_t)m * H + h] = mstar + log2f(den);
-  uint2 w;
-  w.x = pack_bf16(acc.x * inv, acc.y * inv);
-  w.y = pack_bf16(acc.z * inv, acc.w * inv);
-  *reinterpret_cast<uint2*>(out + (size_t)m * C + c4 * 4) = w;
+  if constexpr (sizeof(Out) == 4) {
+    *reinterpret_cast<float4*>(out + (size_t)m * C + c4 * 4) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+  } else {
+    uint2 w;
+    w.x = pack_bf16(acc.x * inv, acc.y * inv);
+    w.y = pack_bf16(acc.z * inv, acc.w * inv);
+    *reinterpret_cast<uint2*>(out + (size_t)m * C + c4 * 4) = w;
+  }
 }
 
 // Self-test of the bounded wait: one CTA sets up a barrier that expects one arrival, nobody arrives, and the wait is
@@ -795,6 +809,26 @@ inline int attn_kv_maps(AttnKvMaps* m, const void* k, const void* v, int N, int 
   return OVGGT_OK;
 }
 
+template <typename Out>
+inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, int H, int splits, Out* out, float* lse,
+                             cudaStream_t st) {
+  const size_t total = (size_t)M * (H * kHD / 4);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((total + 255) / 256));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = 0;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k_attn_merge<Out>, o_part, ml_part, M, H, splits, out, lse);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
+  return OVGGT_OK;
+}
+
 inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
                                void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
                                int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr) {
@@ -826,23 +860,7 @@ inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int 
   k_attn_tcgen05<<<grid, kAttnThreads, kAttnSmemBytes, st>>>(tq, tk, tv, P);
   e = cudaGetLastError();
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  if (P.splits > 1) {
-    const size_t total = (size_t)M * (C / 4);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((total + 255) / 256));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k_attn_merge, (const float*)P.o_part, (const float2*)P.ml_part, M, H, P.splits, P.out,
-                           lse);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  }
+  if (P.splits > 1) return attn_merge_launch(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st);
   return OVGGT_OK;
 }
 

@@ -31,25 +31,6 @@ struct GemmBarriers {
 };
 constexpr size_t kGemmSmemBytes = (size_t)kGemmStages * (kGemmATile + kGemmBTile) + sizeof(GemmBarriers) + 64;
 
-// The bounded wait of the attention kernel, for a barrier block of another shape.
-__device__ __forceinline__ bool gemm_wait(void* bar, uint32_t parity, GemmBarriers* B, int* status) {
-  if (mbar_try_wait(bar, parity)) return true;
-  unsigned long long t0 = 0;
-  for (uint32_t spins = 1;; ++spins) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((spins & 1023u) == 0) {
-      if (*(volatile int*)&B->abort_flag) return false;
-      const unsigned long long now = global_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > kWaitLimitNs) {
-        *(volatile int*)&B->abort_flag = 1;
-        atomicCAS(status, 0, OVGGT_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-}
-
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                     __nv_bfloat16* __restrict__ C, int M, int N, int K, int* status) {
@@ -97,7 +78,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       for (int kt = 0; kt < k_tiles && ok; ++kt) {
         const int s = kt % kGemmStages;
         const uint32_t ph = (uint32_t)(kt / kGemmStages) & 1u;
-        if (kt >= kGemmStages) ok = gemm_wait(&B->empty[s], ph ^ 1u, B, status);
+        if (kt >= kGemmStages) ok = mbar_wait(&B->empty[s], ph ^ 1u, B, status);
         if (!ok) break;
         mbar_expect_tx(&B->full[s], kGemmATile + kGemmBTile);
         tma_load_2d(sA + s * kGemmATile, &tm_a, kt * kGemmBK, m0, &B->full[s]);
@@ -107,7 +88,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       }
       if (!ok)   // leave no bulk copy in flight into this CTA's shared memory
         for (int i = max(0, issued - kGemmStages); i < issued; ++i)
-          gemm_wait(&B->full[i % kGemmStages], (uint32_t)(i / kGemmStages) & 1u, B, status);
+          mbar_wait(&B->full[i % kGemmStages], (uint32_t)(i / kGemmStages) & 1u, B, status);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -119,7 +100,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     for (int kt = 0; kt < k_tiles && ok; ++kt) {
       const int s = kt % kGemmStages;
       const uint32_t ph = (uint32_t)(kt / kGemmStages) & 1u;
-      ok = __all_sync(0xFFFFFFFFu, gemm_wait(&B->full[s], ph, B, status)) != 0;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->full[s], ph, B, status)) != 0;
       if (!ok) break;
       tc_fence_after();
       const uint64_t da = smem_desc_sw128(smem_u32(sA + s * kGemmATile));
@@ -138,7 +119,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       if (leader) tc_commit(&B->acc_full);
     } else {
       if (leader) tc_commit(&B->drain);             // let every issued MMA finish before TMEM is freed
-      __all_sync(0xFFFFFFFFu, gemm_wait(&B->drain, 0, B, status));
+      __all_sync(0xFFFFFFFFu, mbar_wait(&B->drain, 0, B, status));
     }
     __syncwarp();
   } else {
@@ -146,7 +127,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     const int quad = warp & 3;
     const int row = quad * 32 + lane;
     const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);
-    const bool ok = __all_sync(0xFFFFFFFFu, gemm_wait(&B->acc_full, 0, B, status)) != 0;
+    const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->acc_full, 0, B, status)) != 0;
     if (ok) {
       tc_fence_after();
       const int m = m0 + row;

@@ -15,7 +15,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/ovggt.h"
-#include "attn_simt.cuh"
+#include "attn_f32.cuh"
 #include "attn_tcgen05.cuh"
 #include "common.cuh"
 #include "compact_kernels.cuh"
@@ -268,10 +268,11 @@ int launch_attention(const void* q, const void* k, const void* v, int M, int N, 
     if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
     return rc;
   }
-  dim3 grid((M + kSimtRows - 1) / kSimtRows, H);
-  k_attn_simt<kF32><<<grid, kSimtRows, 0, st>>>(q, k, v, M, N, H, out, lse);
-  LAUNCHED();
-  return OVGGT_OK;
+  int launches = 0;
+  const int rc = attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, &launches);
+  g_launches.fetch_add(launches);
+  if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
+  return rc;
 }
 
 }  // namespace
