@@ -51,6 +51,7 @@ struct F32Params {
   float2* ml_part;        // [splits, M, H]
   float* lse;             // [M, H] or nullptr
   int* status;            // or nullptr
+  int wait_first;         // as in AttnParams
 };
 
 // A pair of floats as three bf16 pairs.
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
   const int n_tiles = min(P.tiles_total, t_begin + P.tiles_per_split) - t_begin;   // >= 1 by construction
   const int C = P.H * kHD;
 
+  if (P.wait_first) pdl_wait();
   if (threadIdx.x == 0) {
     mbar_init(&B->k_full, kF32Converters);
     mbar_init(&B->v_full, kF32Converters);
@@ -326,6 +328,7 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols) : "memory");
   }
+  if (!P.wait_first) pdl_wait();
 }
 
 // ---------------------------------------------------------------- host side
@@ -352,7 +355,7 @@ inline int attn_f32_choose_splits(int M, int N, int H) {
 
 // scratch: attn_tcgen05_scratch_bytes, or nullptr (the KV range is then not split).
 inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out, void* scratch,
-                           int* status, cudaStream_t st, float* lse, int* launches) {
+                           int* status, cudaStream_t st, float* lse, bool beside_previous, int* launches) {
   const int C = H * kHD;
   F32Params P;
   P.q = static_cast<const float*>(q);
@@ -368,10 +371,11 @@ inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, i
   P.ml_part = reinterpret_cast<float2*>(static_cast<char*>(scratch) + (size_t)kMaxSplits * M * C * 4);
   P.lse = lse;
   P.status = status;
-  cudaError_t e = cudaFuncSetAttribute(k_attn_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32SmemBytes);
+  P.wait_first = beside_previous ? 0 : 1;
+  static std::atomic<uint64_t> smem_set{0};
+  cudaError_t e = allow_smem(k_attn_f32, kF32SmemBytes, smem_set);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  k_attn_f32<<<dim3((M + kBM - 1) / kBM, H, P.splits), kAttnThreads, kF32SmemBytes, st>>>(P);
-  e = cudaGetLastError();
+  e = launch_dependent(k_attn_f32, dim3((M + kBM - 1) / kBM, H, P.splits), kAttnThreads, 1, kF32SmemBytes, st, true, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   *launches = 1;
   if (P.splits > 1) {

@@ -155,6 +155,12 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
   return d;
 }
 
+// The same for an MN-major operand wider than one 64-column swizzle atom: columns 64 and up lie `gap` bytes after the
+// first 64 (the leading byte offset).
+__device__ __forceinline__ uint64_t smem_desc_sw128_mn(uint32_t saddr, uint32_t gap) {
+  return (smem_desc_sw128(saddr) & ~((uint64_t)0x3FFF << 16)) | ((uint64_t)((gap >> 4) & 0x3FFFu) << 16);
+}
+
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128.
 __host__ __device__ constexpr uint32_t idesc_bf16(int n, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
@@ -293,6 +299,9 @@ struct AttnParams {
   float2* ml_part;        // [splits, M, H]    (reference maximum in log2 units, row sum)
   float* lse;             // [M, H] or nullptr: log2 of each row's softmax denominator (reference + log2 of the sum)
   int* status;
+  // The kernel before this one in the stream: 1 - it wrote what is read here, wait for it first; 0 - it did not, but runs
+  // beside this one (the selection of the same step), and this kernel must not end before it.
+  int wait_first;
 };
 
 __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm)
@@ -314,6 +323,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const int n_tiles = min(P.tiles_total, t_begin + P.tiles_per_split) - t_begin;   // >= 1 by construction
   const int C = P.H * kHD;
 
+  if (P.wait_first) pdl_wait();
   // The producer's elected thread sets the barriers up and sends the first loads (Q and the first K/V tile) on their
   // way at once, so that they travel while tensor memory is allocated and the CTA meets at its first barrier.
   if (warp == 4 && lane == 0) {
@@ -652,6 +662,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols) : "memory");
   }
+  if (!P.wait_first) pdl_wait();
 }
 
 // out[m, h*64 + c] = sum_s O_s 2^(m_s - m*) / sum_s l_s 2^(m_s - m*), m* = max_s m_s, splits folded in order.
@@ -665,7 +676,7 @@ __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_
   const size_t total = (size_t)M * (C / 4);
   // launched with programmatic stream serialisation: its CTAs may become resident while the last attention CTAs
   // drain; the partials are complete and visible once this wait returns
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   if (idx >= total) return;
   const int m = (int)(idx / (C / 4)), c4 = (int)(idx % (C / 4)), h = (c4 * 4) / kHD;
   float2 ml[kMaxSplits];
@@ -813,25 +824,16 @@ template <typename Out>
 inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, int H, int splits, Out* out, float* lse,
                              cudaStream_t st) {
   const size_t total = (size_t)M * (H * kHD / 4);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((total + 255) / 256));
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_attn_merge<Out>, o_part, ml_part, M, H, splits, out, lse);
-  if (e == cudaSuccess) e = cudaGetLastError();
+  cudaError_t e = launch_dependent(k_attn_merge<Out>, dim3((unsigned)((total + 255) / 256)), 256, 1, 0, st, true, o_part,
+                                   ml_part, M, H, splits, out, lse);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   return OVGGT_OK;
 }
 
 inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
                                void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
-                               int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr) {
+                               int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr,
+                               bool beside_previous = false) {
   const int C = H * kHD;
   CUtensorMap tq;
   AttnKvMaps local;
@@ -854,11 +856,12 @@ inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int 
   P.status = status;
   P.kmax2 = kmax2;
   P.lse = lse;
-  cudaError_t e = cudaFuncSetAttribute(k_attn_tcgen05, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnSmemBytes);
+  P.wait_first = beside_previous ? 0 : 1;
+  static std::atomic<uint64_t> smem_set{0};
+  cudaError_t e = allow_smem(k_attn_tcgen05, kAttnSmemBytes, smem_set);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   dim3 grid((M + kBM - 1) / kBM, H, P.splits);
-  k_attn_tcgen05<<<grid, kAttnThreads, kAttnSmemBytes, st>>>(tq, tk, tv, P);
-  e = cudaGetLastError();
+  e = launch_dependent(k_attn_tcgen05, grid, kAttnThreads, 1, kAttnSmemBytes, st, true, tq, tk, tv, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   if (P.splits > 1) return attn_merge_launch(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st);
   return OVGGT_OK;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/ovggt.h"
 
 namespace ovggt {
@@ -85,6 +87,56 @@ __device__ __forceinline__ bool index_ok(long long i, long long n, int* status) 
 #else
 __device__ __forceinline__ bool index_ok(long long, long long, int*) { return true; }
 #endif
+
+// Programmatic dependent launch.  A kernel launched with it may start while the one before it in the stream drains;
+// pdl_wait returns once that one has completed and its writes are visible (at once when the kernel was launched plainly).
+// pdl_trigger lets the kernel after this one start as soon as every CTA of this one has come here or ended.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, int threads, int cluster, size_t smem, cudaStream_t st,
+                                    bool pdl, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster;
+    attr[n].val.clusterDim.y = 1;
+    attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Opt a kernel in to `bytes` of dynamic shared memory, and its SMs to the largest shared-memory carve-out: an SM whose
+// carve-out was set up for a kernel with little shared memory has to drain before a CTA of the attention (115 KB) can join
+// it, so a selection running beside the attention would keep its SMs to itself.  Once per kernel and device (the calls
+// are safe to repeat, so threads may race here).
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t bytes, std::atomic<uint64_t>& done, bool carveout = true) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev < 64 && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess && carveout) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess && dev < 64) done.fetch_or(bit);
+  return e;
+}
 
 // ---- block-wide primitives for a block of up to 1024 threads; `sh` holds >= 33 words.
 

@@ -19,6 +19,7 @@
 #include "attn_tcgen05.cuh"
 #include "common.cuh"
 #include "compact_kernels.cuh"
+#include "front_kernel.cuh"
 #include "gemm_tcgen05.cuh"
 #include "score_kernels.cuh"
 #include "select_kernel.cuh"
@@ -56,6 +57,9 @@ int colsum_parts(int rows) { return std::max(1, std::min(kMaxColsumParts, (rows 
 
 // CTAs per cluster of the selection kernels: about 2K candidates per CTA, at most 8 (the portable limit).
 int select_cluster_ctas(int N) { return std::max(1, std::min(kSelectMaxCtas, (N + 2047) / 2048)); }
+// The fused kernel: one CTA, which needs no cluster barriers, up to the size where its passes over the positions and the
+// rows of the key sums' corrections outweigh them; then a full cluster.
+int compress_ctas(int N, int M) { return N <= 1024 && M <= 128 ? 1 : kSelectMaxCtas; }
 
 template <typename... KArgs, typename... Args>
 cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, int ncta, size_t smem, cudaStream_t st, Args... args) {
@@ -70,7 +74,7 @@ cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, int ncta, size_t
   attr.val.clusterDim.y = 1;
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = ncta > 1 ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -86,77 +90,6 @@ int launch_row_norms(const void* x, int rows, int C, int dtype, float* s, cudaSt
   return OVGGT_OK;
 }
 
-// part: [colsum_parts(rows), C] floats; ksum: [C] floats.
-int launch_diversity(const void* K, int rows, int C, int dtype, float* part, float* ksum, float* d,
-                     cudaStream_t st) {
-  if (rows <= 0) return OVGGT_OK;
-  const int nvec = C * elem_bytes(dtype) / 16;
-  const int parts = colsum_parts(rows);
-  const int rpc = (rows + parts - 1) / parts;
-  const int threads = std::min(256, (nvec + 31) / 32 * 32);
-  if (dtype == kBF16) k_colsum_partial<kBF16><<<parts, threads, 0, st>>>((const uint4*)K, rows, nvec, rpc, part);
-  else                k_colsum_partial<kF32><<<parts, threads, 0, st>>>((const uint4*)K, rows, nvec, rpc, part);
-  LAUNCHED();
-  k_colsum_final<<<(C + 31) / 32, 1024, 0, st>>>(part, parts, C, ksum);
-  LAUNCHED();
-  const int grid = std::min((rows + 7) / 8, 148 * 8);
-  const size_t smem = (size_t)C * 4;
-  if (dtype == kBF16)
-    k_diversity<kBF16><<<grid, 256, smem, st>>>((const uint4*)K, rows, nvec, ksum, 1, nullptr, d, grid, nullptr, 0,
-                                                nullptr);
-  else
-    k_diversity<kF32><<<grid, 256, smem, st>>>((const uint4*)K, rows, nvec, ksum, 1, nullptr, d, grid, nullptr, 0,
-                                               nullptr);
-  LAUNCHED();
-  return OVGGT_OK;
-}
-
-constexpr int kColsumSlices = 8;
-
-// Diversity from the per-CTA column sums the last compaction left (nparts rows of part): no pass over K for the sums.
-// slices: [kColsumSlices, C] floats of scratch, then the column sums [C], then one arrival counter per 32 columns
-// (colsum_scratch_bytes(C) in all; the counters zero before the first use).
-size_t colsum_scratch_bytes(int C) { return ((size_t)(kColsumSlices + 1) * C * 4 + ((size_t)(C + 31) / 32) * 4 + 255) / 256 * 256; }
-// The same launch also computes the residual norms s_raw [resid_rows] of the new frame when resid is given.
-int launch_diversity_from_parts(const void* K, int rows, int C, int dtype, const float* part, int nparts, float* slices,
-                                float* d, const void* resid, int resid_rows, float* s_raw, cudaStream_t st) {
-  if (rows <= 0) return OVGGT_OK;
-  const int nvec = C * elem_bytes(dtype) / 16;
-  float* ksum = slices + (size_t)kColsumSlices * C;
-  int* arrived = reinterpret_cast<int*>(ksum + C);
-  k_colsum_final_sliced<<<dim3((C + 31) / 32, kColsumSlices), 1024, 0, st>>>(part, nparts, C, slices, ksum, arrived);
-  LAUNCHED();
-  const int grid = std::min((rows + 63) / 64, 148 * 8);   // eight rows per warp: the centroid registers are loaded once
-  const size_t smem = (size_t)C * 4;
-  const int norm_ctas = resid ? (resid_rows + 7) / 8 : 0;
-  if (dtype == kBF16)
-    k_diversity<kBF16><<<grid + norm_ctas, 256, smem, st>>>((const uint4*)K, rows, nvec, ksum, 1, nullptr, d, grid,
-                                                            (const uint4*)resid, resid_rows, s_raw);
-  else
-    k_diversity<kF32><<<grid + norm_ctas, 256, smem, st>>>((const uint4*)K, rows, nvec, ksum, 1, nullptr, d, grid,
-                                                           (const uint4*)resid, resid_rows, s_raw);
-  LAUNCHED();
-  return OVGGT_OK;
-}
-
-// Compaction that also leaves per-CTA column sums of the keys it writes; *nparts = number of partial rows written.
-int launch_compact_colsum(const void* ks, const void* vs, const int* surv, int n_keep, int C, int dtype, void* kd,
-                          void* vd, float* part, int* nparts, cudaStream_t st, int n_src, int* status) {
-  *nparts = 0;
-  if (n_keep <= 0) return OVGGT_OK;
-  const int nvec = C * elem_bytes(dtype) / 16;
-  const int grid = std::min((n_keep + 31) / 32, 148 * 8);   // four survivors (K and V rows) per warp
-  if (dtype == kBF16)
-    k_compact_colsum<kBF16><<<grid, 256, 0, st>>>((const uint4*)ks, (const uint4*)vs, surv, n_keep, nvec, (uint4*)kd,
-                                                  (uint4*)vd, part, n_src, status);
-  else
-    k_compact_colsum<kF32><<<grid, 256, 0, st>>>((const uint4*)ks, (const uint4*)vs, surv, n_keep, nvec, (uint4*)kd,
-                                                 (uint4*)vd, part, n_src, status);
-  LAUNCHED();
-  *nparts = grid;
-  return OVGGT_OK;
-}
-
 int launch_compact(const void* ks, const void* vs, const int* surv, int n_keep, int C, int dtype, void* kd,
                    void* vd, cudaStream_t st, int n_src, int* status) {
   if (n_keep <= 0) return OVGGT_OK;
@@ -164,25 +97,6 @@ int launch_compact(const void* ks, const void* vs, const int* surv, int n_keep, 
   const int grid = std::min((2 * n_keep + 7) / 8, 148 * 8);
   k_compact<<<grid, 256, 0, st>>>((const uint4*)ks, (const uint4*)vs, surv, n_keep, nvec, (uint4*)kd, (uint4*)vd, n_src,
                                   status);
-  LAUNCHED();
-  return OVGGT_OK;
-}
-
-// Diversity against sums given as n_slices rows (see k_diversity); the frame's residual norms ride in the same
-// launch when resid is given; the folded sums go to ksum_out when it is given.
-int launch_diversity_sliced(const void* K, int rows, int C, int dtype, const float* ksum, int n_slices, float* ksum_out,
-                            float* d, const void* resid, int resid_rows, float* s_raw, cudaStream_t st) {
-  if (rows <= 0) return OVGGT_OK;
-  const int nvec = C * elem_bytes(dtype) / 16;
-  const int grid = std::min((rows + 63) / 64, 148 * 8);
-  const size_t smem = (size_t)C * 4;
-  const int norm_ctas = resid ? (resid_rows + 7) / 8 : 0;
-  if (dtype == kBF16)
-    k_diversity<kBF16><<<grid + norm_ctas, 256, smem, st>>>((const uint4*)K, rows, nvec, ksum, n_slices, ksum_out, d,
-                                                            grid, (const uint4*)resid, resid_rows, s_raw);
-  else
-    k_diversity<kF32><<<grid + norm_ctas, 256, smem, st>>>((const uint4*)K, rows, nvec, ksum, n_slices, ksum_out, d,
-                                                           grid, (const uint4*)resid, resid_rows, s_raw);
   LAUNCHED();
   return OVGGT_OK;
 }
@@ -199,6 +113,35 @@ int launch_colsum(const void* K, int rows, int C, int dtype, float* part, float*
   k_colsum_final<<<(C + 31) / 32, 1024, 0, st>>>(part, parts, C, ksum);
   LAUNCHED();
   return OVGGT_OK;
+}
+
+// One launch for whatever A asks for: append, diversity, residual norms.  Two CTAs per SM, fewer when there are fewer
+// than eight items a CTA.
+int launch_front(const FrontArgs& A, int C, int dtype, cudaStream_t st) {
+  const int nvec = C * elem_bytes(dtype) / 16;
+  const long items = (long)A.M + (A.ksum ? front_score_items(A.n) : 0) + (A.resid ? front_score_items(A.M) : 0);
+  if (items == 0) return OVGGT_OK;
+  const int grid = (int)std::min<long>((items + kFrontThreads / 32 - 1) / (kFrontThreads / 32), 148 * 2);
+  const size_t smem = (size_t)C * 4;
+  const auto kernel = dtype == kBF16 ? k_front<kBF16> : k_front<kF32>;
+  static std::atomic<uint64_t> smem_set[2];
+  CK(allow_smem(kernel, std::max<size_t>(smem, 48 * 1024), smem_set[dtype == kBF16 ? 1 : 0], false));
+  CK(launch_dependent(kernel, dim3(grid), kFrontThreads, 1, smem, st, true, A, nvec));
+  g_launches.fetch_add(1);
+  return OVGGT_OK;
+}
+
+// d of all rows of K against their own column sums.  part: [colsum_parts(rows), C] floats; ksum: [C] floats.
+int launch_diversity(const void* K, int rows, int C, int dtype, float* part, float* ksum, float* d, cudaStream_t st) {
+  if (rows <= 0) return OVGGT_OK;
+  int rc = launch_colsum(K, rows, C, dtype, part, ksum, st);
+  if (rc) return rc;
+  FrontArgs A = {};
+  A.n = rows;
+  A.k_cache = static_cast<uint4*>(const_cast<void*>(K));     // (read only: nothing is appended)
+  A.ksum = ksum;
+  A.d = d;
+  return launch_front(A, C, dtype, st);
 }
 
 // Supp. D, attention-weight criterion: s[j] = mean over the M queries and the heads of the attention key j of the
@@ -230,46 +173,27 @@ int launch_qk_scores(const void* q, const void* k, int M, int C, int n_heads, in
   return OVGGT_OK;
 }
 
-// The hole-filling move (and, with delta, what it does to the key column sums).
+// The hole-filling moves by themselves.
 int launch_fill_holes(void* kc, void* vc, const int* msrc, const int* mdst, const int* mj, const int* n_moves, int max_moves,
-                      int C, int dtype, int* slot_meta, float* delta, cudaStream_t st, int rows_cap, int n_meta,
-                      int* status) {
+                      int C, int dtype, int* slot_meta, cudaStream_t st, int rows_cap, int n_meta, int* status) {
   const int nvec = C * elem_bytes(dtype) / 16;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kFillSlices * kFillClusterCtas);
-  cfg.blockDim = dim3(kFillThreads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kFillClusterCtas;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  cudaError_t e;
-  if (dtype == kBF16)
-    e = cudaLaunchKernelEx(&cfg, k_fill_holes<kBF16>, (uint4*)kc, (uint4*)vc, msrc, mdst, mj, n_moves, max_moves, nvec,
-                           slot_meta, delta, rows_cap, n_meta, status);
-  else
-    e = cudaLaunchKernelEx(&cfg, k_fill_holes<kF32>, (uint4*)kc, (uint4*)vc, msrc, mdst, mj, n_moves, max_moves, nvec,
-                           slot_meta, delta, rows_cap, n_meta, status);
-  if (e != cudaSuccess) return cuda_fail(e);
+  k_fill_holes<<<std::min((max_moves + 7) / 8, 148 * 4), 256, 0, st>>>((uint4*)kc, (uint4*)vc, msrc, mdst, mj, n_moves,
+                                                                      max_moves, nvec, slot_meta, rows_cap, n_meta, status);
   LAUNCHED();
   return OVGGT_OK;
 }
 
 int launch_attention(const void* q, const void* k, const void* v, int M, int N, int H, int dtype, void* out,
                      void* scratch, int* status, cudaStream_t st, AttnKvMaps* maps = nullptr,
-                     const float* kmax2 = nullptr, float* lse = nullptr) {
+                     const float* kmax2 = nullptr, float* lse = nullptr, bool beside_previous = false) {
   if (dtype == kBF16) {
-    int rc = attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, 0, kmax2, lse);
+    int rc = attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, 0, kmax2, lse, beside_previous);
     if (rc == OVGGT_OK) g_launches.fetch_add(attn_tcgen05_num_launches(M, N, H));
     if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
     return rc;
   }
   int launches = 0;
-  const int rc = attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, &launches);
+  const int rc = attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, &launches);
   g_launches.fetch_add(launches);
   if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
   return rc;
@@ -302,19 +226,19 @@ struct LayerState {
   float *s_raw, *d, *r;
   int* surv;
   int* n_keep_dev;
-  float* colsum_part = nullptr;   // stable layout: [148 * 8, C] per-CTA column sums of the keys the last compaction wrote
-  int colsum_nparts = 0;          // 0: not available (the next step sums the keys itself)
+  int *move_src = nullptr, *move_dst = nullptr, *n_moves_dev = nullptr;   // rows that come and rows that go
   // hole-filling layout
-  int *move_src = nullptr, *move_dst = nullptr, *move_j = nullptr, *tail_move = nullptr, *n_moves_dev = nullptr;
+  int *move_j = nullptr, *tail_move = nullptr;
+  int* hole_stamp = nullptr;      // [B + M] stamp of the last compress that left a move into the slot
+  int stamp = 0;
   bool moves_pending = false;     // the last compress left moves that the next append (or a flush) carries out
-  float* moves_delta = nullptr;   // where that move leaves its corrections of the key column sums, or nullptr
-  float* ksum[2] = {nullptr, nullptr};   // [1 + kFillSlices, C]: the key column sums a step uses, then the move's corrections
-  int kcur = 0;                   // which of the two the next diversity launch reads
-  bool ksum_valid = false;        // ksum[kcur] describes the cached keys (else: recompute)
+  float* ksum[2] = {nullptr, nullptr};   // [C]: column sums of the cached keys; a compress writes the next ones to the other
+  int kcur = 0;                   // which of the two describes the cached keys
+  bool ksum_valid = false;        // it does (else: recompute)
   int since_refresh = 0;
   float* kmax2 = nullptr;         // [n_heads] running upper bound of the squared per-head key norms (bf16 caches)
   AttnKvMaps maps[2];             // tensor maps of the K/V buffers, re-encoded only when the row count changes
-  int64_t scores_frame = -1;      // frame whose s_raw and d were already enqueued on the side stream
+  int64_t norms_frame = -1;       // frame whose residual norms the front launch already took
   size_t kv_bytes = 0;
 };
 
@@ -330,11 +254,12 @@ struct ovggt_cache {
   bool decided_register = false;
   int64_t decided_demote = -1;
   // shared scratch
-  float *colsum_part = nullptr, *ksum = nullptr;
+  float* colsum_part = nullptr;
   float *qk_part = nullptr, *qk_sum = nullptr;       // OVGGT_SCORE_QK: column sums of the frame's queries
   float *attn_lse = nullptr, *attn_part = nullptr;   // OVGGT_SCORE_ATTN: log2 softmax denominators [M, H], per-head sums [H, M]
   void* attn_scratch = nullptr;
   int* status = nullptr;
+  size_t zeroed_bytes = 0;                           // the status block and the key-norm bounds behind it
   // two sets of staging buffers for ovggt_layer_step_host: the copies of one step overlap the kernels of the step before
   char *stage_q[2] = {}, *stage_k[2] = {}, *stage_v[2] = {}, *stage_r[2] = {}, *stage_o[2] = {};
   float* stage_conf[2] = {};
@@ -426,7 +351,7 @@ bool config_ok(const ovggt_config* c, int* err) {
     }
     if ((int64_t)c->budget[l] + M > (1 << 30)) return false;
     // the fused selection kernel keeps all B + M candidates of a layer in the shared memory of one cluster
-    const int N = c->budget[l] + (int)M, ncta = select_cluster_ctas(N);
+    const int N = c->budget[l] + (int)M, ncta = compress_ctas(N, (int)M);
     if (compress_smem_bytes((N + ncta - 1) / ncta, c->grid_h * c->grid_w, (int)M) > kSmemLimit) {
       *err = OVGGT_ERR_UNSUPPORTED;
       return false;
@@ -461,14 +386,13 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
     off[i++] = L.take(R * 4);           // r
     off[i++] = L.take(R * 4);           // survivors
     off[i++] = L.take(64);              // n_keep, n_moves
-    off[i++] = L.take((size_t)c->n_heads * 4);   // bound of the key norms
     if (fill) {
       for (int b = 0; b < 2; ++b) off[i++] = L.take(R * 4);                                  // slots
-      for (int b = 0; b < 4; ++b) off[i++] = L.take((size_t)M * 4);                          // move lists
-      for (int b = 0; b < 2; ++b) off[i++] = L.take((size_t)(1 + kFillSlices) * C * 4);      // column sums + corrections
-    } else {
-      off[i++] = L.take((size_t)148 * 8 * C * 4);   // column-sum partials of the compaction
+      for (int b = 0; b < 2; ++b) off[i++] = L.take((size_t)M * 4);                          // move_j, tail_move
+      off[i++] = L.take(R * 4);                                                              // hole stamps
     }
+    for (int b = 0; b < 2; ++b) off[i++] = L.take((size_t)M * 4);                            // move_src, move_dst
+    for (int b = 0; b < 2; ++b) off[i++] = L.take((size_t)C * 4);                            // column sums
     if (h) {
       LayerState& S = h->layers[l];
       i = 0;
@@ -484,25 +408,23 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
       S.surv = reinterpret_cast<int*>(base + off[i++]);
       S.n_keep_dev = reinterpret_cast<int*>(base + off[i++]);
       S.n_moves_dev = S.n_keep_dev + 4;
-      S.kmax2 = reinterpret_cast<float*>(base + off[i++]);
       if (fill) {
         for (int b = 0; b < 2; ++b) S.slot[b] = reinterpret_cast<int*>(base + off[i++]);
-        S.move_src = reinterpret_cast<int*>(base + off[i++]);
-        S.move_dst = reinterpret_cast<int*>(base + off[i++]);
         S.move_j = reinterpret_cast<int*>(base + off[i++]);
         S.tail_move = reinterpret_cast<int*>(base + off[i++]);
-        for (int b = 0; b < 2; ++b) S.ksum[b] = reinterpret_cast<float*>(base + off[i++]);
-      } else {
-        S.colsum_part = reinterpret_cast<float*>(base + off[i++]);
+        S.hole_stamp = reinterpret_cast<int*>(base + off[i++]);
       }
+      S.move_src = reinterpret_cast<int*>(base + off[i++]);
+      S.move_dst = reinterpret_cast<int*>(base + off[i++]);
+      for (int b = 0; b < 2; ++b) S.ksum[b] = reinterpret_cast<float*>(base + off[i++]);
       S.budget = c->budget[l];
       S.kv_bytes = 2 * (size_t)nkv * R * C * eb;
     }
   }
   const size_t o_part = L.take((size_t)kMaxColsumParts * C * 4);
-  const size_t o_ksum = L.take(colsum_scratch_bytes(C));
   const size_t o_attn = L.take(ovggt_k_attention_scratch_bytes(M, max_rows, c->n_heads));
-  const size_t o_status = L.take(64);
+  // what starts at zero lies together: the status word, then every layer's bound of the key norms
+  const size_t o_status = L.take(64 + (size_t)c->n_layers * c->n_heads * 4);
   const bool qk = c->score_mode == OVGGT_SCORE_QK;
   const size_t o_qk = qk ? L.take((size_t)(colsum_parts(M) + 1) * C * 4) : 0;
   const bool aw = c->score_mode == OVGGT_SCORE_ATTN;
@@ -514,9 +436,11 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
   }
   if (h) {
     h->colsum_part = reinterpret_cast<float*>(base + o_part);
-    h->ksum = reinterpret_cast<float*>(base + o_ksum);
     h->attn_scratch = base + o_attn;
     h->status = reinterpret_cast<int*>(base + o_status);
+    h->zeroed_bytes = 64 + (size_t)c->n_layers * c->n_heads * 4;
+    for (int l = 0; l < c->n_layers; ++l)
+      h->layers[l].kmax2 = reinterpret_cast<float*>(base + o_status + 64) + (size_t)l * c->n_heads;
     if (aw) {
       h->attn_lse = reinterpret_cast<float*>(base + o_aw);
       h->attn_part = h->attn_lse + (size_t)M * c->n_heads;
@@ -617,11 +541,10 @@ extern "C" int ovggt_cache_create(const ovggt_config* cfg, ovggt_cache** out) {
       (void)cudaGetLastError();
     }
   }
-  cudaError_t e = cudaMemset(h->status, 0, 64);
-  if (e == cudaSuccess) e = cudaMemset(h->ksum, 0, colsum_scratch_bytes(h->C));   // (its arrival counters)
-  for (LayerState& S : h->layers)
-    if (e == cudaSuccess) e = cudaMemset(S.kmax2, 0, (size_t)cfg->n_heads * 4);
-
+  cudaError_t e = cudaMemset(h->status, 0, h->zeroed_bytes);
+  for (LayerState& S : h->layers) {
+    if (e == cudaSuccess && S.hole_stamp) e = cudaMemset(S.hole_stamp, 0, ((size_t)S.budget + h->M) * 4);
+  }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     delete h;
@@ -684,82 +607,79 @@ int flush_moves(ovggt_cache* h, LayerState& S, cudaStream_t st) {
   if (!S.moves_pending) return OVGGT_OK;
   ProfScope ps(h, OVGGT_PROF_COMPACT, st);
   int rc = launch_fill_holes(S.kbuf[S.kv], S.vbuf[S.kv], S.move_src, S.move_dst, S.move_j, S.n_moves_dev, h->M, h->C,
-                             h->cfg.dtype, S.slot[S.cur], S.moves_delta, st, S.budget + h->M, S.budget, h->status);
+                             h->cfg.dtype, S.slot[S.cur], st, S.budget + h->M, S.budget, h->status);
   if (rc) return rc;
   S.moves_pending = false;
-  S.moves_delta = nullptr;
   return OVGGT_OK;
 }
 
-// Eq. 2: the append itself; in the hole-filling layout the same launch first carries out the moves the previous
-// compress left (they empty exactly the slots the new frame goes into).
-int enqueue_append(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st) {
+// The front of a step, one launch: the append (Eq. 2; in the hole-filling layout with the moves the previous compress
+// left, which empty exactly the slots the new frame goes into), the diversity of the cached rows (Sec. 3.2), which
+// depends on nothing the frame brings, and with_norms the residual norms of the new rows (Eq. 5).
+int enqueue_front(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, bool with_norms, cudaStream_t st) {
   int rc = validate_attend(h, layer, io);
   if (rc) return rc;
   LayerState& S = h->layers[layer];
   h->last_stream = st;
-  const int M = h->M, C = h->C, nvec = C * h->elem / 16, b = S.cur, kb = S.kv;
-  ProfScope ps(h, OVGGT_PROF_APPEND, st);
-  if (!fill_layout(h)) {
-    const int grid = std::min((2 * M + 7) / 8, 148 * 8);
-    k_append<<<grid, 256, 0, st>>>((const uint4*)io->k, (const uint4*)io->v, M, nvec, S.n, (long long)io->frame_id,
-                                   (uint4*)S.kbuf[kb], (uint4*)S.vbuf[kb], S.ids[b], S.flags[b], S.stored[b], S.slot[b],
-                                   key_norm_bound(h, S));
-    LAUNCHED();
-    return OVGGT_OK;
+  const int M = h->M, C = h->C, b = S.cur, kb = S.kv;
+  const bool diversity = ranks_by_diversity(h->cfg.score_mode) && S.n > 0;
+  if (diversity && (!S.ksum_valid || S.since_refresh >= kColsumRefreshEvery)) {
+    // Column sums of the cached keys afresh: after an import or the step that filled the cache up, and every
+    // kColsumRefreshEvery-th step; otherwise each compress continues them.
+    rc = flush_moves(h, S, st);
+    if (rc) return rc;
+    ProfScope ps(h, OVGGT_PROF_DIVERSITY, st);
+    rc = launch_colsum(S.kbuf[kb], S.n, C, h->cfg.dtype, h->colsum_part, S.ksum[S.kcur], st);
+    if (rc) return rc;
+    S.ksum_valid = true;
+    S.since_refresh = 0;
   }
-  AppendFillArgs A;
+  ProfScope ps(h, OVGGT_PROF_APPEND, st);
+  FrontArgs A = {};
   A.k_new = (const uint4*)io->k; A.v_new = (const uint4*)io->v;
   A.M = M; A.n = S.n; A.frame_id = (long long)io->frame_id;
   A.k_cache = (uint4*)S.kbuf[kb]; A.v_cache = (uint4*)S.vbuf[kb];
   A.ids = S.ids[b]; A.flags = S.flags[b]; A.stored = S.stored[b]; A.slot = S.slot[b];
   A.kmax2 = key_norm_bound(h, S);
   A.B = S.budget;
-  const bool pending = S.moves_pending;
-  A.tail_move = pending ? S.tail_move : nullptr;
-  A.move_dst = S.move_dst; A.move_j = S.move_j; A.n_moves_ptr = S.n_moves_dev;
-  A.delta = pending ? S.moves_delta : nullptr;
+  if (S.moves_pending) {
+    A.tail_move = S.tail_move; A.move_dst = S.move_dst; A.move_j = S.move_j; A.n_moves_ptr = S.n_moves_dev;
+    A.hole_stamp = S.hole_stamp; A.stamp = S.stamp;
+  }
+  if (diversity) { A.ksum = S.ksum[S.kcur]; A.d = S.d; }
+  if (with_norms) { A.resid = (const uint4*)io->resid; A.s_raw = S.s_raw; }
   A.status = h->status;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kFillSlices * kFillClusterCtas);
-  cfg.blockDim = dim3(kAppendFillThreads);
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kFillClusterCtas;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = h->cfg.dtype == kBF16 ? cudaLaunchKernelEx(&cfg, k_append_fill<kBF16>, A, nvec)
-                                        : cudaLaunchKernelEx(&cfg, k_append_fill<kF32>, A, nvec);
-  if (e != cudaSuccess) return cuda_fail(e);
-  LAUNCHED();
+  rc = launch_front(A, C, h->cfg.dtype, st);
+  if (rc) return rc;
   S.moves_pending = false;
-  S.moves_delta = nullptr;
+  S.norms_frame = with_norms ? io->frame_id : -1;
   return OVGGT_OK;
 }
 
 // The attention over all n + M rows, and the bookkeeping that closes the attend half.  Attention does not care in
 // which order the cached rows lie, so it reads the K/V buffer front to back in either layout.
-int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st) {
+// beside_previous: what was enqueued on st just before is the same step's selection, which the attention does not wait for.
+int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st, int N, int kb,
+                      bool beside_previous = false) {
   LayerState& S = h->layers[layer];
-  const int kb = S.kv;
   int rc;
   {
     ProfScope ps(h, OVGGT_PROF_ATTENTION, st);
-    rc = launch_attention(io->q, S.kbuf[kb], S.vbuf[kb], h->M, S.n + h->M, h->cfg.n_heads, h->cfg.dtype, io->out,
+    rc = launch_attention(io->q, S.kbuf[kb], S.vbuf[kb], h->M, N, h->cfg.n_heads, h->cfg.dtype, io->out,
                           h->attn_scratch, h->status, st, &S.maps[kb], key_norm_bound(h, S),
-                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr);
+                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous);
   }
-  if (rc) return rc;
+  return rc;
+}
+
+// The bookkeeping that closes the attend half.
+void close_attend(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
   if (h->first_frame < 0) {
     h->first_frame = io->frame_id;
     h->last_registration = io->frame_id;   // the first frame is the initial anchor
   }
   S.pending = true;
   S.pending_frame = io->frame_id;
-  return OVGGT_OK;
 }
 
 // Query-key mode (Supp. D): the criterion of the new frame's rows, from the frame's own q and k; kept in the layer's
@@ -779,51 +699,6 @@ int enqueue_received_scores(ovggt_cache* h, LayerState& S, const ovggt_frame_io*
                                    S.s_raw, st);
 }
 
-// Eq. 5 and the diversity score of Sec. 3.2 for the frame io describes: everything the selection needs that does not
-// depend on the anchor decision.  Reads the cached keys [0, n) and the frame's residual, so it may run before the
-// frame's K/V are appended.
-int enqueue_scores(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io, cudaStream_t st) {
-  const ovggt_config& c = h->cfg;
-  const int M = h->M, C = h->C, n = S.n, kb = S.kv;
-  const bool hybrid = ranks_by_diversity(c.score_mode) && n > 0;
-  // query-key and attention-weight modes: s_raw was written by the attend half; the residual is not read
-  const void* resid = scored_at_attend(c.score_mode) ? nullptr : io->resid;
-  int rc = OVGGT_OK;
-  if (!hybrid) {
-    if (!resid) return OVGGT_OK;
-    ProfScope ps(h, OVGGT_PROF_ROW_NORMS, st);
-    return launch_row_norms(resid, M, C, c.dtype, S.s_raw, st);
-  }
-  if (fill_layout(h)) {
-    // Column sums of the cached keys: continued from the last step's sums and the corrections its move left, or
-    // summed afresh (first steps, after an import, every kColsumRefreshEvery-th step); the residual norms ride in
-    // the diversity launch either way.
-    ProfScope ps(h, OVGGT_PROF_DIVERSITY, st);
-    const bool fresh = !S.ksum_valid || S.since_refresh >= kColsumRefreshEvery;
-    if (fresh) {
-      rc = launch_colsum(S.kbuf[kb], n, C, c.dtype, h->colsum_part, S.ksum[S.kcur], st);
-      if (rc) return rc;
-      S.since_refresh = 0;
-    } else {
-      S.since_refresh += 1;
-    }
-    return launch_diversity_sliced(S.kbuf[kb], n, C, c.dtype, S.ksum[S.kcur], fresh ? 1 : 1 + kFillSlices,
-                                   S.ksum[S.kcur ^ 1], S.d, resid, M, S.s_raw, st);
-  }
-  if (S.colsum_nparts > 0) {   // stable layout, sums left by the last compaction
-    ProfScope ps(h, OVGGT_PROF_DIVERSITY, st);
-    return launch_diversity_from_parts(S.kbuf[kb], n, C, c.dtype, S.colsum_part, S.colsum_nparts, h->ksum, S.d,
-                                       resid, M, S.s_raw, st);
-  }
-  if (resid) {
-    ProfScope ps(h, OVGGT_PROF_ROW_NORMS, st);
-    rc = launch_row_norms(resid, M, C, c.dtype, S.s_raw, st);
-  }
-  if (rc) return rc;
-  ProfScope ps(h, OVGGT_PROF_DIVERSITY, st);
-  return launch_diversity(S.kbuf[kb], n, C, c.dtype, h->colsum_part, h->ksum, S.d, st);
-}
-
 // `mirrored`: the anchor decision of the frame as another handle took it (camera head, Supp. C) instead of the rule
 // of Sec. 3.3 applied to rho.
 struct MirroredDecision { bool registered; int64_t demoted_frame; };
@@ -840,7 +715,7 @@ int validate_compress(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, c
   }
   const LayerState& S = h->layers[layer];
   if (!S.pending || io->frame_id != S.pending_frame) return OVGGT_ERR_FRAME_ORDER;
-  const int N = S.n + h->M, ncta = select_cluster_ctas(N);
+  const int N = S.n + h->M, ncta = compress_ctas(N, h->M);
   if (compress_smem_bytes((N + ncta - 1) / ncta, h->Np, h->M) > kSmemLimit)
     return OVGGT_ERR_UNSUPPORTED;   // (create already refuses such budgets)
   // The anchor state belongs to the whole handle and moves forward only: a layer that comes with a frame older
@@ -883,6 +758,23 @@ void take_decision(ovggt_cache* h, const ovggt_frame_io* io, const MirroredDecis
   }
 }
 
+// Residual norms of a few rows (the camera head's one) are taken inside the selection kernel: a launch costs more.
+constexpr int kNormsInsideRows = 64;
+bool norms_pending(const ovggt_cache* h, const LayerState& S, const ovggt_frame_io* io) {
+  return !scored_at_attend(h->cfg.score_mode) && S.norms_frame != io->frame_id;
+}
+bool norms_inside(const ovggt_cache* h, const LayerState& S, const ovggt_frame_io* io) {
+  return norms_pending(h, S, io) && h->M <= kNormsInsideRows;
+}
+
+// Does the compress of the pending frame leave the column sums of the keys that stay?  It knows the rows that come and
+// go as move lists, which name exactly those unless the cache of the hole-filling layout fills up in this very step
+// (rows of the frame then already lie below slot B); the sums are taken afresh after that one.
+bool continues_sums(const ovggt_cache* h, const LayerState& S) {
+  return ranks_by_diversity(h->cfg.score_mode) &&
+         !(h->cfg.compaction == OVGGT_COMPACT_FILL_HOLES && S.n + h->M > S.budget && S.n < S.budget);
+}
+
 // Parameter block of the fused selection kernel for the layer's pending frame.
 CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
   const ovggt_config& c = h->cfg;
@@ -910,6 +802,13 @@ CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io
   P.slot_src = S.slot[b]; P.slot_dst = S.slot[b ^ 1];
   P.move_src = S.move_src; P.move_dst = S.move_dst; P.move_j = S.move_j; P.tail_move = S.tail_move;
   P.n_moves_out = S.n_moves_dev;
+  P.hole_stamp = S.hole_stamp; P.stamp = ++S.stamp;
+  // the norms: already taken by the front launch, by a launch of their own, or (a few rows) inside the selection
+  P.resid = norms_inside(h, S, io) ? static_cast<const uint4*>(io->resid) : nullptr;
+  P.k_cache = reinterpret_cast<const uint4*>(S.kbuf[S.kv]);
+  P.nvec = h->C * h->elem / 16;
+  P.ksum = S.n > 0 ? S.ksum[S.kcur] : nullptr;
+  P.ksum_next = continues_sums(h, S) ? S.ksum[S.kcur ^ 1] : nullptr;
   return P;
 }
 
@@ -917,6 +816,13 @@ CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io
 void close_compress(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
   const ovggt_config& c = h->cfg;
   const int N = S.n + h->M, n_keep = std::min(N, S.budget);
+  S.ksum_valid = continues_sums(h, S);
+  if (S.ksum_valid) S.kcur ^= 1;
+  S.since_refresh += 1;
+  // Some rows leave: the survivors above slot B have to move into the slots that open below it.  The selection kernel has
+  // left the pairs; the next append of this layer carries them out (flush_moves for other readers).
+  if (c.compaction == OVGGT_COMPACT_FILL_HOLES && N > S.budget) S.moves_pending = true;
+  S.norms_frame = -1;
   const int per_anchor = c.camera_head ? 1 : c.anchor_tokens;
   if (io->frame_id == h->first_frame && c.protect_first_frame) S.n_prot_init = h->M;
   if (h->decided_register) S.n_prot_hist += per_anchor;
@@ -930,71 +836,43 @@ void close_compress(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
   S.frames_seen += 1;
 }
 
-// Does the hole-filling move of this step also leave corrections of the key column sums?  They continue the sums the
-// step's diversity launch used and wrote to ksum[kcur ^ 1], and describe the next cache only if every slot below B
-// held a cached row (n == B: steady state).
-bool move_leaves_corrections(const ovggt_cache* h, const LayerState& S) {
-  return ranks_by_diversity(h->cfg.score_mode) && h->C * h->elem / 16 <= kCompactSumMaxVec && S.n == S.budget;
-}
-
 // The compress half on stream st.  The stable gather writes another buffer, so the whole half may run beside an
-// attention that still reads this one; the hole-filling moves are only recorded here (see enqueue_append).
+// attention that still reads this one; the hole-filling moves are only recorded here (see enqueue_front).
 int compress_impl(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st_sel,
                   const MirroredDecision* mirrored = nullptr) {
-  const cudaStream_t st_move = st_sel;
   int rc = validate_compress(h, layer, io, mirrored);
   if (rc) return rc;
   LayerState& S = h->layers[layer];
   const ovggt_config& c = h->cfg;
-  const int M = h->M, C = h->C, n = S.n, N = n + M, B = S.budget, b = S.cur, kb = S.kv;
-  const int64_t t = io->frame_id;
-  const bool fill = fill_layout(h);
+  const int M = h->M, C = h->C, N = S.n + M, B = S.budget, kb = S.kv;
   take_decision(h, io, mirrored);     // nothing below can fail on an argument any more
-  h->last_stream = st_move;
+  h->last_stream = st_sel;
 
-  const bool prelaunched = S.scores_frame == t;    // ovggt_layer_step already enqueued them on st_sel
-  S.scores_frame = -1;
-  if (!prelaunched) {
-    rc = enqueue_scores(h, S, io, st_sel);
+  if (norms_pending(h, S, io) && !norms_inside(h, S, io)) {
+    ProfScope ps(h, OVGGT_PROF_ROW_NORMS, st_sel);
+    rc = launch_row_norms(io->resid, M, C, c.dtype, S.s_raw, st_sel);
     if (rc) return rc;
   }
   const CompressParams P = select_params(h, S, io);
-  const int ncta = select_cluster_ctas(N);
+  const int ncta = compress_ctas(N, M);
   const size_t smem = compress_smem_bytes((N + ncta - 1) / ncta, h->Np, M);
-  CK(cudaFuncSetAttribute(k_compress_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
+  const auto kernel = c.dtype == kBF16 ? (ncta == 1 ? k_compress_select<kBF16, true> : k_compress_select<kBF16, false>)
+                                       : (ncta == 1 ? k_compress_select<kF32, true> : k_compress_select<kF32, false>);
+  static std::atomic<uint64_t> smem_set[4];
+  CK(allow_smem(kernel, kSmemLimit, smem_set[(c.dtype == kBF16 ? 2 : 0) + (ncta == 1 ? 1 : 0)]));
   {
     ProfScope ps(h, OVGGT_PROF_SELECT, st_sel);
-    CK(launch_cluster(k_compress_select, dim3(ncta), ncta, smem, st_sel, P));
-    LAUNCHED();
+    CK(launch_dependent(kernel, dim3(ncta), kSelectThreads, ncta, smem, st_sel, true, P));
+    g_launches.fetch_add(1);
   }
-  const int n_keep = std::min(N, B);
-  if (fill) {
-    // Some rows leave: the survivors above slot B have to move into the slots that open below it.  The selection
-    // kernel has left the pairs; the next append of this layer carries them out (flush_moves for other readers).
-    S.ksum_valid = false;
-    if (N > B) {
-      const bool delta = move_leaves_corrections(h, S);
-      S.moves_pending = true;
-      S.moves_delta = delta ? S.ksum[S.kcur ^ 1] + C : nullptr;
-      if (delta) {
-        S.kcur ^= 1;
-        S.ksum_valid = true;
-      }
-    }
-  } else {
-    ProfScope ps(h, OVGGT_PROF_COMPACT, st_move);
-    const bool fuse = ranks_by_diversity(c.score_mode) && C * h->elem / 16 <= kCompactSumMaxVec;
-    S.colsum_nparts = 0;
-    if (fuse)
-      rc = launch_compact_colsum(S.kbuf[kb], S.vbuf[kb], S.surv, n_keep, C, c.dtype, S.kbuf[kb ^ 1], S.vbuf[kb ^ 1],
-                                 S.colsum_part, &S.colsum_nparts, st_move, N, h->status);
-    else
-      rc = launch_compact(S.kbuf[kb], S.vbuf[kb], S.surv, n_keep, C, c.dtype, S.kbuf[kb ^ 1], S.vbuf[kb ^ 1], st_move, N,
-                          h->status);
+  if (!fill_layout(h)) {
+    ProfScope ps(h, OVGGT_PROF_COMPACT, st_sel);
+    rc = launch_compact(S.kbuf[kb], S.vbuf[kb], S.surv, std::min(N, B), C, c.dtype, S.kbuf[kb ^ 1], S.vbuf[kb ^ 1], st_sel,
+                        N, h->status);
     if (rc) return rc;
-    S.kv = kb ^ 1;
   }
   close_compress(h, S, io);
+  if (!fill_layout(h)) S.kv = kb ^ 1;
   return OVGGT_OK;
 }
 
@@ -1018,52 +896,27 @@ int compress_all_layers(ovggt_cache* h, const ovggt_frame_io* ios, cudaStream_t 
   take_decision(h, &ios[0], nullptr);
   h->last_stream = st;
   const int nvec = C * h->elem / 16;
-  CK(cudaFuncSetAttribute(k_compress_select_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
   for (int l0 = 0; l0 < L; l0 += kMaxBatchLayers) {
     const int cnt = std::min(kMaxBatchLayers, L - l0);
-    // ---- scores: diversity of the cached keys and the frame's residual norms
+    // ---- the frame's residual norms (the diversity of the cached rows was taken by each layer's attend half)
     {
-      ProfScope ps(h, OVGGT_PROF_DIVERSITY, st);
-      DiversityBatch db;
-      int grid_x = 1;
-      // Every CTA first folds its layer's column sums (up to 1 + 16 rows of C floats, from L2) and then streams key
-      // rows: the more rows a CTA takes the less that set-up weighs, as long as the launch still fills the machine a
-      // few times over.  (24 layers x 12288 rows, bf16: 0.57 of the copy bandwidth at 64 rows per CTA, 0.67 at 128,
-      // 0.72 at 256, 0.71 at 512.)
-      int rows_per_cta = 64;
-      {
-        long total_rows = 0;
-        for (int i = 0; i < cnt; ++i)
-          if (ranks_by_diversity(c.score_mode)) total_rows += h->layers[l0 + i].n;
-        while (rows_per_cta < 256 && total_rows / (2 * rows_per_cta) >= 148 * 4) rows_per_cta *= 2;
-      }
+      NormBatch nb = {};
+      bool any = false;
       for (int i = 0; i < cnt; ++i) {
         LayerState& S = h->layers[l0 + i];
-        S.scores_frame = -1;
-        const bool hybrid = ranks_by_diversity(c.score_mode) && S.n > 0;
-        DiversityArgs& A = db.a[i];
-        A = DiversityArgs{};
-        A.resid = scored_at_attend(c.score_mode) ? nullptr : (const uint4*)ios[l0 + i].resid;
-        A.resid_rows = M; A.s_raw = S.s_raw;
-        if (hybrid) {
-          const bool fresh = !S.ksum_valid || S.since_refresh >= kColsumRefreshEvery;
-          if (fresh) {
-            int rc = launch_colsum(S.kbuf[S.kv], S.n, C, c.dtype, h->colsum_part, S.ksum[S.kcur], st);
-            if (rc) return rc;
-            S.since_refresh = 0;
-          } else {
-            S.since_refresh += 1;
-          }
-          A.K = (const uint4*)S.kbuf[S.kv]; A.rows = S.n;
-          A.ksum = S.ksum[S.kcur]; A.n_slices = fresh ? 1 : 1 + kFillSlices; A.ksum_out = S.ksum[S.kcur ^ 1];
-          A.d = S.d;
-          A.div_ctas = std::min((S.n + rows_per_cta - 1) / rows_per_cta, 148 * 8);
+        if (norms_pending(h, S, &ios[l0 + i]) && !norms_inside(h, S, &ios[l0 + i])) {
+          nb.x[i] = (const uint4*)ios[l0 + i].resid;
+          nb.s[i] = S.s_raw;
+          any = true;
         }
-        grid_x = std::max(grid_x, A.div_ctas + (M + 7) / 8);
       }
-      if (c.dtype == kBF16) k_diversity_batched<kBF16><<<dim3(grid_x, cnt), 256, (size_t)C * 4, st>>>(db, nvec);
-      else                  k_diversity_batched<kF32><<<dim3(grid_x, cnt), 256, (size_t)C * 4, st>>>(db, nvec);
-      LAUNCHED();
+      if (any) {
+        ProfScope ps(h, OVGGT_PROF_ROW_NORMS, st);
+        const dim3 grid((M + 7) / 8, cnt);
+        if (c.dtype == kBF16) k_row_norms_batched<kBF16><<<grid, 256, 0, st>>>(nb, M, nvec);
+        else                  k_row_norms_batched<kF32><<<grid, 256, 0, st>>>(nb, M, nvec);
+        LAUNCHED();
+      }
     }
     // ---- flags, Eq. 6-8, compacted meta, move pairs: one cluster per layer
     {
@@ -1075,23 +928,14 @@ int compress_all_layers(ovggt_cache* h, const ovggt_frame_io* ios, cudaStream_t 
         cb.p[i] = select_params(h, S, &ios[l0 + i]);
         n_max = std::max(n_max, S.n + M);
       }
-      const int ncta = select_cluster_ctas(n_max);
+      const int ncta = compress_ctas(n_max, M);
+      const auto kernel =
+          c.dtype == kBF16 ? (ncta == 1 ? k_compress_select_batched<kBF16, true> : k_compress_select_batched<kBF16, false>)
+                           : (ncta == 1 ? k_compress_select_batched<kF32, true> : k_compress_select_batched<kF32, false>);
+      CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
       const size_t smem = compress_smem_bytes((n_max + ncta - 1) / ncta, h->Np, M);
-      CK(launch_cluster(k_compress_select_batched, dim3(ncta, cnt), ncta, smem, st, cb));
+      CK(launch_cluster(kernel, dim3(ncta, cnt), ncta, smem, st, cb));
       LAUNCHED();
-    }
-    // ---- the moves of the layers that evict are left to each layer's next append
-    for (int i = 0; i < cnt; ++i) {
-      LayerState& S = h->layers[l0 + i];
-      S.ksum_valid = false;
-      if (S.n + M <= S.budget) continue;
-      const bool delta = move_leaves_corrections(h, S);
-      S.moves_pending = true;
-      S.moves_delta = delta ? S.ksum[S.kcur ^ 1] + C : nullptr;
-      if (delta) {
-        S.kcur ^= 1;
-        S.ksum_valid = true;
-      }
     }
     for (int i = 0; i < cnt; ++i) close_compress(h, h->layers[l0 + i], &ios[l0 + i]);
   }
@@ -1101,11 +945,13 @@ int compress_all_layers(ovggt_cache* h, const ovggt_frame_io* ios, cudaStream_t 
 
 extern "C" int ovggt_layer_attend(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int rc = enqueue_append(h, layer, io, st);
+  int rc = enqueue_front(h, layer, io, false, st);
   if (rc) return rc;
-  rc = enqueue_attention(h, layer, io, st);
+  LayerState& S = h->layers[layer];
+  rc = enqueue_attention(h, layer, io, st, S.n + h->M, S.kv);
   if (rc) return rc;
-  rc = enqueue_qk_scores(h, h->layers[layer], io, st);
+  close_attend(h, S, io);
+  rc = enqueue_qk_scores(h, S, io, st);
   if (rc) return rc;
   return enqueue_received_scores(h, h->layers[layer], io, st);
 }
@@ -1151,35 +997,46 @@ extern "C" int ovggt_layer_step(ovggt_cache* h, int32_t layer, const ovggt_frame
     if (rc) return rc;
     return ovggt_layer_compress(h, layer, io, stream);
   }
-  // Scoring and selection (Eq. 5-8) read the cache and the new rows but not the attention's output, so they run on
-  // the handle's second, higher-priority stream beside the attention:
-  //   stream:  append (+ the previous step's moves) . fork ... attention ........................ join
-  //   side:                                            scores, selection [, stable gather] ....../
-  // The stable gather writes the other K/V buffer.  The hole-filling moves would write the buffer the attention
-  // reads; they wait for the next append of the layer, which has to touch the same slots anyway.
+  // The selection (Eq. 6-8) reads the scores and, for the key sums, rows of the cache, but not the attention's output, so
+  // the two run side by side.  The selection goes first: it is one small cluster, and once the attention holds every SM
+  // it would wait for the first of its CTAs to end.
+  //   hole filling:  stream: front, selection, attention.  The attention is launched programmatically behind the selection
+  //                  and starts when that has started; its moves wait for the layer's next append, which has to touch
+  //                  the same slots anyway (the attention reads the buffer they would write).
+  //   stable gather: stream: front, fork, selection, gather, join.  side: attention.  The gather writes the other buffer.
+  // The query-key scores need only the frame itself: they run on the second stream beside the front.
   rc = validate_attend(h, layer, io);
   if (rc) return rc;
   LayerState& S = h->layers[layer];
-  rc = enqueue_append(h, layer, io, st);
-  if (rc) return rc;
-  CK(cudaEventRecord(h->ev_fork, st));
-  CK(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-  rc = enqueue_qk_scores(h, S, io, h->side);
-  if (rc == OVGGT_OK) rc = enqueue_scores(h, S, io, h->side);
-  if (rc == OVGGT_OK) {
-    S.scores_frame = io->frame_id;
-    rc = enqueue_attention(h, layer, io, st);
+  const int N = S.n + h->M, kb = S.kv;
+  const bool qk = h->cfg.score_mode == OVGGT_SCORE_QK, stable = !fill_layout(h);
+  if (qk) {
+    CK(cudaEventRecord(h->ev_fork, st));
+    CK(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+    rc = enqueue_qk_scores(h, S, io, h->side);
+    const cudaError_t e = cudaEventRecord(h->ev_join, h->side);
+    if (e != cudaSuccess) return cuda_fail(e);
   }
-  if (rc == OVGGT_OK) rc = compress_impl(h, layer, io, h->side);
-  // join: whatever happened, the caller's stream is ordered after the side work
-  S.scores_frame = -1;
-  h->last_stream = st;
-  cudaError_t e1 = cudaEventRecord(h->ev_join, h->side);
-  cudaError_t e2 = cudaStreamWaitEvent(st, h->ev_join, 0);
+  if (rc == OVGGT_OK) rc = enqueue_front(h, layer, io, !scored_at_attend(h->cfg.score_mode), st);
+  if (qk) CK(cudaStreamWaitEvent(st, h->ev_join, 0));
   if (rc) return rc;
-  if (e1 != cudaSuccess) return cuda_fail(e1);
-  if (e2 != cudaSuccess) return cuda_fail(e2);
-  return OVGGT_OK;
+  if (stable) {
+    CK(cudaEventRecord(h->ev_fork, st));
+    CK(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+  }
+  close_attend(h, S, io);
+  rc = compress_impl(h, layer, io, st);
+  // (a compress that is refused, as for a frame older than the last anchor decision, leaves the frame attended)
+  const int ra = enqueue_attention(h, layer, io, stable ? h->side : st, N, kb, !stable && rc == OVGGT_OK);
+  if (rc == OVGGT_OK) rc = ra;
+  h->last_stream = st;
+  if (stable) {   // whatever happened, the caller's stream is ordered after the side work
+    const cudaError_t e1 = cudaEventRecord(h->ev_join, h->side);
+    const cudaError_t e2 = cudaStreamWaitEvent(st, h->ev_join, 0);
+    if (rc == OVGGT_OK && e1 != cudaSuccess) rc = cuda_fail(e1);
+    if (rc == OVGGT_OK && e2 != cudaSuccess) rc = cuda_fail(e2);
+  }
+  return rc;
 }
 
 extern "C" int ovggt_cache_set_key_bound(ovggt_cache* h, int32_t enable) {
@@ -1370,10 +1227,9 @@ extern "C" int ovggt_cache_import(ovggt_cache* h, int32_t layer, const int64_t* 
     CK(cudaDeviceSynchronize());
   }
   S.n = n;
-  S.colsum_nparts = 0;          // the imported keys have not been summed
-  S.ksum_valid = false;
+  S.ksum_valid = false;         // the imported keys have not been summed
   S.moves_pending = false;      // (whatever was pending concerned rows that are gone)
-  S.moves_delta = nullptr;
+  S.norms_frame = -1;
   S.pending = false;
   S.n_prot_init = n_init;
   S.n_prot_hist = n_hist;
@@ -1390,8 +1246,10 @@ extern "C" int ovggt_cache_import(ovggt_cache* h, int32_t layer, const int64_t* 
 
 extern "C" int ovggt_cache_reset(ovggt_cache* h) {
   if (!h) return OVGGT_ERR_INVALID_ARG;
+  // (the second stream's work is joined into the caller's before a call returns, and the next call may come on another
+  // stream: hence the wait)
+  CK(cudaMemsetAsync(h->status, 0, h->zeroed_bytes, h->last_stream));
   CK(cudaStreamSynchronize(h->last_stream));
-  if (h->side) CK(cudaStreamSynchronize(h->side));
   for (LayerState& S : h->layers) {
     S.n = 0;
     S.cur = 0;
@@ -1400,19 +1258,15 @@ extern "C" int ovggt_cache_reset(ovggt_cache* h) {
     S.pending_frame = -1;
     S.n_prot_init = S.n_prot_hist = 0;
     S.last_N = S.last_keep = 0;
-    S.colsum_nparts = 0;
     S.ksum_valid = false;
     S.moves_pending = false;
-    S.moves_delta = nullptr;
     S.since_refresh = 0;
-    S.scores_frame = -1;
-    CK(cudaMemset(S.kmax2, 0, (size_t)h->cfg.n_heads * 4));
+    S.norms_frame = -1;
   }
   h->anchors.clear();
   h->first_frame = h->last_registration = h->decided_frame = -1;
   h->decided_register = false;
   h->decided_demote = -1;
-  CK(cudaMemset(h->status, 0, 64));
   return OVGGT_OK;
 }
 
@@ -1535,11 +1389,12 @@ extern "C" int ovggt_k_select(const float* r, const uint8_t* flags, int32_t N, i
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int* status = reinterpret_cast<int*>(scratch);
   const int ncta = select_cluster_ctas(N);
-  const size_t smem = select_smem_bytes((N + ncta - 1) / ncta, 0);
+  const size_t smem = select_smem_bytes((N + ncta - 1) / ncta);
   if (smem > kSmemLimit) return OVGGT_ERR_UNSUPPORTED;
-  CK(cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
+  const auto kernel = ncta == 1 ? k_select<true> : k_select<false>;
+  CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
   CK(cudaMemsetAsync(status, 0, 4, st));
-  CK(launch_cluster(k_select, dim3(ncta, batch), ncta, smem, st, r, flags, (int)N, (int)B, (int*)survivors, status));
+  CK(launch_cluster(kernel, dim3(ncta, batch), ncta, smem, st, r, flags, (int)N, (int)B, (int*)survivors, status));
   LAUNCHED();
   return OVGGT_OK;
 }

@@ -1,4 +1,4 @@
-// Scoring kernels: residual norms (Eq. 5), key column sums and key diversity (Sec. 3.2).
+// Scoring kernels: residual norms (Eq. 5), key column sums, the criteria of the scoring probe (Supp. D).
 // All of them stream rows of [rows, C] once with 16-byte loads and accumulate in fp32 in an
 // order that depends only on the shapes, so results are reproducible run to run.
 #pragma once
@@ -120,190 +120,64 @@ __global__ void __launch_bounds__(1024) k_colsum_final(const float* __restrict__
   }
 }
 
-// Stage 2 for many partials (the compaction kernel leaves one per CTA): CTA (x, y) folds the partials
-// p = y, y + gridDim.y, ... of its 32 columns into slice y; the CTA of a column block that finishes last folds the
-// gridDim.y slices, in slice order, into ksum.  arrived: one counter per column block, zero before and after.
-__global__ void __launch_bounds__(1024) k_colsum_final_sliced(const float* __restrict__ part, int nparts, int C,
-                                                              float* __restrict__ ksum_slices,
-                                                              float* __restrict__ ksum, int* __restrict__ arrived) {
-  __shared__ float sh[32][33];
-  __shared__ int is_last;
-  const int cx = threadIdx.x & 31, py = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + cx;
-  float acc = 0.0f;
-  if (c < C) {
-#pragma unroll 8
-    for (int p = blockIdx.y + py * gridDim.y; p < nparts; p += 32 * gridDim.y) acc += part[(size_t)p * C + c];
-  }
-  sh[py][cx] = acc;
-  __syncthreads();
-  if (py == 0 && c < C) {
-    float t = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) t += sh[i][cx];
-    ksum_slices[(size_t)blockIdx.y * C + c] = t;
-    __threadfence();
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int old = atomicAdd(&arrived[blockIdx.x], 1);
-    is_last = old == (int)gridDim.y - 1;
-    if (is_last) arrived[blockIdx.x] = 0;
-  }
-  __syncthreads();
-  if (is_last && py == 0 && c < C) {
-    __threadfence();
-    float t = 0.0f;
-    for (int y = 0; y < (int)gridDim.y; ++y) t += __ldcg(&ksum_slices[(size_t)y * C + c]);
-    ksum[c] = t;
-  }
-}
-
-// d[row] = 1 - (k_row . ksum) / (|k_row| |ksum|); the cosine with the centroid equals the cosine
-// with the column sum.  ksum is given as n_slices rows of C floats that every CTA adds up in row order (one row: the
-// sums themselves; more: a base row plus corrections, as the hole-filling compaction leaves them).  A zero vector has cosine 0.  One warp per pair of rows; ksum is staged in shared memory
-// once per CTA and, for rows of up to 128 vectors, kept in registers by the lanes that meet its columns;
-// |ksum|^2 is folded by every warp in the same order, so all CTAs agree on it.
-struct DiversityArgs {
-  const uint4* K; int rows;                 // cached keys [rows, C]
-  const float* ksum; int n_slices;          // [n_slices, C]
-  float* ksum_out;                          // [C] or nullptr
-  float* d;                                 // [rows]
-  int div_ctas;                             // CTAs [0, div_ctas) of the launch work on d; later ones on the norms
-  const uint4* resid; int resid_rows;       // [resid_rows, C] or nullptr
-  float* s_raw;                             // [resid_rows]
-};
-
-template <int DT>
-__device__ __forceinline__ void diversity_body(const DiversityArgs& A, int nvec, float* sh_ksum) {
-  constexpr int VEC = VecOf<DT>::n;
-  const uint4* __restrict__ K = A.K;
-  const float* __restrict__ ksum = A.ksum;
-  float* __restrict__ ksum_out = A.ksum_out;
-  float* __restrict__ d = A.d;
-  const int rows = A.rows, n_slices = A.n_slices, div_ctas = A.div_ctas;
-  // CTAs past the first div_ctas carry a second, independent job in the same launch: the residual norms of
-  // Eq. 5 (one warp per row), so that a step pays one launch for both scores.
-  if ((int)blockIdx.x >= div_ctas) {
-    const int row = (int)((((int)blockIdx.x - div_ctas) * (unsigned)blockDim.x + threadIdx.x) >> 5);
-    if (A.resid != nullptr && row < A.resid_rows) warp_row_norm<DT>(A.resid, row, nvec, A.s_raw);
-    return;
-  }
-  const int C = nvec * VEC;
+// out = (x - mean) / sqrt(var + 1e-5) per row of x [rows, 8 nvec] (bf16), fp32 arithmetic; one warp per row, which stays
+// in registers for rows of up to 128 vectors.  Scaffold (the LayerNorm before a projection), fused with the conversions
+// around it: the three launches it replaces moved 6 bytes per element each way.
+__global__ void __launch_bounds__(256) k_layer_norm_bf16(const uint4* __restrict__ x, int rows, int nvec, uint4* __restrict__ out) {
+  pdl_wait();
+  const int row = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+  if (row >= rows) return;
   const int lane = threadIdx.x & 31;
-  const int warps_total = (int)((div_ctas * (unsigned)blockDim.x) >> 5);
-  // Two rows per iteration, eight 16-byte loads per lane in flight (rows of up to 128 vectors; longer rows loop).
-  // The first pair is requested before the centroid is staged, so that its DRAM latency runs under the set-up.
-  int row = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5) * 2;
-  uint4 u[2][4];
-  auto load_pair = [&](int r0, int v0) {
-    const uint4* p0 = K + (size_t)r0 * nvec;
-    const uint4* p1 = p0 + (r0 + 1 < rows ? nvec : 0);
+  const uint4* p = x + (size_t)row * nvec;
+  const float inv_c = 1.0f / (8.0f * (float)nvec);
+  uint4 u[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (v0 + 32 * i < nvec) {
-        u[0][i] = ld_nc(p0 + v0 + 32 * i);
-        u[1][i] = ld_nc(p1 + v0 + 32 * i);
-      }
-  };
-  if (row < rows) load_pair(row, lane);
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {   // ksum: [n_slices, C], folded in slice order
-    float t = ksum[c];
-    for (int sl = 1; sl < n_slices; ++sl) t += ksum[(size_t)sl * C + c];
-    sh_ksum[c] = t;
-    if (ksum_out != nullptr && blockIdx.x == 0) ksum_out[c] = t;   // the folded sums, for whoever continues from them
-  }
-  __syncthreads();
-  float kn = 0.0f;
-  for (int v = lane; v < nvec; v += 32)
-#pragma unroll
-    for (int e = 0; e < VEC; e += 4) {
-      const float4 k4 = *reinterpret_cast<const float4*>(sh_ksum + v * VEC + e);
-      kn = __fmaf_rn(k4.x, k4.x, kn);
-      kn = __fmaf_rn(k4.y, k4.y, kn);
-      kn = __fmaf_rn(k4.z, k4.z, kn);
-      kn = __fmaf_rn(k4.w, k4.w, kn);
-    }
-  kn = warp_sum(kn);
-  // A lane meets the same columns in every row; when a row fits one round of loads (nvec <= 128) the lane keeps
-  // its 4 x VEC centroid values in registers, and the row loop does not touch shared memory at all.
-  const bool in_regs = nvec <= 128;
-  float kreg[4][VEC];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int e = 0; e < VEC; e += 4) {
-      float4 k4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (in_regs && lane + 32 * i < nvec) k4 = *reinterpret_cast<const float4*>(sh_ksum + (lane + 32 * i) * VEC + e);
-      kreg[i][e] = k4.x; kreg[i][e + 1] = k4.y; kreg[i][e + 2] = k4.z; kreg[i][e + 3] = k4.w;
-    }
-  for (; row < rows; row += 2 * warps_total) {
-    const bool two = row + 1 < rows;
-    float dot[2] = {0.0f, 0.0f}, nrm[2] = {0.0f, 0.0f};
+  for (int i = 0; i < 4; ++i) u[i] = lane + 32 * i < nvec ? p[lane + 32 * i] : make_uint4(0u, 0u, 0u, 0u);
+  auto each = [&](auto fn) {                       // fn(vector index, its eight values)
     for (int v0 = lane; v0 < nvec; v0 += 128) {
-      if (v0 != lane) load_pair(row, v0);
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (v0 + 32 * i < nvec) {
-          float ks[VEC];
-          if (in_regs) {
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) ks[e] = kreg[i][e];
-          } else {
-            // 16-byte reads: consecutive lanes are VEC floats apart, which scalar reads would serialise eight ways
-#pragma unroll
-            for (int e = 0; e < VEC; e += 4)
-              *reinterpret_cast<float4*>(ks + e) =
-                  *reinterpret_cast<const float4*>(sh_ksum + (v0 + 32 * i) * VEC + e);
-          }
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            float f[VEC];
-            unpack<DT>(u[r][i], f);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) {
-              dot[r] = __fmaf_rn(f[e], ks[e], dot[r]);
-              nrm[r] = __fmaf_rn(f[e], f[e], nrm[r]);
-            }
-          }
+          float f[8];
+          unpack<kBF16>(v0 == lane ? u[i] : p[v0 + 32 * i], f);
+          fn(v0 + 32 * i, f);
         }
     }
-    const int next = row + 2 * warps_total;
-    if (next < rows) load_pair(next, lane);           // the next pair travels during the reductions
+  };
+  float s = 0.0f;
+  each([&](int, const float* f) {
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const float dt = warp_sum(dot[r]), nr = warp_sum(nrm[r]);
-      if (lane == 0 && (r == 0 || two)) {
-        float cosv = 0.0f;
-        if (nr > 0.0f && kn > 0.0f) cosv = __fdiv_rn(dt, __fmul_rn(__fsqrt_rn(nr), __fsqrt_rn(kn)));
-        d[row + r] = 1.0f - cosv;
-      }
+    for (int e = 0; e < 8; ++e) s += f[e];
+  });
+  const float mean = warp_sum(s) * inv_c;
+  float q = 0.0f;
+  each([&](int, const float* f) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) q = __fmaf_rn(f[e] - mean, f[e] - mean, q);
+  });
+  const float rstd = rsqrtf(warp_sum(q) * inv_c + 1e-5f);
+  each([&](int v, const float* f) {
+    uint4 w;
+    uint32_t* ww = reinterpret_cast<uint32_t*>(&w);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn((f[2 * e] - mean) * rstd, (f[2 * e + 1] - mean) * rstd);
+      ww[e] = *reinterpret_cast<const uint32_t*>(&h);
     }
-  }
+    out[(size_t)row * nvec + v] = w;
+  });
 }
 
-template <int DT>
-__global__ void __launch_bounds__(256) k_diversity(const uint4* __restrict__ K, int rows, int nvec,
-                                                   const float* __restrict__ ksum, int n_slices,
-                                                   float* __restrict__ ksum_out,
-                                                   float* __restrict__ d, int div_ctas,
-                                                   const uint4* __restrict__ resid, int resid_rows,
-                                                   float* __restrict__ s_raw) {
-  extern __shared__ __align__(16) float sh_ksum[];
-  const DiversityArgs A{K, rows, ksum, n_slices, ksum_out, d, div_ctas, resid, resid_rows, s_raw};
-  diversity_body<DT>(A, nvec, sh_ksum);
-}
-
-// Both scores of several layers in one launch: blockIdx.y = position in the batch, every layer with its own cache,
-// sums and residual; the grid's x extent is the largest layer's, smaller layers leave their surplus CTAs idle.
+// The residual norms of several layers in one launch: blockIdx.y = position in the batch.
 constexpr int kMaxScoreBatch = 32;
-struct DiversityBatch {
-  DiversityArgs a[kMaxScoreBatch];
+struct NormBatch {
+  const uint4* x[kMaxScoreBatch];
+  float* s[kMaxScoreBatch];
 };
 template <int DT>
-__global__ void __launch_bounds__(256) k_diversity_batched(const __grid_constant__ DiversityBatch batch, int nvec) {
-  extern __shared__ __align__(16) float sh_ksum[];
-  diversity_body<DT>(batch.a[blockIdx.y], nvec, sh_ksum);
+__global__ void __launch_bounds__(256) k_row_norms_batched(const __grid_constant__ NormBatch batch, int rows, int nvec) {
+  const int row = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+  if (row < rows && batch.x[blockIdx.y] != nullptr) warp_row_norm<DT>(batch.x[blockIdx.y], row, nvec, batch.s[blockIdx.y]);
 }
 
 // Supp. D, attention-weight criterion: part[h, j] = sum_i 2^(c q_i,h . k_j,h - lse[i, h]), the attention key j of the

@@ -1,45 +1,107 @@
-// Budgeted selection (Eq. 8) as a radix select over a thread-block cluster, and the fused per-step kernel
-// that prepares its input: anchor flags (Sec. 3.3), activation smoothing (Eq. 6), hybrid priorities (Eq. 7).
+// Budgeted selection (Eq. 8) over a thread-block cluster, and the fused per-step kernel that prepares its input: anchor
+// flags (Sec. 3.3), activation smoothing (Eq. 6), hybrid priorities (Eq. 7).
 //
-// A cluster of up to 8 CTAs x 1024 threads splits the N candidates into contiguous position ranges, one per
-// CTA, held in that CTA's shared memory.  Protected rows get the largest possible key, so "every protected
-// row plus the B - |P| best evictable rows" is simply "the B largest keys"; ties at the threshold are
-// admitted in position order, so the result is unique.  The B-th largest key is found with four 8-bit
-// most-significant-digit passes; per-CTA digit histograms and counts are combined through distributed
-// shared memory with one cluster barrier per pass.
+// A cluster of up to 8 CTAs x 512 threads splits the N candidates into contiguous position ranges, one per CTA, held in
+// that CTA's shared memory.  Protected rows get the largest possible key, so "every protected row plus the B - |P| best
+// evictable rows" is simply "the B largest keys", ties by position: a row stays if its key is above T, or equal to T and
+// its position at most posT, where (T, posT) is the B-th candidate in that order.
+//
+// What bounds it is latency: under 1 MB is touched, but every step depends on the one before, and a cluster barrier costs
+// about a microsecond.  So the usual way to T takes three: one to exchange the groups' ranges (Eq. 7), one after which
+// every CTA reads all CTAs' 512-bin histograms of the priorities and finds the bin of the B-th row, one after which every
+// CTA reads the few candidates of that bin and ranks them by comparison; the counts that place each CTA's output travel
+// with them.  When the bin is crowded (many equal or nearly equal priorities) four 8-bit radix passes over the keys find
+// T instead, which takes a barrier each.  A warp then owns a contiguous range of positions and writes survivors, meta
+// and moves with ballots, so that neighbouring lanes write neighbouring words.  (Radix passes for every step, a
+// contiguous range per thread, and a separate exchange for the moves took 36 us at 17758 candidates and 18 us at 325.)
 #pragma once
 
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "score_kernels.cuh"
 
 namespace ovggt {
 
 namespace cg = cooperative_groups;
 
 constexpr int kSelectThreads = 512;   // 512 x 64 registers: half an SM, so a CTA fits beside an attention CTA
+constexpr int kSelectWarps = kSelectThreads / 32;
 constexpr int kSelectMaxCtas = 8;
+constexpr int kSelectBins = kSelectThreads;       // a thread per bin; the last bin holds the protected rows
+constexpr int kSelectCtaCands = 64, kSelectAllCands = 256;   // candidates of the threshold bin, per CTA and in all
 constexpr uint32_t kKeyProtected = 0xFFFFFFFFu;   // above the key of +inf (0xFF800000)
 
-struct SelectShared {
-  int hist[2][256];          // this CTA's digit histogram, double-buffered across passes (read by the cluster)
-  int tot[256];              // cluster-wide digit counts of the current pass
-  int scan[64];
-  float fscan[64];
-  int digit, krem;
-  int pub_gt, pub_eq;        // this CTA's counts of keys above / equal to the threshold, read by the cluster
-  float pub_lo_h, pub_hi_h, pub_lo_n, pub_hi_n;
-  int all_gt[kSelectMaxCtas], all_eq[kSelectMaxCtas];   // the whole cluster's counts, gathered by one warp
-  int pub_up, pub_down;      // hole filling: survivors above the low range / evicted rows inside it, this CTA
-  int all_up[kSelectMaxCtas], all_down[kSelectMaxCtas];
-  float mm[4];               // cluster-wide lo_h, hi_h, lo_n, hi_n
+// The CTAs that share a problem.  A single CTA needs no cluster: its barrier is the block's, which costs a tenth.
+template <bool SINGLE>
+struct Peers {
+  __device__ __forceinline__ static int count() {
+    if constexpr (SINGLE) return 1;
+    else return (int)cg::this_cluster().num_blocks();
+  }
+  __device__ __forceinline__ static int rank() {
+    if constexpr (SINGLE) return 0;
+    else return (int)cg::this_cluster().block_rank();
+  }
+  __device__ __forceinline__ static void sync() {
+    if constexpr (SINGLE) __syncthreads();
+    else cg::this_cluster().sync();
+  }
+  // Before a CTA leaves: nobody reads its shared memory any more.  Orders no memory, so it waits for no stores.
+  __device__ __forceinline__ static void leave() {
+    if constexpr (!SINGLE) {
+      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    }
+  }
+  template <typename T>
+  __device__ __forceinline__ static T* of(T* p, int r) {   // the same object in CTA r
+    if constexpr (SINGLE) return p;
+    else return cg::this_cluster().map_shared_rank(p, r);
+  }
+  static constexpr int kMax = SINGLE ? 1 : kSelectMaxCtas;
 };
+
+struct SelectShared {
+  union {
+    int hist[kSelectBins];     // this CTA's histogram, read by the cluster between the second and the third barrier
+    int radix[2][256];         // digit histograms of the radix passes, double-buffered (read by the cluster)
+    struct { uint32_t key[kSelectAllCands]; int pos[kSelectAllCands]; } all;   // the cluster's candidates, gathered
+  };
+  union {
+    struct { uint32_t key[kSelectCtaCands]; int pos[kSelectCtaCands]; } cand;  // this CTA's candidates, read by the cluster;
+                                                                              // pos: position | kCandUp | kCandDown
+    int tot[256];              // radix passes: cluster-wide digit counts
+  };
+  union {                      // scratch of block-wide reductions, one at a time
+    int scan[64];
+    uint32_t red[kSelectWarps][6];
+    int wtot[kSelectWarps][3];
+  };
+  uint32_t pub_mm[6], mm[6];   // ranges (as keys) of this CTA, of the cluster
+  int n_cand, keep_before;
+  int pub_keep, pub_up, pub_down, pub_eq, pub_pos;   // counts of this CTA, read by the cluster
+  int cnt_bin[kSelectMaxCtas], cnt_keep[kSelectMaxCtas], cnt_up[kSelectMaxCtas], cnt_down[kSelectMaxCtas];
+  int digit, krem;             // (also: the threshold bin and the rank inside it)
+  uint32_t T;
+  int posT;
+};
+constexpr int kCandUp = 1 << 31, kCandDown = 1 << 30, kCandPos = kCandDown - 1;
 
 // Range of positions owned by CTA `rank` when N positions are split over `ncta` CTAs.
 __device__ __forceinline__ void cta_range(int N, int ncta, int rank, int* begin, int* end) {
   const int span = (N + ncta - 1) / ncta;
   *begin = min(N, rank * span);
   *end = min(N, *begin + span);
+}
+// Range of a CTA's positions owned by one of its warps.
+__device__ __forceinline__ void warp_range(int cnt, int warp, int* lo, int* hi) {
+  const int span = ((cnt + kSelectWarps - 1) / kSelectWarps + 31) & ~31;
+  *lo = min(cnt, warp * span);
+  *hi = min(cnt, *lo + span);
+}
+__device__ __forceinline__ float key_value(uint32_t key) {   // inverse of rank_key
+  return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
 }
 
 // Warp 0 finds the digit whose bin holds the krem-th largest remaining key, given bin counts tot[256].
@@ -87,111 +149,76 @@ __device__ __noinline__ void digit_histogram(const uint32_t* keys, int cnt, uint
   }
 }
 
-// keys[0 .. cnt): this CTA's keys for positions [begin, begin + cnt).  Finds the B largest keys of the whole
-// cluster (ties by position), writes the surviving global positions, ascending, to survivors[] and marks the
-// kept local positions in keep[] (cnt bytes).  Returns the cluster-wide survivor count, min(N, B).
-// *my_base receives the index in survivors[] of this CTA's first survivor.
-__device__ inline int cluster_select(cg::cluster_group& cluster, const uint32_t* keys, uint8_t* keep, int begin,
-                                     int cnt, int N, int B, int* survivors, SelectShared* sh, int* my_base,
-                                     int* bad) {
+// Sum over the block, added to *out (shared memory, zeroed by the caller and synchronised around the call).
+__device__ __forceinline__ void block_add(int x, int* out) {
+  x = __reduce_add_sync(0xFFFFFFFFu, x);
+  if ((threadIdx.x & 31) == 0 && x != 0) atomicAdd(out, x);
+}
+
+// (T, posT) of the B-th largest of the cluster's keys by radix passes, for any distribution of keys; N > B >= 1.  Returns
+// whether more protected rows than B exist (only the first B of them can then stay).  keys[0 .. cnt): this CTA's keys.
+template <bool SINGLE>
+__device__ __noinline__ bool radix_threshold(const uint32_t* keys, int begin, int cnt, int B, SelectShared* sh) {
+  using G = Peers<SINGLE>;
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int ncta = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-  const bool keep_all = N <= B;
-  uint32_t T = 0;
-  int need_eq = 0;
-  if (!keep_all) {
-    uint32_t prefix = 0, mask = 0;
-    int krem = B;
-    int buf = 0;
+  const int ncta = G::count(), rank = G::rank();
+  G::sync();                                    // (the histograms below lie over data the cluster may still read)
+  uint32_t prefix = 0, mask = 0;
+  int krem = B, buf = 0;
 #pragma unroll 1
-    for (int shift = 24; shift >= 0; shift -= 8, buf ^= 1) {
-      int* hist = sh->hist[buf];
-      for (int b = tid; b < 256; b += nthr) hist[b] = 0;
-      __syncthreads();
-      digit_histogram(keys, cnt, mask, prefix, shift, hist);
-      cluster.sync();
-      // every CTA folds all histograms and finds the same digit
-      if (tid < 256) {
-        int v[kSelectMaxCtas];
+  for (int shift = 24; shift >= 0; shift -= 8, buf ^= 1) {
+    int* hist = sh->radix[buf];
+    for (int b = tid; b < 256; b += nthr) hist[b] = 0;
+    __syncthreads();
+    digit_histogram(keys, cnt, mask, prefix, shift, hist);
+    G::sync();
+    // every CTA folds all histograms and finds the same digit
+    if (tid < 256) {
+      int v[G::kMax];
 #pragma unroll
-        for (int r = 0; r < kSelectMaxCtas; ++r)      // all remote loads in flight before the first add
-          v[r] = r < ncta ? cluster.map_shared_rank(hist, r)[tid] : 0;
-        int t = 0;
+      for (int r = 0; r < G::kMax; ++r)      // all remote loads in flight before the first add
+        v[r] = r < ncta ? G::of(hist, r)[tid] : 0;
+      int t = 0;
 #pragma unroll
-        for (int r = 0; r < kSelectMaxCtas; ++r) t += v[r];
-        sh->tot[tid] = t;
-      }
-      __syncthreads();
-      find_digit(sh->tot, krem, sh);
-      __syncthreads();
-      prefix |= (uint32_t)sh->digit << shift;
-      mask |= 255u << shift;
-      krem = sh->krem;
+      for (int r = 0; r < G::kMax; ++r) t += v[r];
+      sh->tot[tid] = t;
     }
-    T = prefix;
-    need_eq = krem;
+    __syncthreads();
+    find_digit(sh->tot, krem, sh);
+    __syncthreads();
+    prefix |= (uint32_t)sh->digit << shift;
+    mask |= 255u << shift;
+    krem = sh->krem;
   }
-  // Thread t owns the contiguous local positions [t*chunk, (t+1)*chunk).
+  // the krem-th tie, counted over the CTAs in order: its position
   const int chunk = (cnt + nthr - 1) / nthr;
   const int lo = min(cnt, tid * chunk), hi = min(cnt, lo + chunk);
-  // One exchange settles everything: with (keys above T, keys equal to T) of every CTA, each CTA knows how
-  // many of its ties are admitted (ties go to the lower position, i.e. to the lower rank first) and where its
-  // survivors start in the output.
-  int cnt_gt = 0, cnt_eq = 0;
-  if (keep_all) {
-    cnt_gt = hi - lo;
-  } else {
-    for (int i = lo; i < hi; ++i) {
-      const uint32_t key = keys[i];
-      cnt_gt += key > T;
-      cnt_eq += key == T;
-    }
-  }
-  int gt_total, eq_total;
-  block_excl_scan_int(cnt_gt, sh->scan, &gt_total);
-  int eq_rank = block_excl_scan_int(cnt_eq, sh->scan, &eq_total);   // ties before this thread's, within the CTA
+  int eq = 0, eq_total;
+  for (int i = lo; i < hi; ++i) eq += keys[i] == prefix;
+  int before = block_excl_scan_int(eq, sh->scan, &eq_total);
   if (tid == 0) {
-    sh->pub_gt = gt_total;
     sh->pub_eq = eq_total;
+    sh->pub_pos = -1;
   }
-  cluster.sync();
-  if (tid < ncta) {                                   // one remote read per lane instead of ncta per thread
-    sh->all_gt[tid] = *cluster.map_shared_rank(&sh->pub_gt, tid);
-    sh->all_eq[tid] = *cluster.map_shared_rank(&sh->pub_eq, tid);
-  }
-  __syncthreads();
-  int before = 0, all = 0, eq_before = 0, eq_all = 0;
+  G::sync();
+  int eq_all = 0;
   for (int r = 0; r < ncta; ++r) {
-    const int e = sh->all_eq[r], gcount = sh->all_gt[r];
-    const int adm = keep_all ? 0 : max(0, min(e, need_eq - eq_all));   // ties of rank r that are admitted
-    if (r < rank) {
-      before += gcount + adm;
-      eq_before += e;
-    }
-    all += gcount + adm;
+    const int e = *G::of(&sh->pub_eq, r);
+    if (r < rank) before += e;
     eq_all += e;
   }
-  eq_rank += eq_before;
-  // more protected rows than the budget holds: only the first B of them can stay
-  *bad = (!keep_all && T == kKeyProtected && eq_all > need_eq) ? 1 : 0;
-  int cnt_keep = 0;
-  for (int i = lo; i < hi; ++i) {
-    bool k = true;
-    if (!keep_all) {
-      const uint32_t key = keys[i];
-      k = key > T || (key == T && eq_rank++ < need_eq);
-    }
-    keep[i] = k ? 1 : 0;
-    cnt_keep += k;
+  if (before < krem && before + eq >= krem)          // one thread of the cluster
+    for (int i = lo; i < hi; ++i)
+      if (keys[i] == prefix && ++before == krem) sh->pub_pos = begin + i;
+  G::sync();
+  if (tid == 0) {
+    int p = -1;
+    for (int r = 0; r < ncta; ++r) p = max(p, *G::of(&sh->pub_pos, r));
+    sh->T = prefix;
+    sh->posT = p;
   }
-  int keep_total;
-  int base = block_excl_scan_int(cnt_keep, sh->scan, &keep_total);
-  *my_base = before;
-  base += before;
-  for (int i = lo; i < hi; ++i)
-    if (keep[i]) survivors[base++] = begin + i;
   __syncthreads();
-  return all;
+  return prefix == kKeyProtected && eq_all > krem;
 }
 
 // Single-CTA pick used for the small top-A choice over the confidence map: marks the A largest of cnt keys
@@ -235,45 +262,101 @@ __device__ inline void block_top_mark(const uint32_t* keys, uint8_t* keep, int c
   __syncthreads();
 }
 
-// Shared memory a CTA of the selection kernels needs for `span` owned positions (+ np confidence entries).
-__host__ __device__ inline size_t select_smem_bytes(int span, int np) {
-  return ((sizeof(SelectShared) + 15) & ~(size_t)15) + (size_t)span * 4 + 2 * (((size_t)span + 15) & ~(size_t)15) +
-         (size_t)np * 4 + (((size_t)np + 15) & ~(size_t)15) + 16;
+__host__ __device__ inline size_t select_header_bytes() { return (sizeof(SelectShared) + 15) & ~(size_t)15; }
+
+// Shared memory a CTA of the stand-alone selection needs for `span` owned positions: their keys.
+__host__ __device__ inline size_t select_smem_bytes(int span) { return select_header_bytes() + (((size_t)span * 4 + 15) & ~(size_t)15); }
+
+// The fused per-step kernel keeps, per position, the value or key (4 bytes), bin and flag (2), id (8), stored score (4)
+// and slot (4) on chip, the frame's m raw residual norms and the np confidence keys and marks; the fold of the key sums'
+// corrections at the end needs five rows of kDeltaCols floats over the same place.
+constexpr int kDeltaCols = 1024;
+__host__ __device__ inline size_t compress_smem_bytes(int span, int np, int m) {
+  const size_t s4 = ((size_t)span + 3) & ~(size_t)3, m4 = ((size_t)m + 3) & ~(size_t)3, np4 = ((size_t)np + 3) & ~(size_t)3;
+  const size_t body = s4 * (8 + 3 * 4) + ((s4 + 7) & ~(size_t)7) * 2 + m4 * 4 + np4 * 4 + np4;
+  const size_t fold = (size_t)5 * kDeltaCols * 4;
+  return select_header_bytes() + (body > fold ? body : fold);
 }
 
-// The fused per-step kernel also keeps the ids, stored scores and physical slots of its positions (16 bytes each)
-// and the frame's raw residual norms (m floats) on chip.
-__host__ __device__ inline size_t compress_smem_bytes(int span, int np, int m) {
-  return select_smem_bytes(span, np) + (((size_t)span * 8 + 15) & ~(size_t)15) +
-         2 * (((size_t)span * 4 + 15) & ~(size_t)15) + (((size_t)m * 4 + 15) & ~(size_t)15) + 16;
+// Per-warp totals of the rows that stay, and of two marked kinds of rows, for the warp's range of positions; then the
+// block's exclusive prefix of them.  `row(i, keep, up, down)` classifies a position.  All threads call it.
+template <typename F>
+__device__ __forceinline__ void warp_totals(int lo, int hi, SelectShared* sh, F row, int* keep0, int* up0, int* down0) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int k = 0, u = 0, d = 0;
+  for (int i = lo + lane; i < hi; i += 32) {
+    bool keep, up, down;
+    row(i, keep, up, down);
+    k += keep;
+    u += up;
+    d += down;
+  }
+  k = __reduce_add_sync(0xFFFFFFFFu, k);
+  u = __reduce_add_sync(0xFFFFFFFFu, u);
+  d = __reduce_add_sync(0xFFFFFFFFu, d);
+  if (lane == 0) {
+    sh->wtot[warp][0] = k;
+    sh->wtot[warp][1] = u;
+    sh->wtot[warp][2] = d;
+  }
+  __syncthreads();
+  const bool mine = lane < warp;                     // (16 warps: the lanes of one warp cover them)
+  *keep0 = __reduce_add_sync(0xFFFFFFFFu, mine ? sh->wtot[lane][0] : 0);
+  *up0 = __reduce_add_sync(0xFFFFFFFFu, mine ? sh->wtot[lane][1] : 0);
+  *down0 = __reduce_add_sync(0xFFFFFFFFu, mine ? sh->wtot[lane][2] : 0);
 }
 
 // ---- standalone selection over given priorities: one cluster per independent problem (blockIdx.y)
 
+template <bool SINGLE>
 __global__ void __launch_bounds__(kSelectThreads) k_select(const float* __restrict__ r,
                                                            const uint8_t* __restrict__ flags_in, int N, int B,
                                                            int* __restrict__ survivors, int* status) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  cg::cluster_group cluster = cg::this_cluster();
-  SelectShared* sh = reinterpret_cast<SelectShared*>(smem);
-  unsigned char* p = smem + ((sizeof(SelectShared) + 15) & ~15);
-  const int ncta = (int)cluster.num_blocks();
+  extern __shared__ __align__(16) unsigned char smem_select[];
+  using G = Peers<SINGLE>;
+  SelectShared* sh = reinterpret_cast<SelectShared*>(smem_select);
+  uint32_t* keys = reinterpret_cast<uint32_t*>(smem_select + select_header_bytes());
+  const int ncta = G::count(), rank = G::rank();
   int begin, end;
-  cta_range(N, ncta, (int)cluster.block_rank(), &begin, &end);
-  const int cnt = end - begin, span = (N + ncta - 1) / ncta;
-  uint32_t* keys = reinterpret_cast<uint32_t*>(p);
-  uint8_t* keep = p + (size_t)span * 4;
+  cta_range(N, ncta, rank, &begin, &end);
+  const int cnt = end - begin;
   const size_t prob = blockIdx.y;
   const float* rr = r + prob * (size_t)N;
   const uint8_t* ff = flags_in + prob * (size_t)N;
   for (int i = threadIdx.x; i < cnt; i += blockDim.x)
     keys[i] = ff[begin + i] != 0 ? kKeyProtected : rank_key(rr[begin + i]);
   __syncthreads();
-  int my_base, bad;
-  const int n_keep = cluster_select(cluster, keys, keep, begin, cnt, N, B, survivors + prob * (size_t)min(N, B), sh,
-                                    &my_base, &bad);
-  if ((bad || n_keep != min(N, B)) && threadIdx.x == 0 && status) atomicCAS(status, 0, OVGGT_ERR_DEVICE_STATUS);
-  cluster.sync();   // no CTA may exit while others still read its shared memory
+  uint32_t T = 0;
+  int posT = N;
+  bool bad = false;
+  if (N > B) {
+    bad = radix_threshold<SINGLE>(keys, begin, cnt, B, sh);
+    T = sh->T;
+    posT = sh->posT;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int lo, hi, j, u0, d0;
+  warp_range(cnt, warp, &lo, &hi);
+  auto kept = [&](int i) { return keys[i] > T || (keys[i] == T && begin + i <= posT); };
+  warp_totals(lo, hi, sh, [&](int i, bool& k, bool& u, bool& d) { k = kept(i); u = d = false; }, &j, &u0, &d0);
+  if (threadIdx.x == kSelectThreads - 32) sh->pub_keep = j + sh->wtot[warp][0];   // (the last warp knows the total)
+  G::sync();
+  int all = 0;
+  for (int q = 0; q < ncta; ++q) {
+    const int c = *G::of(&sh->pub_keep, q);
+    if (q < rank) j += c;
+    all += c;
+  }
+  int* out = survivors + prob * (size_t)min(N, B);
+  for (int i0 = lo; i0 < hi; i0 += 32) {
+    const int i = i0 + lane;
+    const bool k = i < hi && kept(i);
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, k);
+    if (k) out[j + __popc(m & ((1u << lane) - 1))] = begin + i;
+    j += __popc(m);
+  }
+  if ((bad || all != min(N, B)) && threadIdx.x == 0 && status) atomicCAS(status, 0, OVGGT_ERR_DEVICE_STATUS);
+  G::leave();
 }
 
 // ---- the fused per-step kernel
@@ -302,14 +385,20 @@ struct CompressParams {
   // Hole-filling layout (fill != 0): the K/V row of logical position g lives in slot slot_src[g] (g < n) or g
   // (new rows); the K/V rows are not gathered.  Survivors whose slot is >= B have to move into the slots < B
   // that evicted rows leave: the i-th such survivor (in logical order) goes to the i-th such slot (in the logical
-  // order of the rows that leave).  The kernel writes the pairs and the survivors' slots; the move kernel that
-  // follows copies the rows and patches slot_dst[move_j[i]] = move_dst[i].
+  // order of the rows that leave).  The kernel writes the pairs, the survivors' slots, and the step's stamp beside every
+  // slot that will be filled; the layer's next append copies the rows and patches slot_dst[move_j[i]] = move_dst[i].
+  // Stable layout: the lists hold the admitted new rows and the evicted cached rows (positions = rows), for the sums below.
   int fill;
   const int* slot_src;              // [n]
   int* slot_dst;                    // [<= B]
   int* move_src; int* move_dst; int* move_j;   // [<= M] each
   int* tail_move;                   // [M]: for slot B + i, the index of the move that empties it, or -1
   int* n_moves_out;
+  int* hole_stamp; int stamp;       // [B]
+  const uint4* resid;               // [M, C] or nullptr: compute the residual norms here instead of reading s_raw (small M)
+  // Column sums of the keys that stay: ksum_next = ksum (or 0) + admitted keys - evicted keys; ksum_next nullptr: not asked for.
+  const uint4* k_cache; int nvec;
+  const float* ksum; float* ksum_next;   // [C]
 };
 
 // Eq. 6 for new-frame token j (aux tokens keep their raw score); s_raw: the frame's M residual norms.
@@ -332,245 +421,492 @@ __device__ __forceinline__ float smoothed_score(const CompressParams& P, const f
   return v;
 }
 
+// ksum_next = ksum + (keys admitted - keys evicted) by the whole cluster.  src / dst: the slots of na admitted and nd
+// evicted rows (src nullptr: the na rows from n on).  A warp takes every 8 ncta-th row of one half of the columns, the
+// eight warps of a half are folded in two rounds, the CTAs in rank order: a fixed order, whatever the timing.
+template <int DT, bool SINGLE>
+__device__ __noinline__ void fold_key_sums(const CompressParams& P, const int* src, const int* dst, int na, int nd,
+                                              float* park /* [4][kDeltaCols] */, float* part /* [kDeltaCols] */) {
+  constexpr int VEC = VecOf<DT>::n, VB = kDeltaCols / VEC, PER = VB / 64, Q = 4 / PER;   // vectors per block, per lane; rows in flight
+  using G = Peers<SINGLE>;
+  const int ncta = G::count(), rank = G::rank();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = warp & 1, grp = warp >> 1;
+  const int C = P.nvec * VEC, stride = 8 * ncta;
+  for (int v0 = 0; v0 < P.nvec; v0 += VB) {
+    float acc[PER * VEC];
+#pragma unroll
+    for (int e = 0; e < PER * VEC; ++e) acc[e] = 0.0f;
+    const int vl = v0 + half * (VB / 2) + lane;       // this lane's vectors: vl, vl + 32, ...
+    auto load = [&](int row, uint4* u) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+        if (vl + 32 * i < P.nvec) u[i] = P.k_cache[(size_t)row * P.nvec + vl + 32 * i];
+    };
+    auto add = [&](const uint4* u, float sign) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+        if (vl + 32 * i < P.nvec) {
+          float f[VEC];
+          unpack<DT>(u[i], f);
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) acc[i * VEC + e] = __fmaf_rn(f[e], sign, acc[i * VEC + e]);
+        }
+    };
+    const int most = max(na, nd);
+    int ra = 0, rb = 0;                               // lane l: the rows of the warp's turn 32 x + l
+    for (int i = rank * 8 + grp, turn = 0; i < most; i += Q * stride, turn += Q) {
+      if ((turn & 31) == 0) {
+        const int k = i + lane * stride;
+        ra = k < na ? (src ? __ldcg(src + k) : P.n + k) : 0;
+        rb = k < nd ? __ldcg(dst + k) : 0;
+      }
+      uint4 a[Q][PER], b[Q][PER];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int k = i + q * stride, xa = __shfl_sync(0xFFFFFFFFu, ra, (turn + q) & 31), xb = __shfl_sync(0xFFFFFFFFu, rb, (turn + q) & 31);
+        if (k < na) load(xa, a[q]);
+        if (k < nd) load(xb, b[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int k = i + q * stride;
+        if (k < na) add(a[q], 1.0f);
+        if (k < nd) add(b[q], -1.0f);
+      }
+    }
+    // (element-major: neighbouring lanes meet neighbouring banks)
+    auto slot = [&](int s, int i, int e) -> float& {
+      return park[s * kDeltaCols + e * VB + half * (VB / 2) + lane + 32 * i];
+    };
+    if (grp >= 4) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) slot(grp - 4, i, e) = acc[i * VEC + e];
+    }
+    __syncthreads();
+    if (grp < 4) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) slot(grp, i, e) += acc[i * VEC + e];
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < kDeltaCols; c += blockDim.x)
+      part[c] = ((park[c] + park[kDeltaCols + c]) + park[2 * kDeltaCols + c]) + park[3 * kDeltaCols + c];
+    G::sync();
+    for (int x = rank * kSelectThreads + threadIdx.x; x < kDeltaCols; x += kSelectThreads * ncta) {
+      const int c = v0 * VEC + (x & (VB - 1)) * VEC + x / VB;   // the column whose sum lies at x
+      if (c >= C) continue;
+      float v[G::kMax];                               // all remote reads in flight before the first add
+#pragma unroll
+      for (int q = 0; q < G::kMax; ++q) v[q] = q < ncta ? G::of(part, q)[x] : 0.0f;
+      float t = P.ksum ? P.ksum[c] : 0.0f;
+#pragma unroll
+      for (int q = 0; q < G::kMax; ++q) t += v[q];
+      P.ksum_next[c] = t;
+    }
+    if (v0 + VB < P.nvec) G::sync();             // (part is written again)
+  }
+}
+
+template <int DT, bool SINGLE>
 __device__ __forceinline__ void compress_select_body(const CompressParams& P, unsigned char* smem) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const int ncta = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  using G = Peers<SINGLE>;
+  const int ncta = G::count(), rank = G::rank();
   SelectShared* sh = reinterpret_cast<SelectShared*>(smem);
-  unsigned char* p = smem + ((sizeof(SelectShared) + 15) & ~15);
-  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int n = P.n, M = P.M, N = n + M, Np = P.grid_h * P.grid_w;
   int begin, end;
   cta_range(N, ncta, rank, &begin, &end);
-  const int cnt = end - begin, span = (N + ncta - 1) / ncta, span16 = (span + 15) & ~15;
-  uint32_t* keys = reinterpret_cast<uint32_t*>(p);        // [span] values, then the priorities' keys, in place
+  const int cnt = end - begin, span4 = ((N + ncta - 1) / ncta + 3) & ~3;
+  unsigned char* p = smem + select_header_bytes();
+  long long* sid = reinterpret_cast<long long*>(p);               // ids of the owned positions
+  uint32_t* keys = reinterpret_cast<uint32_t*>(sid + ((span4 + 1) & ~1));   // their values, then the priorities' keys, in place
   float* val = reinterpret_cast<float*>(keys);
-  uint8_t* fl = p + (size_t)span * 4;                      // [span] protection flags of the owned positions
-  uint8_t* keep = fl + span16;                             // [span]
-  uint32_t* ckeys = reinterpret_cast<uint32_t*>(keep + span16);   // [Np] confidence keys
-  uint8_t* cmark = reinterpret_cast<uint8_t*>(ckeys + Np);        // [Np]
-  unsigned char* q8 = smem + ((select_smem_bytes(span, Np) + 15) & ~(size_t)15);
-  long long* sid = reinterpret_cast<long long*>(q8);              // [span] ids of the owned positions
-  float* sst = reinterpret_cast<float*>(q8 + (((size_t)span * 8 + 15) & ~(size_t)15));   // [span] their stored scores
-  int* ssl = reinterpret_cast<int*>(sst + (((size_t)span + 3) & ~(size_t)3));   // [span] their physical slots
-  float* sraw = reinterpret_cast<float*>(ssl + (((size_t)span + 3) & ~(size_t)3)); // [M] the frame's residual norms
+  float* sst = reinterpret_cast<float*>(keys + span4);            // their stored scores
+  int* ssl = reinterpret_cast<int*>(sst + span4);                 // their physical slots
+  float* sraw = reinterpret_cast<float*>(ssl + span4);            // [M] the frame's residual norms
+  uint32_t* ckeys = reinterpret_cast<uint32_t*>(sraw + ((M + 3) & ~3));   // [Np] confidence keys
+  uint16_t* bf = reinterpret_cast<uint16_t*>(ckeys + ((Np + 3) & ~3));    // flag << 14 | bin of the owned positions
+  uint8_t* cmark = reinterpret_cast<uint8_t*>(bf + ((span4 + 7) & ~7));   // [Np] the most confident patches
+  const bool hybrid = P.mode == OVGGT_SCORE_HYBRID, choose = N > P.B;
+  pdl_wait();
+  pdl_trigger();   // an attention queued behind this kernel reads nothing of it: it starts as soon as this one runs
+  const bool own_rank = P.override_r == nullptr;                  // rank the priorities computed here
 
   // -- anchor registration (Sec. 3.3): the A most confident patch tokens of the new frame, ties to the lower
-  //    index.  Every CTA computes the same marks and uses those of the positions it owns.
-  const bool reg = P.register_anchor && P.A > 0;
+  //    index.  Every CTA that owns new rows computes the same marks and uses those of the positions it owns.
+  const bool reg = P.register_anchor && P.A > 0 && end > n;
   if (reg) {
     for (int i = tid; i < Np; i += nthr) ckeys[i] = rank_key(P.conf[i]);
     __syncthreads();
     block_top_mark(ckeys, cmark, Np, P.A, sh);
   }
 
-  // -- protection flags and values of the owned positions.  A CTA that owns new rows first stages the frame's raw
-  //    norms (Eq. 6 reads each nine times); all global loads of four positions are issued before any is used.
+  // -- protection flags and values of the owned positions, and the ranges of the evictable ones (as keys): cached group,
+  //    new group (Eq. 7), ranked values.  A CTA that owns new rows first stages the frame's raw norms (Eq. 6 reads each
+  //    nine times); all global loads of four positions are issued before any is used.
+  sh->hist[tid] = 0;
+  if (tid == 0) sh->n_cand = sh->pub_up = sh->pub_down = sh->keep_before = 0;
   if (end > n) {
-    for (int j = tid; j < M; j += nthr) sraw[j] = P.s_raw[j];
+    if (P.resid != nullptr) {
+      for (int j = warp; j < M; j += kSelectWarps) warp_row_norm<DT>(P.resid, j, P.nvec, sraw);
+    } else {
+      for (int j = tid; j < M; j += nthr) sraw[j] = P.s_raw[j];
+    }
     __syncthreads();
   }
-  for (int i0 = tid; i0 < cnt; i0 += 4 * nthr) {
-    uint8_t f4[4];
-    long long id4[4];
-    float d4[4], st4[4];
-    int sl4[4];
+  uint32_t mn[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, mx[3] = {0u, 0u, 0u};
+  // (a thread touches its own positions only, so the three passes need no barrier; all loads of a pass are independent)
+#pragma unroll 4
+  for (int i = tid; i < cnt; i += nthr) {
+    const int g = begin + i;
+    int sl = g;
+    float st = 0.0f;
+    if (g < n) {
+      st = P.stored_src[g];
+      if (P.fill) {
+        sl = P.slot_src[g];
+        if (!index_ok(sl, P.B + P.M, P.status)) sl = g;
+      }
+    }
+    bf[i] = (uint16_t)((P.flags_src[g] & 3) << 14);
+    sid[i] = P.ids_src[g];
+    sst[i] = st;
+    ssl[i] = sl;
+  }
+  if (hybrid)
+#pragma unroll 4
+    for (int i = tid; i < cnt; i += nthr) val[i] = begin + i < n ? P.d[ssl[i]] : 0.0f;
+#pragma unroll 1
+  for (int i = tid; i < cnt; i += nthr) {
+    const int g = begin + i;
+    int f = bf[i] >> 14;
+    float x;
+    if (g >= n) {
+      const int j = g - n;
+      if (P.protect_new) f = P.protect_new;
+      if (reg && j >= P.n_special && cmark[j - P.n_special]) f = OVGGT_FLAG_HIST;
+      x = smoothed_score(P, sraw, j);
+      sst[i] = x;                // the score the row keeps
+    } else {
+      if (P.demote_frame >= 0 && f == OVGGT_FLAG_HIST && sid[i] / M == P.demote_frame) f = OVGGT_FLAG_EVICTABLE;
+      x = hybrid ? val[i] : sst[i];
+    }
+    if (P.mode == OVGGT_SCORE_RANDOM) x = random_priority(P.step_key, sid[i]);   // Supp. A: uniform, fresh per step
+    bf[i] = (uint16_t)(f << 14);
+    val[i] = x;
+    if (f == 0) {
+      const uint32_t k = rank_key(x);
+      if (x == x) {              // (a NaN takes no part in its group's range)
+        const bool cached = g < n;
+        mn[0] = cached ? min(mn[0], k) : mn[0];
+        mx[0] = cached ? max(mx[0], k) : mx[0];
+        mn[1] = cached ? mn[1] : min(mn[1], k);
+        mx[1] = cached ? mx[1] : max(mx[1], k);
+      }
+      const float v = own_rank ? x : P.override_r[g];
+      if (fabsf(v) < INFINITY) {
+        const uint32_t kv = rank_key(v);
+        mn[2] = min(mn[2], kv);
+        mx[2] = max(mx[2], kv);
+      }
+    }
+  }
+  if (hybrid || choose) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * nthr, g = begin + i;
-      sl4[u] = g;
-      if (i < cnt) {
-        f4[u] = P.flags_src[g];
-        id4[u] = P.ids_src[g];
-        if (g < n) {
-          st4[u] = P.stored_src[g];
-          if (P.fill) {
-            sl4[u] = P.slot_src[g];
-            if (!index_ok(sl4[u], P.B + P.M, P.status)) sl4[u] = g;
+    for (int q = 0; q < 3; ++q) {
+      mn[q] = __reduce_min_sync(0xFFFFFFFFu, mn[q]);
+      mx[q] = __reduce_max_sync(0xFFFFFFFFu, mx[q]);
+    }
+    if (lane == 0)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        sh->red[warp][2 * q] = mn[q];
+        sh->red[warp][2 * q + 1] = mx[q];
+      }
+    __syncthreads();
+    if (warp < 6) {                                   // one warp per quantity: lanes are the block's warps
+      const bool is_max = warp & 1;
+      const uint32_t v = lane < kSelectWarps ? sh->red[lane][warp] : (is_max ? 0u : 0xFFFFFFFFu);
+      const uint32_t r = is_max ? __reduce_max_sync(0xFFFFFFFFu, v) : __reduce_min_sync(0xFFFFFFFFu, v);
+      if (lane == 0) sh->pub_mm[warp] = r;
+    }
+    G::sync();
+    if (warp < 6) {                                   // lanes are the CTAs of the cluster
+      const bool is_max = warp & 1;
+      const uint32_t v = lane < ncta ? G::of(sh, lane)->pub_mm[warp] : (is_max ? 0u : 0xFFFFFFFFu);
+      const uint32_t r = is_max ? __reduce_max_sync(0xFFFFFFFFu, v) : __reduce_min_sync(0xFFFFFFFFu, v);
+      if (lane == 0) sh->mm[warp] = r;
+    }
+    __syncthreads();
+  }
+
+  // -- Eq. 7, and a bin for every priority: equal steps of the priority (hybrid, random), or equal steps of its key, which
+  //    is logarithmic (residual norms spread over octaves; given priorities may do anything).  Bins only have to be
+  //    monotone; how evenly they fill decides how few candidates the last stage ranks.
+  const float lo_h = key_value(sh->mm[0]), hi_h = key_value(sh->mm[1]), lo_n = key_value(sh->mm[2]), hi_n = key_value(sh->mm[3]);
+  const bool linear = own_rank && (hybrid || P.mode == OVGGT_SCORE_RANDOM);
+  const uint32_t bin_key0 = sh->mm[4];
+  const float bin_lo = linear ? (hybrid ? 0.0f : key_value(bin_key0)) : 0.0f;
+  const float bin_hi = linear ? (hybrid ? fmaxf(P.beta, 1.0f - P.beta) : key_value(sh->mm[5]))
+                              : (float)(sh->mm[5] > bin_key0 ? sh->mm[5] - bin_key0 : 0u);
+  const float bin_scale = bin_hi - bin_lo > 0.0f && bin_hi - bin_lo < INFINITY ? (float)(kSelectBins - 1) / (bin_hi - bin_lo) : 0.0f;
+#pragma unroll 1
+  for (int i = tid; i < ((cnt + 31) & ~31); i += nthr) {
+    bool prot = false;
+    if (i < cnt) {
+      const int g = begin + i;
+      const int f = bf[i] >> 14;
+      float r;
+      uint32_t key;
+      int bin;
+      prot = f != 0;
+      if (prot) {
+        r = INFINITY;
+        key = kKeyProtected;
+        bin = kSelectBins - 1;
+      } else {
+        if (hybrid) {
+          const float lo = g < n ? lo_h : lo_n, hi = g < n ? hi_h : hi_n;
+          const float w = g < n ? 1.0f - P.beta : P.beta;
+          r = hi > lo ? __fmul_rn(w, __fdiv_rn(val[i] - lo, hi - lo))
+                      : ((g >= n && P.lone_new >= 0.0f) ? __fmul_rn(w, P.lone_new) : 0.0f);
+        } else {
+          r = val[i];
+        }
+        const float v = own_rank ? r : P.override_r[g];
+        key = rank_key(v);
+        const float steps = linear ? __fmul_rn(v - bin_lo, bin_scale) : (key > bin_key0 ? __fmul_rn((float)(key - bin_key0), bin_scale) : 0.0f);
+        bin = (int)fminf((float)(kSelectBins - 2), fmaxf(0.0f, steps));
+        if (choose) atomicAdd(&sh->hist[bin], 1);
+      }
+      // The kernel's own priority, also when an override is ranked instead.  Where it can be told from its key it is
+      // written with the survivors: a cluster barrier waits for the global stores before it.
+      if (!own_rank || !(prot || fabsf(r) < INFINITY)) P.r_out[g] = r;
+      keys[i] = key;
+      bf[i] = (uint16_t)(f << 14 | bin);
+    }
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, prot);
+    if (m != 0 && lane == 0) atomicAdd(&sh->hist[kSelectBins - 1], __popc(m));
+  }
+
+  // -- Eq. 8: (T, posT), and what the lower ranks of the cluster keep and move
+  const bool fill = P.fill != 0;
+  auto is_up = [&](int i) { return fill ? ssl[i] >= P.B : begin + i >= n; };
+  uint32_t T = 0;
+  int posT = N, keep_before = begin, up_before = 0, down_before = 0, keep_all = N, up_all = 0, down_all = 0;
+  bool bad = false;
+  auto classify = [&](int i, bool& keep, bool& up, bool& down) {
+    const uint32_t key = keys[i];
+    keep = key > T || (key == T && begin + i <= posT);
+    const bool u = choose && is_up(i);
+    up = keep && u;
+    down = choose && !keep && !u;
+  };
+  int wlo, whi, kw = 0, uw = 0, dw = 0;                // this warp's positions, and what the block's lower warps hold
+  warp_range(cnt, warp, &wlo, &whi);
+  if (!choose) {
+    __syncthreads();
+    kw = wlo;                                          // everything stays
+  } else {
+    G::sync();
+    {
+      // thread t looks at bin (last - t): every CTA finds the bin of the B-th row for itself
+      const int b = kSelectBins - 1 - tid;
+      int v[G::kMax], tot = 0, before = 0;
+#pragma unroll
+      for (int r = 0; r < G::kMax; ++r) v[r] = r < ncta ? G::of(sh, r)->hist[b] : 0;
+#pragma unroll
+      for (int r = 0; r < G::kMax; ++r) {
+        tot += v[r];
+        before += r < rank ? v[r] : 0;
+      }
+      int above = tot;                                 // inclusive over the warp's lanes, then over its lower warps
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, above, o);
+        if (lane >= o) above += y;
+      }
+      if (lane == 31) sh->wtot[warp][0] = above;
+      __syncthreads();
+      above += __reduce_add_sync(0xFFFFFFFFu, lane < warp ? sh->wtot[lane][0] : 0) - tot;
+      if (above < P.B && above + tot >= P.B) {
+        sh->digit = b;
+        sh->krem = P.B - above;
+#pragma unroll
+        for (int r = 0; r < G::kMax; ++r) sh->cnt_bin[r] = v[r];
+      }
+      __syncthreads();
+      block_add(b > sh->digit ? before : 0, &sh->keep_before);   // rows the lower ranks keep in the bins above
+    }
+    const int bstar = sh->digit;
+    int cands = 0;
+    bool crowded = bstar == kSelectBins - 1;           // (more protected rows than B: an error the slow way reports)
+    for (int r = 0; r < ncta; ++r) {
+      cands += sh->cnt_bin[r];
+      crowded |= sh->cnt_bin[r] > kSelectCtaCands;
+    }
+    crowded |= cands > kSelectAllCands;
+    if (!crowded) {
+      int up = 0, down = 0;
+#pragma unroll 1
+      for (int i = tid; i < cnt; i += nthr) {
+        const int bin = bf[i] & (kSelectBins - 1);
+        const bool u = is_up(i);
+        up += bin > bstar && u;
+        down += bin < bstar && !u;
+        if (bin == bstar) {
+          const int c = atomicAdd(&sh->n_cand, 1);     // (in whatever order: they are ranked by key and position)
+          if (c < kSelectCtaCands) {
+            sh->cand.key[c] = keys[i];
+            sh->cand.pos[c] = (begin + i) | (u ? kCandUp : kCandDown);
           }
         }
       }
-    }
-    if (P.mode == OVGGT_SCORE_HYBRID) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * nthr, g = begin + i;
-        d4[u] = (i < cnt && g < n) ? P.d[sl4[u]] : 0.0f;
+      block_add(up, &sh->pub_up);
+      block_add(down, &sh->pub_down);
+      G::sync();
+      uint32_t key = 0;
+      int pos = 0, owner = 0, idx = tid;
+      if (tid < cands) {
+        while (idx >= sh->cnt_bin[owner]) idx -= sh->cnt_bin[owner++];
+        const SelectShared* o = G::of(sh, owner);
+        key = sh->all.key[tid] = o->cand.key[idx];
+        pos = sh->all.pos[tid] = o->cand.pos[idx];
       }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * nthr, g = begin + i;
-      if (i < cnt) {
-        uint8_t f = f4[u] & 3;
-        float x, keepscore;
-        if (g >= n) {
-          const int j = g - n;
-          if (P.protect_new) f = (uint8_t)P.protect_new;
-          if (reg && j >= P.n_special && cmark[j - P.n_special]) f = OVGGT_FLAG_HIST;
-          x = smoothed_score(P, sraw, j);
-          keepscore = x;           // the score the row keeps
-        } else {
-          if (P.demote_frame >= 0 && f == OVGGT_FLAG_HIST && id4[u] / M == P.demote_frame) f = OVGGT_FLAG_EVICTABLE;
-          x = (P.mode == OVGGT_SCORE_HYBRID) ? d4[u] : st4[u];
-          keepscore = st4[u];
+      if (tid >= cands && tid < ((cands + 3) & ~3)) {  // (the ranking loop reads four at a time)
+        sh->all.key[tid] = 0;
+        sh->all.pos[tid] = kCandPos;
+      }
+      if (tid >= nthr - 32 && lane < ncta) {
+        sh->cnt_up[lane] = G::of(sh, lane)->pub_up;
+        sh->cnt_down[lane] = G::of(sh, lane)->pub_down;
+      }
+      __syncthreads();
+      const int krem = sh->krem;
+      if (tid < cands) {
+        int before = 0;
+        const int at = pos & kCandPos;
+        for (int j = 0; j < cands; j += 4) {
+          const uint4 k4 = *reinterpret_cast<const uint4*>(&sh->all.key[j]);
+          const int4 p4 = *reinterpret_cast<const int4*>(&sh->all.pos[j]);
+          before += (k4.x > key || (k4.x == key && (p4.x & kCandPos) < at)) + (k4.y > key || (k4.y == key && (p4.y & kCandPos) < at)) +
+                    (k4.z > key || (k4.z == key && (p4.z & kCandPos) < at)) + (k4.w > key || (k4.w == key && (p4.w & kCandPos) < at));
         }
-        if (P.mode == OVGGT_SCORE_RANDOM) x = random_priority(P.step_key, id4[u]);   // Supp. A: uniform, fresh per step
-        fl[i] = f;
-        val[i] = x;
-        sid[i] = id4[u];
-        sst[i] = keepscore;
-        ssl[i] = sl4[u];
+        if (before == krem - 1) {
+          sh->T = key;
+          sh->posT = pos & kCandPos;
+        }
+        const bool in = before < krem;
+        if (in && owner < rank) atomicAdd(&sh->keep_before, 1);
+        if (in && (pos & kCandUp)) atomicAdd(&sh->cnt_up[owner], 1);
+        if (!in && (pos & kCandDown)) atomicAdd(&sh->cnt_down[owner], 1);
       }
-    }
-  }
-  __syncthreads();
-
-  // -- Eq. 7: min-max of each group over the whole cluster
-  float lo_h = INFINITY, hi_h = -INFINITY, lo_n = INFINITY, hi_n = -INFINITY;
-  if (P.mode == OVGGT_SCORE_HYBRID) {
-    for (int i = tid; i < cnt; i += nthr)
-      if (fl[i] == 0) {
-        const float x = val[i];
-        if (begin + i < n) { lo_h = fminf(lo_h, x); hi_h = fmaxf(hi_h, x); }
-        else               { lo_n = fminf(lo_n, x); hi_n = fmaxf(hi_n, x); }
-      }
-    block_minmax(lo_h, hi_h, sh->fscan, &lo_h, &hi_h);
-    block_minmax(lo_n, hi_n, sh->fscan, &lo_n, &hi_n);
-    if (tid == 0) {
-      sh->pub_lo_h = lo_h; sh->pub_hi_h = hi_h; sh->pub_lo_n = lo_n; sh->pub_hi_n = hi_n;
-    }
-    cluster.sync();
-    if (tid < 32) {                                   // one warp gathers: lane r reads CTA r's four values
-      float a = INFINITY, b = -INFINITY, c2 = INFINITY, d2 = -INFINITY;
-      if (tid < ncta) {
-        const SelectShared* o = cluster.map_shared_rank(sh, tid);
-        a = o->pub_lo_h; b = o->pub_hi_h; c2 = o->pub_lo_n; d2 = o->pub_hi_n;
-      }
-#pragma unroll
-      for (int off = 4; off > 0; off >>= 1) {         // kSelectMaxCtas = 8 lanes carry values
-        a = fminf(a, __shfl_xor_sync(0xFFFFFFFFu, a, off));
-        b = fmaxf(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
-        c2 = fminf(c2, __shfl_xor_sync(0xFFFFFFFFu, c2, off));
-        d2 = fmaxf(d2, __shfl_xor_sync(0xFFFFFFFFu, d2, off));
-      }
-      if (tid == 0) { sh->mm[0] = a; sh->mm[1] = b; sh->mm[2] = c2; sh->mm[3] = d2; }
-    }
-    __syncthreads();
-    lo_h = sh->mm[0]; hi_h = sh->mm[1]; lo_n = sh->mm[2]; hi_n = sh->mm[3];
-  }
-  for (int i = tid; i < cnt; i += nthr) {
-    const int g = begin + i;
-    float r;
-    uint32_t key;
-    if (fl[i] != 0) {
-      r = INFINITY;
-      key = kKeyProtected;
+      __syncthreads();
+      T = sh->T;
+      posT = sh->posT;
+      keep_before = sh->keep_before;
+      keep_all = P.B;
+      warp_totals(wlo, whi, sh, classify, &kw, &uw, &dw);
     } else {
-      if (P.mode == OVGGT_SCORE_HYBRID) {
-        const float lo = g < n ? lo_h : lo_n, hi = g < n ? hi_h : hi_n;
-        const float w = g < n ? 1.0f - P.beta : P.beta;
-        r = hi > lo ? __fmul_rn(w, __fdiv_rn(val[i] - lo, hi - lo))
-                    : ((g >= n && P.lone_new >= 0.0f) ? __fmul_rn(w, P.lone_new) : 0.0f);
-      } else {
-        r = val[i];
+      bad = radix_threshold<SINGLE>(keys, begin, cnt, P.B, sh);
+      T = sh->T;
+      posT = sh->posT;
+      warp_totals(wlo, whi, sh, classify, &kw, &uw, &dw);
+      if (tid == nthr - 32) {                          // the last warp: its prefix and its own count are the CTA's total
+        sh->pub_keep = kw + sh->wtot[kSelectWarps - 1][0];
+        sh->pub_up = uw + sh->wtot[kSelectWarps - 1][1];
+        sh->pub_down = dw + sh->wtot[kSelectWarps - 1][2];
       }
-      key = rank_key(P.override_r ? P.override_r[g] : r);
-    }
-    P.r_out[g] = r;          // the kernel's own priority, also when an override is ranked instead
-    keys[i] = key;
-  }
-  __syncthreads();
-
-  // -- Eq. 8
-  int my_base, bad;
-  const int n_keep = cluster_select(cluster, keys, keep, begin, cnt, N, P.B, P.survivors, sh, &my_base, &bad);
-
-  // -- compacted meta of this CTA's survivors (order preserved)
-  const int chunk = (cnt + nthr - 1) / nthr;
-  const int lo = min(cnt, tid * chunk), hi = min(cnt, lo + chunk);
-  int my_j;       // compacted index of this thread's first survivor
-  {
-    int c = 0;
-    for (int i = lo; i < hi; ++i) c += keep[i];
-    int tot;
-    my_j = my_base + block_excl_scan_int(c, sh->scan, &tot);
-    int j = my_j;
-    for (int i = lo; i < hi; ++i)
-      if (keep[i]) {
-        if (j < P.B) {
-          P.ids_dst[j] = sid[i];
-          P.flags_dst[j] = fl[i];
-          P.stored_dst[j] = sst[i];
-          if (P.fill) P.slot_dst[j] = ssl[i];
-        }
-        ++j;
+      G::sync();
+      if (tid < ncta) {
+        const SelectShared* o = G::of(sh, tid);
+        sh->cnt_keep[tid] = o->pub_keep;
+        sh->cnt_up[tid] = o->pub_up;
+        sh->cnt_down[tid] = o->pub_down;
       }
-  }
-  if (rank == 0 && tid == 0) {
-    *P.n_keep_out = n_keep;
-    if (bad || n_keep != min(N, P.B)) atomicCAS(P.status, 0, OVGGT_ERR_DEVICE_STATUS);
-  }
-  if (P.fill) {
-    // -- hole filling: pair the survivors that sit above slot B with the slots below B whose rows leave
-    int up = 0, down = 0;
-    for (int i = lo; i < hi; ++i) {
-      up += keep[i] && ssl[i] >= P.B;
-      down += !keep[i] && ssl[i] < P.B;
+      __syncthreads();
+      keep_before = keep_all = 0;
+      for (int r = 0; r < ncta; ++r) {
+        if (r < rank) keep_before += sh->cnt_keep[r];
+        keep_all += sh->cnt_keep[r];
+      }
     }
-    int up_tot, down_tot;
-    int up_rank = block_excl_scan_int(up, sh->scan, &up_tot);
-    int down_rank = block_excl_scan_int(down, sh->scan, &down_tot);
-    if (tid == 0) {
-      sh->pub_up = up_tot;
-      sh->pub_down = down_tot;
-    }
-    cluster.sync();
-    if (tid < ncta) {
-      sh->all_up[tid] = *cluster.map_shared_rank(&sh->pub_up, tid);
-      sh->all_down[tid] = *cluster.map_shared_rank(&sh->pub_down, tid);
-    }
-    __syncthreads();
-    int up_all = 0, down_all = 0;
     for (int r = 0; r < ncta; ++r) {
       if (r < rank) {
-        up_rank += sh->all_up[r];
-        down_rank += sh->all_down[r];
+        up_before += sh->cnt_up[r];
+        down_before += sh->cnt_down[r];
       }
-      up_all += sh->all_up[r];
-      down_all += sh->all_down[r];
+      up_all += sh->cnt_up[r];
+      down_all += sh->cnt_down[r];
     }
-    int j = my_j;
-    for (int i = lo; i < hi; ++i) {
-      if (keep[i]) {
-        if (ssl[i] >= P.B && up_rank < M) {
-          P.move_src[up_rank] = ssl[i];
-          P.move_j[up_rank] = j;
-          if (ssl[i] - P.B < M) P.tail_move[ssl[i] - P.B] = up_rank;
-          ++up_rank;
-        }
-        ++j;
-      } else if (ssl[i] < P.B) {
-        if (down_rank < M) P.move_dst[down_rank++] = ssl[i];
-      } else if (ssl[i] - P.B < M) {
-        P.tail_move[ssl[i] - P.B] = -1;           // a row above slot B that leaves: its slot is simply free
+  }
+
+  // -- survivors, compacted meta (order preserved), and the lists of rows that come and go
+  int j0 = keep_before + kw, u0 = up_before + uw, d0 = down_before + dw;
+  const unsigned below = (1u << lane) - 1;
+#pragma unroll 1
+  for (int i0 = wlo; i0 < whi; i0 += 32) {
+    const int i = i0 + lane, g = begin + i;
+    bool keep = false, up = false, down = false;
+    if (i < whi) classify(i, keep, up, down);
+    const unsigned mk = __ballot_sync(0xFFFFFFFFu, keep), mu = __ballot_sync(0xFFFFFFFFu, up),
+                   md = __ballot_sync(0xFFFFFFFFu, down);
+    const int j = j0 + __popc(mk & below), iu = u0 + __popc(mu & below), id = d0 + __popc(md & below);
+    j0 += __popc(mk);
+    u0 += __popc(mu);
+    d0 += __popc(md);
+    if (i < whi) {
+      const int slot = ssl[i];
+      const float r = keys[i] == kKeyProtected ? INFINITY : key_value(keys[i]);
+      if (own_rank && (keys[i] == kKeyProtected || fabsf(r) < INFINITY)) P.r_out[g] = r;
+      if (keep && j < P.B) {
+        P.survivors[j] = g;
+        P.ids_dst[j] = sid[i];
+        P.flags_dst[j] = (uint8_t)(bf[i] >> 14);
+        P.stored_dst[j] = sst[i];
+        if (fill) P.slot_dst[j] = slot;
       }
+      if (up && iu < M) {
+        P.move_src[iu] = slot;
+        if (fill) P.move_j[iu] = j;
+      }
+      if (down && id < M) {
+        P.move_dst[id] = slot;
+        if (fill) P.hole_stamp[slot] = P.stamp;
+      }
+      // which move empties a slot above B: none if its row leaves (or if the list is full: an inconsistency, see below)
+      if (fill && slot >= P.B && slot - P.B < M) P.tail_move[slot - P.B] = up && iu < M ? iu : -1;
     }
-    // slots above B that no row occupies yet (the cache has just filled up) hold nothing to move
-    if (rank == 0)
-      for (int i = max(0, N - P.B) + tid; i < M; i += nthr) P.tail_move[i] = -1;
-    if (rank == 0 && tid == 0) {
+  }
+  // slots above B that no row occupies yet (the cache has just filled up) hold nothing to move
+  if (fill && rank == 0)
+    for (int i = max(0, N - P.B) + tid; i < M; i += nthr) P.tail_move[i] = -1;
+  if (rank == 0 && tid == 0) {
+    *P.n_keep_out = keep_all;
+    if (bad || keep_all != min(N, P.B)) atomicCAS(P.status, 0, OVGGT_ERR_DEVICE_STATUS);
+    if (fill) {
       // the two counts agree whenever the slots below min(N, B) were all occupied, which the layout guarantees
       const bool consistent = up_all == down_all && up_all <= M;
       *P.n_moves_out = consistent ? up_all : 0;
       if (!consistent) atomicCAS(P.status, 0, OVGGT_ERR_DEVICE_STATUS);
     }
   }
-  cluster.sync();   // no CTA may exit while others still read its shared memory
+  if (P.ksum_next != nullptr) {
+    G::sync();                                    // the lists are complete; the staged rows are not needed any more
+    float* fold = reinterpret_cast<float*>(p);
+    fold_key_sums<DT, SINGLE>(P, choose ? P.move_src : nullptr, P.move_dst, choose ? min(up_all, M) : M, choose ? min(down_all, M) : 0,
+                      fold, fold + 4 * kDeltaCols);
+  }
+  G::leave();
 }
 
-__global__ void __launch_bounds__(kSelectThreads) k_compress_select(const CompressParams P) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  compress_select_body(P, smem);
+template <int DT, bool SINGLE>
+__global__ void __launch_bounds__(kSelectThreads, 2) k_compress_select(const __grid_constant__ CompressParams P) {
+  extern __shared__ __align__(16) unsigned char smem_select[];
+  compress_select_body<DT, SINGLE>(P, smem_select);
 }
 
 // The same step for several layers in one launch (Sec. 3.2: every layer has its own budget B^(l) and cache): one
@@ -579,9 +915,10 @@ constexpr int kMaxBatchLayers = 32;
 struct CompressBatch {
   CompressParams p[kMaxBatchLayers];
 };
-__global__ void __launch_bounds__(kSelectThreads) k_compress_select_batched(const __grid_constant__ CompressBatch batch) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  compress_select_body(batch.p[blockIdx.y], smem);
+template <int DT, bool SINGLE>
+__global__ void __launch_bounds__(kSelectThreads, 2) k_compress_select_batched(const __grid_constant__ CompressBatch batch) {
+  extern __shared__ __align__(16) unsigned char smem_select[];
+  compress_select_body<DT, SINGLE>(batch.p[blockIdx.y], smem_select);
 }
 
 }  // namespace ovggt
