@@ -7,6 +7,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Optional, Sequence
 
 import numpy as np
@@ -135,8 +136,10 @@ def _check(code: int, where: str) -> None:
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # (the current stream's handle without building a Stream object around it)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -144,6 +147,24 @@ def _dptr(t: Optional[torch.Tensor]) -> Optional[int]:
         return None
     assert t.is_cuda and t.is_contiguous()
     return t.data_ptr()
+
+
+def _dptr0(t: Optional[torch.Tensor]) -> int:
+    """_dptr with 0 for None."""
+    if t is None:
+        return 0
+    assert t.is_cuda and t.is_contiguous()
+    return t.data_ptr()
+
+
+def _hptr0(t: Optional[torch.Tensor]) -> int:
+    return 0 if t is None else t.data_ptr()
+
+
+# struct ovggt_frame_io as bytes: the per-frame calls fill one buffer per handle in a single pack instead of building a
+# ctypes structure field by field, which cost a small step more host time than its launches.
+_FRAME_IO = struct.Struct("@qPPPPPfPP")
+_NAN = float("nan")
 
 
 def torch_dtype(dtype: int) -> torch.dtype:
@@ -196,6 +217,9 @@ class OvggtCache:
         with torch.cuda.device(self.device):
             _check(lib().ovggt_cache_create(C.byref(self.cfg), C.byref(h)), "ovggt_cache_create")
         self._h = h
+        self._hv = h.value
+        self._io_buf = C.create_string_buffer(_FRAME_IO.size)
+        self._io_at = C.addressof(self._io_buf)
 
     @classmethod
     def from_stream(cls, cfg, **over) -> "OvggtCache":
@@ -211,7 +235,7 @@ class OvggtCache:
     def destroy(self) -> None:
         if getattr(self, "_h", None):
             lib().ovggt_cache_destroy(self._h)
-            self._h = None
+            self._h = self._hv = None
 
     def __del__(self):
         try:
@@ -230,14 +254,18 @@ class OvggtCache:
 
     def layer_attend(self, layer, frame_id, q, k, v, out=None, stream=None) -> torch.Tensor:
         out = self.new_out() if out is None else out
-        io = self._io(frame_id, q=q, k=k, v=v, out=out)
-        _check(lib().ovggt_layer_attend(self._h, layer, C.byref(io), _stream_ptr(stream)), "ovggt_layer_attend")
+        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _dptr0(q), _dptr0(k), _dptr0(v), 0, 0, _NAN, 0, _dptr0(out))
+        code = _LIB.ovggt_layer_attend_at(self._hv, layer, self._io_at, _stream_ptr(stream))
+        if code:
+            _check(code, "ovggt_layer_attend")
         return out
 
     def layer_compress(self, layer, frame_id, resid, conf=None, rho=float("nan"), score_override=None,
                        stream=None) -> None:
-        io = self._io(frame_id, resid=resid, conf=conf, rho=rho, score_override=score_override)
-        _check(lib().ovggt_layer_compress(self._h, layer, C.byref(io), _stream_ptr(stream)), "ovggt_layer_compress")
+        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), 0, 0, 0, _dptr0(resid), _dptr0(conf), rho, _dptr0(score_override), 0)
+        code = _LIB.ovggt_layer_compress_at(self._hv, layer, self._io_at, _stream_ptr(stream))
+        if code:
+            _check(code, "ovggt_layer_compress")
 
     def layers_compress(self, frame_id, resids, conf=None, rho=float("nan"), score_overrides=None, stream=None) -> None:
         """ovggt_layers_compress: resids[l] (and optionally score_overrides[l]) per layer, one call for all layers."""
@@ -256,9 +284,11 @@ class OvggtCache:
         return bool(reg.value), int(dem.value)
 
     def camera_compress(self, layer, frame_id, resid, registered, demoted_frame, score_override=None, stream=None) -> None:
-        io = self._io(frame_id, resid=resid, score_override=score_override)
-        _check(lib().ovggt_camera_compress(self._h, layer, C.byref(io), int(bool(registered)), int(demoted_frame),
-                                           _stream_ptr(stream)), "ovggt_camera_compress")
+        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), 0, 0, 0, _dptr0(resid), 0, _NAN, _dptr0(score_override), 0)
+        code = _LIB.ovggt_camera_compress_at(self._hv, layer, self._io_at, 1 if registered else 0, int(demoted_frame),
+                                             _stream_ptr(stream))
+        if code:
+            _check(code, "ovggt_camera_compress")
 
     @classmethod
     def camera(cls, *, n_layers=1, n_heads=16, head_dim=64, budget=144, k_max=3, beta=0.5, protect_first_frame=1,
@@ -271,14 +301,20 @@ class OvggtCache:
     def layer_step(self, layer, frame_id, q, k, v, resid, conf=None, rho=float("nan"), score_override=None,
                    out=None, stream=None) -> torch.Tensor:
         out = self.new_out() if out is None else out
-        io = self._io(frame_id, q, k, v, resid, conf, rho, score_override, out)
-        _check(lib().ovggt_layer_step(self._h, layer, C.byref(io), _stream_ptr(stream)), "ovggt_layer_step")
+        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _dptr0(q), _dptr0(k), _dptr0(v), _dptr0(resid), _dptr0(conf), rho,
+                            _dptr0(score_override), _dptr0(out))
+        code = _LIB.ovggt_layer_step_at(self._hv, layer, self._io_at, _stream_ptr(stream))
+        if code:
+            _check(code, "ovggt_layer_step")
         return out
 
     def layer_step_host(self, layer, frame_id, q, k, v, resid, conf, rho, out, stream=None) -> None:
         """All tensors are host (ideally pinned) torch tensors; the copies run inside the call."""
-        io = self._io(frame_id, q, k, v, resid, conf, rho, None, out, host=True)
-        _check(lib().ovggt_layer_step_host(self._h, layer, C.byref(io), _stream_ptr(stream)), "ovggt_layer_step_host")
+        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _hptr0(q), _hptr0(k), _hptr0(v), _hptr0(resid), _hptr0(conf), rho, 0,
+                            _hptr0(out))
+        code = _LIB.ovggt_layer_step_host_at(self._hv, layer, self._io_at, _stream_ptr(stream))
+        if code:
+            _check(code, "ovggt_layer_step_host")
 
     def stats(self, layer=0) -> dict:
         st = OvggtStats()
