@@ -772,21 +772,26 @@ inline int make_rows_map(CUtensorMap* map, const void* base, int rows, int C, in
   return OVGGT_OK;
 }
 
-// Number of KV splits: minimise (waves of CTAs over 2 x 148 slots) x (tiles per CTA + fixed overhead).
+// Number of KV splits, from a model in nanoseconds fitted to a sweep of 1 to 16 splits over eighteen shapes (69 x 325 x 4
+// heads to 1374 x 34142 x 16): waves of CTAs over 2 x 148 slots; 1.25 us per tile for a CTA that has its SM to itself,
+// 1.85 us where two share one; 4 us per CTA for set-up and epilogue; a merge is 3 us and passes over the partial outputs
+// (write and read) at 6 TB/s.  The merge is what short KV ranges cannot pay: 1041 x 1041 x 16 takes 14.5 us unsplit and
+// 20.6 us in two splits, whose CTAs alone would be faster.
 inline int attn_choose_splits(int M, int N, int H) {
   const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kBN - 1) / kBN;
   const long slots = (long)kCtasPerSm * 148;
   int best = 1;
-  long best_cost = -1;
+  long best_ns = -1;
   for (int s = 1; s <= kMaxSplits && s <= tiles; ++s) {
     const int per = (tiles + s - 1) / s;
     const int eff = (tiles + per - 1) / per;
     if (eff != s) continue;
     const long ctas = (long)q_tiles * H * s;
     const long waves = (ctas + slots - 1) / slots;
-    const long cost = waves * (per + 384 / kBN) + (s > 1 ? 256 / kBN : 0);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
+    const long ns = waves * (per * (ctas <= 148 ? 1250l : 1850l) + 4000) +
+                    (s > 1 ? 3000 + (long)s * M * H * kHD * 8 / 6000 : 0);
+    if (best_ns < 0 || ns < best_ns) {
+      best_ns = ns;
       best = s;
     }
   }
