@@ -354,6 +354,14 @@ int ovggt_k_attention_bounded(const void* q, const void* k, const void* v, int32
  * multiple of 64 and N of 8 (OVGGT_ERR_UNSUPPORTED otherwise).  device_status: device int, as for ovggt_k_attention. */
 int ovggt_k_gemm_bf16(const void* A, const void* B, int32_t M, int32_t N, int32_t K, void* C, int32_t* device_status,
                       void* stream);
+/* The same product with what usually follows it in the epilogue.  t = bf16(A B), or bf16(gelu(bf16(A B))) (the exact,
+ * erf-based GELU) with gelu != 0.  n_outs = 1: t to outs[0] [M, N]; 2 or 3: column block i of t to outs[i] [M, N / n_outs]
+ * (a QKV product; N / n_outs a multiple of 8); 0: t is not stored.  residual [M, N] and sum [M, N], both or neither:
+ * sum = bf16(residual + t).  outs is a host array of device pointers; sum may not be residual or A. */
+int ovggt_k_linear_bf16(const void* A, const void* B, int32_t M, int32_t N, int32_t K, void* const* outs, int32_t n_outs,
+                        int32_t gelu, const void* residual, void* sum, int32_t* device_status, void* stream);
+/* out [rows, C] = LayerNorm of the rows of x (bf16, no affine part, epsilon 1e-5, fp32 arithmetic); C a multiple of 8. */
+int ovggt_k_layer_norm_bf16(const void* x, int32_t rows, int32_t C, void* out, void* stream);
 
 #ifdef __cplusplus
 }

@@ -33,6 +33,7 @@ EXPORTED = [
     "ovggt_strerror", "ovggt_last_cuda_error", "ovggt_k_row_norms", "ovggt_k_diversity_scratch_bytes",
     "ovggt_k_diversity", "ovggt_k_diversity_static", "ovggt_k_select", "ovggt_k_compact", "ovggt_k_attention_scratch_bytes",
     "ovggt_k_attention", "ovggt_k_key_norm_bound", "ovggt_k_attention_bounded", "ovggt_k_gemm_bf16",
+    "ovggt_k_linear_bf16", "ovggt_k_layer_norm_bf16",
 ]
 
 
@@ -125,7 +126,17 @@ def lib():
         L.ovggt_k_attention.argtypes = [vp, vp, vp, i32, i32, i32, i32, vp, vp, vp, vp]
         L.ovggt_k_key_norm_bound.argtypes = [vp, i32, i32, vp, vp]
         L.ovggt_k_gemm_bf16.argtypes = [vp, vp, i32, i32, i32, vp, vp, vp]
+        L.ovggt_k_linear_bf16.argtypes = [vp, vp, i32, i32, i32, C.POINTER(vp), i32, i32, vp, vp, vp, vp]
+        L.ovggt_k_layer_norm_bf16.argtypes = [vp, i32, i32, vp, vp]
         L.ovggt_k_attention_bounded.argtypes = [vp, vp, vp, i32, i32, i32, vp, vp, vp, vp, vp]
+        assert _FRAME_IO.size == C.sizeof(OvggtFrameIO)
+        for name in ("ovggt_layer_attend", "ovggt_layer_compress", "ovggt_layer_step", "ovggt_layer_step_host"):
+            f = L[name]                                   # (a second function object: the frame as a plain address)
+            f.argtypes = [vp, i32, vp, vp]
+            setattr(L, name + "_at", f)
+        f = L["ovggt_camera_compress"]
+        f.argtypes = [vp, i32, vp, i32, i64, vp]
+        L.ovggt_camera_compress_at = f
         _LIB = L
     return _LIB
 
@@ -447,6 +458,20 @@ def k_gemm_bf16(a: torch.Tensor, b: torch.Tensor, out=None, status=None, stream=
            "ovggt_k_gemm_bf16")
     if own:
         _check(int(status[0].item()), "ovggt_k_gemm_bf16 (device status)")
+    return out
+
+
+def k_linear_bf16(a, b, outs=(), gelu=False, residual=None, sum_out=None, status=None, stream=None) -> None:
+    """t = a [M, K] @ b [K, N] (then GELU); its column blocks to outs; sum_out = residual + t.  Nothing is allocated."""
+    M, K = a.shape
+    _check(lib().ovggt_k_linear_bf16(_dptr(a), _dptr(b), M, b.shape[1], K, (C.c_void_p * 3)(*[_dptr(o) for o in outs]), len(outs),
+                                     int(gelu), _dptr(residual), _dptr(sum_out), _dptr(status), _stream_ptr(stream)),
+           "ovggt_k_linear_bf16")
+
+
+def k_layer_norm_bf16(x: torch.Tensor, out: torch.Tensor, stream=None) -> torch.Tensor:
+    _check(lib().ovggt_k_layer_norm_bf16(_dptr(x), x.shape[0], x.shape[1], _dptr(out), _stream_ptr(stream)),
+           "ovggt_k_layer_norm_bf16")
     return out
 
 

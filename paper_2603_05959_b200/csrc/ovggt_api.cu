@@ -1444,15 +1444,46 @@ extern "C" int ovggt_k_attention_bounded(const void* q, const void* k, const voi
                           nullptr, kmax2);
 }
 
-extern "C" int ovggt_k_gemm_bf16(const void* A, const void* Bm, int32_t M, int32_t N, int32_t K, void* C,
-                                 int32_t* device_status, void* stream) {
-  if (!A || !Bm || !C || !device_status || M < 1 || N < 1 || K < 1) return OVGGT_ERR_INVALID_ARG;
-  if (K % 64 != 0 || N % 8 != 0) return OVGGT_ERR_UNSUPPORTED;
-  if (!aligned16(A) || !aligned16(Bm) || !aligned16(C)) return OVGGT_ERR_MISALIGNED;
-  int rc = gemm_tcgen05_launch(A, Bm, C, M, N, K, device_status, static_cast<cudaStream_t>(stream));
+extern "C" int ovggt_k_linear_bf16(const void* A, const void* Bm, int32_t M, int32_t N, int32_t K, void* const* outs,
+                                   int32_t n_outs, int32_t gelu, const void* residual, void* sum, int32_t* device_status,
+                                   void* stream) {
+  if (!A || !Bm || !device_status || M < 1 || N < 1 || K < 1 || n_outs < 0 || n_outs > 3 || (n_outs > 0 && !outs) ||
+      (residual != nullptr) != (sum != nullptr) || (n_outs == 0 && !sum))
+    return OVGGT_ERR_INVALID_ARG;
+  if (K % 64 != 0 || N % 8 != 0 || (n_outs > 1 && (N % n_outs != 0 || (N / n_outs) % 8 != 0))) return OVGGT_ERR_UNSUPPORTED;
+  if (!aligned16(A) || !aligned16(Bm) || !aligned16(residual) || !aligned16(sum)) return OVGGT_ERR_MISALIGNED;
+  GemmArgs P = {};
+  P.M = M; P.N = N; P.K = K;
+  for (int i = 0; i < n_outs; ++i) {
+    if (!outs[i]) return OVGGT_ERR_INVALID_ARG;
+    if (!aligned16(outs[i])) return OVGGT_ERR_MISALIGNED;
+    P.out[i] = static_cast<__nv_bfloat16*>(outs[i]);
+  }
+  P.part = n_outs > 1 ? N / n_outs : N;
+  P.gelu = gelu != 0;
+  P.residual = static_cast<const __nv_bfloat16*>(residual);
+  P.sum = static_cast<__nv_bfloat16*>(sum);
+  P.status = device_status;
+  int rc = gemm_tcgen05_launch(A, Bm, P, static_cast<cudaStream_t>(stream));
   if (rc == OVGGT_OK) g_launches.fetch_add(1);
   if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
   return rc;
+}
+
+extern "C" int ovggt_k_gemm_bf16(const void* A, const void* Bm, int32_t M, int32_t N, int32_t K, void* C,
+                                 int32_t* device_status, void* stream) {
+  if (!C) return OVGGT_ERR_INVALID_ARG;
+  return ovggt_k_linear_bf16(A, Bm, M, N, K, &C, 1, 0, nullptr, nullptr, device_status, stream);
+}
+
+extern "C" int ovggt_k_layer_norm_bf16(const void* x, int32_t rows, int32_t C, void* out, void* stream) {
+  if (rows == 0) return OVGGT_OK;
+  if (!x || !out || rows < 0 || C < 8 || C % 8 != 0) return OVGGT_ERR_INVALID_ARG;
+  if (!aligned16(x) || !aligned16(out)) return OVGGT_ERR_MISALIGNED;
+  CK(launch_dependent(k_layer_norm_bf16, dim3((rows + 7) / 8), 256, 1, 0, static_cast<cudaStream_t>(stream), true,
+                      (const uint4*)x, (int)rows, (int)(C / 8), (uint4*)out));
+  g_launches.fetch_add(1);
+  return OVGGT_OK;
 }
 
 // ------------------------------------------------------------------ allocation-free diversity

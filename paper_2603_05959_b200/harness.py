@@ -108,19 +108,58 @@ class _Timer:
         return t
 
 
-class _Matmul:
-    """x @ W of the scaffold: torch's matmul, or the library's own tcgen05 GEMM (ovggt_k_gemm_bf16).  Either way it is
-    scaffold time, not the streaming step's."""
+class _Scaffold:
+    """The dense products of a workload and what surrounds them: on torch, or on the library's own kernels
+    (ovggt_k_linear_bf16 with GELU, residual sum and the split of a QKV product in its epilogue; ovggt_k_layer_norm_bf16;
+    buffers that are kept between frames).  Both round to bf16 at the same places.  Either way it is scaffold time, not
+    the streaming step's."""
 
     def __init__(self, kind: str, device):
         assert kind in ("torch", "library")
-        self.kind = kind
+        self.library = kind == "library"
+        self.device = device
         self.status = torch.zeros(16, dtype=torch.int32, device=device)
+        self._kept = {}
 
-    def __call__(self, x: torch.Tensor, w: torch.Tensor, stream=None) -> torch.Tensor:
-        if self.kind == "torch":
-            return x @ w
-        return B.k_gemm_bf16(x.contiguous(), w, status=self.status, stream=stream)
+    def kept(self, name, shape) -> torch.Tensor:
+        t = self._kept.get(name)
+        if t is None:
+            t = self._kept[name] = torch.empty(shape, dtype=torch.bfloat16, device=self.device)
+        return t
+
+    def layer_norm(self, x, stream=None):
+        if self.library:
+            return B.k_layer_norm_bf16(x, self.kept("ln", x.shape), stream)
+        return torch.nn.functional.layer_norm(x.float(), (x.shape[-1],)).to(x.dtype)
+
+    def qkv(self, x, w, stream=None):
+        """The three [M, C] column blocks of x W."""
+        M, C = x.shape[0], w.shape[1] // 3
+        if self.library:
+            out = [self.kept("qkv%d" % i, (M, C)) for i in range(3)]
+            B.k_linear_bf16(x, w, out, status=self.status, stream=stream)
+            return out
+        y = x @ w
+        return [y[:, i * C:(i + 1) * C].contiguous() for i in range(3)]
+
+    def add_product(self, x, a, w, out=None, product=None, stream=None):
+        """x + a W, to `out` if given; the product itself to `product` if given."""
+        if self.library:
+            out = torch.empty_like(x) if out is None else out
+            B.k_linear_bf16(a, w, () if product is None else (product,), residual=x, sum_out=out, status=self.status,
+                            stream=stream)
+            return out
+        y = a @ w
+        if product is not None:
+            product.copy_(y)
+        return torch.add(x, y, out=out) if out is not None else x + y
+
+    def gelu_product(self, x, w, stream=None):
+        if self.library:
+            h = self.kept("hidden", (x.shape[0], w.shape[1]))
+            B.k_linear_bf16(x, w, (h,), gelu=True, status=self.status, stream=stream)
+            return h
+        return torch.nn.functional.gelu(x @ w)
 
     def check(self) -> None:
         assert int(self.status[0].item()) == 0
@@ -140,7 +179,7 @@ class ProjectionStack:
     def __init__(self, cfg: gen.StreamConfig, device, compaction: int = B.COMPACT_FILL_HOLES, matmul: str = "library"):
         assert cfg.dtype == gen.DTYPE_BF16
         self.cfg, self.device = cfg, device
-        self.mm = _Matmul(matmul, device)
+        self.mm = _Scaffold(matmul, device)
         self.cache = B.OvggtCache.from_stream(cfg, device=device, compaction=compaction)
         g = torch.Generator(device=device)
         g.manual_seed(cfg.seed)
@@ -154,27 +193,25 @@ class ProjectionStack:
     def frame(self, t: int, x: torch.Tensor, resid: List[torch.Tensor], conf: torch.Tensor, rho: float, stream,
               lib: Optional[_Timer] = None) -> torch.Tensor:
         """x: [M, C] patch embeddings of frame t (bf16).  resid[l]: the layer's synthetic residual rows."""
-        C = self.cfg.dim
-        for l in range(self.cfg.n_layers):
+        L, mm = self.cfg.n_layers, self.mm
+        x = x.contiguous()
+        for l in range(L):
             # embeddings are N(0, 1) over 1024 columns and the weights N(0, 0.02): q, k, v come out near N(0, 0.4)
-            qkv = self.mm(x, self.w_qkv[l], stream)
-            q, k, v = (qkv[:, i * C:(i + 1) * C].contiguous() for i in range(3))
+            q, k, v = mm.qkv(x, self.w_qkv[l], stream)
             ov = self.tap(t, l, q, k, v, resid[l]) if self.tap else None
             run = lambda: self.cache.layer_step(l, t, q, k, v, resid[l], conf, rho, score_override=ov, out=self.out,
                                                 stream=stream)
             lib(run) if lib else run()
             if self.after:
                 self.after(t, l, self.out)
-            x = x + self.mm(self.out, self.w_o[l], stream)
+            # (the frame's result is the caller's; what is passed between the layers is kept)
+            x = mm.add_product(x, self.out, self.w_o[l], out=None if l + 1 == L else mm.kept("x%d" % (l & 1), x.shape),
+                               stream=stream)
         return x
 
     def destroy(self) -> None:
         self.mm.check()
         self.cache.destroy()
-
-
-def _layer_norm(x: torch.Tensor) -> torch.Tensor:
-    return torch.nn.functional.layer_norm(x.float(), (x.shape[-1],)).to(x.dtype)
 
 
 class Aggregator:
@@ -192,7 +229,7 @@ class Aggregator:
         (ovggt_k_attention with N = M: the same kernel that serves the cache); "torch" uses torch's SDPA.
         matmul: "library" runs every projection and MLP product on ovggt_k_gemm_bf16; "torch" on torch's matmul."""
         self.batched_compress = batched_compress
-        self.mm = _Matmul(matmul, device)
+        self.mm = _Scaffold(matmul, device)
         self.frame_attention = frame_attention
         M, H = cfg.tokens_per_frame, cfg.n_heads
         self._fa_scratch = torch.empty(B.lib().ovggt_k_attention_scratch_bytes(M, M, H), dtype=torch.uint8, device=device)
@@ -211,35 +248,37 @@ class Aggregator:
         self.tap: Optional[Callable] = None
         self.after: Optional[Callable] = None
 
-    def _mlp(self, w, h, stream=None):
-        return self.mm(torch.nn.functional.gelu(self.mm(_layer_norm(h), w["fc1"], stream)), w["fc2"], stream)
-
     def frame(self, t: int, x: torch.Tensor, conf: torch.Tensor, rho: float, stream,
               lib: Optional[_Timer] = None) -> torch.Tensor:
-        cfg = self.cfg
-        C, H, M = cfg.dim, cfg.n_heads, cfg.tokens_per_frame
+        cfg, mm = self.cfg, self.mm
+        C, H, M, L = cfg.dim, cfg.n_heads, cfg.tokens_per_frame, cfg.n_layers
         resids, overrides = [], []
-        for l in range(cfg.n_layers):
+        x = x.contiguous()
+        keep = (lambda name: mm.kept(name, (M, C)))
+        for l in range(L):
             w = self.blocks[l]["frame"]
-            qkv = self.mm(_layer_norm(x), w["qkv"], stream)
+            fq, fk, fv = mm.qkv(mm.layer_norm(x, stream), w["qkv"], stream)
             if self.frame_attention == "library":
-                fq, fk, fv = (qkv[:, i * C:(i + 1) * C].contiguous() for i in range(3))
                 a = B.k_attention(fq, fk, fv, H, out=self._fa_out, scratch=self._fa_scratch, status=self._fa_status,
                                   stream=stream)
             else:
-                q3 = qkv.view(M, 3, H, C // H).permute(1, 2, 0, 3)                               # [3, H, M, d]
-                a = torch.nn.functional.scaled_dot_product_attention(q3[0], q3[1], q3[2]).permute(1, 0, 2).reshape(M, C)
-            x = x + self.mm(a, w["o"], stream)
-            x = x + self._mlp(w, x, stream)
+                q3 = [y.view(M, H, C // H).permute(1, 0, 2) for y in (fq, fk, fv)]               # [H, M, d]
+                a = torch.nn.functional.scaled_dot_product_attention(*q3).permute(1, 0, 2).reshape(M, C)
+            x = mm.add_product(x, a, w["o"], out=keep("frame attended"), stream=stream)
+            x = mm.add_product(x, mm.gelu_product(mm.layer_norm(x, stream), w["fc1"], stream), w["fc2"],
+                               out=keep("frame out"), stream=stream)
             w = self.blocks[l]["global"]
-            qkv = self.mm(_layer_norm(x), w["qkv"], stream)
-            q, k, v = (qkv[:, i * C:(i + 1) * C].contiguous() for i in range(3))
+            q, k, v = mm.qkv(mm.layer_norm(x, stream), w["qkv"], stream)
             att = lambda: self.cache.layer_attend(l, t, q, k, v, out=self.out, stream=stream)
             lib(att) if lib else att()
             if self.after:
                 self.after(t, l, self.out)
-            h = x + self.mm(self.out, w["o"], stream)
-            r = self._mlp(w, h, stream).contiguous()
+            h = mm.add_product(x, self.out, w["o"], out=keep("global attended"), stream=stream)
+            # the block's MLP output is the layer's residual, read by its compress: one buffer per layer
+            r = keep("resid%d" % (l if self.batched_compress else 0))
+            # (the frame's result is the caller's; what is passed between the layers is kept)
+            x = mm.add_product(h, mm.gelu_product(mm.layer_norm(h, stream), w["fc1"], stream), w["fc2"],
+                               out=None if l + 1 == L else keep("global out"), product=r, stream=stream)
             ov = self.tap(t, l, q, k, v, r) if self.tap else None
             if self.batched_compress:
                 resids.append(r)
@@ -247,7 +286,6 @@ class Aggregator:
             else:
                 cmp_ = lambda: self.cache.layer_compress(l, t, r, conf, rho, score_override=ov, stream=stream)
                 lib(cmp_) if lib else cmp_()
-            x = h + r
         if self.batched_compress:
             ovs = overrides if any(o is not None for o in overrides) else None
             cmp_ = lambda: self.cache.layers_compress(t, resids, conf, rho, score_overrides=ovs, stream=stream)
