@@ -4,18 +4,19 @@
 //
 // Not part of the streaming step itself: it is what a model wraps around it (QKV / output projections, MLP), provided
 // so that the 24-layer workloads can run their scaffold on hand-written kernels too.
-//   CTA tile 128 x 128, K in steps of 64: A tile [128 rows, 64 k] K-major (16 KB), B tile [64 k, 128 n] as two
-//   [64 k, 64 n] boxes, N-major as the tensor lies in memory (2 x 8 KB), read by one N = 128 MMA per 16 k whose
-//   descriptor names the distance between the boxes; three stages;
-//   warp 0 produces (TMA), warp 1 issues the MMAs, accumulators in TMEM columns [0, 128), warps 2-5 read them back (one
-//   thread per output row), finish and store.
-// At these sizes (1041 or 1374 rows, N and K of 1024 to 4096) a product is 72 to 352 tiles of 2 to 9 us each, so it is
-// the number of tiles in flight that matters, not the peak rate of one: 96 KB of stages let two CTAs share an SM (one
-// fills or drains while the other multiplies), and a product with fewer tiles than SMs is cut along K over a cluster
-// of two CTAs, each of which finishes half of the columns with the other's partial sums, sent through distributed shared
-// memory.  The kernel is launched programmatically behind its predecessor, so set-up runs under that one's drain.
-// (Before: N = 64 MMAs, four stages and one CTA per SM, no split: 17.9 / 8.9 / 16.6 / 22.7 us for the QKV, output, first
-// and second MLP product of 1041 rows, and 45 element-wise launches per layer around them.)
+//   CTA tile 128 x BN (256 or 128), K in steps of 64: A tile [128 rows, 64 k] K-major (16 KB), B tile [64 k, BN n] as
+//   [64 k, 64 n] boxes, N-major as the tensor lies in memory (8 KB each), read by one N = BN MMA per 16 k whose descriptor
+//   names the distance between the boxes; 192 KB of stages, one CTA per SM;
+//   warp 16 produces (TMA), warp 17 issues the MMAs, accumulators in BN TMEM columns; warps 0-15 read them back, one thread
+//   per output row and quarter of the columns, finish, and store whole lines by way of shared memory.
+// What bounds it at these sizes (1041 or 1374 rows, N and K of 1024 to 4096): one wave of CTAs whose loads all come from
+// L2, and shared memory, which the MMA reads and TMA writes at 128 bytes a clock each at N = 128 (half the tensor rate)
+// and at 94 at N = 256; hence the wide tile, all of shared memory in flight, and K cut over a cluster of two or four CTAs
+// where a product has few tiles: each CTA finishes its share of the columns with the others' partial sums, sent through
+// distributed shared memory into the stages.  The kernel is launched programmatically behind its predecessor and
+// prefetches its part of B (weights, as a rule) into L2 while that one drains.
+// Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 10.5 / 7.3 / 14.1 / 14.8 us, against
+// 13.9 / 9.2 / 18.1 / 19.4 with 128 x 128 tiles of three stages and four epilogue warps that stored row by row.
 // Requirements: K a multiple of 64, N a multiple of 8 (TMA row pitch of 16 bytes), 16-byte aligned bases.  Every
 // barrier wait is bounded (about one second); on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the
 // common teardown, after the MMAs it issued have drained.
@@ -27,21 +28,21 @@
 
 namespace ovggt {
 
-constexpr int kGemmBM = 128, kGemmBN = 128, kGemmBK = 64, kGemmStages = 3;
-constexpr int kGemmThreads = 192;
+constexpr int kGemmBM = 128, kGemmBK = 64;
+constexpr int kGemmEpilogueWarps = 16, kGemmThreads = (kGemmEpilogueWarps + 2) * 32;
 constexpr int kGemmATile = kGemmBM * kGemmBK * 2;          // 16 KB
 constexpr int kGemmBBox = kGemmBK * 64 * 2;                // 8 KB: [64 k, 64 n]
-constexpr int kGemmBTile = 2 * kGemmBBox;                  // 16 KB
-constexpr int kGemmTmemCols = 128;
-constexpr int kGemmExchange = kGemmBM * (kGemmBN / 2) * 4; // 32 KB: half a tile of fp32 partial sums from the other CTA
+constexpr int kGemmMaxStages = 6;
+__host__ __device__ constexpr int gemm_stage_bytes(int bn) { return kGemmATile + bn / 64 * kGemmBBox; }
+__host__ __device__ constexpr int gemm_stages(int bn) { return bn == 256 ? 4 : 6; }
 
 struct GemmBarriers {
-  unsigned long long full[kGemmStages], empty[kGemmStages], acc_full, drain;
+  unsigned long long full[kGemmMaxStages], empty[kGemmMaxStages], acc_full, drain;
   uint32_t tmem_base;
   int abort_flag;
 };
-__host__ __device__ constexpr size_t gemm_smem_bytes(bool split) {
-  return (size_t)kGemmStages * (kGemmATile + kGemmBTile) + (split ? kGemmExchange : 0) + sizeof(GemmBarriers) + 64;
+__host__ __device__ constexpr size_t gemm_smem_bytes(int bn) {
+  return (size_t)gemm_stages(bn) * gemm_stage_bytes(bn) + sizeof(GemmBarriers) + 64;
 }
 
 struct GemmArgs {
@@ -55,24 +56,35 @@ struct GemmArgs {
   int* status;
 };
 
-__device__ __forceinline__ float gelu_exact(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
+// x Phi(x) = x erfc(-x / sqrt 2) / 2 for a pair.  erfc(z), z >= 0, by the Chebyshev fit of Press et al. (Numerical Recipes,
+// erfcc): t exp(-z^2 + q(t)), t = 1 / (1 + z / 2), fractional error below 1.2e-7 everywhere; Phi(x) = 1 - erfc / 2 above 0.
+__device__ __forceinline__ float2 gelu2(float2 x) {
+  const float2 z = make_float2(fabsf(x.x) * 0.70710678118654752f, fabsf(x.y) * 0.70710678118654752f);
+  const float2 t = make_float2(__fdividef(1.0f, fmaf(0.5f, z.x, 1.0f)), __fdividef(1.0f, fmaf(0.5f, z.y, 1.0f)));
+  auto both = [](float c) { return make_float2(c, c); };
+  float2 q = fma2(t, both(0.17087277f), both(-0.82215223f));
+  q = fma2(q, t, both(1.48851587f));
+  q = fma2(q, t, both(-1.13520398f));
+  q = fma2(q, t, both(0.27886807f));
+  q = fma2(q, t, both(-0.18628806f));
+  q = fma2(q, t, both(0.09678418f));
+  q = fma2(q, t, both(0.37409196f));
+  q = fma2(q, t, both(1.00002368f));
+  q = fma2(q, t, both(-1.26551223f));
+  q = fma2(z, make_float2(-z.x, -z.y), q);
+  const float e0 = 0.5f * t.x * ex2(q.x * 1.4426950408889634f), e1 = 0.5f * t.y * ex2(q.y * 1.4426950408889634f);
+  return make_float2(x.x * (x.x > 0.0f ? 1.0f - e0 : e0), x.y * (x.y > 0.0f ? 1.0f - e1 : e1));
+}
 
-// Eight finished columns [n, n + 8) of row m.
-__device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, const float* acc) {
-  uint4 t;
-  uint32_t* w = reinterpret_cast<uint32_t*>(&t);
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    w[e] = pack_bf16(acc[2 * e], acc[2 * e + 1]);
-    if (P.gelu)
-      w[e] = pack_bf16(gelu_exact(__uint_as_float(w[e] << 16)), gelu_exact(__uint_as_float(w[e] & 0xFFFF0000u)));
-  }
+// Finished bf16 columns [n, n + 8) of row m: where the caller wants them.
+__device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, const uint4& t) {
   if (P.out[0] != nullptr) {
     const int i = n / P.part;       // (8 columns lie in one part: its width is a multiple of 8)
     __nv_bfloat16* o = i == 0 ? P.out[0] : (i == 1 ? P.out[1] : P.out[2]);
     *reinterpret_cast<uint4*>(o + (size_t)m * P.part + (n - i * P.part)) = t;
   }
   if (P.residual != nullptr) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(&t);
     const uint4 r = *reinterpret_cast<const uint4*>(P.residual + (size_t)m * P.N + n);
     const uint32_t* rw = reinterpret_cast<const uint32_t*>(&r);
     uint4 s;
@@ -85,28 +97,30 @@ __device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, con
   }
 }
 
-// SPLIT: launched as clusters of two CTAs, neighbours in x, each with half of the K steps of one tile.
-template <bool SPLIT>
-__global__ void __launch_bounds__(kGemmThreads, SPLIT ? 1 : 2)
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
+}
+
+// SPLIT > 1: launched as clusters of SPLIT CTAs, neighbours in x, each with its part of the K steps of one tile.
+template <int BN, int SPLIT>
+__global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                     const __grid_constant__ GemmArgs P) {
+  constexpr int kStages = gemm_stages(BN), kStage = gemm_stage_bytes(BN);
+  constexpr int kProducer = kGemmEpilogueWarps, kIssuer = kGemmEpilogueWarps + 1;
   extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sA = smem;
-  unsigned char* sB = sA + kGemmStages * kGemmATile;
-  float* xch = reinterpret_cast<float*>(sB + kGemmStages * kGemmBTile);     // [64 columns][128 rows], SPLIT only
-  GemmBarriers* B = reinterpret_cast<GemmBarriers*>(sB + kGemmStages * kGemmBTile + (SPLIT ? kGemmExchange : 0));
+  GemmBarriers* B = reinterpret_cast<GemmBarriers*>(smem + kStages * kStage);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * kGemmBM, n0 = (SPLIT ? blockIdx.x >> 1 : blockIdx.x) * kGemmBN;
-  const int half = SPLIT ? (int)(blockIdx.x & 1) : 0;
-  const int k_all = P.K / kGemmBK;
-  const int k_begin = SPLIT && half ? (k_all + 1) / 2 : 0, k_tiles = (SPLIT && !half ? (k_all + 1) / 2 : k_all) - k_begin;
-  bool aligned = (smem_u32(smem) & 1023u) == 0;     // the 128-byte swizzle needs 1024-byte aligned tiles
+  const int m0 = blockIdx.y * kGemmBM, n0 = (int)(blockIdx.x / SPLIT) * BN, part = (int)(blockIdx.x % SPLIT);
+  const int k_all = P.K / kGemmBK, k_begin = k_all * part / SPLIT, k_tiles = k_all * (part + 1) / SPLIT - k_begin;
+  const bool aligned = (smem_u32(smem) & 1023u) == 0;     // the 128-byte swizzle needs 1024-byte aligned tiles
   if (!aligned && threadIdx.x == 0) atomicCAS(P.status, 0, OVGGT_ERR_DEVICE_STATUS);
+  pdl_trigger();
 
-  if (warp == 0 && lane == 0) {
+  if (warp == kProducer && lane == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_a) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_b) : "memory");
-    for (int s = 0; s < kGemmStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&B->full[s], 1);
       mbar_init(&B->empty[s], 1);
     }
@@ -115,10 +129,13 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     B->abort_flag = aligned ? 0 : 1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // the CTAs of one column of tiles share its part of B out among them
+    for (int kt = (int)blockIdx.y; kt < k_tiles; kt += (int)gridDim.y)
+      for (int x = 0; x < BN && n0 + x < P.N; x += 64) tma_prefetch_2d(&tm_b, n0 + x, (k_begin + kt) * kGemmBK);
   }
-  if (warp == 1) {
+  if (warp == kIssuer) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&B->tmem_base)),
-                 "r"((uint32_t)kGemmTmemCols)
+                 "r"((uint32_t)BN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -126,44 +143,45 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *(volatile uint32_t*)&B->tmem_base;
-  if constexpr (SPLIT) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   pdl_wait();
 
   bool ok = aligned;
-  if (warp == 0) {
+  if (warp == kProducer) {
     // ------------------------------------------------ TMA producer
     if (lane == 0) {
       int issued = 0;
       for (int kt = 0; kt < k_tiles && ok; ++kt) {
-        const int s = kt % kGemmStages;
-        const uint32_t ph = (uint32_t)(kt / kGemmStages) & 1u;
-        if (kt >= kGemmStages) ok = mbar_wait(&B->empty[s], ph ^ 1u, B, P.status);
+        const int s = kt % kStages;
+        const uint32_t ph = (uint32_t)(kt / kStages) & 1u;
+        if (kt >= kStages) ok = mbar_wait(&B->empty[s], ph ^ 1u, B, P.status);
         if (!ok) break;
         const int k0 = (k_begin + kt) * kGemmBK;
-        mbar_expect_tx(&B->full[s], kGemmATile + kGemmBTile);
-        tma_load_2d(sA + s * kGemmATile, &tm_a, k0, m0, &B->full[s]);
-        tma_load_2d(sB + s * kGemmBTile, &tm_b, n0, k0, &B->full[s]);
-        tma_load_2d(sB + s * kGemmBTile + kGemmBBox, &tm_b, n0 + 64, k0, &B->full[s]);
+        unsigned char* st = smem + s * kStage;
+        mbar_expect_tx(&B->full[s], kStage);
+        tma_load_2d(st, &tm_a, k0, m0, &B->full[s]);
+#pragma unroll
+        for (int x = 0; x < BN / 64; ++x)
+          tma_load_2d(st + kGemmATile + x * kGemmBBox, &tm_b, n0 + x * 64, k0, &B->full[s]);
         ++issued;
       }
       if (!ok)   // leave no bulk copy in flight into this CTA's shared memory
-        for (int i = max(0, issued - kGemmStages); i < issued; ++i)
-          mbar_wait(&B->full[i % kGemmStages], (uint32_t)(i / kGemmStages) & 1u, B, P.status);
+        for (int i = max(0, issued - kStages); i < issued; ++i)
+          mbar_wait(&B->full[i % kStages], (uint32_t)(i / kStages) & 1u, B, P.status);
     }
     __syncwarp();
-  } else if (warp == 1) {
+  } else if (warp == kIssuer) {
     // ------------------------------------------------ MMA issuer (whole warp in step, one elected lane issues)
     const bool leader = elect_one();
     const uint32_t tm = __reduce_or_sync(0xFFFFFFFFu, tmem);
-    constexpr uint32_t idesc = idesc_bf16(kGemmBN, true);       // A K-major, B N-major
+    constexpr uint32_t idesc = idesc_bf16(BN, true);            // A K-major, B N-major
     for (int kt = 0; kt < k_tiles && ok; ++kt) {
-      const int s = kt % kGemmStages;
-      const uint32_t ph = (uint32_t)(kt / kGemmStages) & 1u;
+      const int s = kt % kStages;
+      const uint32_t ph = (uint32_t)(kt / kStages) & 1u;
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->full[s], ph, B, P.status)) != 0;
       if (!ok) break;
       tc_fence_after();
-      const uint64_t da = smem_desc_sw128(smem_u32(sA + s * kGemmATile));
-      const uint64_t db = smem_desc_sw128_mn(smem_u32(sB + s * kGemmBTile), kGemmBBox);
+      const uint64_t da = smem_desc_sw128(smem_u32(smem + s * kStage));
+      const uint64_t db = smem_desc_sw128_mn(smem_u32(smem + s * kStage + kGemmATile), kGemmBBox);
       if (leader) {
 #pragma unroll
         for (int kk = 0; kk < kGemmBK / 16; ++kk)   // A: 16 k = 32 bytes inside the swizzled row; B: 16 k-rows = 2048 bytes
@@ -173,6 +191,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     }
     if (ok) {
       if (leader) tc_commit(&B->acc_full);
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->acc_full, 0, B, P.status)) != 0;
     } else if (aligned) {
       if (leader) tc_commit(&B->drain);             // let every issued MMA finish before TMEM is freed
       __all_sync(0xFFFFFFFFu, mbar_wait(&B->drain, 0, B, P.status));
@@ -182,68 +201,100 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->acc_full, 0, B, P.status)) != 0;
     tc_fence_after();
   }
-  // ------------------------------------------------ epilogue: warps 2..5 own the TMEM lane quarters 2, 3, 0, 1
-  const int quad = warp & 3;
-  const int row = quad * 32 + lane, m = m0 + row;
+  // ------------------------------------------------ epilogue: warps 0-15; the stages are free now
+  constexpr int kShare = BN / SPLIT, kSides = kShare >= 64 ? 4 : 2, kCols = kShare / kSides;   // columns of this CTA, of a warp
+  constexpr int kUnits = kCols / 8;                        // 16-byte units of a row
+  const int quad = warp & 3, row = quad * 32 + lane, side = warp >> 2;
   const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);
-  if (!SPLIT) {
-    if (warp >= 2 && ok) {
+  float* xch = reinterpret_cast<float*>(smem);             // [SPLIT - 1][kShare][128 rows] partial sums of this CTA's columns
+  const bool store = side < kSides && ok;                  // (the producer and the issuer are past the last side)
+  if constexpr (SPLIT > 1) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();                                        // no CTA of the cluster reads its stages any more
+    if (store) {
+#pragma unroll 1
+      for (int d = 1; d < SPLIT; ++d) {
+        const int to = (part + d) % SPLIT;                 // slot d - 1 at the receiver: the sender is d before it
+        float* dst = cluster.map_shared_rank(xch, to) + (size_t)((d - 1) * kShare + side * kCols) * kGemmBM + row;
+#pragma unroll 1
+        for (int j = 0; j < kCols; j += 16) {
+          uint32_t o[16];
+          tmem_ld16(t_row + to * kShare + side * kCols + j, o);
+          tmem_wait_ld();
 #pragma unroll
-      for (int j = 0; j < kGemmBN / 32; ++j) {
-        uint32_t o[32];
-        tmem_ld32(t_row + j * 32, o);
-        tmem_wait_ld();
-        if (m < P.M) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int n = n0 + j * 32 + e * 8;
-            if (n < P.N) gemm_store8(P, m, n, reinterpret_cast<const float*>(o) + 8 * e);   // (N is a multiple of 8)
-          }
+          for (int e = 0; e < 16; ++e) dst[(j + e) * kGemmBM] = __uint_as_float(o[e]);
         }
-      }
-    }
-  } else {
-    // This CTA finishes the columns [64 half, 64 half + 64) of the tile; the other half's partial sums go to the peer.
-    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
-    float* peer = cluster.map_shared_rank(xch, (int)cluster.block_rank() ^ 1);
-    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");      // the peer has started: its shared memory is there
-    if (warp >= 2 && ok) {
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        uint32_t o[32];
-        tmem_ld32(t_row + (half ^ 1) * 64 + j * 32, o);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 32; ++e) peer[(j * 32 + e) * kGemmBM + row] = __uint_as_float(o[e]);
       }
     }
     cluster.sync();
-    if (warp >= 2 && ok) {
+  }
+  if (store) {
+    uint4* stage = reinterpret_cast<uint4*>(smem + (SPLIT - 1) * kShare * kGemmBM * 4) + warp * 32 * kUnits;
+#pragma unroll 1
+    for (int j = 0; j < kCols; j += 16) {
+      uint32_t o[16];
+      tmem_ld16(t_row + part * kShare + side * kCols + j, o);
+      tmem_wait_ld();
+      float v[16];
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        uint32_t o[32];
-        tmem_ld32(t_row + half * 64 + j * 32, o);
-        tmem_wait_ld();
-        if (m < P.M) {
+      for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(o[e]);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int n = n0 + half * 64 + j * 32 + e * 8;
-            float v[8];
+      for (int d = 0; d < SPLIT - 1; ++d)
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(o[8 * e + i]) + xch[(j * 32 + e * 8 + i) * kGemmBM + row];
-            if (n < P.N) gemm_store8(P, m, n, v);
+        for (int e = 0; e < 16; ++e) v[e] += xch[(size_t)(d * kShare + side * kCols + j + e) * kGemmBM + row];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        uint4 t;
+        uint32_t* w = reinterpret_cast<uint32_t*>(&t);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          w[e] = pack_bf16(v[8 * u + 2 * e], v[8 * u + 2 * e + 1]);
+          if (P.gelu) {
+            const float2 g = gelu2(make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xFFFF0000u)));
+            w[e] = pack_bf16(g.x, g.y);
           }
         }
+        stage[lane * kUnits + ((j / 8 + u) ^ (lane & (kUnits - 1)))] = t;
       }
+    }
+    __syncwarp();
+#pragma unroll 4
+    for (int i = lane; i < 32 * kUnits; i += 32) {         // whole lines of a row by neighbouring lanes
+      const int r = i / kUnits, u = i % kUnits, m = m0 + quad * 32 + r, n = n0 + part * kShare + side * kCols + u * 8;
+      if (m < P.M && n < P.N) gemm_store8(P, m, n, stage[r * kUnits + (u ^ (r & (kUnits - 1)))]);   // (N is a multiple of 8)
     }
   }
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
+  if (warp == kIssuer) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kGemmTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)BN) : "memory");
   }
+}
+
+// Tile width and K split, from a model in nanoseconds fitted to a sweep over seventeen shapes (333 to 1374 rows, N and K 512
+// to 4096): 310 per K step of a 256-wide tile, 265 of a 128-wide one (half the work: shared memory bounds it); set-up and
+// epilogue by variant; one CTA per SM, so 148 CTAs, 74 clusters of two or 33 of four at a time.
+struct GemmPlan { int bn, split; };
+inline GemmPlan gemm_plan(int M, int N, int K) {
+  static const int kFixed[2][3] = {{3500, 4800, 4800}, {4800, 6400, 7000}}, kResident[3] = {148, 74, 33};
+  const int tiles_m = (M + kGemmBM - 1) / kGemmBM, steps = K / kGemmBK;
+  GemmPlan best{256, 1};
+  long best_ns = -1;
+  for (int w = 1; w >= 0; --w)
+    for (int j = 0; j < 3; ++j) {
+      const int bn = w ? 256 : 128, split = 1 << j;
+      if (split > 1 && steps < 2 * split) continue;
+      const long tiles = (long)tiles_m * ((N + bn - 1) / bn), waves = (tiles + kResident[j] - 1) / kResident[j];
+      const long ns = waves * ((long)((steps + split - 1) / split) * (w ? 310 : 265) + kFixed[w][j]);
+      if (best_ns < 0 || ns < best_ns) {
+        best_ns = ns;
+        best = {bn, split};
+      }
+    }
+  return best;
 }
 
 inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P, cudaStream_t st) {
@@ -252,15 +303,17 @@ inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P,
   if (rc) return rc;
   rc = make_rows_map(&tb, Bm, P.K, P.N, kGemmBK);          // 64 n-columns x 64 k-rows per box
   if (rc) return rc;
-  const int tiles_n = (P.N + kGemmBN - 1) / kGemmBN, tiles_m = (P.M + kGemmBM - 1) / kGemmBM;
-  // Half the SMs or fewer busy and a K loop long enough to halve: two CTAs a tile.
-  const bool split = tiles_n * tiles_m <= 74 && P.K >= 1024;
-  static std::atomic<uint64_t> smem_set[2];
-  const auto kernel = split ? k_gemm_bf16_tcgen05<true> : k_gemm_bf16_tcgen05<false>;
-  cudaError_t e = allow_smem(kernel, gemm_smem_bytes(split), smem_set[split ? 1 : 0]);
+  const GemmPlan plan = gemm_plan(P.M, P.N, P.K);
+  const int tiles_n = (P.N + plan.bn - 1) / plan.bn, tiles_m = (P.M + kGemmBM - 1) / kGemmBM;
+  using Kernel = void (*)(CUtensorMap, CUtensorMap, GemmArgs);
+  static const Kernel kernels[2][3] = {{k_gemm_bf16_tcgen05<128, 1>, k_gemm_bf16_tcgen05<128, 2>, k_gemm_bf16_tcgen05<128, 4>},
+                                       {k_gemm_bf16_tcgen05<256, 1>, k_gemm_bf16_tcgen05<256, 2>, k_gemm_bf16_tcgen05<256, 4>}};
+  static std::atomic<uint64_t> smem_set[2][3];
+  const int i = plan.bn == 256 ? 1 : 0, j = plan.split / 2;
+  const size_t smem = gemm_smem_bytes(plan.bn);
+  cudaError_t e = allow_smem(kernels[i][j], smem, smem_set[i][j]);
   if (e == cudaSuccess)
-    e = launch_dependent(kernel, dim3(split ? 2 * tiles_n : tiles_n, tiles_m), kGemmThreads, split ? 2 : 1, gemm_smem_bytes(split), st, true,
-                         ta, tb, P);
+    e = launch_dependent(kernels[i][j], dim3(tiles_n * plan.split, tiles_m), kGemmThreads, plan.split, smem, st, true, ta, tb, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   return OVGGT_OK;
 }

@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(1024) k_colsum_final(const float* __restrict__
 // in registers for rows of up to 128 vectors.  Scaffold (the LayerNorm before a projection), fused with the conversions
 // around it: the three launches it replaces moved 6 bytes per element each way.
 __global__ void __launch_bounds__(256) k_layer_norm_bf16(const uint4* __restrict__ x, int rows, int nvec, uint4* __restrict__ out) {
+  pdl_trigger();
   pdl_wait();
   const int row = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
   if (row >= rows) return;
