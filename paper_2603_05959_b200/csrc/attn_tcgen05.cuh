@@ -666,19 +666,17 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 }
 
 // out[m, h*64 + c] = sum_s O_s 2^(m_s - m*) / sum_s l_s 2^(m_s - m*), m* = max_s m_s, splits folded in order.
-// One thread per 4 columns; all loads of a thread are issued before the arithmetic that needs them.
+// One thread per 4 columns, blockIdx.x = row; all loads of a thread are issued before the arithmetic that needs them.
 template <typename Out>
 __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_part, const float2* __restrict__ ml_part,
                                                     int M, int H, int splits, Out* __restrict__ out,
                                                     float* __restrict__ lse) {
-  const int C = H * kHD;
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t total = (size_t)M * (C / 4);
+  pdl_trigger();
+  const int C = H * kHD, c4 = (int)(blockIdx.y * blockDim.x + threadIdx.x), m = (int)blockIdx.x, h = (c4 * 4) / kHD;
   // launched with programmatic stream serialisation: its CTAs may become resident while the last attention CTAs
   // drain; the partials are complete and visible once this wait returns
   pdl_wait();
-  if (idx >= total) return;
-  const int m = (int)(idx / (C / 4)), c4 = (int)(idx % (C / 4)), h = (c4 * 4) / kHD;
+  if (c4 * 4 >= C) return;
   float2 ml[kMaxSplits];
   float4 o[kMaxSplits];
 #pragma unroll
@@ -828,8 +826,8 @@ inline int attn_kv_maps(AttnKvMaps* m, const void* k, const void* v, int N, int 
 template <typename Out>
 inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, int H, int splits, Out* out, float* lse,
                              cudaStream_t st) {
-  const size_t total = (size_t)M * (H * kHD / 4);
-  cudaError_t e = launch_dependent(k_attn_merge<Out>, dim3((unsigned)((total + 255) / 256)), 256, 1, 0, st, true, o_part,
+  const int c4 = H * kHD / 4, threads = std::min(256, (c4 + 31) / 32 * 32);
+  cudaError_t e = launch_dependent(k_attn_merge<Out>, dim3(M, (c4 + threads - 1) / threads), threads, 1, 0, st, true, o_part,
                                    ml_part, M, H, splits, out, lse);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   return OVGGT_OK;

@@ -56,6 +56,9 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
   const int items = A.M + n_div + n_norm;
   const bool pending = A.tail_move != nullptr;
 
+  // The selection behind this kernel may take its place early; behind a front of a few CTAs, which ends sooner than that is
+  // worth, it only gets in the way (camera head: 84 us a pass without, 93 with).
+  if (gridDim.x >= 148) pdl_trigger();
   pdl_wait();
   uint4 u[4][4];
   // the first 128 vectors of an item's rows: the new K and V row and what sits in their slot, or four rows to score
