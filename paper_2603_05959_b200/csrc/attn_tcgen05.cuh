@@ -667,7 +667,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 
 // out[m, h*64 + c] = sum_s O_s 2^(m_s - m*) / sum_s l_s 2^(m_s - m*), m* = max_s m_s, splits folded in order.
 // One thread per 4 columns, blockIdx.x = row; all loads of a thread are issued before the arithmetic that needs them.
-template <typename Out>
+template <typename Out, int MAXS>
 __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_part, const float2* __restrict__ ml_part,
                                                     int M, int H, int splits, Out* __restrict__ out,
                                                     float* __restrict__ lse) {
@@ -677,22 +677,22 @@ __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_
   // drain; the partials are complete and visible once this wait returns
   pdl_wait();
   if (c4 * 4 >= C) return;
-  float2 ml[kMaxSplits];
-  float4 o[kMaxSplits];
+  float2 ml[MAXS];
+  float4 o[MAXS];
 #pragma unroll
-  for (int s = 0; s < kMaxSplits; ++s)
+  for (int s = 0; s < MAXS; ++s)
     if (s < splits) {
       ml[s] = ml_part[((size_t)s * M + m) * H + h];
       o[s] = *reinterpret_cast<const float4*>(o_part + ((size_t)s * M + m) * C + c4 * 4);
     }
   float mstar = -INFINITY;
 #pragma unroll
-  for (int s = 0; s < kMaxSplits; ++s)
+  for (int s = 0; s < MAXS; ++s)
     if (s < splits) mstar = fmaxf(mstar, ml[s].x);
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float den = 0.0f;
 #pragma unroll
-  for (int s = 0; s < kMaxSplits; ++s)
+  for (int s = 0; s < MAXS; ++s)
     if (s < splits) {
       const float w = exp2f(ml[s].x - mstar);
       acc.x = fmaf(w, o[s].x, acc.x);
@@ -827,7 +827,8 @@ template <typename Out>
 inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, int H, int splits, Out* out, float* lse,
                              cudaStream_t st) {
   const int c4 = H * kHD / 4, threads = std::min(256, (c4 + 31) / 32 * 32);
-  cudaError_t e = launch_dependent(k_attn_merge<Out>, dim3(M, (c4 + threads - 1) / threads), threads, 1, 0, st, true, o_part,
+  const auto kernel = splits <= 4 ? k_attn_merge<Out, 4> : (splits <= 8 ? k_attn_merge<Out, 8> : k_attn_merge<Out, kMaxSplits>);
+  cudaError_t e = launch_dependent(kernel, dim3(M, (c4 + threads - 1) / threads), threads, 1, 0, st, true, o_part,
                                    ml_part, M, H, splits, out, lse);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   return OVGGT_OK;

@@ -724,6 +724,13 @@ int validate_compress(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, c
   return OVGGT_OK;
 }
 
+// The rule of Sec. 3.3 for a frame whose decision has not been taken: does it become a historical anchor?
+bool wants_registration(const ovggt_cache* h, const ovggt_frame_io* io) {
+  const ovggt_config& c = h->cfg;
+  return io->frame_id != h->first_frame && c.anchor_tokens > 0 && c.k_max > 0 && io->conf != nullptr && io->rho < c.tau &&
+         io->frame_id - h->last_registration >= c.min_anchor_interval;
+}
+
 // Anchor decision of frame t (Sec. 3.3), taken once and shared by all layers.
 void take_decision(ovggt_cache* h, const ovggt_frame_io* io, const MirroredDecision* mirrored) {
   const ovggt_config& c = h->cfg;
@@ -746,8 +753,7 @@ void take_decision(ovggt_cache* h, const ovggt_frame_io* io, const MirroredDecis
         h->anchors.erase(it);
       }
     }
-  } else if (t != h->first_frame && c.anchor_tokens > 0 && c.k_max > 0 && io->conf != nullptr && io->rho < c.tau &&
-             t - h->last_registration >= c.min_anchor_interval) {
+  } else if (wants_registration(h, io)) {
     h->decided_register = true;
     h->anchors.push_back(t);
     h->last_registration = t;
@@ -1078,7 +1084,12 @@ extern "C" int ovggt_layer_step_host(ovggt_cache* h, int32_t layer, const ovggt_
     CK(cudaMemcpyAsync(h->stage_v[p], io->v, bytes, cudaMemcpyHostToDevice, cs));
     CK(cudaMemcpyAsync(h->stage_r[p], io->resid, bytes, cudaMemcpyHostToDevice, cs));
   }
-  if (io->conf) CK(cudaMemcpyAsync(h->stage_conf[p], io->conf, (size_t)h->Np * 4, cudaMemcpyHostToDevice, cs));
+  // Only a frame that becomes an anchor has its confidence map read: a copy of its own between two frames' inputs costs the
+  // bus some 4 us a step (11 MB a frame take 207).
+  const bool reads_conf = h->decided_frame == io->frame_id ? h->decided_register
+                                                           : h->first_frame >= 0 && wants_registration(h, io);
+  if (io->conf && reads_conf)
+    CK(cudaMemcpyAsync(h->stage_conf[p], io->conf, (size_t)h->Np * 4, cudaMemcpyHostToDevice, cs));
   if (h->copy) {
     CK(cudaEventRecord(h->ev_h2d[p], cs));
     CK(cudaStreamWaitEvent(st, h->ev_h2d[p], 0));
