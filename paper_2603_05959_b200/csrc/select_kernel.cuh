@@ -268,14 +268,13 @@ __host__ __device__ inline size_t select_header_bytes() { return (sizeof(SelectS
 __host__ __device__ inline size_t select_smem_bytes(int span) { return select_header_bytes() + (((size_t)span * 4 + 15) & ~(size_t)15); }
 
 // The fused per-step kernel keeps, per position, the value or key (4 bytes), bin and flag (2), id (8), stored score (4)
-// and slot (4) on chip, the frame's m raw residual norms and the np confidence keys and marks; the fold of the key sums'
-// corrections at the end needs five rows of kDeltaCols floats over the same place.
+// and slot (4) on chip, the frame's m raw residual norms, the np confidence keys and marks, and for the key sums'
+// corrections a list of rows (m that leave, m that come) and a block of sums.
 constexpr int kDeltaCols = 1024;
 __host__ __device__ inline size_t compress_smem_bytes(int span, int np, int m) {
   const size_t s4 = ((size_t)span + 3) & ~(size_t)3, m4 = ((size_t)m + 3) & ~(size_t)3, np4 = ((size_t)np + 3) & ~(size_t)3;
-  const size_t body = s4 * (8 + 3 * 4) + ((s4 + 7) & ~(size_t)7) * 2 + m4 * 4 + np4 * 4 + np4;
-  const size_t fold = (size_t)5 * kDeltaCols * 4;
-  return select_header_bytes() + (body > fold ? body : fold);
+  const size_t body = s4 * (8 + 3 * 4) + ((s4 + 7) & ~(size_t)7) * 2 + m4 * 4 + np4 * 4 + ((np4 + 15) & ~(size_t)15);
+  return select_header_bytes() + body + (size_t)kDeltaCols * 4 + 2 * m4 * 4;
 }
 
 // Per-warp totals of the rows that stay, and of two marked kinds of rows, for the warp's range of positions; then the
@@ -387,7 +386,6 @@ struct CompressParams {
   // that evicted rows leave: the i-th such survivor (in logical order) goes to the i-th such slot (in the logical
   // order of the rows that leave).  The kernel writes the pairs, the survivors' slots, and the step's stamp beside every
   // slot that will be filled; the layer's next append copies the rows and patches slot_dst[move_j[i]] = move_dst[i].
-  // Stable layout: the lists hold the admitted new rows and the evicted cached rows (positions = rows), for the sums below.
   int fill;
   const int* slot_src;              // [n]
   int* slot_dst;                    // [<= B]
@@ -421,92 +419,71 @@ __device__ __forceinline__ float smoothed_score(const CompressParams& P, const f
   return v;
 }
 
-// ksum_next = ksum + (keys admitted - keys evicted) by the whole cluster.  src / dst: the slots of na admitted and nd
-// evicted rows (src nullptr: the na rows from n on).  A warp takes every 8 ncta-th row of one half of the columns, the
-// eight warps of a half are folded in two rounds, the CTAs in rank order: a fixed order, whatever the timing.
+// ksum_next = ksum + (keys admitted - keys evicted) by the whole cluster: each CTA adds up the rows of its list, whose first
+// n_out entries leave and whose others come (< 0: nothing), then the CTAs are folded in rank order.  A warp owns a line of
+// eight vectors of all rows, its four lane groups take every fourth row with eight loads in flight each, so the fold inside
+// the CTA is two shuffles; every order is fixed, whatever the timing.
 template <int DT, bool SINGLE>
-__device__ __noinline__ void fold_key_sums(const CompressParams& P, const int* src, const int* dst, int na, int nd,
-                                              float* park /* [4][kDeltaCols] */, float* part /* [kDeltaCols] */) {
-  constexpr int VEC = VecOf<DT>::n, VB = kDeltaCols / VEC, PER = VB / 64, Q = 4 / PER;   // vectors per block, per lane; rows in flight
+__device__ __noinline__ void fold_key_sums(const CompressParams& P, const int* list, int n_out, int n_list, float* part) {
+  constexpr int VEC = VecOf<DT>::n, VB = kDeltaCols / VEC;        // vectors of a block of columns
   using G = Peers<SINGLE>;
   const int ncta = G::count(), rank = G::rank();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = warp & 1, grp = warp >> 1;
-  const int C = P.nvec * VEC, stride = 8 * ncta;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = lane >> 3;
+  const int C = P.nvec * VEC, share = kDeltaCols / G::kMax;       // columns of a block that a CTA finishes
   for (int v0 = 0; v0 < P.nvec; v0 += VB) {
-    float acc[PER * VEC];
+    float base[(kDeltaCols + kSelectThreads - 1) / kSelectThreads];
 #pragma unroll
-    for (int e = 0; e < PER * VEC; ++e) acc[e] = 0.0f;
-    const int vl = v0 + half * (VB / 2) + lane;       // this lane's vectors: vl, vl + 32, ...
-    auto load = [&](int row, uint4* u) {
+    for (int k = 0; k * kSelectThreads < share; ++k) {
+      const int x = k * kSelectThreads + tid, c = v0 * VEC + rank * share + x;
+      base[k] = P.ksum != nullptr && x < share && c < C ? P.ksum[c] : 0.0f;
+    }
+#pragma unroll 1
+    for (int w = warp; w < VB / 8 && v0 + w * 8 < P.nvec; w += kSelectWarps) {
+      const int vec = v0 + w * 8 + (lane & 7);
+      const bool in = vec < P.nvec;
+      float acc[VEC];
 #pragma unroll
-      for (int i = 0; i < PER; ++i)
-        if (vl + 32 * i < P.nvec) u[i] = P.k_cache[(size_t)row * P.nvec + vl + 32 * i];
-    };
-    auto add = [&](const uint4* u, float sign) {
+      for (int e = 0; e < VEC; ++e) acc[e] = 0.0f;
+#pragma unroll 1
+      for (int e0 = grp; e0 < n_list; e0 += 32) {
+        uint4 u[8];
 #pragma unroll
-      for (int i = 0; i < PER; ++i)
-        if (vl + 32 * i < P.nvec) {
-          float f[VEC];
-          unpack<DT>(u[i], f);
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) acc[i * VEC + e] = __fmaf_rn(f[e], sign, acc[i * VEC + e]);
+        for (int k = 0; k < 8; ++k) {
+          const int slot = e0 + 4 * k < n_list && in ? list[e0 + 4 * k] : -1;
+          u[k] = slot >= 0 ? P.k_cache[(size_t)slot * P.nvec + vec] : make_uint4(0u, 0u, 0u, 0u);
         }
-    };
-    const int most = max(na, nd);
-    int ra = 0, rb = 0;                               // lane l: the rows of the warp's turn 32 x + l
-    for (int i = rank * 8 + grp, turn = 0; i < most; i += Q * stride, turn += Q) {
-      if ((turn & 31) == 0) {
-        const int k = i + lane * stride;
-        ra = k < na ? (src ? __ldcg(src + k) : P.n + k) : 0;
-        rb = k < nd ? __ldcg(dst + k) : 0;
-      }
-      uint4 a[Q][PER], b[Q][PER];
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const int k = i + q * stride, xa = __shfl_sync(0xFFFFFFFFu, ra, (turn + q) & 31), xb = __shfl_sync(0xFFFFFFFFu, rb, (turn + q) & 31);
-        if (k < na) load(xa, a[q]);
-        if (k < nd) load(xb, b[q]);
+        for (int k = 0; k < 8; ++k) {
+          const float sign = e0 + 4 * k < n_out ? -1.0f : 1.0f;
+          float f[VEC];
+          unpack<DT>(u[k], f);
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) acc[e] = __fmaf_rn(f[e], sign, acc[e]);
+        }
       }
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const int k = i + q * stride;
-        if (k < na) add(a[q], 1.0f);
-        if (k < nd) add(b[q], -1.0f);
+      for (int e = 0; e < VEC; ++e) {
+        acc[e] += __shfl_xor_sync(0xFFFFFFFFu, acc[e], 8);
+        acc[e] += __shfl_xor_sync(0xFFFFFFFFu, acc[e], 16);
       }
+      if (grp == 0)
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) part[(w * 8 + lane) * VEC + e] = acc[e];
     }
-    // (element-major: neighbouring lanes meet neighbouring banks)
-    auto slot = [&](int s, int i, int e) -> float& {
-      return park[s * kDeltaCols + e * VB + half * (VB / 2) + lane + 32 * i];
-    };
-    if (grp >= 4) {
-#pragma unroll
-      for (int i = 0; i < PER; ++i)
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) slot(grp - 4, i, e) = acc[i * VEC + e];
-    }
-    __syncthreads();
-    if (grp < 4) {
-#pragma unroll
-      for (int i = 0; i < PER; ++i)
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) slot(grp, i, e) += acc[i * VEC + e];
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < kDeltaCols; c += blockDim.x)
-      part[c] = ((park[c] + park[kDeltaCols + c]) + park[2 * kDeltaCols + c]) + park[3 * kDeltaCols + c];
     G::sync();
-    for (int x = rank * kSelectThreads + threadIdx.x; x < kDeltaCols; x += kSelectThreads * ncta) {
-      const int c = v0 * VEC + (x & (VB - 1)) * VEC + x / VB;   // the column whose sum lies at x
-      if (c >= C) continue;
-      float v[G::kMax];                               // all remote reads in flight before the first add
 #pragma unroll
-      for (int q = 0; q < G::kMax; ++q) v[q] = q < ncta ? G::of(part, q)[x] : 0.0f;
-      float t = P.ksum ? P.ksum[c] : 0.0f;
+    for (int k = 0; k * kSelectThreads < share; ++k) {
+      const int x = k * kSelectThreads + tid, y = rank * share + x, c = v0 * VEC + y;
+      if (x < share && c < C) {
+        float v[G::kMax];                             // all remote reads in flight before the first add
 #pragma unroll
-      for (int q = 0; q < G::kMax; ++q) t += v[q];
-      P.ksum_next[c] = t;
+        for (int q = 0; q < G::kMax; ++q) v[q] = q < ncta ? G::of(part, q)[y] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < G::kMax; ++q) base[k] += v[q];
+        P.ksum_next[c] = base[k];
+      }
     }
-    if (v0 + VB < P.nvec) G::sync();             // (part is written again)
+    if (v0 + VB < P.nvec) G::sync();                  // (part is written again)
   }
 }
 
@@ -530,6 +507,8 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   uint32_t* ckeys = reinterpret_cast<uint32_t*>(sraw + ((M + 3) & ~3));   // [Np] confidence keys
   uint16_t* bf = reinterpret_cast<uint16_t*>(ckeys + ((Np + 3) & ~3));    // flag << 14 | bin of the owned positions
   uint8_t* cmark = reinterpret_cast<uint8_t*>(bf + ((span4 + 7) & ~7));   // [Np] the most confident patches
+  float* part = reinterpret_cast<float*>(cmark + ((Np + 15) & ~15));      // [kDeltaCols] this CTA's corrections of the key sums
+  int* list = reinterpret_cast<int*>(part + kDeltaCols);                  // [2 M] slots of the rows they are made of
   const bool hybrid = P.mode == OVGGT_SCORE_HYBRID, choose = N > P.B;
   pdl_wait();
   pdl_trigger();   // an attention queued behind this kernel reads nothing of it: it starts as soon as this one runs
@@ -555,10 +534,9 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
     } else {
       for (int j = tid; j < M; j += nthr) sraw[j] = P.s_raw[j];
     }
-    __syncthreads();
   }
   uint32_t mn[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, mx[3] = {0u, 0u, 0u};
-  // (a thread touches its own positions only, so the three passes need no barrier; all loads of a pass are independent)
+  // (a thread touches its own positions only, so the passes need no barrier among them; all loads of a pass are independent)
 #pragma unroll 4
   for (int i = tid; i < cnt; i += nthr) {
     const int g = begin + i;
@@ -579,6 +557,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   if (hybrid)
 #pragma unroll 4
     for (int i = tid; i < cnt; i += nthr) val[i] = begin + i < n ? P.d[ssl[i]] : 0.0f;
+  __syncthreads();                                     // the staged norms are complete
 #pragma unroll 1
   for (int i = tid; i < cnt; i += nthr) {
     const int g = begin + i;
@@ -844,9 +823,37 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
     }
   }
 
+  // -- column sums of the keys that stay, before anything is written (a cluster barrier waits for the global stores before
+  //    it).  A CTA takes the rows that leave from its own positions, and of the frame's rows, which the last CTAs own, its
+  //    share, by a look at their keys.
+  const unsigned below = (1u << lane) - 1;
+  if (P.ksum_next != nullptr) {
+    int n_out = 0;
+    if (choose) {
+      int d = dw;
+#pragma unroll 1
+      for (int i0 = wlo; i0 < whi; i0 += 32) {
+        bool keep, up, down = false;
+        if (i0 + lane < whi) classify(i0 + lane, keep, up, down);
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, down);
+        const int at = d + __popc(m & below);
+        if (down && at < M) list[at] = ssl[i0 + lane];
+        d += __popc(m);
+      }
+      n_out = min(M, (int)__reduce_add_sync(0xFFFFFFFFu, lane < kSelectWarps ? sh->wtot[lane][2] : 0));
+    }
+    const int span = (N + ncta - 1) / ncta, per = (M + ncta - 1) / ncta, first = min(M, rank * per), n_in = min(M, first + per) - first;
+    for (int j = tid; j < n_in; j += nthr) {
+      const int g = n + first + j, owner = g / span;
+      const uint32_t key = choose ? G::of(keys, owner)[g - owner * span] : 0u;
+      list[n_out + j] = !choose || key > T || (key == T && g <= posT) ? g : -1;
+    }
+    __syncthreads();
+    fold_key_sums<DT, SINGLE>(P, list, n_out, n_out + n_in, part);
+  }
+
   // -- survivors, compacted meta (order preserved), and the lists of rows that come and go
   int j0 = keep_before + kw, u0 = up_before + uw, d0 = down_before + dw;
-  const unsigned below = (1u << lane) - 1;
 #pragma unroll 1
   for (int i0 = wlo; i0 < whi; i0 += 32) {
     const int i = i0 + lane, g = begin + i;
@@ -869,13 +876,13 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
         P.stored_dst[j] = sst[i];
         if (fill) P.slot_dst[j] = slot;
       }
-      if (up && iu < M) {
+      if (fill && up && iu < M) {
         P.move_src[iu] = slot;
-        if (fill) P.move_j[iu] = j;
+        P.move_j[iu] = j;
       }
-      if (down && id < M) {
+      if (fill && down && id < M) {
         P.move_dst[id] = slot;
-        if (fill) P.hole_stamp[slot] = P.stamp;
+        P.hole_stamp[slot] = P.stamp;
       }
       // which move empties a slot above B: none if its row leaves (or if the list is full: an inconsistency, see below)
       if (fill && slot >= P.B && slot - P.B < M) P.tail_move[slot - P.B] = up && iu < M ? iu : -1;
@@ -893,12 +900,6 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       *P.n_moves_out = consistent ? up_all : 0;
       if (!consistent) atomicCAS(P.status, 0, OVGGT_ERR_DEVICE_STATUS);
     }
-  }
-  if (P.ksum_next != nullptr) {
-    G::sync();                                    // the lists are complete; the staged rows are not needed any more
-    float* fold = reinterpret_cast<float*>(p);
-    fold_key_sums<DT, SINGLE>(P, choose ? P.move_src : nullptr, P.move_dst, choose ? min(up_all, M) : M, choose ? min(down_all, M) : 0,
-                      fold, fold + 4 * kDeltaCols);
   }
   G::leave();
 }
