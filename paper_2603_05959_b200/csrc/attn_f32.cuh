@@ -40,18 +40,21 @@ struct F32Barriers {
   uint32_t tmem_base;
   int abort_flag;
 };
-constexpr size_t kF32SmemBytes = (size_t)3 * kF32QPlane + 6 * kF32KvPlane + sizeof(F32Barriers) + 64;
+constexpr int kF32Planes = 3 * kF32QPlane + 6 * kF32KvPlane;
+static_assert(kJoinStages * kPartBytes <= kF32Planes, "the parts do not fit the operand planes");
+constexpr size_t f32_smem_bytes(bool join) { return (size_t)kF32Planes + sizeof(F32Barriers) + (join ? sizeof(PartJoin) + kJoinTable * 4 : 0) + 64; }
 
 struct F32Params {
   const float *q, *k, *v;
   int M, N, H;
   int splits, tiles_per_split, tiles_total;
   float* out;             // [M, C]            (splits == 1)
-  float* o_part;          // [splits, M, C]
-  float2* ml_part;        // [splits, M, H]
+  float* o_part;          // these as in AttnParams
+  float2* ml_part;
   float* lse;             // [M, H] or nullptr
   int* status;            // or nullptr
-  int wait_first;         // as in AttnParams
+  int wait_first;         // these as in AttnParams
+  unsigned* tickets;
 };
 
 // A pair of floats as three bf16 pairs.
@@ -81,6 +84,8 @@ __device__ __forceinline__ void store_planes(unsigned char* base, int plane_byte
 __device__ constexpr int kSplitA[6] = {2, 0, 1, 1, 0, 0};
 __device__ constexpr int kSplitB[6] = {0, 2, 1, 0, 1, 0};
 
+// JOIN: the parts of a split KV range are joined here (see join_parts).
+template <bool JOIN>
 __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __grid_constant__ F32Params P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   if (smem_u32(smem) & 1023u) {                      // the 128-byte swizzle needs 1024-byte aligned tiles
@@ -90,7 +95,8 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
   unsigned char* sQ = smem;
   unsigned char* sK = sQ + 3 * kF32QPlane;
   unsigned char* sV = sK + 3 * kF32KvPlane;
-  F32Barriers* B = reinterpret_cast<F32Barriers*>(sV + 3 * kF32KvPlane);
+  F32Barriers* B = reinterpret_cast<F32Barriers*>(smem + kF32Planes);
+  PartJoin* J = reinterpret_cast<PartJoin*>(B + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int qt = blockIdx.x, h = blockIdx.y, split = blockIdx.z;
   const int t_begin = split * P.tiles_per_split;
@@ -108,6 +114,8 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
     mbar_init(&B->p_full, 128);
     mbar_init(&B->o_full, 1);
     mbar_init(&B->drain, 1);
+    if constexpr (JOIN)
+      for (int s = 0; s < kJoinStages; ++s) mbar_init(&J->full[s], 1);
     B->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -313,12 +321,23 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
     if (ok && m < P.M) {
       const bool whole = P.splits == 1;
       const float f = whole ? 1.0f / l : 1.0f;
-      float4* dst = reinterpret_cast<float4*>((whole ? P.out + (size_t)m * C : P.o_part + ((size_t)split * P.M + m) * C) + (size_t)h * kHD);
+      const size_t part_row = JOIN ? join_row0(P.M, qt, h, P.splits) + (size_t)split * min(kBM, P.M - qt * kBM) + row
+                                   : (size_t)split * P.M + m;
+      float* part = JOIN ? P.o_part + part_row * kHD : P.o_part + part_row * C + (size_t)h * kHD;
+      float4* dst = reinterpret_cast<float4*>(whole ? P.out + (size_t)m * C + (size_t)h * kHD : part);
 #pragma unroll
       for (int i = 0; i < kHD; i += 4) dst[i / 4] = make_float4(acc[i] * f, acc[i + 1] * f, acc[i + 2] * f, acc[i + 3] * f);
-      if (!whole) P.ml_part[((size_t)split * P.M + m) * P.H + h] = make_float2(mref, l);
+      if (!whole) P.ml_part[JOIN ? part_row : part_row * P.H + h] = make_float2(mref, l);
       if (whole && P.lse != nullptr) P.lse[(size_t)m * P.H + h] = mref + log2f(l);
     }
+    if constexpr (JOIN)
+      if (join_arrive(J, P.tickets + h * gridDim.x + qt, P.splits, ok)) {
+        const int m0 = qt * kBM;
+        const size_t row0 = join_row0(P.M, qt, h, P.splits);
+        join_parts(J, B, smem, reinterpret_cast<float*>(J + 1), P.o_part + row0 * kHD, P.ml_part + row0, min(kBM, P.M - m0),
+                   P.splits, P.out + (size_t)m0 * C + h * kHD, C, P.lse != nullptr ? P.lse + (size_t)m0 * P.H + h : nullptr, P.H,
+                   P.status);
+      }
   }
 
   // ------------------------------------------------ teardown
@@ -355,7 +374,7 @@ inline int attn_f32_choose_splits(int M, int N, int H) {
 
 // scratch: attn_tcgen05_scratch_bytes, or nullptr (the KV range is then not split).
 inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out, void* scratch,
-                           int* status, cudaStream_t st, float* lse, bool beside_previous, int* launches) {
+                           int* status, cudaStream_t st, float* lse, bool beside_previous, unsigned* tickets, int* launches) {
   const int C = H * kHD;
   F32Params P;
   P.q = static_cast<const float*>(q);
@@ -369,20 +388,22 @@ inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, i
   P.out = static_cast<float*>(out);
   P.o_part = static_cast<float*>(scratch);
   P.ml_part = reinterpret_cast<float2*>(static_cast<char*>(scratch) + (size_t)kMaxSplits * M * C * 4);
+  P.tickets = tickets;
   P.lse = lse;
   P.status = status;
   P.wait_first = beside_previous ? 0 : 1;
-  static std::atomic<uint64_t> smem_set{0};
-  cudaError_t e = allow_smem(k_attn_f32, kF32SmemBytes, smem_set);
+  const dim3 grid((M + kBM - 1) / kBM, H, P.splits);
+  // (an fp32 tile of 64 rows takes about as long as a bf16 tile of 128)
+  const bool join = tickets && P.splits > 1 && attn_join_inside((long)grid.x * grid.y * grid.z, P.tiles_per_split);
+  const auto kernel = join ? k_attn_f32<true> : k_attn_f32<false>;
+  static std::atomic<uint64_t> smem_set[2];
+  cudaError_t e = allow_smem(kernel, f32_smem_bytes(join), smem_set[join]);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  e = launch_dependent(k_attn_f32, dim3((M + kBM - 1) / kBM, H, P.splits), kAttnThreads, 1, kF32SmemBytes, st, true, P);
+  e = launch_dependent(kernel, grid, kAttnThreads, 1, f32_smem_bytes(join), st, true, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  *launches = 1;
-  if (P.splits > 1) {
-    *launches = 2;
-    return attn_merge_launch<float>(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st);
-  }
-  return OVGGT_OK;
+  const bool merge = P.splits > 1 && !join;
+  *launches = merge ? 2 : 1;
+  return merge ? attn_merge_launch<float>(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st) : OVGGT_OK;
 }
 
 }  // namespace ovggt

@@ -65,6 +65,13 @@ constexpr int kPolyNum = OVGGT_ATTN_POLY_NUM, kPolyDen = OVGGT_ATTN_POLY_DEN;
 __host__ __device__ constexpr bool pair_on_fma_pipes(int pair) { return (pair * kPolyNum) % kPolyDen < kPolyNum; }
 constexpr int kMaxSplits = 16;
 
+// What the warps that join the parts of a split KV range share (see join_parts).
+constexpr int kJoinStages = 3, kPartBytes = kBM * kHD * 4;
+struct PartJoin {
+  unsigned long long full[kJoinStages];
+  int ok[4], last;
+};
+
 struct AttnBarriers {
   unsigned long long q_full, s_full[2], p_full[2], pv_done, o_full, drain;
   unsigned long long k_full[kKVStages], k_empty[kKVStages], v_full[kKVStages], v_empty[kKVStages];
@@ -73,7 +80,7 @@ struct AttnBarriers {
 };
 
 // (no slack for aligning the base by hand: two CTAs of 114.9 KB must fit one SM; the base is checked instead)
-constexpr size_t kAttnSmemBytes = (size_t)kQBytes + (size_t)kTileBytes * 2 * kKVStages + sizeof(AttnBarriers) + 64;
+constexpr size_t kAttnSmemBytes = (size_t)kQBytes + (size_t)kTileBytes * 2 * kKVStages + sizeof(AttnBarriers) + sizeof(PartJoin) + 64;
 
 // ---------------------------------------------------------------- PTX wrappers
 
@@ -288,6 +295,137 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return d;
 }
 
+// ---------------------------------------------------------------- joining the parts of a split KV range
+
+// A KV range in several parts leaves one un-normalised O, one reference maximum and one row sum per part, which
+//   out = sum_s O_s 2^(m_s - m*) / sum_s l_s 2^(m_s - m*),  m* = max_s m_s,  parts folded in order,
+// makes one: inside the attention kernel (join_parts) where that is cheaper and the caller keeps tickets for it (see
+// attn_join_inside), else in a kernel of its own (k_attn_merge).
+//
+// Inside the attention the CTA that is the last of its tile's parts to take a ticket folds them all, so no launch follows
+// whose CTAs wait for the whole grid and, in a step, for the selection beside it.  Nothing waits: the others just leave,
+// and the ticket counter wraps to zero for the next launch.  A part is 32 KB, fetched from L2: three bulk copies in flight
+// into the operand tiles that are no longer needed keep an SM's L2 port busy, which 128 threads' own loads do not.
+constexpr int kJoinTable = (kMaxSplits + 1) * kBM;      // floats: a weight per part and row, then 1 / denominator per row
+static_assert(kJoinTable * 4 <= kQBytes && kJoinStages * kPartBytes <= 2 * kKVStages * kTileBytes, "the parts do not fit the operand tiles");
+
+__device__ __forceinline__ void softmax_warps_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Where the parts of query tile qt of head h lie: O at [row * 64 + column], (m, l) at [row], part s as many rows after part
+// s - 1 as the tile has, so that one copy fetches a part.
+__device__ __forceinline__ size_t join_row0(int M, int qt, int h, int splits) {
+  return ((size_t)h * M + (size_t)qt * kBM) * splits;
+}
+
+// Called by the 128 softmax threads of every CTA after they have stored their part (ok: the part is complete).  Returns
+// whether this CTA is the last of its tile.
+__device__ __forceinline__ bool join_arrive(PartJoin* J, unsigned* ticket, int splits, bool ok) {
+  if ((threadIdx.x & 31) == 0) J->ok[threadIdx.x >> 5] = ok;
+  __threadfence();
+  asm volatile("fence.proxy.async;" ::: "memory");     // (the parts are read by bulk copies)
+  softmax_warps_sync();
+  if (threadIdx.x == 0) {
+    const bool last = atomicInc(ticket, (unsigned)splits - 1u) == (unsigned)splits - 1u;
+    J->last = last && J->ok[0] && J->ok[1] && J->ok[2] && J->ok[3];
+    __threadfence();
+    asm volatile("fence.proxy.async;" ::: "memory");
+  }
+  softmax_warps_sync();
+  return J->last != 0;
+}
+
+// stage: kJoinStages x 32 KB that nothing else uses any more; table: kJoinTable floats; o, ml: the tile's parts; out, lse:
+// the tile's first row.
+template <typename Out, typename Barriers>
+__device__ __forceinline__ void join_parts(PartJoin* J, Barriers* B, unsigned char* stage, float* table, const float* o,
+                                           const float2* ml, int rows, int splits, Out* out, int C, float* lse, int H, int* status) {
+  const int tid = threadIdx.x, c4 = tid & 15, r0 = tid >> 4;
+  const uint32_t bytes = (uint32_t)rows * kHD * 4;
+  auto fetch = [&](int s) {
+    void* bar = &J->full[s % kJoinStages];
+    mbar_expect_tx(bar, bytes);
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(stage + (s % kJoinStages) * kPartBytes)),
+                 "l"(o + (size_t)s * rows * kHD), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+  };
+  int fetched = min(splits, kJoinStages);
+  if (tid == 0)
+    for (int s = 0; s < fetched; ++s) fetch(s);
+  if (tid < rows) {
+    float2 p[kMaxSplits];
+    float mstar = -INFINITY, den = 0.0f;
+#pragma unroll
+    for (int s = 0; s < kMaxSplits; ++s)
+      if (s < splits) p[s] = __ldcg(ml + (size_t)s * rows + tid);
+#pragma unroll
+    for (int s = 0; s < kMaxSplits; ++s)
+      if (s < splits) mstar = fmaxf(mstar, p[s].x);
+#pragma unroll
+    for (int s = 0; s < kMaxSplits; ++s)
+      if (s < splits) {
+        const float w = exp2f(p[s].x - mstar);
+        table[s * kBM + tid] = w;
+        den = fmaf(w, p[s].y, den);
+      }
+    table[kMaxSplits * kBM + tid] = 1.0f / den;
+    if (lse != nullptr) lse[(size_t)tid * H] = mstar + log2f(den);
+  }
+  softmax_warps_sync();
+  float4 acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool ok = true;                                      // (a wait that ran out skips the arithmetic, not the barriers)
+#pragma unroll 1
+  for (int s = 0; s < splits; ++s) {
+    ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait(&J->full[s % kJoinStages], (uint32_t)(s / kJoinStages) & 1u, B, status)) != 0;
+    if (ok) {
+      const float4* part = reinterpret_cast<const float4*>(stage + (s % kJoinStages) * kPartBytes);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int r = r0 + 8 * i;
+        if (r < rows) {
+          const float w = table[s * kBM + r];
+          const float4 x = part[r * 16 + c4];
+          acc[i].x = fmaf(w, x.x, acc[i].x);
+          acc[i].y = fmaf(w, x.y, acc[i].y);
+          acc[i].z = fmaf(w, x.z, acc[i].z);
+          acc[i].w = fmaf(w, x.w, acc[i].w);
+        }
+      }
+    }
+    if (s + kJoinStages < splits) {
+      softmax_warps_sync();                            // the buffer has been read
+      if (tid == 0 && ok) {
+        fetch(s + kJoinStages);
+        fetched = s + kJoinStages + 1;
+      }
+    }
+  }
+  if (!ok) {                                           // leave no bulk copy in flight into this CTA's shared memory
+    if (tid == 0)
+      for (int s = max(0, fetched - kJoinStages); s < fetched; ++s)
+        mbar_wait(&J->full[s % kJoinStages], (uint32_t)(s / kJoinStages) & 1u, B, status);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int r = r0 + 8 * i;
+    if (r < rows) {
+      const float inv = table[kMaxSplits * kBM + r];
+      if constexpr (sizeof(Out) == 4) {
+        *reinterpret_cast<float4*>(out + (size_t)r * C + c4 * 4) =
+            make_float4(acc[i].x * inv, acc[i].y * inv, acc[i].z * inv, acc[i].w * inv);
+      } else {
+        uint2 w;
+        w.x = pack_bf16(acc[i].x * inv, acc[i].y * inv);
+        w.y = pack_bf16(acc[i].z * inv, acc[i].w * inv);
+        *reinterpret_cast<uint2*>(out + (size_t)r * C + c4 * 4) = w;
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------- the kernel
 
 struct AttnParams {
@@ -295,15 +433,18 @@ struct AttnParams {
   int splits, tiles_per_split, tiles_total;
   const float* kmax2;     // [H] upper bound of |k_j,h|^2 over all N keys, or nullptr (the maximum is tracked)
   __nv_bfloat16* out;     // [M, C]            (splits == 1)
-  float* o_part;          // [splits, M, C]    un-normalised partial outputs
-  float2* ml_part;        // [splits, M, H]    (reference maximum in log2 units, row sum)
+  float* o_part;          // un-normalised partial outputs: [splits, M, C], or by tile where they are joined here (see join_row0)
+  float2* ml_part;        // (reference maximum in log2 units, row sum): [splits, M, H], or by tile
   float* lse;             // [M, H] or nullptr: log2 of each row's softmax denominator (reference + log2 of the sum)
   int* status;
   // The kernel before this one in the stream: 1 - it wrote what is read here, wait for it first; 0 - it did not, but runs
   // beside this one (the selection of the same step), and this kernel must not end before it.
   int wait_first;
+  unsigned* tickets;      // JOIN: [query tiles * H], zero
 };
 
+// JOIN: the parts of a split KV range are joined here (see join_parts).
+template <bool JOIN>
 __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm)
 k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const AttnParams P) {
@@ -316,6 +457,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   unsigned char* sK = sQ + kQBytes;
   unsigned char* sV = sK + kKVStages * kTileBytes;
   AttnBarriers* B = reinterpret_cast<AttnBarriers*>(sV + kKVStages * kTileBytes);
+  PartJoin* J = reinterpret_cast<PartJoin*>(B + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int qt = blockIdx.x, h = blockIdx.y, split = blockIdx.z;
@@ -338,6 +480,8 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     mbar_init(&B->pv_done, 1);
     mbar_init(&B->o_full, 1);
     mbar_init(&B->drain, 1);
+    if constexpr (JOIN)
+      for (int s = 0; s < kJoinStages; ++s) mbar_init(&J->full[s], 1);
     for (int s = 0; s < kKVStages; ++s) {
       mbar_init(&B->k_full[s], 1);
       mbar_init(&B->k_empty[s], 1);
@@ -626,6 +770,9 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       tc_fence_after();
       const int m = qt * kBM + row;
       const float inv = 1.0f / l;
+      const size_t part_row = JOIN ? join_row0(P.M, qt, h, P.splits) + (size_t)split * min(kBM, P.M - qt * kBM) + row
+                                   : (size_t)split * P.M + m;
+      float* part = JOIN ? P.o_part + part_row * kHD : P.o_part + part_row * C + (size_t)h * kHD;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         uint32_t o[32];
@@ -644,15 +791,22 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               dst[e] = w;
             }
           } else {
-            uint4* dst = reinterpret_cast<uint4*>(P.o_part + ((size_t)split * P.M + m) * C + (size_t)h * kHD + j * 32);
+            uint4* dst = reinterpret_cast<uint4*>(part + j * 32);
 #pragma unroll
             for (int e = 0; e < 8; ++e) dst[e] = make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
           }
         }
       }
-      if (P.splits > 1 && m < P.M) P.ml_part[((size_t)split * P.M + m) * P.H + h] = make_float2(mref, l);
+      if (P.splits > 1 && m < P.M) P.ml_part[JOIN ? part_row : part_row * P.H + h] = make_float2(mref, l);
       if (P.splits == 1 && P.lse != nullptr && m < P.M) P.lse[(size_t)m * P.H + h] = mref + log2f(l);
     }
+    if constexpr (JOIN)
+      if (join_arrive(J, P.tickets + h * gridDim.x + qt, P.splits, ok)) {
+        const int m0 = qt * kBM;
+        const size_t row0 = join_row0(P.M, qt, h, P.splits);
+        join_parts(J, B, sK, reinterpret_cast<float*>(sQ), P.o_part + row0 * kHD, P.ml_part + row0, min(kBM, P.M - m0), P.splits,
+                   P.out + (size_t)m0 * C + h * kHD, C, P.lse != nullptr ? P.lse + (size_t)m0 * P.H + h : nullptr, P.H, P.status);
+      }
   }
 
   // ------------------------------------------------ teardown
@@ -665,8 +819,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   if (!P.wait_first) pdl_wait();
 }
 
-// out[m, h*64 + c] = sum_s O_s 2^(m_s - m*) / sum_s l_s 2^(m_s - m*), m* = max_s m_s, splits folded in order.
-// One thread per 4 columns, blockIdx.x = row; all loads of a thread are issued before the arithmetic that needs them.
+// The parts joined by a kernel of its own.  One thread per 4 columns, blockIdx.x = row; all loads of a thread are issued before the arithmetic that needs them.
 template <typename Out, int MAXS>
 __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_part, const float2* __restrict__ ml_part,
                                                     int M, int H, int splits, Out* __restrict__ out,
@@ -770,12 +923,20 @@ inline int make_rows_map(CUtensorMap* map, const void* base, int rows, int C, in
   return OVGGT_OK;
 }
 
+// Whether the parts are joined inside the attention, for `ctas` CTAs of `per` KV tiles: where all of them are resident at once,
+// so that a CTA that joins keeps no other from starting, and done before the selection of the same step, 20 to 30 us, for
+// which a kernel of its own would wait.  Steps of 329 x 3329 x 10 and 605 x 20605 x 5 take 27.3 and 45.5 us joined inside,
+// 30.1 and 50.3 us otherwise; where the selection ends first the launch is the cheaper way, as it uses every SM: 905 x
+// 20905 x 12 (288 CTAs of 55 tiles) takes 93.0 and 90.7 us, 1374 x 17758 x 16 (528 CTAs) 144.1 and 140.3 us.
+constexpr int kJoinMaxTiles = 16;
+inline bool attn_join_inside(long ctas, int per) { return ctas <= (long)kCtasPerSm * 148 && per <= kJoinMaxTiles; }
+
 // Number of KV splits, from a model in nanoseconds fitted to a sweep of 1 to 16 splits over eighteen shapes (69 x 325 x 4
 // heads to 1374 x 34142 x 16): waves of CTAs over 2 x 148 slots; 1.25 us per tile for a CTA that has its SM to itself,
 // 1.85 us where two share one; 4 us per CTA for set-up and epilogue; a merge is 3 us and passes over the partial outputs
-// (write and read) at 6 TB/s.  The merge is what short KV ranges cannot pay: 1041 x 1041 x 16 takes 14.5 us unsplit and
-// 20.6 us in two splits, whose CTAs alone would be faster.
-inline int attn_choose_splits(int M, int N, int H) {
+// (write and read) at 6 TB/s, a join inside the attention 1.5 us and 0.4 us per part.  The merge is what short KV ranges
+// cannot pay: 1041 x 1041 x 16 takes 14.5 us unsplit and 20.6 us in two splits, whose CTAs alone would be faster.
+inline int attn_choose_splits(int M, int N, int H, bool tickets) {
   const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kBN - 1) / kBN;
   const long slots = (long)kCtasPerSm * 148;
   int best = 1;
@@ -786,8 +947,8 @@ inline int attn_choose_splits(int M, int N, int H) {
     if (eff != s) continue;
     const long ctas = (long)q_tiles * H * s;
     const long waves = (ctas + slots - 1) / slots;
-    const long ns = waves * (per * (ctas <= 148 ? 1250l : 1850l) + 4000) +
-                    (s > 1 ? 3000 + (long)s * M * H * kHD * 8 / 6000 : 0);
+    const long merge = tickets && attn_join_inside(ctas, per) ? 1500 + 400l * s : 3000 + (long)s * M * H * kHD * 8 / 6000;
+    const long ns = waves * (per * (ctas <= 148 ? 1250l : 1850l) + 4000) + (s > 1 ? merge : 0);
     if (best_ns < 0 || ns < best_ns) {
       best_ns = ns;
       best = s;
@@ -802,7 +963,8 @@ inline size_t attn_tcgen05_scratch_bytes(int M, int N, int H) {
   return (size_t)kMaxSplits * M * C * 4 + (size_t)kMaxSplits * M * H * 8 + 1024;
 }
 
-inline int attn_tcgen05_num_launches(int M, int N, int H) { return attn_choose_splits(M, N, H) > 1 ? 2 : 1; }
+// Ticket counters of a launch whose parts are joined inside; zero before the first one, and left at zero.
+inline size_t attn_tickets(int M, int H) { return (size_t)((M + kBM - 1) / kBM) * H; }
 
 // Tensor maps of a K/V buffer pair, kept by the caller between launches: a cache that lives in one buffer with a
 // row count that stops changing needs them encoded once, not once per step.
@@ -837,7 +999,7 @@ inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, 
 inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
                                void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
                                int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr,
-                               bool beside_previous = false) {
+                               bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr) {
   const int C = H * kHD;
   CUtensorMap tq;
   AttnKvMaps local;
@@ -851,7 +1013,7 @@ inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int 
   AttnParams P;
   P.M = M; P.N = N; P.H = H;
   P.tiles_total = (N + kBN - 1) / kBN;
-  P.splits = force_splits > 0 ? std::min(force_splits, std::min(kMaxSplits, P.tiles_total)) : attn_choose_splits(M, N, H);
+  P.splits = force_splits > 0 ? std::min(force_splits, std::min(kMaxSplits, P.tiles_total)) : attn_choose_splits(M, N, H, tickets != nullptr);
   P.tiles_per_split = (P.tiles_total + P.splits - 1) / P.splits;
   P.splits = (P.tiles_total + P.tiles_per_split - 1) / P.tiles_per_split;     // no empty split
   P.out = static_cast<__nv_bfloat16*>(out);
@@ -861,14 +1023,18 @@ inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int 
   P.kmax2 = kmax2;
   P.lse = lse;
   P.wait_first = beside_previous ? 0 : 1;
-  static std::atomic<uint64_t> smem_set{0};
-  cudaError_t e = allow_smem(k_attn_tcgen05, kAttnSmemBytes, smem_set);
+  P.tickets = tickets;
+  const dim3 grid((M + kBM - 1) / kBM, H, P.splits);
+  const bool join = tickets && P.splits > 1 && attn_join_inside((long)grid.x * grid.y * grid.z, P.tiles_per_split);
+  const auto kernel = join ? k_attn_tcgen05<true> : k_attn_tcgen05<false>;
+  static std::atomic<uint64_t> smem_set[2];
+  cudaError_t e = allow_smem(kernel, kAttnSmemBytes, smem_set[join]);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  dim3 grid((M + kBM - 1) / kBM, H, P.splits);
-  e = launch_dependent(k_attn_tcgen05, grid, kAttnThreads, 1, kAttnSmemBytes, st, true, tq, tk, tv, P);
+  e = launch_dependent(kernel, grid, kAttnThreads, 1, kAttnSmemBytes, st, true, tq, tk, tv, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  if (P.splits > 1) return attn_merge_launch(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st);
-  return OVGGT_OK;
+  const bool merge = P.splits > 1 && !join;
+  if (launches) *launches = merge ? 2 : 1;
+  return merge ? attn_merge_launch(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st) : OVGGT_OK;
 }
 
 }  // namespace ovggt

@@ -185,15 +185,13 @@ int launch_fill_holes(void* kc, void* vc, const int* msrc, const int* mdst, cons
 
 int launch_attention(const void* q, const void* k, const void* v, int M, int N, int H, int dtype, void* out,
                      void* scratch, int* status, cudaStream_t st, AttnKvMaps* maps = nullptr,
-                     const float* kmax2 = nullptr, float* lse = nullptr, bool beside_previous = false) {
-  if (dtype == kBF16) {
-    int rc = attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, 0, kmax2, lse, beside_previous);
-    if (rc == OVGGT_OK) g_launches.fetch_add(attn_tcgen05_num_launches(M, N, H));
-    if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
-    return rc;
-  }
+                     const float* kmax2 = nullptr, float* lse = nullptr, bool beside_previous = false,
+                     unsigned* tickets = nullptr) {
   int launches = 0;
-  const int rc = attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, &launches);
+  const int rc = dtype == kBF16 ? attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, 0, kmax2, lse,
+                                                      beside_previous, tickets, &launches)
+                                : attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, tickets,
+                                                  &launches);
   g_launches.fetch_add(launches);
   if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
   return rc;
@@ -258,8 +256,9 @@ struct ovggt_cache {
   float *qk_part = nullptr, *qk_sum = nullptr;       // OVGGT_SCORE_QK: column sums of the frame's queries
   float *attn_lse = nullptr, *attn_part = nullptr;   // OVGGT_SCORE_ATTN: log2 softmax denominators [M, H], per-head sums [H, M]
   void* attn_scratch = nullptr;
+  unsigned* attn_tickets = nullptr;
   int* status = nullptr;
-  size_t zeroed_bytes = 0;                           // the status block and the key-norm bounds behind it
+  size_t zeroed_bytes = 0;                           // the status block, the key-norm bounds and the attention's tickets behind it
   // two sets of staging buffers for ovggt_layer_step_host: the copies of one step overlap the kernels of the step before
   char *stage_q[2] = {}, *stage_k[2] = {}, *stage_v[2] = {}, *stage_r[2] = {}, *stage_o[2] = {};
   float* stage_conf[2] = {};
@@ -423,8 +422,9 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
   }
   const size_t o_part = L.take((size_t)kMaxColsumParts * C * 4);
   const size_t o_attn = L.take(ovggt_k_attention_scratch_bytes(M, max_rows, c->n_heads));
-  // what starts at zero lies together: the status word, then every layer's bound of the key norms
-  const size_t o_status = L.take(64 + (size_t)c->n_layers * c->n_heads * 4);
+  // what starts at zero lies together: the status word, then every layer's bound of the key norms, then the attention's tickets
+  const size_t bounds_bytes = (size_t)c->n_layers * c->n_heads * 4, zeroed = 64 + bounds_bytes + attn_tickets(M, c->n_heads) * 4;
+  const size_t o_status = L.take(zeroed);
   const bool qk = c->score_mode == OVGGT_SCORE_QK;
   const size_t o_qk = qk ? L.take((size_t)(colsum_parts(M) + 1) * C * 4) : 0;
   const bool aw = c->score_mode == OVGGT_SCORE_ATTN;
@@ -438,7 +438,8 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
     h->colsum_part = reinterpret_cast<float*>(base + o_part);
     h->attn_scratch = base + o_attn;
     h->status = reinterpret_cast<int*>(base + o_status);
-    h->zeroed_bytes = 64 + (size_t)c->n_layers * c->n_heads * 4;
+    h->zeroed_bytes = zeroed;
+    h->attn_tickets = reinterpret_cast<unsigned*>(base + o_status + 64 + bounds_bytes);
     for (int l = 0; l < c->n_layers; ++l)
       h->layers[l].kmax2 = reinterpret_cast<float*>(base + o_status + 64) + (size_t)l * c->n_heads;
     if (aw) {
@@ -667,7 +668,7 @@ int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, c
     ProfScope ps(h, OVGGT_PROF_ATTENTION, st);
     rc = launch_attention(io->q, S.kbuf[kb], S.vbuf[kb], h->M, N, h->cfg.n_heads, h->cfg.dtype, io->out,
                           h->attn_scratch, h->status, st, &S.maps[kb], key_norm_bound(h, S),
-                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous);
+                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous, h->attn_tickets);
   }
   return rc;
 }
