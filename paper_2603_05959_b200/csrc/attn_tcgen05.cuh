@@ -924,11 +924,12 @@ inline int make_rows_map(CUtensorMap* map, const void* base, int rows, int C, in
 }
 
 // Whether the parts are joined inside the attention, for `ctas` CTAs of `per` KV tiles: where all of them are resident at once,
-// so that a CTA that joins keeps no other from starting, and done before the selection of the same step, 20 to 30 us, for
-// which a kernel of its own would wait.  Steps of 329 x 3329 x 10 and 605 x 20605 x 5 take 27.3 and 45.5 us joined inside,
-// 30.1 and 50.3 us otherwise; where the selection ends first the launch is the cheaper way, as it uses every SM: 905 x
-// 20905 x 12 (288 CTAs of 55 tiles) takes 93.0 and 90.7 us, 1374 x 17758 x 16 (528 CTAs) 144.1 and 140.3 us.
-constexpr int kJoinMaxTiles = 16;
+// so that a CTA that joins keeps no other from starting, and done before the selection of the same step (20 to 40 us), for
+// which a kernel of its own would wait.  Measured over steps of 126 x 8126 x 16 heads to 1374 x 15374 x 5: joining inside
+// saves 1.5 to 3.5 us (329 x 9329 x 12: 39.4 -> 37.0 us) up to 10 tiles, is worth -1 to 1.5 us from 11 to 15 and costs 3 to
+// 5 us from 17 (734 x 9734 x 16: 52.4 -> 55.5 us), where the selection has ended first and a launch of its own can use
+// every SM.
+constexpr int kJoinMaxTiles = 11;
 inline bool attn_join_inside(long ctas, int per) { return ctas <= (long)kCtasPerSm * 148 && per <= kJoinMaxTiles; }
 
 // Number of KV splits, from a model in nanoseconds fitted to a sweep of 1 to 16 splits over eighteen shapes (69 x 325 x 4
