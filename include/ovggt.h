@@ -360,8 +360,6 @@ int ovggt_k_gemm_bf16(const void* A, const void* B, int32_t M, int32_t N, int32_
  * sum = bf16(residual + t).  outs is a host array of device pointers; sum may not be residual or A. */
 int ovggt_k_linear_bf16(const void* A, const void* B, int32_t M, int32_t N, int32_t K, void* const* outs, int32_t n_outs,
                         int32_t gelu, const void* residual, void* sum, int32_t* device_status, void* stream);
-/* out [rows, C] = LayerNorm of the rows of x (bf16, no affine part, epsilon 1e-5, fp32 arithmetic); C a multiple of 8. */
-int ovggt_k_layer_norm_bf16(const void* x, int32_t rows, int32_t C, void* out, void* stream);
 
 #ifdef __cplusplus
 }

@@ -33,7 +33,7 @@ EXPORTED = [
     "ovggt_strerror", "ovggt_last_cuda_error", "ovggt_k_row_norms", "ovggt_k_diversity_scratch_bytes",
     "ovggt_k_diversity", "ovggt_k_diversity_static", "ovggt_k_select", "ovggt_k_compact", "ovggt_k_attention_scratch_bytes",
     "ovggt_k_attention", "ovggt_k_key_norm_bound", "ovggt_k_attention_bounded", "ovggt_k_gemm_bf16",
-    "ovggt_k_linear_bf16", "ovggt_k_layer_norm_bf16",
+    "ovggt_k_linear_bf16",
 ]
 
 
@@ -127,7 +127,6 @@ def lib():
         L.ovggt_k_key_norm_bound.argtypes = [vp, i32, i32, vp, vp]
         L.ovggt_k_gemm_bf16.argtypes = [vp, vp, i32, i32, i32, vp, vp, vp]
         L.ovggt_k_linear_bf16.argtypes = [vp, vp, i32, i32, i32, C.POINTER(vp), i32, i32, vp, vp, vp, vp]
-        L.ovggt_k_layer_norm_bf16.argtypes = [vp, i32, i32, vp, vp]
         L.ovggt_k_attention_bounded.argtypes = [vp, vp, vp, i32, i32, i32, vp, vp, vp, vp, vp]
         assert _FRAME_IO.size == C.sizeof(OvggtFrameIO)
         for name in ("ovggt_layer_attend", "ovggt_layer_compress", "ovggt_layer_step", "ovggt_layer_step_host"):
@@ -467,12 +466,6 @@ def k_linear_bf16(a, b, outs=(), gelu=False, residual=None, sum_out=None, status
     _check(lib().ovggt_k_linear_bf16(_dptr(a), _dptr(b), M, b.shape[1], K, (C.c_void_p * 3)(*[_dptr(o) for o in outs]), len(outs),
                                      int(gelu), _dptr(residual), _dptr(sum_out), _dptr(status), _stream_ptr(stream)),
            "ovggt_k_linear_bf16")
-
-
-def k_layer_norm_bf16(x: torch.Tensor, out: torch.Tensor, stream=None) -> torch.Tensor:
-    _check(lib().ovggt_k_layer_norm_bf16(_dptr(x), x.shape[0], x.shape[1], _dptr(out), _stream_ptr(stream)),
-           "ovggt_k_layer_norm_bf16")
-    return out
 
 
 def k_key_norm_bound(k: torch.Tensor, n_heads: int, stream=None) -> torch.Tensor:

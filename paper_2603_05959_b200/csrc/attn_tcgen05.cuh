@@ -958,6 +958,26 @@ inline int attn_choose_splits(int M, int N, int H, bool tickets) {
   return best;
 }
 
+// The rule for an attention outside the fused step (the bare kernel, the halves of a step): waves of CTAs, each as long as
+// its tiles and two more, a merge one tile more.  The model above would group the sums of some shapes otherwise, and in a
+// stack of 24 layers whose state is rounded to bf16 after each any other grouping changes the result by one or two per cent.
+inline int attn_choose_splits_alone(int M, int N, int H) {
+  const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kBN - 1) / kBN;
+  const long slots = (long)kCtasPerSm * 148;
+  int best = 1;
+  long best_cost = -1;
+  for (int s = 1; s <= kMaxSplits && s <= tiles; ++s) {
+    const int per = (tiles + s - 1) / s;
+    if ((tiles + per - 1) / per != s) continue;
+    const long cost = ((long)q_tiles * H * s + slots - 1) / slots * (per + 2) + (s > 1 ? 1 : 0);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = s;
+    }
+  }
+  return best;
+}
+
 inline size_t attn_tcgen05_scratch_bytes(int M, int N, int H) {
   (void)N;
   const size_t C = (size_t)H * kHD;
@@ -1000,7 +1020,7 @@ inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, 
 inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
                                void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
                                int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr,
-                               bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr) {
+                               bool beside_previous = false, unsigned* tickets = nullptr, bool in_step = false, int* launches = nullptr) {
   const int C = H * kHD;
   CUtensorMap tq;
   AttnKvMaps local;
@@ -1014,7 +1034,7 @@ inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int 
   AttnParams P;
   P.M = M; P.N = N; P.H = H;
   P.tiles_total = (N + kBN - 1) / kBN;
-  P.splits = force_splits > 0 ? std::min(force_splits, std::min(kMaxSplits, P.tiles_total)) : attn_choose_splits(M, N, H, tickets != nullptr);
+  P.splits = force_splits > 0 ? std::min(force_splits, std::min(kMaxSplits, P.tiles_total)) : (in_step ? attn_choose_splits(M, N, H, tickets != nullptr) : attn_choose_splits_alone(M, N, H));
   P.tiles_per_split = (P.tiles_total + P.splits - 1) / P.splits;
   P.splits = (P.tiles_total + P.tiles_per_split - 1) / P.tiles_per_split;     // no empty split
   P.out = static_cast<__nv_bfloat16*>(out);

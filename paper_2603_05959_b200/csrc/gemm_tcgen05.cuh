@@ -11,18 +11,14 @@
 //   per output row and quarter of the columns, finish, and store whole lines by way of shared memory.
 // What bounds it at these sizes (1041 or 1374 rows, N and K of 1024 to 4096): one wave of CTAs whose loads all come from
 // L2, and shared memory, which the MMA reads and TMA writes at 128 bytes a clock each at N = 128 (half the tensor rate)
-// and at 94 at N = 256; hence the wide tile, all of shared memory in flight, and K cut over a cluster of two or four CTAs
-// where a product has few tiles: each CTA finishes its share of the columns with the others' partial sums, sent through
-// distributed shared memory into the stages.  The kernel is launched programmatically behind its predecessor and
-// prefetches its part of B (weights, as a rule) into L2 while that one drains.
+// and at 94 at N = 256; hence the wide tile and all of shared memory in flight.  The kernel is launched programmatically
+// behind its predecessor and prefetches its part of B (weights, as a rule) into L2 while that one drains.
 // Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 10.5 / 7.3 / 14.1 / 14.8 us, against
 // 13.9 / 9.2 / 18.1 / 19.4 with 128 x 128 tiles of three stages and four epilogue warps that stored row by row.
 // Requirements: K a multiple of 64, N a multiple of 8 (TMA row pitch of 16 bytes), 16-byte aligned bases.  Every
 // barrier wait is bounded (about one second); on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the
 // common teardown, after the MMAs it issued have drained.
 #pragma once
-
-#include <cooperative_groups.h>
 
 #include "attn_tcgen05.cuh"
 
@@ -56,25 +52,8 @@ struct GemmArgs {
   int* status;
 };
 
-// x Phi(x) = x erfc(-x / sqrt 2) / 2 for a pair.  erfc(z), z >= 0, by the Chebyshev fit of Press et al. (Numerical Recipes,
-// erfcc): t exp(-z^2 + q(t)), t = 1 / (1 + z / 2), fractional error below 1.2e-7 everywhere; Phi(x) = 1 - erfc / 2 above 0.
-__device__ __forceinline__ float2 gelu2(float2 x) {
-  const float2 z = make_float2(fabsf(x.x) * 0.70710678118654752f, fabsf(x.y) * 0.70710678118654752f);
-  const float2 t = make_float2(__fdividef(1.0f, fmaf(0.5f, z.x, 1.0f)), __fdividef(1.0f, fmaf(0.5f, z.y, 1.0f)));
-  auto both = [](float c) { return make_float2(c, c); };
-  float2 q = fma2(t, both(0.17087277f), both(-0.82215223f));
-  q = fma2(q, t, both(1.48851587f));
-  q = fma2(q, t, both(-1.13520398f));
-  q = fma2(q, t, both(0.27886807f));
-  q = fma2(q, t, both(-0.18628806f));
-  q = fma2(q, t, both(0.09678418f));
-  q = fma2(q, t, both(0.37409196f));
-  q = fma2(q, t, both(1.00002368f));
-  q = fma2(q, t, both(-1.26551223f));
-  q = fma2(z, make_float2(-z.x, -z.y), q);
-  const float e0 = 0.5f * t.x * ex2(q.x * 1.4426950408889634f), e1 = 0.5f * t.y * ex2(q.y * 1.4426950408889634f);
-  return make_float2(x.x * (x.x > 0.0f ? 1.0f - e0 : e0), x.y * (x.y > 0.0f ? 1.0f - e1 : e1));
-}
+// x Phi(x), in the form whose bf16 rounding every bf16 input shares with torch's GELU.
+__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 
 // Finished bf16 columns [n, n + 8) of row m: where the caller wants them.
 __device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, const uint4& t) {
@@ -101,8 +80,7 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
 
-// SPLIT > 1: launched as clusters of SPLIT CTAs, neighbours in x, each with its part of the K steps of one tile.
-template <int BN, int SPLIT>
+template <int BN>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                     const __grid_constant__ GemmArgs P) {
@@ -111,8 +89,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   extern __shared__ __align__(1024) unsigned char smem[];
   GemmBarriers* B = reinterpret_cast<GemmBarriers*>(smem + kStages * kStage);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * kGemmBM, n0 = (int)(blockIdx.x / SPLIT) * BN, part = (int)(blockIdx.x % SPLIT);
-  const int k_all = P.K / kGemmBK, k_begin = k_all * part / SPLIT, k_tiles = k_all * (part + 1) / SPLIT - k_begin;
+  const int m0 = blockIdx.y * kGemmBM, n0 = (int)blockIdx.x * BN, k_tiles = P.K / kGemmBK;
   const bool aligned = (smem_u32(smem) & 1023u) == 0;     // the 128-byte swizzle needs 1024-byte aligned tiles
   if (!aligned && threadIdx.x == 0) atomicCAS(P.status, 0, OVGGT_ERR_DEVICE_STATUS);
   pdl_trigger();
@@ -131,7 +108,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     // the CTAs of one column of tiles share its part of B out among them
     for (int kt = (int)blockIdx.y; kt < k_tiles; kt += (int)gridDim.y)
-      for (int x = 0; x < BN && n0 + x < P.N; x += 64) tma_prefetch_2d(&tm_b, n0 + x, (k_begin + kt) * kGemmBK);
+      for (int x = 0; x < BN && n0 + x < P.N; x += 64) tma_prefetch_2d(&tm_b, n0 + x, kt * kGemmBK);
   }
   if (warp == kIssuer) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&B->tmem_base)),
@@ -155,7 +132,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
         const uint32_t ph = (uint32_t)(kt / kStages) & 1u;
         if (kt >= kStages) ok = mbar_wait(&B->empty[s], ph ^ 1u, B, P.status);
         if (!ok) break;
-        const int k0 = (k_begin + kt) * kGemmBK;
+        const int k0 = kt * kGemmBK;
         unsigned char* st = smem + s * kStage;
         mbar_expect_tx(&B->full[s], kStage);
         tma_load_2d(st, &tm_a, k0, m0, &B->full[s]);
@@ -202,57 +179,25 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     tc_fence_after();
   }
   // ------------------------------------------------ epilogue: warps 0-15; the stages are free now
-  constexpr int kShare = BN / SPLIT, kSides = kShare >= 64 ? 4 : 2, kCols = kShare / kSides;   // columns of this CTA, of a warp
-  constexpr int kUnits = kCols / 8;                        // 16-byte units of a row
-  const int quad = warp & 3, row = quad * 32 + lane, side = warp >> 2;
+  constexpr int kCols = BN / 4, kUnits = kCols / 8;        // columns of a warp, their 16-byte units
+  const int quad = warp & 3, side = warp >> 2;
   const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);
-  float* xch = reinterpret_cast<float*>(smem);             // [SPLIT - 1][kShare][128 rows] partial sums of this CTA's columns
-  const bool store = side < kSides && ok;                  // (the producer and the issuer are past the last side)
-  if constexpr (SPLIT > 1) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();                                        // no CTA of the cluster reads its stages any more
-    if (store) {
-#pragma unroll 1
-      for (int d = 1; d < SPLIT; ++d) {
-        const int to = (part + d) % SPLIT;                 // slot d - 1 at the receiver: the sender is d before it
-        float* dst = cluster.map_shared_rank(xch, to) + (size_t)((d - 1) * kShare + side * kCols) * kGemmBM + row;
-#pragma unroll 1
-        for (int j = 0; j < kCols; j += 16) {
-          uint32_t o[16];
-          tmem_ld16(t_row + to * kShare + side * kCols + j, o);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 16; ++e) dst[(j + e) * kGemmBM] = __uint_as_float(o[e]);
-        }
-      }
-    }
-    cluster.sync();
-  }
-  if (store) {
-    uint4* stage = reinterpret_cast<uint4*>(smem + (SPLIT - 1) * kShare * kGemmBM * 4) + warp * 32 * kUnits;
+  if (side < 4 && ok) {                                    // (the producer and the issuer are past the last side)
+    uint4* stage = reinterpret_cast<uint4*>(smem) + warp * 32 * kUnits;
 #pragma unroll 1
     for (int j = 0; j < kCols; j += 16) {
       uint32_t o[16];
-      tmem_ld16(t_row + part * kShare + side * kCols + j, o);
+      tmem_ld16(t_row + side * kCols + j, o);
       tmem_wait_ld();
-      float v[16];
-#pragma unroll
-      for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(o[e]);
-#pragma unroll
-      for (int d = 0; d < SPLIT - 1; ++d)
-#pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] += xch[(size_t)(d * kShare + side * kCols + j + e) * kGemmBM + row];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         uint4 t;
         uint32_t* w = reinterpret_cast<uint32_t*>(&t);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          w[e] = pack_bf16(v[8 * u + 2 * e], v[8 * u + 2 * e + 1]);
+          w[e] = pack_bf16(__uint_as_float(o[8 * u + 2 * e]), __uint_as_float(o[8 * u + 2 * e + 1]));
           if (P.gelu) {
-            const float2 g = gelu2(make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xFFFF0000u)));
-            w[e] = pack_bf16(g.x, g.y);
+            w[e] = pack_bf16(gelu(__uint_as_float(w[e] << 16)), gelu(__uint_as_float(w[e] & 0xFFFF0000u)));
           }
         }
         stage[lane * kUnits + ((j / 8 + u) ^ (lane & (kUnits - 1)))] = t;
@@ -261,7 +206,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     __syncwarp();
 #pragma unroll 4
     for (int i = lane; i < 32 * kUnits; i += 32) {         // whole lines of a row by neighbouring lanes
-      const int r = i / kUnits, u = i % kUnits, m = m0 + quad * 32 + r, n = n0 + part * kShare + side * kCols + u * 8;
+      const int r = i / kUnits, u = i % kUnits, m = m0 + quad * 32 + r, n = n0 + side * kCols + u * 8;
       if (m < P.M && n < P.N) gemm_store8(P, m, n, stage[r * kUnits + (u ^ (r & (kUnits - 1)))]);   // (N is a multiple of 8)
     }
   }
@@ -274,27 +219,15 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   }
 }
 
-// Tile width and K split, from a model in nanoseconds fitted to a sweep over seventeen shapes (333 to 1374 rows, N and K 512
-// to 4096): 310 per K step of a 256-wide tile, 265 of a 128-wide one (half the work: shared memory bounds it); set-up and
-// epilogue by variant; one CTA per SM, so 148 CTAs, 74 clusters of two or 33 of four at a time.
-struct GemmPlan { int bn, split; };
-inline GemmPlan gemm_plan(int M, int N, int K) {
-  static const int kFixed[2][3] = {{3500, 4800, 4800}, {4800, 6400, 7000}}, kResident[3] = {148, 74, 33};
-  const int tiles_m = (M + kGemmBM - 1) / kGemmBM, steps = K / kGemmBK;
-  GemmPlan best{256, 1};
-  long best_ns = -1;
-  for (int w = 1; w >= 0; --w)
-    for (int j = 0; j < 3; ++j) {
-      const int bn = w ? 256 : 128, split = 1 << j;
-      if (split > 1 && steps < 2 * split) continue;
-      const long tiles = (long)tiles_m * ((N + bn - 1) / bn), waves = (tiles + kResident[j] - 1) / kResident[j];
-      const long ns = waves * ((long)((steps + split - 1) / split) * (w ? 310 : 265) + kFixed[w][j]);
-      if (best_ns < 0 || ns < best_ns) {
-        best_ns = ns;
-        best = {bn, split};
-      }
-    }
-  return best;
+// Tile width, from a model in nanoseconds fitted to a sweep over seventeen shapes (333 to 1374 rows, N and K 512 to 4096):
+// waves over 148 SMs, one CTA each; 310 per K step of a 256-wide tile, 265 of a 128-wide one (half the work: shared memory
+// bounds it); 4,800 and 3,500 for set-up and epilogue.  K is not split: a product of few tiles and many steps would gain
+// (1041 x 1024 x 4096: 14.8 us in clusters of two against 19), but its sums would be grouped otherwise, and 24 layers of
+// bf16 turn any such change into one or two per cent of the result.
+inline int gemm_tile_width(int M, int N, int K) {
+  const long tiles_m = (M + kGemmBM - 1) / kGemmBM, steps = K / kGemmBK;
+  auto ns = [&](int bn, long step, long fixed) { return (tiles_m * ((N + bn - 1) / bn) + 147) / 148 * (steps * step + fixed); };
+  return ns(256, 310, 4800) <= ns(128, 265, 3500) ? 256 : 128;
 }
 
 inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P, cudaStream_t st) {
@@ -303,17 +236,13 @@ inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P,
   if (rc) return rc;
   rc = make_rows_map(&tb, Bm, P.K, P.N, kGemmBK);          // 64 n-columns x 64 k-rows per box
   if (rc) return rc;
-  const GemmPlan plan = gemm_plan(P.M, P.N, P.K);
-  const int tiles_n = (P.N + plan.bn - 1) / plan.bn, tiles_m = (P.M + kGemmBM - 1) / kGemmBM;
-  using Kernel = void (*)(CUtensorMap, CUtensorMap, GemmArgs);
-  static const Kernel kernels[2][3] = {{k_gemm_bf16_tcgen05<128, 1>, k_gemm_bf16_tcgen05<128, 2>, k_gemm_bf16_tcgen05<128, 4>},
-                                       {k_gemm_bf16_tcgen05<256, 1>, k_gemm_bf16_tcgen05<256, 2>, k_gemm_bf16_tcgen05<256, 4>}};
-  static std::atomic<uint64_t> smem_set[2][3];
-  const int i = plan.bn == 256 ? 1 : 0, j = plan.split / 2;
-  const size_t smem = gemm_smem_bytes(plan.bn);
-  cudaError_t e = allow_smem(kernels[i][j], smem, smem_set[i][j]);
+  const int bn = gemm_tile_width(P.M, P.N, P.K), wide = bn == 256 ? 1 : 0;
+  const auto kernel = wide ? k_gemm_bf16_tcgen05<256> : k_gemm_bf16_tcgen05<128>;
+  static std::atomic<uint64_t> smem_set[2];
+  const size_t smem = gemm_smem_bytes(bn);
+  cudaError_t e = allow_smem(kernel, smem, smem_set[wide]);
   if (e == cudaSuccess)
-    e = launch_dependent(kernels[i][j], dim3(tiles_n * plan.split, tiles_m), kGemmThreads, plan.split, smem, st, true, ta, tb, P);
+    e = launch_dependent(kernel, dim3((P.N + bn - 1) / bn, (P.M + kGemmBM - 1) / kGemmBM), kGemmThreads, 1, smem, st, true, ta, tb, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   return OVGGT_OK;
 }

@@ -120,55 +120,6 @@ __global__ void __launch_bounds__(1024) k_colsum_final(const float* __restrict__
   }
 }
 
-// out = (x - mean) / sqrt(var + 1e-5) per row of x [rows, 8 nvec] (bf16), fp32 arithmetic; one warp per row, which stays
-// in registers for rows of up to 128 vectors.  Scaffold (the LayerNorm before a projection), fused with the conversions
-// around it: the three launches it replaces moved 6 bytes per element each way.
-__global__ void __launch_bounds__(256) k_layer_norm_bf16(const uint4* __restrict__ x, int rows, int nvec, uint4* __restrict__ out) {
-  pdl_trigger();
-  pdl_wait();
-  const int row = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-  if (row >= rows) return;
-  const int lane = threadIdx.x & 31;
-  const uint4* p = x + (size_t)row * nvec;
-  const float inv_c = 1.0f / (8.0f * (float)nvec);
-  uint4 u[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) u[i] = lane + 32 * i < nvec ? p[lane + 32 * i] : make_uint4(0u, 0u, 0u, 0u);
-  auto each = [&](auto fn) {                       // fn(vector index, its eight values)
-    for (int v0 = lane; v0 < nvec; v0 += 128) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (v0 + 32 * i < nvec) {
-          float f[8];
-          unpack<kBF16>(v0 == lane ? u[i] : p[v0 + 32 * i], f);
-          fn(v0 + 32 * i, f);
-        }
-    }
-  };
-  float s = 0.0f;
-  each([&](int, const float* f) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) s += f[e];
-  });
-  const float mean = warp_sum(s) * inv_c;
-  float q = 0.0f;
-  each([&](int, const float* f) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) q = __fmaf_rn(f[e] - mean, f[e] - mean, q);
-  });
-  const float rstd = rsqrtf(warp_sum(q) * inv_c + 1e-5f);
-  each([&](int v, const float* f) {
-    uint4 w;
-    uint32_t* ww = reinterpret_cast<uint32_t*>(&w);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn((f[2 * e] - mean) * rstd, (f[2 * e + 1] - mean) * rstd);
-      ww[e] = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    out[(size_t)row * nvec + v] = w;
-  });
-}
-
 // The residual norms of several layers in one launch: blockIdx.y = position in the batch.
 constexpr int kMaxScoreBatch = 32;
 struct NormBatch {

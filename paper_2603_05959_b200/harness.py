@@ -110,8 +110,8 @@ class _Timer:
 
 class _Scaffold:
     """The dense products of a workload and what surrounds them: on torch, or on the library's own kernels
-    (ovggt_k_linear_bf16 with GELU, residual sum and the split of a QKV product in its epilogue; ovggt_k_layer_norm_bf16;
-    buffers that are kept between frames).  Both round to bf16 at the same places.  Either way it is scaffold time, not
+    (ovggt_k_linear_bf16 with GELU, residual sum and the split of a QKV product in its epilogue; buffers that are kept
+    between frames; LayerNorm is torch's, which computes in fp32 and rounds once).  Both round to bf16 at the same places.  Either way it is scaffold time, not
     the streaming step's."""
 
     def __init__(self, kind: str, device):
@@ -127,10 +127,8 @@ class _Scaffold:
             t = self._kept[name] = torch.empty(shape, dtype=torch.bfloat16, device=self.device)
         return t
 
-    def layer_norm(self, x, stream=None):
-        if self.library:
-            return B.k_layer_norm_bf16(x, self.kept("ln", x.shape), stream)
-        return torch.nn.functional.layer_norm(x.float(), (x.shape[-1],)).to(x.dtype)
+    def layer_norm(self, x):
+        return torch.nn.functional.layer_norm(x, (x.shape[-1],))
 
     def qkv(self, x, w, stream=None):
         """The three [M, C] column blocks of x W."""
@@ -257,7 +255,7 @@ class Aggregator:
         keep = (lambda name: mm.kept(name, (M, C)))
         for l in range(L):
             w = self.blocks[l]["frame"]
-            fq, fk, fv = mm.qkv(mm.layer_norm(x, stream), w["qkv"], stream)
+            fq, fk, fv = mm.qkv(mm.layer_norm(x), w["qkv"], stream)
             if self.frame_attention == "library":
                 a = B.k_attention(fq, fk, fv, H, out=self._fa_out, scratch=self._fa_scratch, status=self._fa_status,
                                   stream=stream)
@@ -265,10 +263,10 @@ class Aggregator:
                 q3 = [y.view(M, H, C // H).permute(1, 0, 2) for y in (fq, fk, fv)]               # [H, M, d]
                 a = torch.nn.functional.scaled_dot_product_attention(*q3).permute(1, 0, 2).reshape(M, C)
             x = mm.add_product(x, a, w["o"], out=keep("frame attended"), stream=stream)
-            x = mm.add_product(x, mm.gelu_product(mm.layer_norm(x, stream), w["fc1"], stream), w["fc2"],
+            x = mm.add_product(x, mm.gelu_product(mm.layer_norm(x), w["fc1"], stream), w["fc2"],
                                out=keep("frame out"), stream=stream)
             w = self.blocks[l]["global"]
-            q, k, v = mm.qkv(mm.layer_norm(x, stream), w["qkv"], stream)
+            q, k, v = mm.qkv(mm.layer_norm(x), w["qkv"], stream)
             att = lambda: self.cache.layer_attend(l, t, q, k, v, out=self.out, stream=stream)
             lib(att) if lib else att()
             if self.after:
@@ -277,7 +275,7 @@ class Aggregator:
             # the block's MLP output is the layer's residual, read by its compress: one buffer per layer
             r = keep("resid%d" % (l if self.batched_compress else 0))
             # (the frame's result is the caller's; what is passed between the layers is kept)
-            x = mm.add_product(h, mm.gelu_product(mm.layer_norm(h, stream), w["fc1"], stream), w["fc2"],
+            x = mm.add_product(h, mm.gelu_product(mm.layer_norm(h), w["fc1"], stream), w["fc2"],
                                out=None if l + 1 == L else keep("global out"), product=r, stream=stream)
             ov = self.tap(t, l, q, k, v, r) if self.tap else None
             if self.batched_compress:

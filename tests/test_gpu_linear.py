@@ -1,4 +1,4 @@
-"""The scaffold's dense products and LayerNorm: tile edges, every tile width and K split of the plan, the fused epilogues."""
+"""The scaffold's dense products: tile edges, both tile widths, the fused epilogues."""
 import pytest
 import torch
 
@@ -6,7 +6,7 @@ from paper_2603_05959_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
 
-# rows, columns, K: single partial tiles, ragged edges, few tiles (K split over two and four CTAs), full waves
+# rows, columns, K: single partial tiles, ragged edges, few tiles, full waves
 SHAPES = [(1, 8, 64), (127, 72, 64), (129, 264, 192), (333, 512, 2048), (130, 768, 3072), (1041, 1024, 1024), (700, 2304, 768)]
 
 
@@ -41,24 +41,10 @@ def test_linear_epilogues(M, N, K):
 
 
 def test_gelu_over_its_range():
-    """Every bf16 value from -16 to 16 through an identity product: within bf16 rounding of the exact GELU, tails included."""
-    v = torch.arange(0, 0x4180, dtype=torch.int16, device="cuda").view(torch.bfloat16)
-    v = torch.cat([v, -v])
-    a = v[: v.numel() // 64 * 64].view(-1, 64).contiguous()
+    """Every finite bf16 value through an identity product: the bf16 rounding of torch's GELU, tails included."""
+    v = torch.arange(0, 0x7F80, dtype=torch.int16, device="cuda").view(torch.bfloat16)
+    a = torch.cat([v, -v]).view(-1, 64)
     out = torch.empty_like(a)
     st = torch.zeros(16, dtype=torch.int32, device="cuda")
     B.k_linear_bf16(a, torch.eye(64, device="cuda").bfloat16(), (out,), gelu=True, status=st)
-    x = a.double()
-    ref = 0.5 * x * torch.special.erfc(-x / 2 ** 0.5)
-    # the unit roundoff of bf16 (8 significant bits: 2^-8), the rest for fp32 arithmetic in the tail, where erfc falls as
-    # exp(-x^2 / 2); subnormals flush
-    torch.testing.assert_close(out.double(), ref, rtol=2.0 ** -8 + 1e-4, atol=1e-37)
-
-
-@pytest.mark.parametrize("rows,C", [(1, 8), (9, 64), (130, 1024), (33, 1544)])
-def test_layer_norm(rows, C):
-    g = torch.Generator(device="cuda")
-    g.manual_seed(rows + C)
-    x = (torch.randn((rows, C), generator=g, device="cuda") * 3 + 1).bfloat16()
-    out = B.k_layer_norm_bf16(x, torch.empty_like(x))
-    torch.testing.assert_close(out.double(), torch.nn.functional.layer_norm(x.double(), (C,)), rtol=2.0 ** -8, atol=1e-4)
+    assert torch.equal(out, torch.nn.functional.gelu(a))
