@@ -10,8 +10,11 @@
 // about a microsecond.  So the usual way to T takes three: one to exchange the groups' ranges (Eq. 7), one after which
 // every CTA reads all CTAs' 512-bin histograms of the priorities and finds the bin of the B-th row, one after which every
 // CTA reads the few candidates of that bin and ranks them by comparison; the counts that place each CTA's output travel
-// with them.  When the bin is crowded (many equal or nearly equal priorities) four 8-bit radix passes over the keys find
-// T instead, which takes a barrier each.  A warp then owns a contiguous range of positions and writes survivors, meta
+// with them.  A crowded bin is histogrammed once more in 256 finer ones with the range of keys in each: a stream whose
+// frames recur fills its cache with copies of the same scores, and the finer bin then holds nothing but ties, which go by
+// position alone (a step of 1374 x 5470 x 16 in stored-score mode, after 10,000 frames that recur: 69.4 us with radix passes
+// alone, 58.9 us so).  What is still crowded and not one key takes four 8-bit radix passes,
+// a barrier each.  A warp then owns a contiguous range of positions and writes survivors, meta
 // and moves with ballots, so that neighbouring lanes write neighbouring words.  (Radix passes for every step, a
 // contiguous range per thread, and a separate exchange for the moves took 36 us at 17758 candidates and 18 us at 325.)
 #pragma once
@@ -29,6 +32,7 @@ constexpr int kSelectThreads = 512;   // 512 x 64 registers: half an SM, so a CT
 constexpr int kSelectWarps = kSelectThreads / 32;
 constexpr int kSelectMaxCtas = 8;
 constexpr int kSelectBins = kSelectThreads;       // a thread per bin; the last bin holds the protected rows
+constexpr int kSelectSubBins = 256;               // of a crowded bin
 constexpr int kSelectCtaCands = 64, kSelectAllCands = 256;   // candidates of the threshold bin, per CTA and in all
 constexpr uint32_t kKeyProtected = 0xFFFFFFFFu;   // above the key of +inf (0xFF800000)
 
@@ -221,6 +225,105 @@ __device__ __noinline__ bool radix_threshold(const uint32_t* keys, int begin, in
   return prefix == kKeyProtected && eq_all > krem;
 }
 
+// The bin of the target-th row from the top, of the cluster's histograms hist[0 .. bins), into sh->digit, its rank inside
+// the bin into sh->krem and the CTAs' shares of the bin into sh->cnt_bin; what the lower ranks hold in the bins above is
+// added to sh->keep_before.  Thread t looks at bin (last - t); every CTA finds the bin for itself.
+template <bool SINGLE>
+__device__ __forceinline__ void find_bin(int* hist, int bins, int target, SelectShared* sh) {
+  using G = Peers<SINGLE>;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ncta = G::count(), rank = G::rank(), b = bins - 1 - tid;
+  int v[G::kMax], tot = 0, before = 0;
+#pragma unroll
+  for (int r = 0; r < G::kMax; ++r) v[r] = b >= 0 && r < ncta ? G::of(hist, r)[b] : 0;
+#pragma unroll
+  for (int r = 0; r < G::kMax; ++r) {
+    tot += v[r];
+    before += r < rank ? v[r] : 0;
+  }
+  int above = tot;                                     // inclusive over the warp's lanes, then over its lower warps
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xFFFFFFFFu, above, o);
+    if (lane >= o) above += y;
+  }
+  if (lane == 31) sh->wtot[warp][0] = above;
+  __syncthreads();
+  above += __reduce_add_sync(0xFFFFFFFFu, lane < warp ? sh->wtot[lane][0] : 0) - tot;
+  if (above < target && above + tot >= target) {
+    sh->digit = b;
+    sh->krem = target - above;
+#pragma unroll
+    for (int r = 0; r < G::kMax; ++r) sh->cnt_bin[r] = v[r];
+  }
+  __syncthreads();
+  block_add(b > sh->digit ? before : 0, &sh->keep_before);
+}
+
+// Finer bins of a crowded one: equal steps of the key between its edges (monotone, so a key may be a step off).
+struct SubBins {
+  uint32_t lo;
+  float scale;
+  __device__ __forceinline__ int of(uint32_t key) const {
+    return key > lo ? (int)fminf((float)(kSelectSubBins - 1), (float)(key - lo) * scale) : 0;
+  }
+};
+
+// The threshold bin, bf's sh->digit, in finer ones: as find_bin, for the sh->krem-th row of it.  Returns whether the finer
+// bin holds one key only, which is then sh->T.  mem: 3 kSelectSubBins words that the cluster may read until the next barrier.
+template <bool SINGLE>
+__device__ __noinline__ bool refine_bin(const uint32_t* keys, const uint16_t* bf, int cnt, SubBins sub, uint32_t* mem, SelectShared* sh) {
+  using G = Peers<SINGLE>;
+  const int tid = threadIdx.x, lane = tid & 31, bstar = sh->digit, target = sh->krem;
+  int* hist = reinterpret_cast<int*>(mem);
+  uint32_t *lo = mem + kSelectSubBins, *hi = lo + kSelectSubBins;
+  if (tid < kSelectSubBins) {
+    hist[tid] = 0;
+    lo[tid] = 0xFFFFFFFFu;
+    hi[tid] = 0;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int i = tid; i < cnt; i += (int)blockDim.x)
+    if ((bf[i] & (kSelectBins - 1)) == bstar) {
+      const uint32_t key = keys[i];
+      const int b = sub.of(key);
+      atomicAdd(&hist[b], 1);
+      atomicMin(&lo[b], key);
+      atomicMax(&hi[b], key);
+    }
+  G::sync();
+  find_bin<SINGLE>(hist, kSelectSubBins, target, sh);
+  const int b = sh->digit;
+  const uint32_t first = __reduce_min_sync(0xFFFFFFFFu, lane < G::count() ? G::of(lo, lane)[b] : 0xFFFFFFFFu);
+  const uint32_t last = __reduce_max_sync(0xFFFFFFFFu, lane < G::count() ? G::of(hi, lane)[b] : 0u);
+  if (tid == 0) sh->T = first;
+  __syncthreads();
+  return first == last;
+}
+
+// Where all rows of the threshold bin have the key sh->T: the position of the last one that stays, of those in this CTA (N:
+// all of its own, -1: none).  The lower ranks' ties come first, then the lower positions.
+__device__ __noinline__ int last_tie(const uint32_t* keys, int begin, int cnt, int N, int rank, SelectShared* sh) {
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  int mine = sh->krem;
+  for (int r = 0; r < rank; ++r) mine -= sh->cnt_bin[r];
+  int pos = mine >= sh->cnt_bin[rank] ? N : -1;
+  if (mine > 0 && pos < 0) {
+    const int chunk = (cnt + nthr - 1) / nthr, lo = min(cnt, tid * chunk), hi = min(cnt, lo + chunk);
+    const uint32_t T = sh->T;
+    int eq = 0, all;
+    for (int i = lo; i < hi; ++i) eq += keys[i] == T;
+    int before = block_excl_scan_int(eq, sh->scan, &all);
+    if (before < mine && before + eq >= mine)          // one thread
+      for (int i = lo; i < hi; ++i)
+        if (keys[i] == T && ++before == mine) sh->posT = begin + i;
+    __syncthreads();
+    pos = sh->posT;
+  }
+  __syncthreads();                                     // (the counts have been read)
+  return pos;
+}
+
 // Single-CTA pick used for the small top-A choice over the confidence map: marks the A largest of cnt keys
 // in keep[], ties to the lower index.
 __device__ inline void block_top_mark(const uint32_t* keys, uint8_t* keep, int cnt, int A, SelectShared* sh) {
@@ -271,6 +374,7 @@ __host__ __device__ inline size_t select_smem_bytes(int span) { return select_he
 // and slot (4) on chip, the frame's m raw residual norms, the np confidence keys and marks, and for the key sums'
 // corrections a list of rows (m that leave, m that come) and a block of sums.
 constexpr int kDeltaCols = 1024;
+static_assert(3 * kSelectSubBins <= kDeltaCols, "the finer bins lie in the block of sums");
 __host__ __device__ inline size_t compress_smem_bytes(int span, int np, int m) {
   const size_t s4 = ((size_t)span + 3) & ~(size_t)3, m4 = ((size_t)m + 3) & ~(size_t)3, np4 = ((size_t)np + 3) & ~(size_t)3;
   const size_t body = s4 * (8 + 3 * 4) + ((s4 + 7) & ~(size_t)7) * 2 + m4 * 4 + np4 * 4 + ((np4 + 15) & ~(size_t)15);
@@ -691,52 +795,42 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
     kw = wlo;                                          // everything stays
   } else {
     G::sync();
-    {
-      // thread t looks at bin (last - t): every CTA finds the bin of the B-th row for itself
-      const int b = kSelectBins - 1 - tid;
-      int v[G::kMax], tot = 0, before = 0;
-#pragma unroll
-      for (int r = 0; r < G::kMax; ++r) v[r] = r < ncta ? G::of(sh, r)->hist[b] : 0;
-#pragma unroll
-      for (int r = 0; r < G::kMax; ++r) {
-        tot += v[r];
-        before += r < rank ? v[r] : 0;
-      }
-      int above = tot;                                 // inclusive over the warp's lanes, then over its lower warps
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, above, o);
-        if (lane >= o) above += y;
-      }
-      if (lane == 31) sh->wtot[warp][0] = above;
-      __syncthreads();
-      above += __reduce_add_sync(0xFFFFFFFFu, lane < warp ? sh->wtot[lane][0] : 0) - tot;
-      if (above < P.B && above + tot >= P.B) {
-        sh->digit = b;
-        sh->krem = P.B - above;
-#pragma unroll
-        for (int r = 0; r < G::kMax; ++r) sh->cnt_bin[r] = v[r];
-      }
-      __syncthreads();
-      block_add(b > sh->digit ? before : 0, &sh->keep_before);   // rows the lower ranks keep in the bins above
-    }
+    find_bin<SINGLE>(sh->hist, kSelectBins, P.B, sh);
     const int bstar = sh->digit;
-    int cands = 0;
+    int cands = 0, sstar = -1;
     bool crowded = bstar == kSelectBins - 1;           // (more protected rows than B: an error the slow way reports)
-    for (int r = 0; r < ncta; ++r) {
-      cands += sh->cnt_bin[r];
-      crowded |= sh->cnt_bin[r] > kSelectCtaCands;
+    auto count = [&]() {
+      cands = 0;
+      for (int r = 0; r < ncta; ++r) {
+        cands += sh->cnt_bin[r];
+        crowded |= sh->cnt_bin[r] > kSelectCtaCands;
+      }
+      crowded |= cands > kSelectAllCands;
+    };
+    count();
+    // a crowded bin in finer ones, equal steps of the key between its edges (monotone, so a key may be a step off)
+    SubBins sub = {0, 1.0f};
+    bool ties = false;
+    if (!SINGLE && crowded && bstar < kSelectBins - 1) {   // (one CTA's radix passes are cheap: no cluster barriers)
+      const float step = bin_scale > 0.0f ? 1.0f / bin_scale : 0.0f, e0 = (float)bstar * step, e1 = (float)(bstar + 1) * step;
+      sub.lo = linear ? rank_key(bin_lo + e0) : bin_key0 + (uint32_t)e0;
+      const uint32_t hi = linear ? rank_key(bin_lo + e1) : bin_key0 + (uint32_t)e1;
+      if (hi > sub.lo) sub.scale = (float)kSelectSubBins / (float)(hi - sub.lo);
+      ties = refine_bin<SINGLE>(keys, bf, cnt, sub, reinterpret_cast<uint32_t*>(part), sh);   // (the block of sums is not in use yet)
+      sstar = sh->digit;
+      crowded = false;
+      count();
     }
-    crowded |= cands > kSelectAllCands;
     if (!crowded) {
       int up = 0, down = 0;
 #pragma unroll 1
       for (int i = tid; i < cnt; i += nthr) {
-        const int bin = bf[i] & (kSelectBins - 1);
+        int side = (bf[i] & (kSelectBins - 1)) - bstar;
+        if (!SINGLE && side == 0 && sstar >= 0) side = sub.of(keys[i]) - sstar;
         const bool u = is_up(i);
-        up += bin > bstar && u;
-        down += bin < bstar && !u;
-        if (bin == bstar) {
+        up += side > 0 && u;
+        down += side < 0 && !u;
+        if (side == 0) {
           const int c = atomicAdd(&sh->n_cand, 1);     // (in whatever order: they are ranked by key and position)
           if (c < kSelectCtaCands) {
             sh->cand.key[c] = keys[i];
@@ -790,9 +884,14 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       keep_all = P.B;
       warp_totals(wlo, whi, sh, classify, &kw, &uw, &dw);
     } else {
-      bad = radix_threshold<SINGLE>(keys, begin, cnt, P.B, sh);
-      T = sh->T;
-      posT = sh->posT;
+      if (!SINGLE && ties) {
+        T = sh->T;
+        posT = last_tie(keys, begin, cnt, N, rank, sh);
+      } else {
+        bad = radix_threshold<SINGLE>(keys, begin, cnt, P.B, sh);
+        T = sh->T;
+        posT = sh->posT;
+      }
       warp_totals(wlo, whi, sh, classify, &kw, &uw, &dw);
       if (tid == nthr - 32) {                          // the last warp: its prefix and its own count are the CTA's total
         sh->pub_keep = kw + sh->wtot[kSelectWarps - 1][0];
