@@ -192,10 +192,10 @@ int ovggt_camera_compress(ovggt_cache* camera, int32_t layer, const ovggt_frame_
                           int64_t demoted_frame, void* stream);
 
 /* ovggt_layer_attend and ovggt_layer_compress of one (frame, layer): the whole hot path.  Scoring and selection
- * read the cache and the new rows but not the attention's output, so they are enqueued on a second stream that the
- * handle owns (a host object, created by ovggt_cache_create), forked from and joined back into `stream` with
- * events, and run beside the attention; so does the stable gather, which writes another buffer.  The hole-filling
- * moves would write the buffer the attention reads: the selection only records them, and the layer's next append
+ * read the cache and the new rows but not the attention's output, so the attention runs beside them: launched
+ * programmatically behind the selection on `stream`, or, in the stable layout, on a second stream that the handle owns (a
+ * host object, created by ovggt_cache_create), forked and joined with events, beside the selection and the gather, which
+ * writes another buffer.  The hole-filling moves would write the buffer the attention reads: the selection only records them, and the layer's next append
  * (which touches the same slots) carries them out first; ovggt_cache_export flushes them.  For the caller the call
  * is still asynchronous and ordered on `stream` alone. */
 int ovggt_layer_step(ovggt_cache* cache, int32_t layer, const ovggt_frame_io* io, void* stream);

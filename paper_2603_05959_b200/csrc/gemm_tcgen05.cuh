@@ -13,8 +13,9 @@
 // L2, and shared memory, which the MMA reads and TMA writes at 128 bytes a clock each at N = 128 (half the tensor rate)
 // and at 94 at N = 256; hence the wide tile and all of shared memory in flight.  The kernel is launched programmatically
 // behind its predecessor and prefetches its part of B (weights, as a rule) into L2 while that one drains.
-// Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 10.5 / 7.3 / 14.1 / 14.8 us, against
-// 13.9 / 9.2 / 18.1 / 19.4 with 128 x 128 tiles of three stages and four epilogue warps that stored row by row.
+// Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 9.8 / 7.7 / 14.1 / 20.5 us, against
+// 13.9 / 9.2 / 18.1 / 19.4 with 128 x 128 tiles of three stages and four epilogue warps that stored row by row (the second
+// and the fourth of those with K split over two CTAs, see gemm_tile_width).
 // Requirements: K a multiple of 64, N a multiple of 8 (TMA row pitch of 16 bytes), 16-byte aligned bases.  Every
 // barrier wait is bounded (about one second); on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the
 // common teardown, after the MMAs it issued have drained.
@@ -222,7 +223,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
 // Tile width, from a model in nanoseconds fitted to a sweep over seventeen shapes (333 to 1374 rows, N and K 512 to 4096):
 // waves over 148 SMs, one CTA each; 310 per K step of a 256-wide tile, 265 of a 128-wide one (half the work: shared memory
 // bounds it); 4,800 and 3,500 for set-up and epilogue.  K is not split: a product of few tiles and many steps would gain
-// (1041 x 1024 x 4096: 14.8 us in clusters of two against 19), but its sums would be grouped otherwise, and 24 layers of
+// (1041 x 1024 x 4096: 14.8 us in clusters of two against 20.5), but its sums would be grouped otherwise, and 24 layers of
 // bf16 turn any such change into one or two per cent of the result.
 inline int gemm_tile_width(int M, int N, int K) {
   const long tiles_m = (M + kGemmBM - 1) / kGemmBM, steps = K / kGemmBK;

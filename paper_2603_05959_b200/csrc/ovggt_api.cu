@@ -269,8 +269,8 @@ struct ovggt_cache {
   float w_center = 0, w_edge = 0, w_corner = 0;
   cudaStream_t last_stream = nullptr;
   int max_rows = 0;
-  // ovggt_layer_step scores the cache (diversity, residual norms) on a second, higher-priority stream while the
-  // attention runs: the scores do not depend on the attention.  Host objects only; absent if creation failed.
+  // Second stream of ovggt_layer_step: the attention beside the selection and the gather of the stable layout, the
+  // query-key scores beside the front.  Host objects only; absent if creation failed.
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool overlap = true;            // ovggt_cache_set_overlap
