@@ -4,16 +4,17 @@
 //
 // Not part of the streaming step itself: it is what a model wraps around it (QKV / output projections, MLP), provided
 // so that the 24-layer workloads can run their scaffold on hand-written kernels too.
-//   CTA tile 128 x BN (256 or 128), K in steps of 64: A tile [128 rows, 64 k] K-major (16 KB), B tile [64 k, BN n] as
+//   CTA tile 128 x BN (256, 128 or 64), K in steps of 64: A tile [128 rows, 64 k] K-major (16 KB), B tile [64 k, BN n] as
 //   [64 k, 64 n] boxes, N-major as the tensor lies in memory (8 KB each), read by one N = BN MMA per 16 k whose descriptor
 //   names the distance between the boxes; 192 KB of stages, one CTA per SM;
 //   warp 16 produces (TMA), warp 17 issues the MMAs, accumulators in BN TMEM columns; warps 0-15 read them back, one thread
 //   per output row and quarter of the columns, finish, and store whole lines by way of shared memory.
 // What bounds it at these sizes (1041 or 1374 rows, N and K of 1024 to 4096): one wave of CTAs whose loads all come from
-// L2, and shared memory, which the MMA reads and TMA writes at 128 bytes a clock each at N = 128 (half the tensor rate)
-// and at 94 at N = 256; hence the wide tile and all of shared memory in flight.  The kernel is launched programmatically
+// L2, each at the 64 bytes a clock that an SM takes in (260 ns for the 32 KB of a 128-wide K step, however many CTAs run);
+// hence the widest tile where a product has tiles enough for every SM, the narrowest where it has few, and all of shared
+// memory in flight.  The kernel is launched programmatically
 // behind its predecessor and prefetches its part of B (weights, as a rule) into L2 while that one drains.
-// Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 9.8 / 7.7 / 14.1 / 20.5 us, against
+// Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 9.7 / 6.3 / 14.1 / 17.0 us, against
 // 13.9 / 9.2 / 18.1 / 19.4 with 128 x 128 tiles of three stages and four epilogue warps that stored row by row (the second
 // and the fourth of those with K split over two CTAs, see gemm_tile_width).
 // Requirements: K a multiple of 64, N a multiple of 8 (TMA row pitch of 16 bytes), 16-byte aligned bases.  Every
@@ -29,9 +30,9 @@ constexpr int kGemmBM = 128, kGemmBK = 64;
 constexpr int kGemmEpilogueWarps = 16, kGemmThreads = (kGemmEpilogueWarps + 2) * 32;
 constexpr int kGemmATile = kGemmBM * kGemmBK * 2;          // 16 KB
 constexpr int kGemmBBox = kGemmBK * 64 * 2;                // 8 KB: [64 k, 64 n]
-constexpr int kGemmMaxStages = 6;
+constexpr int kGemmMaxStages = 8;
 __host__ __device__ constexpr int gemm_stage_bytes(int bn) { return kGemmATile + bn / 64 * kGemmBBox; }
-__host__ __device__ constexpr int gemm_stages(int bn) { return bn == 256 ? 4 : 6; }
+__host__ __device__ constexpr int gemm_stages(int bn) { return bn == 256 ? 4 : (bn == 128 ? 6 : 8); }
 
 struct GemmBarriers {
   unsigned long long full[kGemmMaxStages], empty[kGemmMaxStages], acc_full, drain;
@@ -220,15 +221,16 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   }
 }
 
-// Tile width, from a model in nanoseconds fitted to a sweep over seventeen shapes (333 to 1374 rows, N and K 512 to 4096):
-// waves over 148 SMs, one CTA each; 310 per K step of a 256-wide tile, 265 of a 128-wide one (half the work: shared memory
-// bounds it); 4,800 and 3,500 for set-up and epilogue.  K is not split: a product of few tiles and many steps would gain
-// (1041 x 1024 x 4096: 14.8 us in clusters of two against 20.5), but its sums would be grouped otherwise, and 24 layers of
+// Tile width, from a model in nanoseconds fitted to a sweep over twenty shapes (261 to 1374 rows, N 768 to 4096, K 1024 to
+// 4096): waves over 148 SMs, one CTA each; 350, 260 and 217 per K step of a 256-, 128- and 64-wide tile (loads: 48, 32 and
+// 24 KB); 4,200, 3,100 and 2,400 for set-up and epilogue.  1041 x 1024 x 4096 takes 26.8, 20.5 and 17.0 us.  K is not
+// split: that product would gain (14.8 us in clusters of two), but its sums would be grouped otherwise, and 24 layers of
 // bf16 turn any such change into one or two per cent of the result.
 inline int gemm_tile_width(int M, int N, int K) {
   const long tiles_m = (M + kGemmBM - 1) / kGemmBM, steps = K / kGemmBK;
   auto ns = [&](int bn, long step, long fixed) { return (tiles_m * ((N + bn - 1) / bn) + 147) / 148 * (steps * step + fixed); };
-  return ns(256, 310, 4800) <= ns(128, 265, 3500) ? 256 : 128;
+  const long wide = ns(256, 350, 4200), middle = ns(128, 260, 3100), narrow = ns(64, 217, 2400);
+  return wide <= middle && wide <= narrow ? 256 : (middle <= narrow ? 128 : 64);
 }
 
 inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P, cudaStream_t st) {
@@ -237,11 +239,11 @@ inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P,
   if (rc) return rc;
   rc = make_rows_map(&tb, Bm, P.K, P.N, kGemmBK);          // 64 n-columns x 64 k-rows per box
   if (rc) return rc;
-  const int bn = gemm_tile_width(P.M, P.N, P.K), wide = bn == 256 ? 1 : 0;
-  const auto kernel = wide ? k_gemm_bf16_tcgen05<256> : k_gemm_bf16_tcgen05<128>;
-  static std::atomic<uint64_t> smem_set[2];
+  const int bn = gemm_tile_width(P.M, P.N, P.K);
+  const auto kernel = bn == 256 ? k_gemm_bf16_tcgen05<256> : (bn == 128 ? k_gemm_bf16_tcgen05<128> : k_gemm_bf16_tcgen05<64>);
+  static std::atomic<uint64_t> smem_set[3];
   const size_t smem = gemm_smem_bytes(bn);
-  cudaError_t e = allow_smem(kernel, smem, smem_set[wide]);
+  cudaError_t e = allow_smem(kernel, smem, smem_set[bn == 256 ? 0 : (bn == 128 ? 1 : 2)]);
   if (e == cudaSuccess)
     e = launch_dependent(kernel, dim3((P.N + bn - 1) / bn, (P.M + kGemmBM - 1) / kGemmBM), kGemmThreads, 1, smem, st, true, ta, tb, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }

@@ -1,4 +1,4 @@
-"""The scaffold's dense products: tile edges, both tile widths, the fused epilogues."""
+"""The scaffold's dense products: tile edges, every tile width, the fused epilogues."""
 import pytest
 import torch
 
@@ -6,8 +6,10 @@ from paper_2603_05959_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
 
-# rows, columns, K: single partial tiles, ragged edges, few tiles, full waves
-SHAPES = [(1, 8, 64), (127, 72, 64), (129, 264, 192), (333, 512, 2048), (130, 768, 3072), (1041, 1024, 1024), (700, 2304, 768)]
+# rows, columns, K: single partial tiles, ragged edges, few tiles (64 wide), one wave of 128
+# and of 256 wide
+SHAPES = [(1, 8, 64), (127, 72, 64), (129, 264, 192), (333, 512, 2048), (130, 768, 3072), (1041, 1024, 1024), (700, 2304, 768),
+          (1041, 4096, 64)]
 
 
 def _ab(M, N, K):
