@@ -932,36 +932,12 @@ inline int make_rows_map(CUtensorMap* map, const void* base, int rows, int C, in
 constexpr int kJoinMaxTiles = 11;
 inline bool attn_join_inside(long ctas, int per) { return ctas <= (long)kCtasPerSm * 148 && per <= kJoinMaxTiles; }
 
-// Number of KV splits, from a model in nanoseconds fitted to a sweep of 1 to 16 splits over eighteen shapes (69 x 325 x 4
-// heads to 1374 x 34142 x 16): waves of CTAs over 2 x 148 slots; 1.25 us per tile for a CTA that has its SM to itself,
-// 1.85 us where two share one; 4 us per CTA for set-up and epilogue; a merge is 3 us and passes over the partial outputs
-// (write and read) at 6 TB/s, a join inside the attention 1.5 us and 0.4 us per part.  The merge is what short KV ranges
-// cannot pay: 1041 x 1041 x 16 takes 14.5 us unsplit and 20.6 us in two splits, whose CTAs alone would be faster.
-inline int attn_choose_splits(int M, int N, int H, bool tickets) {
-  const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kBN - 1) / kBN;
-  const long slots = (long)kCtasPerSm * 148;
-  int best = 1;
-  long best_ns = -1;
-  for (int s = 1; s <= kMaxSplits && s <= tiles; ++s) {
-    const int per = (tiles + s - 1) / s;
-    const int eff = (tiles + per - 1) / per;
-    if (eff != s) continue;
-    const long ctas = (long)q_tiles * H * s;
-    const long waves = (ctas + slots - 1) / slots;
-    const long merge = tickets && attn_join_inside(ctas, per) ? 1500 + 400l * s : 3000 + (long)s * M * H * kHD * 8 / 6000;
-    const long ns = waves * (per * (ctas <= 148 ? 1250l : 1850l) + 4000) + (s > 1 ? merge : 0);
-    if (best_ns < 0 || ns < best_ns) {
-      best_ns = ns;
-      best = s;
-    }
-  }
-  return best;
-}
-
-// The rule for an attention outside the fused step (the bare kernel, the halves of a step): waves of CTAs, each as long as
-// its tiles and two more, a merge one tile more.  The model above would group the sums of some shapes otherwise, and in a
-// stack of 24 layers whose state is rounded to bf16 after each any other grouping changes the result by one or two per cent.
-inline int attn_choose_splits_alone(int M, int N, int H) {
+// Number of KV splits: waves of CTAs over 2 x 148 slots, each as long as its tiles and two more (set-up, epilogue), a merge
+// one tile more.  How many parts a range is cut into decides the bits of the output: each part rounds P to bf16 under a
+// reference of its own, so another number of parts moves the result by some 3e-3 of its norm (1374 x 9566 x 16 in three
+// parts instead of five), on a single step as on a stack of layers.  Hence one rule for every caller, and a change of it is
+// a change of results.
+inline int attn_choose_splits(int M, int N, int H) {
   const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kBN - 1) / kBN;
   const long slots = (long)kCtasPerSm * 148;
   int best = 1;
@@ -1020,7 +996,7 @@ inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, 
 inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
                                void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
                                int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr,
-                               bool beside_previous = false, unsigned* tickets = nullptr, bool in_step = false, int* launches = nullptr) {
+                               bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr) {
   const int C = H * kHD;
   CUtensorMap tq;
   AttnKvMaps local;
@@ -1034,7 +1010,7 @@ inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int 
   AttnParams P;
   P.M = M; P.N = N; P.H = H;
   P.tiles_total = (N + kBN - 1) / kBN;
-  P.splits = force_splits > 0 ? std::min(force_splits, std::min(kMaxSplits, P.tiles_total)) : (in_step ? attn_choose_splits(M, N, H, tickets != nullptr) : attn_choose_splits_alone(M, N, H));
+  P.splits = force_splits > 0 ? std::min(force_splits, std::min(kMaxSplits, P.tiles_total)) : attn_choose_splits(M, N, H);
   P.tiles_per_split = (P.tiles_total + P.splits - 1) / P.splits;
   P.splits = (P.tiles_total + P.tiles_per_split - 1) / P.tiles_per_split;     // no empty split
   P.out = static_cast<__nv_bfloat16*>(out);

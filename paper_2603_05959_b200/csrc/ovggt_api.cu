@@ -186,10 +186,10 @@ int launch_fill_holes(void* kc, void* vc, const int* msrc, const int* mdst, cons
 int launch_attention(const void* q, const void* k, const void* v, int M, int N, int H, int dtype, void* out,
                      void* scratch, int* status, cudaStream_t st, AttnKvMaps* maps = nullptr,
                      const float* kmax2 = nullptr, float* lse = nullptr, bool beside_previous = false,
-                     unsigned* tickets = nullptr, bool in_step = false) {
+                     unsigned* tickets = nullptr) {
   int launches = 0;
   const int rc = dtype == kBF16 ? attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, 0, kmax2, lse,
-                                                      beside_previous, tickets, in_step, &launches)
+                                                      beside_previous, tickets, &launches)
                                 : attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, tickets,
                                                   &launches);
   g_launches.fetch_add(launches);
@@ -661,14 +661,14 @@ int enqueue_front(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, bool 
 // which order the cached rows lie, so it reads the K/V buffer front to back in either layout.
 // beside_previous: what was enqueued on st just before is the same step's selection, which the attention does not wait for.
 int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st, int N, int kb,
-                      bool beside_previous = false, bool in_step = false) {
+                      bool beside_previous = false) {
   LayerState& S = h->layers[layer];
   int rc;
   {
     ProfScope ps(h, OVGGT_PROF_ATTENTION, st);
     rc = launch_attention(io->q, S.kbuf[kb], S.vbuf[kb], h->M, N, h->cfg.n_heads, h->cfg.dtype, io->out,
                           h->attn_scratch, h->status, st, &S.maps[kb], key_norm_bound(h, S),
-                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous, h->attn_tickets, in_step);
+                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous, h->attn_tickets);
   }
   return rc;
 }
@@ -1034,7 +1034,7 @@ extern "C" int ovggt_layer_step(ovggt_cache* h, int32_t layer, const ovggt_frame
   close_attend(h, S, io);
   rc = compress_impl(h, layer, io, st);
   // (a compress that is refused, as for a frame older than the last anchor decision, leaves the frame attended)
-  const int ra = enqueue_attention(h, layer, io, stable ? h->side : st, N, kb, !stable && rc == OVGGT_OK, true);
+  const int ra = enqueue_attention(h, layer, io, stable ? h->side : st, N, kb, !stable && rc == OVGGT_OK);
   if (rc == OVGGT_OK) rc = ra;
   h->last_stream = st;
   if (stable) {   // whatever happened, the caller's stream is ordered after the side work
