@@ -301,27 +301,27 @@ __device__ __noinline__ bool refine_bin(const uint32_t* keys, const uint16_t* bf
   return first == last;
 }
 
-// Where all rows of the threshold bin have the key sh->T: the position of the last one that stays, of those in this CTA (N:
-// all of its own, -1: none).  The lower ranks' ties come first, then the lower positions.
+// Where all rows of the threshold bin have the key sh->T: up to which position those of this CTA stay (N: all of its own, -1:
+// none).  The lower ranks' ties come first, then the lower positions; the CTA that holds the last one to stay leaves its
+// position in sh->pub_pos, the others -1, so that after the next barrier all can judge rows of any CTA.
 __device__ __noinline__ int last_tie(const uint32_t* keys, int begin, int cnt, int N, int rank, SelectShared* sh) {
   const int tid = threadIdx.x, nthr = blockDim.x;
   int mine = sh->krem;
   for (int r = 0; r < rank; ++r) mine -= sh->cnt_bin[r];
-  int pos = mine >= sh->cnt_bin[rank] ? N : -1;
-  if (mine > 0 && pos < 0) {
+  const bool holds = mine > 0 && mine <= sh->cnt_bin[rank];
+  if (tid == 0) sh->pub_pos = -1;
+  if (holds) {
     const int chunk = (cnt + nthr - 1) / nthr, lo = min(cnt, tid * chunk), hi = min(cnt, lo + chunk);
     const uint32_t T = sh->T;
     int eq = 0, all;
     for (int i = lo; i < hi; ++i) eq += keys[i] == T;
     int before = block_excl_scan_int(eq, sh->scan, &all);
-    if (before < mine && before + eq >= mine)          // one thread
+    if (before < mine && before + eq >= mine)            // one thread
       for (int i = lo; i < hi; ++i)
-        if (keys[i] == T && ++before == mine) sh->posT = begin + i;
-    __syncthreads();
-    pos = sh->posT;
+        if (keys[i] == T && ++before == mine) sh->pub_pos = begin + i;
   }
-  __syncthreads();                                     // (the counts have been read)
-  return pos;
+  __syncthreads();
+  return holds ? sh->pub_pos : (mine > 0 ? N : -1);
 }
 
 // Single-CTA pick used for the small top-A choice over the confidence map: marks the A largest of cnt keys
@@ -899,13 +899,18 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
         sh->pub_down = dw + sh->wtot[kSelectWarps - 1][2];
       }
       G::sync();
-      if (tid < ncta) {
-        const SelectShared* o = G::of(sh, tid);
-        sh->cnt_keep[tid] = o->pub_keep;
-        sh->cnt_up[tid] = o->pub_up;
-        sh->cnt_down[tid] = o->pub_down;
+      if (warp == 0) {                                 // lanes are the CTAs of the cluster
+        const SelectShared* o = G::of(sh, min(lane, ncta - 1));
+        if (lane < ncta) {
+          sh->cnt_keep[lane] = o->pub_keep;
+          sh->cnt_up[lane] = o->pub_up;
+          sh->cnt_down[lane] = o->pub_down;
+        }
+        const int pos = __reduce_max_sync(0xFFFFFFFFu, o->pub_pos);
+        if (lane == 0) sh->posT = pos;
       }
       __syncthreads();
+      posT = sh->posT;                                 // (of the whole cluster, also where ties were settled by each CTA)
       keep_before = keep_all = 0;
       for (int r = 0; r < ncta; ++r) {
         if (r < rank) keep_before += sh->cnt_keep[r];
