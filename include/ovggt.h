@@ -148,7 +148,8 @@ size_t ovggt_workspace_bytes(const ovggt_config* cfg);
  * workspace on the legacy default stream and synchronises.
  * OVGGT_ERR_BUDGET_TOO_SMALL if a layer's budget cannot hold the protected set (Eq. 9).
  * OVGGT_ERR_UNSUPPORTED if a layer's B + M candidates do not fit the selection kernel, which keeps them in the
- * shared memory of one 8-CTA cluster (about 18 bytes per candidate and CTA: B + M up to roughly 90,000). */
+ * shared memory of one 8-CTA cluster (22 bytes per candidate, and 9 per token of a frame in each CTA: B + M up to about
+ * 83,000 with small frames, 78,600 with 1374 tokens a frame, 56,300 with 8197). */
 int ovggt_cache_create(const ovggt_config* cfg, ovggt_cache** out);
 int ovggt_cache_destroy(ovggt_cache* cache);
 

@@ -60,6 +60,12 @@ int select_cluster_ctas(int N) { return std::max(1, std::min(kSelectMaxCtas, (N 
 // The fused kernel: one CTA, which needs no cluster barriers, up to the size where its passes over the positions and the
 // rows of the key sums' corrections outweigh them; then a full cluster.
 int compress_ctas(int N, int M) { return N <= 1024 && M <= 128 ? 1 : kSelectMaxCtas; }
+size_t compress_smem(int N, int Np, int M, bool room) {
+  const int ncta = compress_ctas(N, M);
+  return compress_smem_bytes((N + ncta - 1) / ncta, ncta, Np, M, room);
+}
+// Whether the key sums' corrections of a layer of that budget have their place beside B + M candidates.
+bool compress_has_room(int B, int Np, int M) { return compress_smem(B + M, Np, M, true) <= kSmemLimit; }
 
 template <typename... KArgs, typename... Args>
 cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, int ncta, size_t smem, cudaStream_t st, Args... args) {
@@ -234,6 +240,7 @@ struct LayerState {
   int kcur = 0;                   // which of the two describes the cached keys
   bool ksum_valid = false;        // it does (else: recompute)
   int since_refresh = 0;
+  bool room = true;               // the selection has a place for the corrections of the key sums (else: afresh each step)
   float* kmax2 = nullptr;         // [n_heads] running upper bound of the squared per-head key norms (bf16 caches)
   AttnKvMaps maps[2];             // tensor maps of the K/V buffers, re-encoded only when the row count changes
   int64_t norms_frame = -1;       // frame whose residual norms the front launch already took
@@ -350,8 +357,7 @@ bool config_ok(const ovggt_config* c, int* err) {
     }
     if ((int64_t)c->budget[l] + M > (1 << 30)) return false;
     // the fused selection kernel keeps all B + M candidates of a layer in the shared memory of one cluster
-    const int N = c->budget[l] + (int)M, ncta = compress_ctas(N, (int)M);
-    if (compress_smem_bytes((N + ncta - 1) / ncta, c->grid_h * c->grid_w, (int)M) > kSmemLimit) {
+    if (compress_smem(c->budget[l] + (int)M, c->grid_h * c->grid_w, (int)M, false) > kSmemLimit) {
       *err = OVGGT_ERR_UNSUPPORTED;
       return false;
     }
@@ -417,6 +423,7 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
       S.move_dst = reinterpret_cast<int*>(base + off[i++]);
       for (int b = 0; b < 2; ++b) S.ksum[b] = reinterpret_cast<float*>(base + off[i++]);
       S.budget = c->budget[l];
+      S.room = compress_has_room(S.budget, Np, M);
       S.kv_bytes = 2 * (size_t)nkv * R * C * eb;
     }
   }
@@ -716,9 +723,7 @@ int validate_compress(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, c
   }
   const LayerState& S = h->layers[layer];
   if (!S.pending || io->frame_id != S.pending_frame) return OVGGT_ERR_FRAME_ORDER;
-  const int N = S.n + h->M, ncta = compress_ctas(N, h->M);
-  if (compress_smem_bytes((N + ncta - 1) / ncta, h->Np, h->M) > kSmemLimit)
-    return OVGGT_ERR_UNSUPPORTED;   // (create already refuses such budgets)
+  if (compress_smem(S.n + h->M, h->Np, h->M, S.room) > kSmemLimit) return OVGGT_ERR_UNSUPPORTED;   // (create already refuses such budgets)
   // The anchor state belongs to the whole handle and moves forward only: a layer that comes with a frame older
   // than the last decision would take that frame's decision a second time.
   if (io->frame_id < h->decided_frame) return OVGGT_ERR_FRAME_ORDER;
@@ -778,7 +783,7 @@ bool norms_inside(const ovggt_cache* h, const LayerState& S, const ovggt_frame_i
 // go as move lists, which name exactly those unless the cache of the hole-filling layout fills up in this very step
 // (rows of the frame then already lie below slot B); the sums are taken afresh after that one.
 bool continues_sums(const ovggt_cache* h, const LayerState& S) {
-  return ranks_by_diversity(h->cfg.score_mode) &&
+  return S.room && ranks_by_diversity(h->cfg.score_mode) &&
          !(h->cfg.compaction == OVGGT_COMPACT_FILL_HOLES && S.n + h->M > S.budget && S.n < S.budget);
 }
 
@@ -814,6 +819,7 @@ CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io
   P.resid = norms_inside(h, S, io) ? static_cast<const uint4*>(io->resid) : nullptr;
   P.k_cache = reinterpret_cast<const uint4*>(S.kbuf[S.kv]);
   P.nvec = h->C * h->elem / 16;
+  P.room = S.room ? 1 : 0;
   P.ksum = S.n > 0 ? S.ksum[S.kcur] : nullptr;
   P.ksum_next = continues_sums(h, S) ? S.ksum[S.kcur ^ 1] : nullptr;
   return P;
@@ -862,7 +868,7 @@ int compress_impl(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaS
   }
   const CompressParams P = select_params(h, S, io);
   const int ncta = compress_ctas(N, M);
-  const size_t smem = compress_smem_bytes((N + ncta - 1) / ncta, h->Np, M);
+  const size_t smem = compress_smem(N, h->Np, M, S.room);
   const auto kernel = c.dtype == kBF16 ? (ncta == 1 ? k_compress_select<kBF16, true> : k_compress_select<kBF16, false>)
                                        : (ncta == 1 ? k_compress_select<kF32, true> : k_compress_select<kF32, false>);
   static std::atomic<uint64_t> smem_set[4];
@@ -940,7 +946,11 @@ int compress_all_layers(ovggt_cache* h, const ovggt_frame_io* ios, cudaStream_t 
           c.dtype == kBF16 ? (ncta == 1 ? k_compress_select_batched<kBF16, true> : k_compress_select_batched<kBF16, false>)
                            : (ncta == 1 ? k_compress_select_batched<kF32, true> : k_compress_select_batched<kF32, false>);
       CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
-      const size_t smem = compress_smem_bytes((n_max + ncta - 1) / ncta, h->Np, M);
+      size_t smem = 0;
+      for (int i = 0; i < cnt; ++i) {
+        const LayerState& S = h->layers[l0 + i];
+        smem = std::max(smem, compress_smem_bytes((S.n + M + ncta - 1) / ncta, ncta, h->Np, M, S.room));
+      }
       CK(launch_cluster(kernel, dim3(ncta, cnt), ncta, smem, st, cb));
       LAUNCHED();
     }

@@ -371,14 +371,17 @@ __host__ __device__ inline size_t select_header_bytes() { return (sizeof(SelectS
 __host__ __device__ inline size_t select_smem_bytes(int span) { return select_header_bytes() + (((size_t)span * 4 + 15) & ~(size_t)15); }
 
 // The fused per-step kernel keeps, per position, the value or key (4 bytes), bin and flag (2), id (8), stored score (4)
-// and slot (4) on chip, the frame's m raw residual norms, the np confidence keys and marks, and for the key sums'
-// corrections a list of rows (m that leave, m that come) and a block of sums.
+// and slot (4) on chip.  Behind them lie the frame's m raw residual norms and the np confidence keys and marks, which the
+// flags and values are made of, and later, in the same place, a block of sums and a list of rows for the key sums' corrections: a
+// CTA lists at most m rows that leave and its share of the m that come.  Largest caches of small frames do without that
+// block (room 0: their sums are taken afresh each step) rather than be refused.
 constexpr int kDeltaCols = 1024;
 static_assert(3 * kSelectSubBins <= kDeltaCols, "the finer bins lie in the block of sums");
-__host__ __device__ inline size_t compress_smem_bytes(int span, int np, int m) {
+__host__ __device__ inline size_t compress_smem_bytes(int span, int ncta, int np, int m, bool room) {
   const size_t s4 = ((size_t)span + 3) & ~(size_t)3, m4 = ((size_t)m + 3) & ~(size_t)3, np4 = ((size_t)np + 3) & ~(size_t)3;
-  const size_t body = s4 * (8 + 3 * 4) + ((s4 + 7) & ~(size_t)7) * 2 + m4 * 4 + np4 * 4 + ((np4 + 15) & ~(size_t)15);
-  return select_header_bytes() + body + (size_t)kDeltaCols * 4 + 2 * m4 * 4;
+  const size_t early = m4 * 4 + np4 * 4 + ((np4 + 15) & ~(size_t)15);
+  const size_t late = room ? (size_t)kDeltaCols * 4 + ((size_t)m + (size_t)((m + ncta - 1) / ncta)) * 4 : 0;
+  return select_header_bytes() + s4 * (8 + 3 * 4) + ((s4 + 7) & ~(size_t)7) * 2 + (early > late ? early : late);
 }
 
 // Per-warp totals of the rows that stay, and of two marked kinds of rows, for the warp's range of positions; then the
@@ -500,6 +503,7 @@ struct CompressParams {
   const uint4* resid;               // [M, C] or nullptr: compute the residual norms here instead of reading s_raw (small M)
   // Column sums of the keys that stay: ksum_next = ksum (or 0) + admitted keys - evicted keys; ksum_next nullptr: not asked for.
   const uint4* k_cache; int nvec;
+  int room;                         // the block of sums and the list have their place in shared memory (needed for ksum_next)
   const float* ksum; float* ksum_next;   // [C]
 };
 
@@ -607,12 +611,12 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   float* val = reinterpret_cast<float*>(keys);
   float* sst = reinterpret_cast<float*>(keys + span4);            // their stored scores
   int* ssl = reinterpret_cast<int*>(sst + span4);                 // their physical slots
-  float* sraw = reinterpret_cast<float*>(ssl + span4);            // [M] the frame's residual norms
+  uint16_t* bf = reinterpret_cast<uint16_t*>(ssl + span4);        // flag << 14 | bin of the owned positions
+  float* sraw = reinterpret_cast<float*>(bf + ((span4 + 7) & ~7));        // [M] the frame's residual norms
   uint32_t* ckeys = reinterpret_cast<uint32_t*>(sraw + ((M + 3) & ~3));   // [Np] confidence keys
-  uint16_t* bf = reinterpret_cast<uint16_t*>(ckeys + ((Np + 3) & ~3));    // flag << 14 | bin of the owned positions
-  uint8_t* cmark = reinterpret_cast<uint8_t*>(bf + ((span4 + 7) & ~7));   // [Np] the most confident patches
-  float* part = reinterpret_cast<float*>(cmark + ((Np + 15) & ~15));      // [kDeltaCols] this CTA's corrections of the key sums
-  int* list = reinterpret_cast<int*>(part + kDeltaCols);                  // [2 M] slots of the rows they are made of
+  uint8_t* cmark = reinterpret_cast<uint8_t*>(ckeys + ((Np + 3) & ~3));   // [Np] the most confident patches
+  float* part = sraw;   // over the last three, which are dead by then: [kDeltaCols] this CTA's corrections of the key sums
+  int* list = reinterpret_cast<int*>(part + kDeltaCols);          // [M + its share of M] slots of the rows they are made of
   const bool hybrid = P.mode == OVGGT_SCORE_HYBRID, choose = N > P.B;
   pdl_wait();
   pdl_trigger();   // an attention queued behind this kernel reads nothing of it: it starts as soon as this one runs
@@ -811,7 +815,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
     // a crowded bin in finer ones, equal steps of the key between its edges (monotone, so a key may be a step off)
     SubBins sub = {0, 1.0f};
     bool ties = false;
-    if (!SINGLE && crowded && bstar < kSelectBins - 1) {   // (one CTA's radix passes are cheap: no cluster barriers)
+    if (!SINGLE && P.room && crowded && bstar < kSelectBins - 1) {   // (one CTA's radix passes are cheap: no cluster barriers)
       const float step = bin_scale > 0.0f ? 1.0f / bin_scale : 0.0f, e0 = (float)bstar * step, e1 = (float)(bstar + 1) * step;
       sub.lo = linear ? rank_key(bin_lo + e0) : bin_key0 + (uint32_t)e0;
       const uint32_t hi = linear ? rank_key(bin_lo + e1) : bin_key0 + (uint32_t)e1;
