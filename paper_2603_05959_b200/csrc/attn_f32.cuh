@@ -125,6 +125,8 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // (K and V, which the front wrote, are read behind the barrier below)
+  if (threadIdx.x == kAttnThreads - 32 && !P.wait_first) drop_stale_lines(reinterpret_cast<const int*>(P.q));
   {  // the query tile's planes: 128 rows x 8 groups of 8 columns, rows past M zero
     float4 x[4], y[4];
 #pragma unroll
@@ -133,8 +135,8 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
       x[i] = y[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (m < P.M) {
         const float4* p = reinterpret_cast<const float4*>(P.q + (size_t)m * C + (size_t)h * kHD + (idx & 7) * 8);
-        x[i] = __ldg(p);
-        y[i] = __ldg(p + 1);
+        x[i] = __ldcg(p);
+        y[i] = __ldcg(p + 1);
       }
     }
 #pragma unroll

@@ -650,7 +650,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             qn2 = fmaf(hi, hi, qn2);
           }
         }
-        bound = sqrtf(qn2 * __ldg(P.kmax2 + h)) * c;
+        bound = sqrtf(qn2 * __ldcg(P.kmax2 + h)) * c;
       }
     }
     for (int idx = 0; idx < 2 * n_tiles && ok; ++idx) {       // idx = 2 * tile + half

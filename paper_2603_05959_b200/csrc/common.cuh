@@ -93,6 +93,15 @@ __device__ __forceinline__ bool index_ok(long long, long long, int*) { return tr
 // pdl_trigger lets the kernel after this one start as soon as every CTA of this one has come here or ended.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A kernel that starts at its predecessor's trigger and does not wait for its end may read what kernels BEFORE that one wrote:
+// those are complete (the predecessor waited for them before it triggered) and their writes are in L2, but this SM's first-level
+// cache may still hold lines from before.  So such data is read by bulk copies or __ldcg, which go to L2, or by plain loads
+// behind a CTA barrier ahead of which one thread has called this: an acquire, which drops the first-level lines.  `word` is
+// any word of global memory.  (Loads of the read-only path, __ldg, are not covered.)
+__device__ __forceinline__ void drop_stale_lines(const int* word) {
+  int x;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(x) : "l"(word) : "memory");
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, int threads, int cluster, size_t smem, cudaStream_t st,
