@@ -19,6 +19,7 @@
 //   warps 5-7  read K and V rows from global memory, split them and write the bf16 planes, 128-byte swizzled, to
 //              shared memory (done once per CTA and tile: cheaper than a pass over the cache that writes planes, and
 //              it needs no scratch memory)
+// A result that is not finite is taken again in plain fp32 arithmetic, which says whether it should be (see plain_row).
 // Every wait is bounded; on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the common teardown.
 #pragma once
 
@@ -39,6 +40,7 @@ struct F32Barriers {
   unsigned long long k_full, k_empty, v_full, v_empty, s_full[2], p_full, o_full, drain;
   uint32_t tmem_base;
   int abort_flag;
+  int odd;                // a result of this CTA is not finite
 };
 constexpr int kF32Planes = 3 * kF32QPlane + 6 * kF32KvPlane;
 static_assert(kJoinStages * kPartBytes <= kF32Planes, "the parts do not fit the operand planes");
@@ -84,6 +86,25 @@ __device__ __forceinline__ void store_planes(unsigned char* base, int plane_byte
 __device__ constexpr int kSplitA[6] = {2, 0, 1, 1, 0, 0};
 __device__ constexpr int kSplitB[6] = {0, 2, 1, 0, 1, 0};
 
+// Takes the rows of this CTA's query tile whose results are not finite again, a warp each; called by the softmax warps, whose
+// register budget covers any function's.  A function, not inline: with its loops in the kernel the softmax loop came out 5
+// to 11 % slower (1374 x 5470 x 16: 209 us without any of this, 211 so, 220 to 232 inline); one per cent is what looking for such
+// rows costs.
+__device__ __noinline__ void redo_rows(const F32Params& P) {
+  const int lane = threadIdx.x & 31, h = blockIdx.y;
+  const PlainRows plain = {P.q, P.k, P.v, P.N, P.H};
+#pragma unroll 1
+  for (int r = threadIdx.x >> 5; r < kBM && (int)blockIdx.x * kBM + r < P.M; r += 4) {
+    const int m = blockIdx.x * kBM + r;
+    float2* o = reinterpret_cast<float2*>(P.out + ((size_t)m * P.H + h) * kHD) + lane;
+    float2 x = *o;
+    if (__any_sync(0xFFFFFFFFu, !(x.x * 0.0f + x.y * 0.0f == 0.0f))) {
+      plain_row<32>(plain, m, h, P.lse, &x.x);
+      *o = x;
+    }
+  }
+}
+
 // JOIN: the parts of a split KV range are joined here (see join_parts).
 template <bool JOIN>
 __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __grid_constant__ F32Params P) {
@@ -116,7 +137,7 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
     mbar_init(&B->drain, 1);
     if constexpr (JOIN)
       for (int s = 0; s < kJoinStages; ++s) mbar_init(&J->full[s], 1);
-    B->abort_flag = 0;
+    B->abort_flag = B->odd = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 4) {
@@ -328,7 +349,11 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
       float* part = JOIN ? P.o_part + part_row * kHD : P.o_part + part_row * C + (size_t)h * kHD;
       float4* dst = reinterpret_cast<float4*>(whole ? P.out + (size_t)m * C + (size_t)h * kHD : part);
 #pragma unroll
-      for (int i = 0; i < kHD; i += 4) dst[i / 4] = make_float4(acc[i] * f, acc[i + 1] * f, acc[i + 2] * f, acc[i + 3] * f);
+      for (int i = 0; i < kHD; i += 4) {
+        const float4 x = make_float4(acc[i] * f, acc[i + 1] * f, acc[i + 2] * f, acc[i + 3] * f);
+        dst[i / 4] = x;
+        if (!JOIN && whole && !all_finite(x)) B->odd = 1;
+      }
       if (!whole) P.ml_part[JOIN ? part_row : part_row * P.H + h] = make_float2(mref, l);
       if (whole && P.lse != nullptr) P.lse[(size_t)m * P.H + h] = mref + log2f(l);
     }
@@ -338,8 +363,10 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
         const size_t row0 = join_row0(P.M, qt, h, P.splits);
         join_parts(J, B, smem, reinterpret_cast<float*>(J + 1), P.o_part + row0 * kHD, P.ml_part + row0, min(kBM, P.M - m0),
                    P.splits, P.out + (size_t)m0 * C + h * kHD, C, P.lse != nullptr ? P.lse + (size_t)m0 * P.H + h : nullptr, P.H,
-                   P.status);
+                   P.status, &B->odd);
       }
+    softmax_warps_sync();
+    if (*(volatile int*)&B->odd) redo_rows(P);
   }
 
   // ------------------------------------------------ teardown
@@ -405,7 +432,7 @@ inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, i
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   const bool merge = P.splits > 1 && !join;
   *launches = merge ? 2 : 1;
-  return merge ? attn_merge_launch<float>(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st) : OVGGT_OK;
+  return merge ? attn_merge_launch<float>(P.o_part, P.ml_part, M, H, P.splits, P.out, lse, st, {P.q, P.k, P.v, N, H}) : OVGGT_OK;
 }
 
 }  // namespace ovggt

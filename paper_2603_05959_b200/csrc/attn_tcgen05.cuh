@@ -295,6 +295,63 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return d;
 }
 
+// ---------------------------------------------------------------- fp32 rows by plain arithmetic
+
+__device__ __forceinline__ bool all_finite(const float4& x) { return fmaf(x.x, 0.0f, x.y * 0.0f) + fmaf(x.z, 0.0f, x.w * 0.0f) == 0.0f; }
+
+// What the fp32 attention reads, for rows that are taken again.
+struct PlainRows {
+  const float *q, *k, *v;
+  int N, H;
+};
+// Query row m of head h over all N KV rows in plain fp32 arithmetic, for the results that are not finite on split operands: an
+// infinity has no remainder to split (inf - inf), and a float above the largest bf16 rounds to one, so those may be NaN where
+// plain fp32 has a number.  LANES lanes (16 or the whole warp) take a row, four KV rows at a time; x: the lane's 64 / LANES
+// columns.
+template <int LANES>
+__device__ __forceinline__ void plain_row(const PlainRows& A, int m, int h, float* lse, float* x) {
+  constexpr int W = kHD / LANES;
+  const int c0 = (threadIdx.x & (LANES - 1)) * W;
+  const unsigned mask = LANES == 32 ? 0xFFFFFFFFu : 0xFFFFu << (threadIdx.x & 16);
+  const size_t C = (size_t)A.H * kHD, at = (size_t)h * kHD + c0;
+  const float c = 1.4426950408889634f * 0.125f;        // log2(e) / sqrt(64)
+  float q[W], mref = -INFINITY, l = 0.0f;
+#pragma unroll
+  for (int e = 0; e < W; ++e) {
+    q[e] = A.q[m * C + at + e] * c;
+    x[e] = 0.0f;
+  }
+#pragma unroll 1
+  for (int r0 = 0; r0 < A.N; r0 += 4) {
+    float s[4], v[4][W];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const size_t row = (size_t)min(r0 + i, A.N - 1) * C + at;
+      s[i] = 0.0f;
+#pragma unroll
+      for (int e = 0; e < W; ++e) {
+        s[i] = fmaf(q[e], A.k[row + e], s[i]);
+        v[i][e] = A.v[row + e];
+      }
+#pragma unroll
+      for (int o = LANES / 2; o > 0; o >>= 1) s[i] += __shfl_xor_sync(mask, s[i], o);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (r0 + i < A.N) {
+        const float mnew = fmaxf(mref, s[i]);          // (a score of -inf is a weight of 0, also before any other)
+        const float corr = mref == -INFINITY ? 0.0f : exp2f(mref - mnew), p = s[i] == -INFINITY ? 0.0f : exp2f(s[i] - mnew);
+        l = fmaf(l, corr, p);
+#pragma unroll
+        for (int e = 0; e < W; ++e) x[e] = fmaf(p, v[i][e], x[e] * corr);
+        mref = mnew;
+      }
+  }
+#pragma unroll
+  for (int e = 0; e < W; ++e) x[e] /= l;
+  if (lse != nullptr && c0 == 0) lse[(size_t)m * A.H + h] = mref + log2f(l);
+}
+
 // ---------------------------------------------------------------- joining the parts of a split KV range
 
 // A KV range in several parts leaves one un-normalised O, one reference maximum and one row sum per part, which
@@ -335,10 +392,11 @@ __device__ __forceinline__ bool join_arrive(PartJoin* J, unsigned* ticket, int s
 }
 
 // stage: kJoinStages x 32 KB that nothing else uses any more; table: kJoinTable floats; o, ml: the tile's parts; out, lse:
-// the tile's first row.
+// the tile's first row; odd (shared memory; fp32 only): set where a result is not finite.
 template <typename Out, typename Barriers>
 __device__ __forceinline__ void join_parts(PartJoin* J, Barriers* B, unsigned char* stage, float* table, const float* o,
-                                           const float2* ml, int rows, int splits, Out* out, int C, float* lse, int H, int* status) {
+                                           const float2* ml, int rows, int splits, Out* out, int C, float* lse, int H, int* status,
+                                           int* odd) {
   const int tid = threadIdx.x, c4 = tid & 15, r0 = tid >> 4;
   const uint32_t bytes = (uint32_t)rows * kHD * 4;
   auto fetch = [&](int s) {
@@ -414,8 +472,9 @@ __device__ __forceinline__ void join_parts(PartJoin* J, Barriers* B, unsigned ch
     if (r < rows) {
       const float inv = table[kMaxSplits * kBM + r];
       if constexpr (sizeof(Out) == 4) {
-        *reinterpret_cast<float4*>(out + (size_t)r * C + c4 * 4) =
-            make_float4(acc[i].x * inv, acc[i].y * inv, acc[i].z * inv, acc[i].w * inv);
+        const float4 x = make_float4(acc[i].x * inv, acc[i].y * inv, acc[i].z * inv, acc[i].w * inv);
+        *reinterpret_cast<float4*>(out + (size_t)r * C + c4 * 4) = x;
+        if (!all_finite(x)) *odd = 1;
       } else {
         uint2 w;
         w.x = pack_bf16(acc[i].x * inv, acc[i].y * inv);
@@ -805,7 +864,8 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const int m0 = qt * kBM;
         const size_t row0 = join_row0(P.M, qt, h, P.splits);
         join_parts(J, B, sK, reinterpret_cast<float*>(sQ), P.o_part + row0 * kHD, P.ml_part + row0, min(kBM, P.M - m0), P.splits,
-                   P.out + (size_t)m0 * C + h * kHD, C, P.lse != nullptr ? P.lse + (size_t)m0 * P.H + h : nullptr, P.H, P.status);
+                   P.out + (size_t)m0 * C + h * kHD, C, P.lse != nullptr ? P.lse + (size_t)m0 * P.H + h : nullptr, P.H, P.status,
+                   nullptr);
       }
   }
 
@@ -823,7 +883,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 template <typename Out, int MAXS>
 __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_part, const float2* __restrict__ ml_part,
                                                     int M, int H, int splits, Out* __restrict__ out,
-                                                    float* __restrict__ lse) {
+                                                    float* __restrict__ lse, PlainRows plain) {
   pdl_trigger();
   const int C = H * kHD, c4 = (int)(blockIdx.y * blockDim.x + threadIdx.x), m = (int)blockIdx.x, h = (c4 * 4) / kHD;
   // launched with programmatic stream serialisation: its CTAs may become resident while the last attention CTAs
@@ -857,7 +917,9 @@ __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_
   const float inv = 1.0f / den;
   if (lse != nullptr && (c4 * 4) % kHD == 0) lse[(size_t)m * H + h] = mstar + log2f(den);
   if constexpr (sizeof(Out) == 4) {
-    *reinterpret_cast<float4*>(out + (size_t)m * C + c4 * 4) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+    float4 x = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+    if (__any_sync(0xFFFFu << (threadIdx.x & 16), !all_finite(x))) plain_row<16>(plain, m, h, lse, &x.x);   // (16 lanes: a row of a head)
+    *reinterpret_cast<float4*>(out + (size_t)m * C + c4 * 4) = x;
   } else {
     uint2 w;
     w.x = pack_bf16(acc.x * inv, acc.y * inv);
@@ -984,11 +1046,11 @@ inline int attn_kv_maps(AttnKvMaps* m, const void* k, const void* v, int N, int 
 
 template <typename Out>
 inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, int H, int splits, Out* out, float* lse,
-                             cudaStream_t st) {
+                             cudaStream_t st, const PlainRows& plain = {}) {
   const int c4 = H * kHD / 4, threads = std::min(256, (c4 + 31) / 32 * 32);
   const auto kernel = splits <= 4 ? k_attn_merge<Out, 4> : (splits <= 8 ? k_attn_merge<Out, 8> : k_attn_merge<Out, kMaxSplits>);
   cudaError_t e = launch_dependent(kernel, dim3(M, (c4 + threads - 1) / threads), threads, 1, 0, st, true, o_part,
-                                   ml_part, M, H, splits, out, lse);
+                                   ml_part, M, H, splits, out, lse, plain);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   return OVGGT_OK;
 }
