@@ -402,8 +402,8 @@ inline int attn_f32_choose_splits(int M, int N, int H) {
 }
 
 // scratch: attn_tcgen05_scratch_bytes, or nullptr (the KV range is then not split).
-inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out, void* scratch,
-                           int* status, cudaStream_t st, float* lse, bool beside_previous, unsigned* tickets, int* launches) {
+static inline int attn_f32_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out, void* scratch,
+                                  int* status, cudaStream_t st, float* lse, bool beside_previous, unsigned* tickets, int* launches) {
   const int C = H * kHD;
   F32Params P;
   P.q = static_cast<const float*>(q);

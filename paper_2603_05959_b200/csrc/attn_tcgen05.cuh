@@ -948,14 +948,14 @@ __global__ void __launch_bounds__(32) k_bounded_wait_selftest(int* status, unsig
 
 // ---------------------------------------------------------------- host side
 
-inline int g_attn_last_error = 0;
+static int g_attn_last_error = 0;
 inline int attn_tcgen05_last_error() { return g_attn_last_error; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-inline EncodeTiledFn encode_tiled_fn() {
+static inline EncodeTiledFn encode_tiled_fn() {
   static EncodeTiledFn fn = nullptr;
   if (!fn) {
     void* p = nullptr;
@@ -1055,10 +1055,10 @@ inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, 
   return OVGGT_OK;
 }
 
-inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
-                               void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
-                               int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr,
-                               bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr) {
+static inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
+                                      void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
+                                      int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr,
+                                      bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr) {
   const int C = H * kHD;
   CUtensorMap tq;
   AttnKvMaps local;

@@ -133,7 +133,8 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, int thr
 // Opt a kernel in to `bytes` of dynamic shared memory, and its SMs to the largest shared-memory carve-out: an SM whose
 // carve-out was set up for a kernel with little shared memory has to drain before a CTA of the attention (115 KB) can join
 // it, so a selection running beside the attention would keep its SMs to itself.  Once per kernel and device (the calls
-// are safe to repeat, so threads may race here).
+// are safe to repeat, so threads may race here).  `done` belongs to this copy of the library: a function that keeps one is static
+// or in an anonymous namespace, since the statics of an inline function would be shared by all copies a process has loaded.
 template <typename K>
 inline cudaError_t allow_smem(K kernel, size_t bytes, std::atomic<uint64_t>& done, bool carveout = true) {
   int dev = 0;

@@ -233,7 +233,7 @@ inline int gemm_tile_width(int M, int N, int K) {
   return wide <= middle && wide <= narrow ? 256 : (middle <= narrow ? 128 : 64);
 }
 
-inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P, cudaStream_t st) {
+static inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmArgs& P, cudaStream_t st) {
   CUtensorMap ta, tb;
   int rc = make_rows_map(&ta, A, P.M, P.K, kGemmBM);       // 64 k-columns x 128 rows per box
   if (rc) return rc;
