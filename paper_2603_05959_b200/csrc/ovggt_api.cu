@@ -31,8 +31,10 @@ namespace {
 std::atomic<uint64_t> g_launches{0};
 std::atomic<int> g_last_cuda_error{0};
 
+// (The runtime keeps a failed call's error until it is asked for it: left there, the next launch would be taken to have failed.)
 inline int cuda_fail(cudaError_t e) {
   g_last_cuda_error.store((int)e);
+  (void)cudaGetLastError();
   return OVGGT_ERR_CUDA;
 }
 #define CK(expr)                                  \
@@ -199,7 +201,7 @@ int launch_attention(const void* q, const void* k, const void* v, int M, int N, 
                                 : attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, tickets,
                                                   &launches);
   g_launches.fetch_add(launches);
-  if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
+  if (rc == OVGGT_ERR_CUDA) cuda_fail((cudaError_t)attn_tcgen05_last_error());
   return rc;
 }
 
@@ -1488,7 +1490,7 @@ extern "C" int ovggt_k_linear_bf16(const void* A, const void* Bm, int32_t M, int
   P.status = device_status;
   int rc = gemm_tcgen05_launch(A, Bm, P, static_cast<cudaStream_t>(stream));
   if (rc == OVGGT_OK) g_launches.fetch_add(1);
-  if (rc == OVGGT_ERR_CUDA) g_last_cuda_error.store(attn_tcgen05_last_error());
+  if (rc == OVGGT_ERR_CUDA) cuda_fail((cudaError_t)attn_tcgen05_last_error());
   return rc;
 }
 
