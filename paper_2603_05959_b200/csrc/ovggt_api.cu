@@ -130,10 +130,10 @@ int launch_front(const FrontArgs& A, int C, int dtype, cudaStream_t st) {
   const long items = (long)A.M + (A.ksum ? front_score_items(A.n) : 0) + (A.resid ? front_score_items(A.M) : 0);
   if (items == 0) return OVGGT_OK;
   const int grid = (int)std::min<long>((items + kFrontThreads / 32 - 1) / (kFrontThreads / 32), 148 * 2);
-  const size_t smem = (size_t)C * 4;
+  const size_t smem = A.ksum ? (size_t)C * 4 : 0;           // (the centroid; rows that are not scored may be of any width)
   const auto kernel = dtype == kBF16 ? k_front<kBF16> : k_front<kF32>;
   static std::atomic<uint64_t> smem_set[2];
-  CK(allow_smem(kernel, std::max<size_t>(smem, 48 * 1024), smem_set[dtype == kBF16 ? 1 : 0], false));
+  if (smem > 48 * 1024) CK(allow_smem(kernel, kSmemLimit, smem_set[dtype == kBF16 ? 1 : 0], false));
   CK(launch_dependent(kernel, dim3(grid), kFrontThreads, 1, smem, st, true, A, nvec));
   g_launches.fetch_add(1);
   return OVGGT_OK;
