@@ -462,8 +462,11 @@ def k_gemm_bf16(a: torch.Tensor, b: torch.Tensor, out=None, status=None, stream=
 
 def k_linear_bf16(a, b, outs=(), gelu=False, residual=None, sum_out=None, status=None, stream=None) -> None:
     """t = a [M, K] @ b [K, N] (then GELU); its column blocks to outs; sum_out = residual + t.  Nothing is allocated."""
-    M, K = a.shape
-    _check(lib().ovggt_k_linear_bf16(_dptr(a), _dptr(b), M, b.shape[1], K, (C.c_void_p * 3)(*[_dptr(o) for o in outs]), len(outs),
+    (M, K), N = a.shape, b.shape[1]
+    assert K == b.shape[0] and all(t.dtype == torch.bfloat16 for t in (a, b, residual, sum_out, *outs) if t is not None)
+    assert all(o.numel() * len(outs) == M * N for o in outs)
+    assert all(t.numel() == M * N for t in (residual, sum_out) if t is not None) and status.numel() * status.element_size() >= 4
+    _check(lib().ovggt_k_linear_bf16(_dptr(a), _dptr(b), M, N, K, (C.c_void_p * 3)(*[_dptr(o) for o in outs]), len(outs),
                                      int(gelu), _dptr(residual), _dptr(sum_out), _dptr(status), _stream_ptr(stream)),
            "ovggt_k_linear_bf16")
 
