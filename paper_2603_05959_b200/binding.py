@@ -175,6 +175,7 @@ def _hptr0(t: Optional[torch.Tensor]) -> int:
 # ctypes structure field by field, which cost a small step more host time than its launches.
 _FRAME_IO = struct.Struct("@qPPPPPfPP")
 _NAN = float("nan")
+_UNPACKED = (struct.error, OverflowError)    # what pack refuses and C conversions take: see OvggtCache._convert
 
 
 def torch_dtype(dtype: int) -> torch.dtype:
@@ -259,12 +260,22 @@ class OvggtCache:
         return OvggtFrameIO(int(frame_id), ptr(q), ptr(k), ptr(v), ptr(resid), ptr(conf), float(rho),
                             ptr(score_override), ptr(out))
 
+    def _convert(self, frame_id, *rest) -> None:
+        """The frame arguments by C's conversions, for values that pack refuses: a rho beyond fp32, an id beyond 64 bits, a
+        number as text."""
+        rest = list(rest)
+        rest[5] = float(rest[5])
+        C.memmove(self._io_buf, C.byref(OvggtFrameIO(int(frame_id), *rest)), _FRAME_IO.size)
+
     def new_out(self) -> torch.Tensor:
         return torch.empty((self.M, self.C), dtype=torch_dtype(self.dtype), device=self.device)
 
     def layer_attend(self, layer, frame_id, q, k, v, out=None, stream=None) -> torch.Tensor:
         out = self.new_out() if out is None else out
-        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _dptr0(q), _dptr0(k), _dptr0(v), 0, 0, _NAN, 0, _dptr0(out))
+        try:
+            _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _dptr0(q), _dptr0(k), _dptr0(v), 0, 0, _NAN, 0, _dptr0(out))
+        except _UNPACKED:
+            self._convert(frame_id, _dptr0(q), _dptr0(k), _dptr0(v), 0, 0, _NAN, 0, _dptr0(out))
         code = _LIB.ovggt_layer_attend_at(self._hv, layer, self._io_at, _stream_ptr(stream))
         if code:
             _check(code, "ovggt_layer_attend")
@@ -272,7 +283,11 @@ class OvggtCache:
 
     def layer_compress(self, layer, frame_id, resid, conf=None, rho=float("nan"), score_override=None,
                        stream=None) -> None:
-        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), 0, 0, 0, _dptr0(resid), _dptr0(conf), rho, _dptr0(score_override), 0)
+        try:
+            _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), 0, 0, 0, _dptr0(resid), _dptr0(conf), rho,
+                                _dptr0(score_override), 0)
+        except _UNPACKED:
+            self._convert(frame_id, 0, 0, 0, _dptr0(resid), _dptr0(conf), rho, _dptr0(score_override), 0)
         code = _LIB.ovggt_layer_compress_at(self._hv, layer, self._io_at, _stream_ptr(stream))
         if code:
             _check(code, "ovggt_layer_compress")
@@ -294,7 +309,10 @@ class OvggtCache:
         return bool(reg.value), int(dem.value)
 
     def camera_compress(self, layer, frame_id, resid, registered, demoted_frame, score_override=None, stream=None) -> None:
-        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), 0, 0, 0, _dptr0(resid), 0, _NAN, _dptr0(score_override), 0)
+        try:
+            _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), 0, 0, 0, _dptr0(resid), 0, _NAN, _dptr0(score_override), 0)
+        except _UNPACKED:
+            self._convert(frame_id, 0, 0, 0, _dptr0(resid), 0, _NAN, _dptr0(score_override), 0)
         code = _LIB.ovggt_camera_compress_at(self._hv, layer, self._io_at, 1 if registered else 0, int(demoted_frame),
                                              _stream_ptr(stream))
         if code:
@@ -311,8 +329,12 @@ class OvggtCache:
     def layer_step(self, layer, frame_id, q, k, v, resid, conf=None, rho=float("nan"), score_override=None,
                    out=None, stream=None) -> torch.Tensor:
         out = self.new_out() if out is None else out
-        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _dptr0(q), _dptr0(k), _dptr0(v), _dptr0(resid), _dptr0(conf), rho,
-                            _dptr0(score_override), _dptr0(out))
+        try:
+            _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _dptr0(q), _dptr0(k), _dptr0(v), _dptr0(resid), _dptr0(conf),
+                                rho, _dptr0(score_override), _dptr0(out))
+        except _UNPACKED:
+            self._convert(frame_id, _dptr0(q), _dptr0(k), _dptr0(v), _dptr0(resid), _dptr0(conf), rho,
+                          _dptr0(score_override), _dptr0(out))
         code = _LIB.ovggt_layer_step_at(self._hv, layer, self._io_at, _stream_ptr(stream))
         if code:
             _check(code, "ovggt_layer_step")
@@ -320,8 +342,11 @@ class OvggtCache:
 
     def layer_step_host(self, layer, frame_id, q, k, v, resid, conf, rho, out, stream=None) -> None:
         """All tensors are host (ideally pinned) torch tensors; the copies run inside the call."""
-        _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _hptr0(q), _hptr0(k), _hptr0(v), _hptr0(resid), _hptr0(conf), rho, 0,
-                            _hptr0(out))
+        try:
+            _FRAME_IO.pack_into(self._io_buf, 0, int(frame_id), _hptr0(q), _hptr0(k), _hptr0(v), _hptr0(resid), _hptr0(conf),
+                                rho, 0, _hptr0(out))
+        except _UNPACKED:
+            self._convert(frame_id, _hptr0(q), _hptr0(k), _hptr0(v), _hptr0(resid), _hptr0(conf), rho, 0, _hptr0(out))
         code = _LIB.ovggt_layer_step_host_at(self._hv, layer, self._io_at, _stream_ptr(stream))
         if code:
             _check(code, "ovggt_layer_step_host")
