@@ -163,6 +163,11 @@ class _Scaffold:
         assert int(self.status[0].item()) == 0
 
 
+def _own(*tensors):
+    """What a caller's hook is given of a frame: tensors of its own, not the buffers that the next layer or frame writes."""
+    return [t.clone() for t in tensors]
+
+
 def _randn(shape, std, device, dtype, gen_):
     return (torch.randn(shape, generator=gen_, device=device, dtype=torch.float32) * std).to(dtype)
 
@@ -196,7 +201,7 @@ class ProjectionStack:
         for l in range(L):
             # embeddings are N(0, 1) over 1024 columns and the weights N(0, 0.02): q, k, v come out near N(0, 0.4)
             q, k, v = mm.qkv(x, self.w_qkv[l], stream)
-            ov = self.tap(t, l, q, k, v, resid[l]) if self.tap else None
+            ov = self.tap(t, l, *_own(q, k, v), resid[l]) if self.tap else None
             run = lambda: self.cache.layer_step(l, t, q, k, v, resid[l], conf, rho, score_override=ov, out=self.out,
                                                 stream=stream)
             lib(run) if lib else run()
@@ -277,7 +282,7 @@ class Aggregator:
             # (the frame's result is the caller's; what is passed between the layers is kept)
             x = mm.add_product(h, mm.gelu_product(mm.layer_norm(h), w["fc1"], stream), w["fc2"],
                                out=None if l + 1 == L else keep("global out"), product=r, stream=stream)
-            ov = self.tap(t, l, q, k, v, r) if self.tap else None
+            ov = self.tap(t, l, *_own(q, k, v, r)) if self.tap else None
             if self.batched_compress:
                 resids.append(r)
                 overrides.append(ov)
