@@ -1444,6 +1444,7 @@ extern "C" int ovggt_k_attention(const void* q, const void* k, const void* v, in
     return OVGGT_ERR_INVALID_ARG;
   if (dtype == kBF16 && (!scratch || !device_status)) return OVGGT_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out)) return OVGGT_ERR_MISALIGNED;
+  if (dtype == kF32 && !aligned16(scratch)) scratch = nullptr;   // (optional there: the KV range is then not split)
   return launch_attention(q, k, v, M, N, n_heads, dtype, out, scratch, device_status, static_cast<cudaStream_t>(stream));
 }
 
