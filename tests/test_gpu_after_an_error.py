@@ -1,10 +1,18 @@
 """A call that fails on the host side of CUDA says so, and leaves nothing behind for the next one."""
+import gc
+
 import pytest
 import torch
 
 from paper_2603_05959_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def collected():
+    yield
+    gc.collect()                                         # (a raised error's frames hold a handle's workspace)
 
 
 def test_a_failed_call_does_not_fail_the_next():

@@ -1,11 +1,19 @@
 """Frame arguments as C converts them: a coverage ratio beyond fp32 is infinite (no anchor), an id beyond 64 bits wraps and is
 refused as out of order, numbers as text or as tensors are numbers."""
+import gc
+
 import pytest
 import torch
 
 from paper_2603_05959_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def collected():
+    yield
+    gc.collect()                                         # (a raised error's frames hold tensors)
 
 
 def test_conversions():

@@ -1,4 +1,6 @@
 """What the scaffold's product refuses: other types than bf16 and sizes that do not fit, also through the models that use it."""
+import gc
+
 import pytest
 import torch
 
@@ -7,6 +9,12 @@ from paper_2603_05959_b200 import harness as H
 from paper_2603_05959_b200 import inputs as gen
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def collected():
+    yield
+    gc.collect()                                         # (a raised error's frames hold tensors)
 
 
 def _t(*shape, dtype=torch.bfloat16):

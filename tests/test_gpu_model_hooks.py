@@ -1,4 +1,6 @@
 """What a model's hook is given of a layer stays the hook's: it may be kept over later layers and frames."""
+import gc
+
 import pytest
 import torch
 
@@ -31,3 +33,5 @@ def test_tapped_tensors_are_kept(model, matmul):
     for a, b in zip(kept, seen):
         assert all(torch.equal(p, q) for p, q in zip(a, b))
     m.destroy()
+    del m, tap, args
+    gc.collect()                                         # (the hook and the model hold one another)

@@ -1,5 +1,7 @@
 """Rows wider than the front's centroid can be in shared memory: modes that rank without it take any width, whatever other
 handles the process has used; the others say so."""
+import gc
+
 import numpy as np
 import pytest
 import torch
@@ -7,6 +9,12 @@ import torch
 from paper_2603_05959_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def collected():
+    yield
+    gc.collect()                                         # (a raised error's frames hold a handle's workspace)
 
 
 def _run(heads, dtype, mode, frames=5):
