@@ -12,12 +12,14 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("grid,cached,heads", [((1, 1), 700, 16),      # one row
                                                ((1, 127), 1025, 3),    # a whole tile
-                                               ((3, 43), 2049, 2),     # one row more, 16 parts
+                                               ((3, 43), 2049, 2),     # one row more; 11 and 12 parts
+                                       ((3, 43), 2860, 2),     # the largest number of parts, 16, of one KV tile (fp32: of three)
                                                ((11, 35), 260, 5),     # few parts
-                                               ((1, 126), 127, 1)],    # one KV tile: nothing to join
+                                               ((1, 126), 127, 1)],    # two KV tiles in one part: nothing to join (fp32: 4, then 6 parts)
                          ids=lambda x: str(x).replace(" ", ""))
 @pytest.mark.parametrize("dtype", [B.DTYPE_BF16, B.DTYPE_F32], ids=["bf16", "f32"])
-def test_joined_parts(grid, cached, heads, dtype):
+@pytest.mark.parametrize("fused", [False, True], ids=["attend", "step"])
+def test_joined_parts(grid, cached, heads, dtype, fused):
     orc.set_threads(8)
     rng = np.random.default_rng(cached)
     n_special = 1 if grid != (1, 1) else 0
@@ -34,13 +36,16 @@ def test_joined_parts(grid, cached, heads, dtype):
     K, V = f32(k0), f32(v0)
     for t in range(2):                                  # the second launch finds the tickets as the first one left them
         q, k, v, resid = (draw(M) for _ in range(4))
-        got = f32(cache.layer_attend(0, n0 // M + t, q, k, v)).astype(np.float64)
+        if fused:                                       # the attention beside the selection of the same step
+            got = f32(cache.layer_step(0, n0 // M + t, q, k, v, resid)).astype(np.float64)
+        else:
+            got = f32(cache.layer_attend(0, n0 // M + t, q, k, v)).astype(np.float64)
+            cache.layer_compress(0, n0 // M + t, resid)
         K, V = np.concatenate([K, f32(k)]), np.concatenate([V, f32(v)])
         ref = orc.attention(f32(q), K, V, heads, 64).astype(np.float64)
         # bf16: outputs are rounded to within 2^-8 of themselves, weights too, but independently of each other; fp32: a score
         # of up to 6 sigma carries a few roundings of 2^-24, weights, sums and outputs a few more
         tol = 2.0 ** -8 if dtype == B.DTYPE_BF16 else 2.0 ** -22 * (8 + 6)
         assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)
-        cache.layer_compress(0, n0 // M + t, resid)
     cache.stats(0)                                      # (raises if a kernel has left a status)
     cache.destroy()

@@ -1,5 +1,5 @@
 """The selection where its threshold bin is crowded: ties, near-ties and dense ranges, on one CTA and on a cluster, against a
-stable sort."""
+stable sort.  (Survivors only: what the same launch leaves of the key sums is checked in test_gpu_key_sums.py.)"""
 import numpy as np
 import pytest
 import torch

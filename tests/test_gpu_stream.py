@@ -208,8 +208,8 @@ def test_largest_budget_the_selection_cluster_holds():
 def test_attention_weight_mode_matches_the_oracle(compaction):
     """The attention-weight criterion of the scoring probe (Supp. D): the attention the frame's tokens receive in
     the frame's own attention, from the attention kernels' log2 denominators and a second pass over the frame's
-    M x M block, against the oracle's materialised softmax on every frame; fp32 (SIMT attention) and bf16 (tcgen05
-    attention, split and merged).  In bf16 a third of the attention kernel's exponentials are cubics of relative
+    M x M block, against the oracle's materialised softmax on every frame; fp32 and bf16 (attention on
+    the tensor pipe, split and merged).  In bf16 a third of the attention kernel's exponentials are cubics of relative
     error 1e-4, which enters every denominator: scores and priorities are compared at 5e-4 of their range there."""
     cfg = gen.config_tiny().replace(score_mode=gen.SCORE_ATTN, n_frames=12, min_anchor_interval=4)
     layer = run_teacher_forced(cfg, cfg.n_frames, attn_frames={11}, compaction=compaction)
