@@ -255,10 +255,9 @@ class OvggtCache:
             pass
 
     def _io(self, frame_id, q=None, k=None, v=None, resid=None, conf=None, rho=float("nan"),
-            score_override=None, out=None, host=False) -> OvggtFrameIO:
-        ptr = (lambda t: None if t is None else t.data_ptr()) if host else _dptr
-        return OvggtFrameIO(int(frame_id), ptr(q), ptr(k), ptr(v), ptr(resid), ptr(conf), float(rho),
-                            ptr(score_override), ptr(out))
+            score_override=None, out=None) -> OvggtFrameIO:
+        return OvggtFrameIO(int(frame_id), _dptr(q), _dptr(k), _dptr(v), _dptr(resid), _dptr(conf), float(rho),
+                            _dptr(score_override), _dptr(out))
 
     def _convert(self, frame_id, *rest) -> None:
         """The frame arguments by C's conversions, for values that pack refuses: a rho beyond fp32, an id beyond 64 bits, a

@@ -1057,7 +1057,7 @@ inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, 
 
 static inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
                                       void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
-                                      int force_splits = 0, const float* kmax2 = nullptr, float* lse = nullptr,
+                                      const float* kmax2 = nullptr, float* lse = nullptr,
                                       bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr) {
   const int C = H * kHD;
   CUtensorMap tq;
@@ -1072,7 +1072,7 @@ static inline int attn_tcgen05_launch(const void* q, const void* k, const void* 
   AttnParams P;
   P.M = M; P.N = N; P.H = H;
   P.tiles_total = (N + kBN - 1) / kBN;
-  P.splits = force_splits > 0 ? std::min(force_splits, std::min(kMaxSplits, P.tiles_total)) : attn_choose_splits(M, N, H);
+  P.splits = attn_choose_splits(M, N, H);
   P.tiles_per_split = (P.tiles_total + P.splits - 1) / P.splits;
   P.splits = (P.tiles_total + P.tiles_per_split - 1) / P.tiles_per_split;     // no empty split
   P.out = static_cast<__nv_bfloat16*>(out);

@@ -148,19 +148,7 @@ inline cudaError_t allow_smem(K kernel, size_t bytes, std::atomic<uint64_t>& don
   return e;
 }
 
-// ---- block-wide primitives for a block of up to 1024 threads; `sh` holds >= 33 words.
-
-__device__ inline int block_sum_int(int x, int* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-  __syncthreads();
-  if (lane == 0) sh[warp] = x;
-  __syncthreads();
-  int t = 0;
-  for (int w = 0; w < nwarp; ++w) t += sh[w];
-  return t;
-}
+// ---- block-wide primitive for a block of up to 1024 threads; `sh` holds >= 32 words.
 
 // Exclusive prefix sum of x over the threads of the block in thread order; *total = block sum.
 __device__ __noinline__ int block_excl_scan_int(int x, int* sh, int* total) {
@@ -181,28 +169,6 @@ __device__ __noinline__ int block_excl_scan_int(int x, int* sh, int* total) {
   }
   *total = tot;
   return base + incl - x;
-}
-
-__device__ __noinline__ void block_minmax(float lo, float hi, float* sh, float* out_lo, float* out_hi) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
-  }
-  __syncthreads();
-  if (lane == 0) {
-    sh[warp] = lo;
-    sh[32 + warp] = hi;
-  }
-  __syncthreads();
-  float a = sh[0], b = sh[32];
-  for (int w = 1; w < nwarp; ++w) {
-    a = fminf(a, sh[w]);
-    b = fmaxf(b, sh[32 + w]);
-  }
-  *out_lo = a;
-  *out_hi = b;
 }
 
 }  // namespace ovggt

@@ -196,7 +196,7 @@ int launch_attention(const void* q, const void* k, const void* v, int M, int N, 
                      const float* kmax2 = nullptr, float* lse = nullptr, bool beside_previous = false,
                      unsigned* tickets = nullptr) {
   int launches = 0;
-  const int rc = dtype == kBF16 ? attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, 0, kmax2, lse,
+  const int rc = dtype == kBF16 ? attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, kmax2, lse,
                                                       beside_previous, tickets, &launches)
                                 : attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, tickets,
                                                   &launches);
