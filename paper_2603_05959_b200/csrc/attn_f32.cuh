@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
 // ---------------------------------------------------------------- host side
 
 // Number of KV splits: waves of CTAs over the 2 x 148 slots, each as long as its tiles plus about two more for the
-// set-up (query planes, tensor memory); a split costs a merge of about three tiles.
+// set-up (query planes, tensor memory); a split costs a merge of about three tiles.  (Also where the parts are joined inside,
+// which is cheaper: a charge of its own there has not been measured, and it would regroup sums.)
 inline int attn_f32_choose_splits(int M, int N, int H) {
   const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kF32BN - 1) / kF32BN;
   const long slots = (long)kCtasPerSm * 148;
@@ -422,7 +423,7 @@ static inline int attn_f32_launch(const void* q, const void* k, const void* v, i
   P.status = status;
   P.wait_first = beside_previous ? 0 : 1;
   const dim3 grid((M + kBM - 1) / kBM, H, P.splits);
-  // (an fp32 tile of 64 rows takes about 1.3 us, a bf16 tile 1.85 us)
+  // (the limit on tiles was measured with bf16 tiles of 192 rows and 1.85 us; one of 64 rows here takes about 1.3 us)
   const bool join = tickets && P.splits > 1 && attn_join_inside((long)grid.x * grid.y * grid.z, P.tiles_per_split);
   const auto kernel = join ? k_attn_f32<true> : k_attn_f32<false>;
   static std::atomic<uint64_t> smem_set[2];

@@ -14,9 +14,8 @@
 // hence the widest tile where a product has tiles enough for every SM, the narrowest where it has few, and all of shared
 // memory in flight.  The kernel is launched programmatically
 // behind its predecessor and prefetches its part of B (weights, as a rule) into L2 while that one drains.
-// Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 9.7 / 6.3 / 14.1 / 17.0 us, against
-// 13.9 / 9.2 / 18.1 / 19.4 with 128 x 128 tiles of three stages and four epilogue warps that stored row by row (the second
-// and the fourth of those with K split over two CTAs, see gemm_tile_width).
+// Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 9.7 / 6.3 / 14.1 / 17.0 us; the
+// first and the third took 13.9 and 18.1 us with 128 x 128 tiles of three stages and four epilogue warps that stored row by row.
 // Requirements: K a multiple of 64, N a multiple of 8 (TMA row pitch of 16 bytes), 16-byte aligned bases.  Every
 // barrier wait is bounded (about one second); on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the
 // common teardown, after the MMAs it issued have drained.
