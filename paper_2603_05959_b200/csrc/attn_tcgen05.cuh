@@ -15,7 +15,8 @@
 //   warp 5      allocates tensor memory and issues tcgen05.mma:  S_h = Q K_h^T  (SS, fp32 in TMEM),
 //               O += P_h V_h (P read from TMEM as the A operand, V MN-major from shared memory); the whole warp
 //               walks the loop so that descriptors stay warp-uniform, one elected lane issues
-//   warps 6-7   only complete the second warpgroup, which hands its registers to the softmax warpgroup
+//   warps 6-7   complete the second warpgroup, which hands its registers to the softmax warpgroup; in a step they take the
+//               key sums that the selection beside this kernel leaves (see take_key_sums)
 // With head_dim 64 a 128 x 128 tile needs 512 tensor-pipe cycles but 1024 cycles of the 16-per-clock
 // exponential unit, so the softmax rounds bound the kernel (a 96-column round is about 1,700 cycles, 1,200 of them
 // the exponential pass, whose instruction mix tops out near 0.15 columns per cycle per scheduler); two CTAs are
@@ -485,6 +486,67 @@ __device__ __forceinline__ void join_parts(PartJoin* J, Barriers* B, unsigned ch
   }
 }
 
+// ---------------------------------------------------------------- key sums beside the attention
+
+// What the selection beside this kernel would otherwise take last, for 6 to 13 us in which the attention's later waves are
+// held back: its eight CTAs can keep too few loads in flight.  Here two warps a CTA that have nothing else to do wait for
+// the selection's end and take four columns each.  A lane adds up every fourth entry of one list, eight rows in flight
+// and the entries of the next eight requested with them; the fold over a list's four lanes, then over the lists in order,
+// is the selection's own (fold_key_sums).  24 layers of 1374 + 8192 rows: 2978 -> 2835 us; the first eight frames of a
+// scene of 8192 rows: 578 -> 546 us; 1374 + 16384: 158.9 -> 156.9 us.
+constexpr int kSumsRows = 8;
+__device__ __forceinline__ void take_key_sums(const KeySums& S, int warp, int warps, int* status) {
+  static_assert(kSumsLists * 4 == 32, "four lanes a list");
+  const int lane = threadIdx.x & 31, r = lane >> 2, groups = S.C / 4;
+  const int per = sums_share(S.M, kSumsLists), n_out = S.out[r];
+  const int left = n_out + max(0, min(S.M, (r + 1) * per) - r * per) - (lane & 3);       // entries from this lane's first on
+  const int longest = __reduce_max_sync(0xFFFFFFFFu, left);
+  const int* list = S.list + r * S.cap + (lane & 3);
+#pragma unroll 1
+  for (int g = warp; g < groups; g += warps) {
+    const uint2* column = S.k_cache + g;
+    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
+    int at[kSumsRows];
+#pragma unroll
+    for (int i = 0; i < kSumsRows; ++i) at[i] = 4 * i < left ? list[4 * i] : kSumsNone;
+#pragma unroll 1
+    for (int e = 0; e < longest; e += 4 * kSumsRows) {
+      uint2 u[kSumsRows];
+#pragma unroll
+      for (int i = 0; i < kSumsRows; ++i) {
+        const int slot = at[i] ^ (at[i] >> 31);            // (~x of a negative x)
+        u[i] = at[i] != kSumsNone && index_ok(slot, S.rows, status) ? column[(size_t)slot * groups] : make_uint2(0u, 0u);
+      }
+#pragma unroll
+      for (int i = 0; i < kSumsRows; ++i) {
+        const float sign = at[i] < 0 ? -1.0f : 1.0f;
+        const int next = e + 4 * (kSumsRows + i);
+        at[i] = next < left ? list[next] : kSumsNone;
+        a0 = __fmaf_rn(__uint_as_float(u[i].x << 16), sign, a0);
+        a1 = __fmaf_rn(__uint_as_float(u[i].x & 0xFFFF0000u), sign, a1);
+        a2 = __fmaf_rn(__uint_as_float(u[i].y << 16), sign, a2);
+        a3 = __fmaf_rn(__uint_as_float(u[i].y & 0xFFFF0000u), sign, a3);
+      }
+    }
+    float4 sum = S.ksum != nullptr ? *reinterpret_cast<const float4*>(S.ksum + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      a0 += __shfl_xor_sync(0xFFFFFFFFu, a0, o);
+      a1 += __shfl_xor_sync(0xFFFFFFFFu, a1, o);
+      a2 += __shfl_xor_sync(0xFFFFFFFFu, a2, o);
+      a3 += __shfl_xor_sync(0xFFFFFFFFu, a3, o);
+    }
+#pragma unroll
+    for (int q = 0; q < kSumsLists; ++q) {
+      sum.x += __shfl_sync(0xFFFFFFFFu, a0, 4 * q);
+      sum.y += __shfl_sync(0xFFFFFFFFu, a1, 4 * q);
+      sum.z += __shfl_sync(0xFFFFFFFFu, a2, 4 * q);
+      sum.w += __shfl_sync(0xFFFFFFFFu, a3, 4 * q);
+    }
+    if (lane == 0) *reinterpret_cast<float4*>(S.ksum_next + 4 * g) = sum;
+  }
+}
+
 // ---------------------------------------------------------------- the kernel
 
 struct AttnParams {
@@ -500,6 +562,7 @@ struct AttnParams {
   // beside this one (the selection of the same step), and this kernel must not end before it.
   int wait_first;
   unsigned* tickets;      // JOIN: [query tiles * H], zero
+  KeySums sums;           // wait_first == 0: what that selection leaves to be added up here
 };
 
 // JOIN: the parts of a split KV range are joined here (see join_parts).
@@ -680,6 +743,10 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       }
     }
     __syncwarp();
+  } else if (P.sums.ksum_next != nullptr) {
+    pdl_wait();                                      // the selection is complete
+    const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+    take_key_sums(P.sums, cta * 2 + (warp - 6), (int)(gridDim.x * gridDim.y * gridDim.z) * 2, P.status);
   }
   } else {
     // ------------------------------------------------ softmax, correction and epilogue (128 threads)
@@ -1058,7 +1125,8 @@ inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, 
 static inline int attn_tcgen05_launch(const void* q, const void* k, const void* v, int M, int N, int H, void* out,
                                       void* scratch, int* status, cudaStream_t st, AttnKvMaps* kv_maps = nullptr,
                                       const float* kmax2 = nullptr, float* lse = nullptr,
-                                      bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr) {
+                                      bool beside_previous = false, unsigned* tickets = nullptr, int* launches = nullptr,
+                                      const KeySums& sums = {}) {
   const int C = H * kHD;
   CUtensorMap tq;
   AttnKvMaps local;
@@ -1083,6 +1151,7 @@ static inline int attn_tcgen05_launch(const void* q, const void* k, const void* 
   P.lse = lse;
   P.wait_first = beside_previous ? 0 : 1;
   P.tickets = tickets;
+  P.sums = sums;
   const dim3 grid((M + kBM - 1) / kBM, H, P.splits);
   const bool join = tickets && P.splits > 1 && attn_join_inside((long)grid.x * grid.y * grid.z, P.tiles_per_split);
   const auto kernel = join ? k_attn_tcgen05<true> : k_attn_tcgen05<false>;

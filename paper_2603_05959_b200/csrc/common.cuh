@@ -103,6 +103,20 @@ __device__ __forceinline__ void drop_stale_lines(const int* word) {
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(x) : "l"(word) : "memory");
 }
 
+// The column sums of the cached keys after a step: those before it, plus the rows that come, less the rows that leave.  The
+// selection takes them itself, or leaves the rows in a list per CTA of its cluster for the attention beside it to take (see
+// take_key_sums); either way the rows of a list are added in the same order, so the sums are the same bits.
+constexpr int kSumsLists = 8;                 // CTAs of the selection's cluster
+constexpr int kSumsNone = 0x7FFFFFFF;         // an entry without a row
+struct KeySums {
+  const uint2* k_cache;                       // [.., C] bf16
+  const float* ksum; float* ksum_next;        // [C] before (nullptr: zero) and after the step; ksum_next nullptr: not asked for
+  const int* list; const int* out;            // as CompressParams::sums_list, sums_out
+  int cap, M, C, rows;                        // rows: of k_cache
+};
+// New rows that a list names, of a frame of M.
+__host__ __device__ constexpr int sums_share(int M, int lists) { return (M + lists - 1) / lists; }
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, int threads, int cluster, size_t smem, cudaStream_t st,
                                     bool pdl, Args... args) {

@@ -194,10 +194,10 @@ int launch_fill_holes(void* kc, void* vc, const int* msrc, const int* mdst, cons
 int launch_attention(const void* q, const void* k, const void* v, int M, int N, int H, int dtype, void* out,
                      void* scratch, int* status, cudaStream_t st, AttnKvMaps* maps = nullptr,
                      const float* kmax2 = nullptr, float* lse = nullptr, bool beside_previous = false,
-                     unsigned* tickets = nullptr) {
+                     unsigned* tickets = nullptr, const KeySums& sums = {}) {
   int launches = 0;
   const int rc = dtype == kBF16 ? attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, kmax2, lse,
-                                                      beside_previous, tickets, &launches)
+                                                      beside_previous, tickets, &launches, sums)
                                 : attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, tickets,
                                                   &launches);
   g_launches.fetch_add(launches);
@@ -266,6 +266,7 @@ struct ovggt_cache {
   float *attn_lse = nullptr, *attn_part = nullptr;   // OVGGT_SCORE_ATTN: log2 softmax denominators [M, H], per-head sums [H, M]
   void* attn_scratch = nullptr;
   unsigned* attn_tickets = nullptr;
+  int *sums_list = nullptr, *sums_out = nullptr;     // rows of the key sums that a step's attention takes (see KeySums)
   int* status = nullptr;
   size_t zeroed_bytes = 0;                           // the status block, the key-norm bounds and the attention's tickets behind it
   // two sets of staging buffers for ovggt_layer_step_host: the copies of one step overlap the kernels of the step before
@@ -438,6 +439,7 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
   const size_t o_qk = qk ? L.take((size_t)(colsum_parts(M) + 1) * C * 4) : 0;
   const bool aw = c->score_mode == OVGGT_SCORE_ATTN;
   const size_t o_aw = aw ? L.take((size_t)2 * M * c->n_heads * 4) : 0;
+  const size_t o_sums = L.take((kSumsLists + (size_t)kSumsLists * (M + sums_share(M, kSumsLists))) * 4);
   size_t o_stage[2][5], o_conf[2];
   for (int p = 0; p < 2; ++p) {
     for (int i = 0; i < 5; ++i) o_stage[p][i] = L.take((size_t)M * C * eb);
@@ -449,6 +451,8 @@ size_t layout_workspace(const ovggt_config* c, ovggt_cache* h) {
     h->status = reinterpret_cast<int*>(base + o_status);
     h->zeroed_bytes = zeroed;
     h->attn_tickets = reinterpret_cast<unsigned*>(base + o_status + 64 + bounds_bytes);
+    h->sums_out = reinterpret_cast<int*>(base + o_sums);
+    h->sums_list = h->sums_out + kSumsLists;
     for (int l = 0; l < c->n_layers; ++l)
       h->layers[l].kmax2 = reinterpret_cast<float*>(base + o_status + 64) + (size_t)l * c->n_heads;
     if (aw) {
@@ -668,16 +672,18 @@ int enqueue_front(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, bool 
 
 // The attention over all n + M rows, and the bookkeeping that closes the attend half.  Attention does not care in
 // which order the cached rows lie, so it reads the K/V buffer front to back in either layout.
-// beside_previous: what was enqueued on st just before is the same step's selection, which the attention does not wait for.
+// beside_previous: what was enqueued on st just before is the same step's selection, which the attention does not wait for;
+// sums: what that one leaves to be added up beside the attention.
 int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st, int N, int kb,
-                      bool beside_previous = false) {
+                      bool beside_previous = false, const KeySums& sums = {}) {
   LayerState& S = h->layers[layer];
   int rc;
   {
     ProfScope ps(h, OVGGT_PROF_ATTENTION, st);
     rc = launch_attention(io->q, S.kbuf[kb], S.vbuf[kb], h->M, N, h->cfg.n_heads, h->cfg.dtype, io->out,
                           h->attn_scratch, h->status, st, &S.maps[kb], key_norm_bound(h, S),
-                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous, h->attn_tickets);
+                          h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous, h->attn_tickets,
+                          sums);
   }
   return rc;
 }
@@ -789,8 +795,29 @@ bool continues_sums(const ovggt_cache* h, const LayerState& S) {
          !(h->cfg.compaction == OVGGT_COMPACT_FILL_HOLES && S.n + h->M > S.budget && S.n < S.budget);
 }
 
-// Parameter block of the fused selection kernel for the layer's pending frame.
-CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
+// Whether the attention of a fused step takes the key sums (see take_key_sums): in the hole-filling layout, whose attention is
+// launched behind the selection, for bf16 rows (the fp32 kernel has no idle warps) and where the selection is a cluster (a
+// single CTA has few rows to add).
+bool sums_beside_attention(const ovggt_cache* h, const LayerState& S) {
+  return fill_layout(h) && h->cfg.dtype == kBF16 && compress_ctas(S.n + h->M, h->M) == kSumsLists && continues_sums(h, S);
+}
+// They as a fused step's attention gets them, once the layer's compress is closed; n: rows cached before the step.
+KeySums key_sums(const ovggt_cache* h, const LayerState& S, int n) {
+  KeySums K = {};
+  K.k_cache = reinterpret_cast<const uint2*>(S.kbuf[S.kv]);
+  K.ksum = n > 0 ? S.ksum[S.kcur ^ 1] : nullptr;
+  K.ksum_next = S.ksum[S.kcur];
+  K.list = h->sums_list;
+  K.out = h->sums_out;
+  K.cap = h->M + sums_share(h->M, kSumsLists);
+  K.M = h->M;
+  K.C = h->C;
+  K.rows = S.budget + h->M;
+  return K;
+}
+
+// Parameter block of the fused selection kernel for the layer's pending frame.  sums_beside: the attention takes the key sums.
+CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io, bool sums_beside = false) {
   const ovggt_config& c = h->cfg;
   const int b = S.cur;
   const bool first = io->frame_id == h->first_frame;
@@ -823,7 +850,10 @@ CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io
   P.nvec = h->C * h->elem / 16;
   P.room = S.room ? 1 : 0;
   P.ksum = S.n > 0 ? S.ksum[S.kcur] : nullptr;
-  P.ksum_next = continues_sums(h, S) ? S.ksum[S.kcur ^ 1] : nullptr;
+  P.ksum_next = continues_sums(h, S) && !sums_beside ? S.ksum[S.kcur ^ 1] : nullptr;
+  P.sums_list = sums_beside ? h->sums_list : nullptr;
+  P.sums_cap = h->M + sums_share(h->M, kSumsLists);
+  P.sums_out = h->sums_out;
   return P;
 }
 
@@ -854,7 +884,7 @@ void close_compress(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
 // The compress half on stream st.  The stable gather writes another buffer, so the whole half may run beside an
 // attention that still reads this one; the hole-filling moves are only recorded here (see enqueue_front).
 int compress_impl(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st_sel,
-                  const MirroredDecision* mirrored = nullptr) {
+                  const MirroredDecision* mirrored = nullptr, bool sums_beside = false) {
   int rc = validate_compress(h, layer, io, mirrored);
   if (rc) return rc;
   LayerState& S = h->layers[layer];
@@ -868,7 +898,7 @@ int compress_impl(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaS
     rc = launch_row_norms(io->resid, M, C, c.dtype, S.s_raw, st_sel);
     if (rc) return rc;
   }
-  const CompressParams P = select_params(h, S, io);
+  const CompressParams P = select_params(h, S, io, sums_beside);
   const int ncta = compress_ctas(N, M);
   const size_t smem = compress_smem(N, h->Np, M, S.room);
   const auto kernel = c.dtype == kBF16 ? (ncta == 1 ? k_compress_select<kBF16, true> : k_compress_select<kBF16, false>)
@@ -1044,9 +1074,13 @@ extern "C" int ovggt_layer_step(ovggt_cache* h, int32_t layer, const ovggt_frame
     CK(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
   }
   close_attend(h, S, io);
-  rc = compress_impl(h, layer, io, st);
+  const bool sums_beside = sums_beside_attention(h, S);
+  const int n = S.n;
+  rc = compress_impl(h, layer, io, st, nullptr, sums_beside);
   // (a compress that is refused, as for a frame older than the last anchor decision, leaves the frame attended)
-  const int ra = enqueue_attention(h, layer, io, stable ? h->side : st, N, kb, !stable && rc == OVGGT_OK);
+  const int ra = enqueue_attention(h, layer, io, stable ? h->side : st, N, kb, !stable && rc == OVGGT_OK,
+                                   sums_beside && rc == OVGGT_OK ? key_sums(h, S, n) : KeySums{});
+  if (sums_beside && rc == OVGGT_OK && ra != OVGGT_OK) S.ksum_valid = false;
   if (rc == OVGGT_OK) rc = ra;
   h->last_stream = st;
   if (stable) {   // whatever happened, the caller's stream is ordered after the side work

@@ -31,6 +31,7 @@ namespace cg = cooperative_groups;
 constexpr int kSelectThreads = 512;   // 512 x 64 registers: half an SM, so a CTA fits beside an attention CTA
 constexpr int kSelectWarps = kSelectThreads / 32;
 constexpr int kSelectMaxCtas = 8;
+static_assert(kSelectMaxCtas == kSumsLists, "a list of key sums per CTA");
 constexpr int kSelectBins = kSelectThreads;       // a thread per bin; the last bin holds the protected rows
 constexpr int kSelectSubBins = 256;               // of a crowded bin
 constexpr int kSelectCtaCands = 64, kSelectAllCands = 256;   // candidates of the threshold bin, per CTA and in all
@@ -380,7 +381,7 @@ static_assert(3 * kSelectSubBins <= kDeltaCols, "the finer bins lie in the block
 __host__ __device__ inline size_t compress_smem_bytes(int span, int ncta, int np, int m, bool room) {
   const size_t s4 = ((size_t)span + 3) & ~(size_t)3, m4 = ((size_t)m + 3) & ~(size_t)3, np4 = ((size_t)np + 3) & ~(size_t)3;
   const size_t early = m4 * 4 + np4 * 4 + ((np4 + 15) & ~(size_t)15);
-  const size_t late = room ? (size_t)kDeltaCols * 4 + ((size_t)m + (size_t)((m + ncta - 1) / ncta)) * 4 : 0;
+  const size_t late = room ? (size_t)kDeltaCols * 4 + ((size_t)m + (size_t)sums_share(m, ncta)) * 4 : 0;
   return select_header_bytes() + s4 * (8 + 3 * 4) + ((s4 + 7) & ~(size_t)7) * 2 + (early > late ? early : late);
 }
 
@@ -505,6 +506,9 @@ struct CompressParams {
   const uint4* k_cache; int nvec;
   int room;                         // the block of sums and the list have their place in shared memory (needed for ksum_next)
   const float* ksum; float* ksum_next;   // [C]
+  // Where the attention beside this kernel takes the sums instead (see KeySums): the list of rows, by CTA of the cluster.
+  int* sums_list; int sums_cap;     // [CTAs][sums_cap]: ~slot of a row that leaves, the slot of one that comes, or kSumsNone
+  int* sums_out;                    // [CTAs] rows that leave
 };
 
 // Eq. 6 for new-frame token j (aux tokens keep their raw score); s_raw: the frame's M residual norms.
@@ -950,7 +954,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       }
       n_out = min(M, (int)__reduce_add_sync(0xFFFFFFFFu, lane < kSelectWarps ? sh->wtot[lane][2] : 0));
     }
-    const int span = (N + ncta - 1) / ncta, per = (M + ncta - 1) / ncta, first = min(M, rank * per), n_in = min(M, first + per) - first;
+    const int span = (N + ncta - 1) / ncta, per = sums_share(M, ncta), first = min(M, rank * per), n_in = min(M, first + per) - first;
     for (int j = tid; j < n_in; j += nthr) {
       const int g = n + first + j, owner = g / span;
       const uint32_t key = choose ? G::of(keys, owner)[g - owner * span] : 0u;
@@ -991,6 +995,11 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       if (fill && down && id < M) {
         P.move_dst[id] = slot;
         P.hole_stamp[slot] = P.stamp;
+        if (P.sums_list != nullptr) P.sums_list[rank * P.sums_cap + min(M - 1, id - down_before)] = ~slot;
+      }
+      if (P.sums_list != nullptr && g >= n) {
+        const int q = (g - n) / sums_share(M, ncta);
+        P.sums_list[q * P.sums_cap + (choose ? min(M, sh->cnt_down[q]) : 0) + (g - n - q * sums_share(M, ncta))] = keep ? slot : kSumsNone;
       }
       // which move empties a slot above B: none if its row leaves (or if the list is full: an inconsistency, see below)
       if (fill && slot >= P.B && slot - P.B < M) P.tail_move[slot - P.B] = up && iu < M ? iu : -1;
@@ -999,6 +1008,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   // slots above B that no row occupies yet (the cache has just filled up) hold nothing to move
   if (fill && rank == 0)
     for (int i = max(0, N - P.B) + tid; i < M; i += nthr) P.tail_move[i] = -1;
+  if (P.sums_list != nullptr && rank == 0 && tid < ncta) P.sums_out[tid] = choose ? min(M, sh->cnt_down[tid]) : 0;
   if (rank == 0 && tid == 0) {
     *P.n_keep_out = keep_all;
     if (bad || keep_all != min(N, P.B)) atomicCAS(P.status, 0, OVGGT_ERR_DEVICE_STATUS);
