@@ -44,6 +44,14 @@ constexpr int kFrontRows = 4;                 // rows of a scoring item
 
 __host__ __device__ inline int front_score_items(int rows) { return (rows + kFrontRows - 1) / kFrontRows; }
 
+// 1 - the cosine of a key with the centroid, which is that with the column sums: their product, the squared norms of both; a
+// zero vector has cosine 0.
+__device__ __forceinline__ float key_diversity(float dot, float nrm, float kn) {
+  float cosv = 0.0f;
+  if (nrm > 0.0f && kn > 0.0f) cosv = __fdiv_rn(dot, __fmul_rn(__fsqrt_rn(nrm), __fsqrt_rn(kn)));
+  return 1.0f - cosv;
+}
+
 template <int DT>
 __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constant__ FrontArgs A, int nvec) {
   constexpr int VEC = VecOf<DT>::n;
@@ -107,12 +115,6 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
       }
     kn = warp_sum(kn);
   }
-  // cosine with the centroid = cosine with the column sums; a zero vector has cosine 0
-  auto diversity = [&](float dot, float nrm) {
-    float cosv = 0.0f;
-    if (nrm > 0.0f && kn > 0.0f) cosv = __fdiv_rn(dot, __fmul_rn(__fsqrt_rn(nrm), __fsqrt_rn(kn)));
-    return 1.0f - cosv;
-  };
   auto centroid = [&](int vec, float* ks) {   // 16-byte reads: consecutive lanes are VEC floats apart
 #pragma unroll
     for (int e = 0; e < VEC; e += 4)
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
       if (m >= 0 && A.ksum != nullptr) {      // (m is the same in all lanes)
         dot = warp_sum(dot);
         nrm = warp_sum(nrm);
-        if (lane == 0) A.d[dst] = diversity(dot, nrm);
+        if (lane == 0) A.d[dst] = key_diversity(dot, nrm, kn);
       }
       if (lane == 0) {
         if (m >= 0) A.slot[A.move_j[m]] = dst;
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
       }
       if (mine) {
         if (norm) A.s_raw[row0 + lane] = __fsqrt_rn(nr);
-        else      A.d[row0 + lane] = diversity(dt, nr);
+        else      A.d[row0 + lane] = key_diversity(dt, nr, kn);
       }
     }
   }

@@ -23,6 +23,7 @@
 #include "gemm_tcgen05.cuh"
 #include "score_kernels.cuh"
 #include "select_kernel.cuh"
+#include "token_kernel.cuh"
 
 using namespace ovggt;
 
@@ -627,6 +628,67 @@ int flush_moves(ovggt_cache* h, LayerState& S, cudaStream_t st) {
   return OVGGT_OK;
 }
 
+// The bookkeeping that closes the attend half.
+void close_attend(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
+  if (h->first_frame < 0) {
+    h->first_frame = io->frame_id;
+    h->last_registration = io->frame_id;   // the first frame is the initial anchor
+  }
+  S.pending = true;
+  S.pending_frame = io->frame_id;
+}
+
+// Whether the layer's attend half is one launch (k_token_attend) and its selection moves the admitted row itself: the camera
+// head's caches, one token a frame, as long as their selection is a single CTA.
+bool takes_token(const ovggt_cache* h, const LayerState& S) {
+  return h->cfg.camera_head && compress_ctas(S.budget + 1, 1) == 1 && h->C * 4 <= 48 * 1024;
+}
+
+// Column sums of the cached keys afresh, where a step needs them and has none: after an import or the step that filled the
+// cache up, and every kColsumRefreshEvery-th step; otherwise each compress continues them.
+int refresh_sums(ovggt_cache* h, LayerState& S, cudaStream_t st) {
+  if (S.ksum_valid && S.since_refresh < kColsumRefreshEvery) return OVGGT_OK;
+  int rc = flush_moves(h, S, st);
+  if (rc) return rc;
+  ProfScope ps(h, OVGGT_PROF_DIVERSITY, st);
+  rc = launch_colsum(S.kbuf[S.kv], S.n, h->C, h->cfg.dtype, h->colsum_part, S.ksum[S.kcur], st);
+  if (rc) return rc;
+  S.ksum_valid = true;
+  S.since_refresh = 0;
+  return OVGGT_OK;
+}
+
+// The attend half of a layer that takes_token.
+int enqueue_token(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st) {
+  int rc = validate_attend(h, layer, io);
+  if (rc) return rc;
+  LayerState& S = h->layers[layer];
+  h->last_stream = st;
+  const int b = S.cur, nvec = h->C * h->elem / 16;
+  const bool diversity = ranks_by_diversity(h->cfg.score_mode) && S.n > 0;
+  if (diversity) {
+    rc = refresh_sums(h, S, st);
+    if (rc) return rc;
+  }
+  ProfScope ps(h, OVGGT_PROF_ATTENTION, st);
+  TokenArgs A = {};
+  A.q = (const uint4*)io->q; A.k_new = (const uint4*)io->k; A.v_new = (const uint4*)io->v;
+  A.k_cache = (uint4*)S.kbuf[S.kv]; A.v_cache = (uint4*)S.vbuf[S.kv];
+  A.out = io->out;
+  A.n = S.n; A.H = h->cfg.n_heads;
+  A.frame_id = (long long)io->frame_id;
+  A.ids = S.ids[b]; A.flags = S.flags[b]; A.stored = S.stored[b]; A.slot = S.slot[b];
+  A.kmax2 = key_norm_bound(h, S);
+  if (diversity) { A.ksum = S.ksum[S.kcur]; A.d = S.d; }
+  const int scoring = diversity ? std::min(148, (front_score_items(S.n) + kTokenWarps - 1) / kTokenWarps) : 0;
+  const auto kernel = h->cfg.dtype == kBF16 ? k_token_attend<kBF16> : k_token_attend<kF32>;
+  CK(launch_dependent(kernel, dim3(A.H + scoring), kTokenThreads, 1, diversity ? (size_t)h->C * 4 : 0, st, true, A, nvec));
+  g_launches.fetch_add(1);
+  S.norms_frame = -1;
+  close_attend(h, S, io);
+  return OVGGT_OK;
+}
+
 // The front of a step, one launch: the append (Eq. 2; in the hole-filling layout with the moves the previous compress
 // left, which empty exactly the slots the new frame goes into), the diversity of the cached rows (Sec. 3.2), which
 // depends on nothing the frame brings, and with_norms the residual norms of the new rows (Eq. 5).
@@ -637,16 +699,9 @@ int enqueue_front(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, bool 
   h->last_stream = st;
   const int M = h->M, C = h->C, b = S.cur, kb = S.kv;
   const bool diversity = ranks_by_diversity(h->cfg.score_mode) && S.n > 0;
-  if (diversity && (!S.ksum_valid || S.since_refresh >= kColsumRefreshEvery)) {
-    // Column sums of the cached keys afresh: after an import or the step that filled the cache up, and every
-    // kColsumRefreshEvery-th step; otherwise each compress continues them.
-    rc = flush_moves(h, S, st);
+  if (diversity) {
+    rc = refresh_sums(h, S, st);
     if (rc) return rc;
-    ProfScope ps(h, OVGGT_PROF_DIVERSITY, st);
-    rc = launch_colsum(S.kbuf[kb], S.n, C, h->cfg.dtype, h->colsum_part, S.ksum[S.kcur], st);
-    if (rc) return rc;
-    S.ksum_valid = true;
-    S.since_refresh = 0;
   }
   ProfScope ps(h, OVGGT_PROF_APPEND, st);
   FrontArgs A = {};
@@ -686,16 +741,6 @@ int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, c
                           sums);
   }
   return rc;
-}
-
-// The bookkeeping that closes the attend half.
-void close_attend(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
-  if (h->first_frame < 0) {
-    h->first_frame = io->frame_id;
-    h->last_registration = io->frame_id;   // the first frame is the initial anchor
-  }
-  S.pending = true;
-  S.pending_frame = io->frame_id;
 }
 
 // Query-key mode (Supp. D): the criterion of the new frame's rows, from the frame's own q and k; kept in the layer's
@@ -844,6 +889,9 @@ CompressParams select_params(ovggt_cache* h, LayerState& S, const ovggt_frame_io
   P.move_src = S.move_src; P.move_dst = S.move_dst; P.move_j = S.move_j; P.tail_move = S.tail_move;
   P.n_moves_out = S.n_moves_dev;
   P.hole_stamp = S.hole_stamp; P.stamp = ++S.stamp;
+  const bool moves_here = fill_layout(h) && takes_token(h, S);
+  P.move_k = moves_here ? reinterpret_cast<uint4*>(S.kbuf[S.kv]) : nullptr;
+  P.move_v = moves_here ? reinterpret_cast<uint4*>(S.vbuf[S.kv]) : nullptr;
   // the norms: already taken by the front launch, by a launch of their own, or (a few rows) inside the selection
   P.resid = norms_inside(h, S, io) ? static_cast<const uint4*>(io->resid) : nullptr;
   P.k_cache = reinterpret_cast<const uint4*>(S.kbuf[S.kv]);
@@ -866,7 +914,7 @@ void close_compress(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
   S.since_refresh += 1;
   // Some rows leave: the survivors above slot B have to move into the slots that open below it.  The selection kernel has
   // left the pairs; the next append of this layer carries them out (flush_moves for other readers).
-  if (c.compaction == OVGGT_COMPACT_FILL_HOLES && N > S.budget) S.moves_pending = true;
+  if (c.compaction == OVGGT_COMPACT_FILL_HOLES && N > S.budget && !takes_token(h, S)) S.moves_pending = true;
   S.norms_frame = -1;
   const int per_anchor = c.camera_head ? 1 : c.anchor_tokens;
   if (io->frame_id == h->first_frame && c.protect_first_frame) S.n_prot_init = h->M;
@@ -994,9 +1042,12 @@ int compress_all_layers(ovggt_cache* h, const ovggt_frame_io* ios, cudaStream_t 
 
 extern "C" int ovggt_layer_attend(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int rc = enqueue_front(h, layer, io, false, st);
+  int rc = check_layer(h, layer);
   if (rc) return rc;
   LayerState& S = h->layers[layer];
+  if (takes_token(h, S)) return enqueue_token(h, layer, io, st);
+  rc = enqueue_front(h, layer, io, false, st);
+  if (rc) return rc;
   rc = enqueue_attention(h, layer, io, st, S.n + h->M, S.kv);
   if (rc) return rc;
   close_attend(h, S, io);

@@ -501,6 +501,7 @@ struct CompressParams {
   int* tail_move;                   // [M]: for slot B + i, the index of the move that empties it, or -1
   int* n_moves_out;
   int* hole_stamp; int stamp;       // [B]
+  uint4 *move_k, *move_v;           // not nullptr (a frame of one row, one CTA): the pair is moved here, not by the next append
   const uint4* resid;               // [M, C] or nullptr: compute the residual norms here instead of reading s_raw (small M)
   // Column sums of the keys that stay: ksum_next = ksum (or 0) + admitted keys - evicted keys; ksum_next nullptr: not asked for.
   const uint4* k_cache; int nvec;
@@ -622,6 +623,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   float* part = sraw;   // over the last three, which are dead by then: [kDeltaCols] this CTA's corrections of the key sums
   int* list = reinterpret_cast<int*>(part + kDeltaCols);          // [M + its share of M] slots of the rows they are made of
   const bool hybrid = P.mode == OVGGT_SCORE_HYBRID, choose = N > P.B;
+  const bool one_leaves = SINGLE && N == P.B + 1;                 // (a cache of one token a frame, at its budget)
   pdl_wait();
   pdl_trigger();   // an attention queued behind this kernel reads nothing of it: it starts as soon as this one runs
   const bool own_rank = P.override_r == nullptr;                  // rank the priorities computed here
@@ -642,7 +644,8 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   if (tid == 0) sh->n_cand = sh->pub_up = sh->pub_down = sh->keep_before = 0;
   if (end > n) {
     if (P.resid != nullptr) {
-      for (int j = warp; j < M; j += kSelectWarps) warp_row_norm<DT>(P.resid, j, P.nvec, sraw);
+      // (from the last warp on: the first ones have positions to load)
+      for (int j = kSelectWarps - 1 - warp; j < M; j += kSelectWarps) warp_row_norm<DT>(P.resid, j, P.nvec, sraw);
     } else {
       for (int j = tid; j < M; j += nthr) sraw[j] = P.s_raw[j];
     }
@@ -771,7 +774,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
         key = rank_key(v);
         const float steps = linear ? __fmul_rn(v - bin_lo, bin_scale) : (key > bin_key0 ? __fmul_rn((float)(key - bin_key0), bin_scale) : 0.0f);
         bin = (int)fminf((float)(kSelectBins - 2), fmaxf(0.0f, steps));
-        if (choose) atomicAdd(&sh->hist[bin], 1);
+        if (choose && !one_leaves) atomicAdd(&sh->hist[bin], 1);
       }
       // The kernel's own priority, also when an override is ranked instead.  Where it can be told from its key it is
       // written with the survivors: a cluster barrier waits for the global stores before it.
@@ -801,6 +804,38 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   if (!choose) {
     __syncthreads();
     kw = wlo;                                          // everything stays
+  } else if (one_leaves) {
+    // the row that leaves: the lowest key, of equal ones the last
+    uint32_t key = 0xFFFFFFFFu;
+    int pos = -1;
+    for (int i = tid; i < cnt; i += nthr)
+      if (keys[i] <= key) {
+        key = keys[i];
+        pos = i;
+      }
+    auto lowest = [&]() {
+      const uint32_t k = __reduce_min_sync(0xFFFFFFFFu, key);
+      pos = __reduce_max_sync(0xFFFFFFFFu, key == k ? pos : -1);
+      key = k;
+    };
+    lowest();
+    if (lane == 0) {
+      sh->red[warp][0] = key;
+      sh->red[warp][1] = (uint32_t)pos;
+    }
+    __syncthreads();
+    key = lane < kSelectWarps ? sh->red[lane][0] : 0xFFFFFFFFu;
+    pos = lane < kSelectWarps ? (int)sh->red[lane][1] : -1;
+    lowest();
+    __syncthreads();                                   // (warp_totals writes over them)
+    T = key;
+    posT = pos - 1;
+    bad = key == kKeyProtected;
+    keep_before = 0;
+    keep_all = P.B;
+    warp_totals(wlo, whi, sh, classify, &kw, &uw, &dw);
+    up_all = __reduce_add_sync(0xFFFFFFFFu, lane < kSelectWarps ? sh->wtot[lane][1] : 0);
+    down_all = __reduce_add_sync(0xFFFFFFFFu, lane < kSelectWarps ? sh->wtot[lane][2] : 0);
   } else {
     G::sync();
     find_bin<SINGLE>(sh->hist, kSelectBins, P.B, sh);
@@ -991,9 +1026,14 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       if (fill && up && iu < M) {
         P.move_src[iu] = slot;
         P.move_j[iu] = j;
+        if (SINGLE && P.move_k != nullptr) {
+          sh->cnt_bin[0] = slot;
+          sh->cnt_bin[1] = j;
+        }
       }
       if (fill && down && id < M) {
         P.move_dst[id] = slot;
+        if (SINGLE && P.move_k != nullptr) sh->cnt_bin[2] = slot;
         P.hole_stamp[slot] = P.stamp;
         if (P.sums_list != nullptr) P.sums_list[rank * P.sums_cap + min(M - 1, id - down_before)] = ~slot;
       }
@@ -1004,6 +1044,16 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       // which move empties a slot above B: none if its row leaves (or if the list is full: an inconsistency, see below)
       if (fill && slot >= P.B && slot - P.B < M) P.tail_move[slot - P.B] = up && iu < M ? iu : -1;
     }
+  }
+  if (SINGLE && P.move_k != nullptr && up_all == 1 && down_all == 1) {
+    __syncthreads();
+    const int src = sh->cnt_bin[0], dst = sh->cnt_bin[2];
+    for (int v = tid; v < P.nvec; v += nthr) {
+      const uint4 k = P.move_k[(size_t)src * P.nvec + v], w = P.move_v[(size_t)src * P.nvec + v];
+      P.move_k[(size_t)dst * P.nvec + v] = k;
+      P.move_v[(size_t)dst * P.nvec + v] = w;
+    }
+    if (tid == 0) P.slot_dst[sh->cnt_bin[1]] = dst;
   }
   // slots above B that no row occupies yet (the cache has just filled up) hold nothing to move
   if (fill && rank == 0)
