@@ -9,16 +9,19 @@
 // tensor memory are not rounded to nearest.  Measured against fp64 the result is as close as that of plain fp32
 // arithmetic.
 //
-// What bounds it: 48 MMAs of 128 x 64 x 16 per 128 x 64 tile, about 1,900 tensor-pipe cycles; the exponentials and the
-// splitting of P take about two thirds of the issue slots in that time, the splitting of K and V a further sixth.  A
-// plain fp32 kernel is bound by the FMA pipes at 64 x 2 x 2 instructions per score instead, an order of magnitude more.
-// One CTA owns 128 query rows of one head and a range of 64-row KV tiles; two CTAs share an SM.
-//   warps 0-3  softmax: one thread per query row; running maximum, P split and written to tensor memory over the scores
-//              it came from, O accumulated in registers
-//   warp 4     allocates tensor memory, issues the MMAs (the whole warp in step, one elected lane)
-//   warps 5-7  read K and V rows from global memory, split them and write the bf16 planes, 128-byte swizzled, to
-//              shared memory (done once per CTA and tile: cheaper than a pass over the cache that writes planes, and
-//              it needs no scratch memory)
+// What bounds it: 48 MMAs of 128 x 64 x 16 per 128 x 64 tile, which take the tensor pipe some 61 cycles each, 5,850 for the two
+// query tiles of a CTA; the softmax of a tile is busy for 2,500 of them, the splitting of a K and V tile for 1,900.  A plain
+// fp32 kernel is bound by the FMA pipes at 64 x 2 x 2 instructions per score instead, an order of magnitude more.
+// One CTA per SM owns 256 query rows of one head, two tiles, and a range of 64-row KV tiles, so that K and V are split once for
+// both tiles and their planes have room for two stages.  1374 x 5470 x 16: 176 us; as two CTAs per SM of one tile and one
+// stage each, whose MMAs waited for the splitting, 215.  (Four MMAs a K step instead of six, those that share a plane of A
+// with B planes side by side, leave no room for a second buffer of scores: 259 us.)
+//   warps 0-7    softmax, four for each tile: one thread per query row; running maximum, P split and written to tensor memory
+//                over the scores it came from, O accumulated in registers
+//   warps 8, 9   issue the MMAs of a tile each (the whole warp in step, one elected lane); warp 8 allocates tensor memory
+//   warps 10-15  read K and V rows from global memory, split them and write the bf16 planes, 128-byte swizzled, to
+//                shared memory (done once per CTA and tile: cheaper than a pass over the cache that writes planes, and
+//                it needs no scratch memory)
 // A result that is not finite is taken again in plain fp32 arithmetic, which says whether it should be (see plain_row).
 // Every wait is bounded; on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the common teardown.
 #pragma once
@@ -28,23 +31,26 @@
 namespace ovggt {
 
 constexpr int kF32BN = 64;                              // KV rows per tile
-constexpr int kF32Converters = 96;                      // threads of warps 5-7
+constexpr int kF32Threads = 512;
+constexpr int kF32Converters = 192;                     // threads of warps 10-15
+constexpr int kF32Stages = 2;                           // of K and V planes
 constexpr int kF32QPlane = kBM * kHD * 2;               // 16 KB
 constexpr int kF32KvPlane = kF32BN * kHD * 2;           // 8 KB
 constexpr int kF32RegsSoftmax = 168, kF32RegsOther = 88;
-static_assert(128 * kF32RegsSoftmax + 128 * kF32RegsOther <= kAttnThreads * kRegsLaunch, "register pool of the CTA exceeded");
-// S_b at columns [96 b, 96 b + 64), the planes of P_b over it at [96 b, 96 b + 96), O of a tile at [192, 256)
+static_assert(256 * kF32RegsSoftmax + 256 * kF32RegsOther <= kF32Threads * kRegsLaunch, "register pool of the CTA exceeded");
+// Of each query tile's 256 columns: S_b at columns [96 b, 96 b + 64), the planes of P_b over it at [96 b, 96 b + 96), O of a tile at [192, 256)
 constexpr int kF32ColBuf = 96, kF32ColO = 192;
 
 struct F32Barriers {
-  unsigned long long k_full, k_empty, v_full, v_empty, s_full[2], p_full, o_full, drain;
+  unsigned long long k_full[kF32Stages], k_empty[kF32Stages], v_full[kF32Stages], v_empty[kF32Stages];
+  unsigned long long s_full[2][2], p_full[2], o_full[2], drain[2];   // by query tile
   uint32_t tmem_base;
   int abort_flag;
-  int odd;                // a result of this CTA is not finite
+  int odd[2];             // a result of the tile is not finite
 };
-constexpr int kF32Planes = 3 * kF32QPlane + 6 * kF32KvPlane;
-static_assert(kJoinStages * kPartBytes <= kF32Planes, "the parts do not fit the operand planes");
-constexpr size_t f32_smem_bytes(bool join) { return (size_t)kF32Planes + sizeof(F32Barriers) + (join ? sizeof(PartJoin) + kJoinTable * 4 : 0) + 64; }
+constexpr int kF32Planes = 2 * 3 * kF32QPlane + kF32Stages * 6 * kF32KvPlane;
+static_assert(2 * kJoinStages * kPartBytes <= kF32Planes, "the parts do not fit the operand planes");
+constexpr size_t f32_smem_bytes(bool join) { return (size_t)kF32Planes + sizeof(F32Barriers) + (join ? 2 * (sizeof(PartJoin) + kJoinTable * 4) : 0) + 64; }
 
 struct F32Params {
   const float *q, *k, *v;
@@ -90,12 +96,12 @@ __device__ constexpr int kSplitB[6] = {0, 2, 1, 0, 1, 0};
 // register budget covers any function's.  A function, not inline: with its loops in the kernel the softmax loop came out 5
 // to 11 % slower (1374 x 5470 x 16: 209 us without any of this, 211 so, 220 to 232 inline); one per cent is what looking for such
 // rows costs.
-__device__ __noinline__ void redo_rows(const F32Params& P) {
+__device__ __noinline__ void redo_rows(const F32Params& P, int qt) {
   const int lane = threadIdx.x & 31, h = blockIdx.y;
   const PlainRows plain = {P.q, P.k, P.v, P.N, P.H};
 #pragma unroll 1
-  for (int r = threadIdx.x >> 5; r < kBM && (int)blockIdx.x * kBM + r < P.M; r += 4) {
-    const int m = blockIdx.x * kBM + r;
+  for (int r = (threadIdx.x >> 5) & 3; r < kBM && qt * kBM + r < P.M; r += 4) {
+    const int m = qt * kBM + r;
     float2* o = reinterpret_cast<float2*>(P.out + ((size_t)m * P.H + h) * kHD) + lane;
     float2 x = *o;
     if (__any_sync(0xFFFFFFFFu, !(x.x * 0.0f + x.y * 0.0f == 0.0f))) {
@@ -107,52 +113,59 @@ __device__ __noinline__ void redo_rows(const F32Params& P) {
 
 // JOIN: the parts of a split KV range are joined here (see join_parts).
 template <bool JOIN>
-__global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __grid_constant__ F32Params P) {
+__global__ void __launch_bounds__(kF32Threads, 1) k_attn_f32(const __grid_constant__ F32Params P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   if (smem_u32(smem) & 1023u) {                      // the 128-byte swizzle needs 1024-byte aligned tiles
     if (threadIdx.x == 0) report_status(P.status, OVGGT_ERR_DEVICE_STATUS);
     return;
   }
-  unsigned char* sQ = smem;
-  unsigned char* sK = sQ + 3 * kF32QPlane;
-  unsigned char* sV = sK + 3 * kF32KvPlane;
+  unsigned char* sQ = smem;                            // [2 tiles][3 planes]
+  unsigned char* sK = sQ + 2 * 3 * kF32QPlane;         // [stages][3 planes]
+  unsigned char* sV = sK + kF32Stages * 3 * kF32KvPlane;
   F32Barriers* B = reinterpret_cast<F32Barriers*>(smem + kF32Planes);
-  PartJoin* J = reinterpret_cast<PartJoin*>(B + 1);
+  PartJoin* J = reinterpret_cast<PartJoin*>(B + 1);    // [2]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qt = blockIdx.x, h = blockIdx.y, split = blockIdx.z;
+  const int h = blockIdx.y, split = blockIdx.z;
+  const int q_tiles = (P.M + kBM - 1) / kBM, tiles = min(2, q_tiles - 2 * (int)blockIdx.x);   // of this CTA
   const int t_begin = split * P.tiles_per_split;
   const int n_tiles = min(P.tiles_total, t_begin + P.tiles_per_split) - t_begin;   // >= 1 by construction
   const int C = P.H * kHD;
 
   if (P.wait_first) pdl_wait();
   if (threadIdx.x == 0) {
-    mbar_init(&B->k_full, kF32Converters);
-    mbar_init(&B->v_full, kF32Converters);
-    mbar_init(&B->k_empty, 1);
-    mbar_init(&B->v_empty, 1);
-    mbar_init(&B->s_full[0], 1);
-    mbar_init(&B->s_full[1], 1);
-    mbar_init(&B->p_full, 128);
-    mbar_init(&B->o_full, 1);
-    mbar_init(&B->drain, 1);
-    if constexpr (JOIN)
-      for (int s = 0; s < kJoinStages; ++s) mbar_init(&J->full[s], 1);
-    B->abort_flag = B->odd = 0;
+    for (int s = 0; s < kF32Stages; ++s) {
+      mbar_init(&B->k_full[s], kF32Converters);
+      mbar_init(&B->v_full[s], kF32Converters);
+      mbar_init(&B->k_empty[s], tiles);
+      mbar_init(&B->v_empty[s], tiles);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&B->s_full[i][0], 1);
+      mbar_init(&B->s_full[i][1], 1);
+      mbar_init(&B->p_full[i], 128);
+      mbar_init(&B->o_full[i], 1);
+      mbar_init(&B->drain[i], 1);
+      B->odd[i] = 0;
+      if constexpr (JOIN)
+        for (int s = 0; s < kJoinStages; ++s) mbar_init(&J[i].full[s], 1);
+    }
+    B->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 4) {
+  if (warp == 8) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&B->tmem_base)),
-                 "r"((uint32_t)kTmemCols)
+                 "r"((uint32_t)(2 * kTmemCols))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   // (K and V, which the front wrote, are read behind the barrier below)
-  if (threadIdx.x == kAttnThreads - 32 && !P.wait_first) drop_stale_lines(reinterpret_cast<const int*>(P.q));
-  {  // the query tile's planes: 128 rows x 8 groups of 8 columns, rows past M zero
-    float4 x[4], y[4];
+  if (threadIdx.x == kF32Threads - 32 && !P.wait_first) drop_stale_lines(reinterpret_cast<const int*>(P.q));
+#pragma unroll 1
+  for (int half = 0; half < tiles; ++half) {           // a query tile's planes: 128 rows x 8 groups of 8 columns, rows past M zero
+    float4 x[2], y[2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = threadIdx.x + i * kAttnThreads, m = qt * kBM + (idx >> 3);
+    for (int i = 0; i < 2; ++i) {
+      const int idx = threadIdx.x + i * kF32Threads, m = (2 * (int)blockIdx.x + half) * kBM + (idx >> 3);
       x[i] = y[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (m < P.M) {
         const float4* p = reinterpret_cast<const float4*>(P.q + (size_t)m * C + (size_t)h * kHD + (idx & 7) * 8);
@@ -161,9 +174,9 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
       }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = threadIdx.x + i * kAttnThreads;
-      store_planes(sQ, kF32QPlane, idx >> 3, idx & 7, x[i], y[i]);
+    for (int i = 0; i < 2; ++i) {
+      const int idx = threadIdx.x + i * kF32Threads;
+      store_planes(sQ + half * 3 * kF32QPlane, kF32QPlane, idx >> 3, idx & 7, x[i], y[i]);
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -172,103 +185,120 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
   tc_fence_after();
   const uint32_t tmem = *(volatile uint32_t*)&B->tmem_base;
 
-  if (warp >= 4) {
+  if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kF32RegsOther));
-    if (warp == 4) {
-      // ------------------------------------------------ MMA issuer: QK(0) | QK(1) PV(0) | QK(2) PV(1) | ...
+    if (warp < 10) {
+      // ------------------------------------------------ MMA issuers, one per query tile: QK(0) | QK(1) PV(0) | QK(2) PV(1) | ...
       // QK(t + 1) goes into the other buffer, whose P(t - 1) the already issued PV(t - 1) reads first (the tensor pipe
       // executes one thread's MMAs in order).
-      const bool leader = elect_one();
-      const uint32_t tm = __reduce_or_sync(0xFFFFFFFFu, tmem);
-      constexpr uint32_t idesc_qk = idesc_bf16(kF32BN, false), idesc_pv = idesc_bf16(kHD, true);
-      const uint64_t dq = smem_desc_sw128(smem_u32(sQ)), dk = smem_desc_sw128(smem_u32(sK)), dv = smem_desc_sw128(smem_u32(sV));
-      auto wait_all = [&](void* bar, uint32_t parity) {
-        return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, B, P.status)) != 0;
-      };
-      auto issue_qk = [&](int t) {
-        if (leader) {
+      const int i = warp - 8;
+      if (i < tiles) {
+        const bool leader = elect_one();
+        const uint32_t tm = __reduce_or_sync(0xFFFFFFFFu, tmem) + i * kTmemCols;
+        constexpr uint32_t idesc_qk = idesc_bf16(kF32BN, false), idesc_pv = idesc_bf16(kHD, true);
+        const uint64_t dq = smem_desc_sw128(smem_u32(sQ + i * 3 * kF32QPlane));
+        const uint64_t dk0 = smem_desc_sw128(smem_u32(sK)), dv0 = smem_desc_sw128(smem_u32(sV));
+        auto wait_all = [&](void* bar, uint32_t parity) {
+          return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, B, P.status)) != 0;
+        };
+        auto issue_qk = [&](int t) {
+          const uint64_t dk = dk0 + (uint64_t)((t & 1) * (3 * kF32KvPlane >> 4));
+          if (leader) {
 #pragma unroll
-          for (int g = 0; g < 6; ++g)
+            for (int g = 0; g < 6; ++g)
 #pragma unroll
-            for (int kk = 0; kk < kHD / 16; ++kk)
-              mma_ss(tm + (t & 1) * kF32ColBuf, dq + (uint64_t)(kSplitA[g] * (kF32QPlane >> 4) + kk * 2),
-                     dk + (uint64_t)(kSplitB[g] * (kF32KvPlane >> 4) + kk * 2), idesc_qk, g > 0 || kk > 0);
-          tc_commit(&B->s_full[t & 1]);
-          tc_commit(&B->k_empty);
+              for (int kk = 0; kk < kHD / 16; ++kk)
+                mma_ss(tm + (t & 1) * kF32ColBuf, dq + (uint64_t)(kSplitA[g] * (kF32QPlane >> 4) + kk * 2),
+                       dk + (uint64_t)(kSplitB[g] * (kF32KvPlane >> 4) + kk * 2), idesc_qk, g > 0 || kk > 0);
+            tc_commit(&B->s_full[i][t & 1]);
+            tc_commit(&B->k_empty[t & 1]);
+          }
+        };
+        bool ok = wait_all(&B->k_full[0], 0);
+        if (ok) {
+          tc_fence_after();
+          issue_qk(0);
         }
-      };
-      bool ok = wait_all(&B->k_full, 0);
-      if (ok) {
-        tc_fence_after();
-        issue_qk(0);
-      }
-      for (int t = 0; t < n_tiles && ok; ++t) {
-        if (t + 1 < n_tiles) {
-          ok = wait_all(&B->k_full, (uint32_t)(t + 1) & 1u);
+        for (int t = 0; t < n_tiles && ok; ++t) {
+          if (t + 1 < n_tiles) {
+            ok = wait_all(&B->k_full[(t + 1) & 1], (uint32_t)((t + 1) >> 1) & 1u);
+            if (!ok) break;
+            tc_fence_after();
+            issue_qk(t + 1);
+          }
+          ok = wait_all(&B->v_full[t & 1], (uint32_t)(t >> 1) & 1u);
+          if (ok) ok = wait_all(&B->p_full[i], (uint32_t)t & 1u);
           if (!ok) break;
           tc_fence_after();
-          issue_qk(t + 1);
-        }
-        ok = wait_all(&B->v_full, (uint32_t)t & 1u);
-        if (ok) ok = wait_all(&B->p_full, (uint32_t)t & 1u);
-        if (!ok) break;
-        tc_fence_after();
-        if (leader) {
+          if (leader) {
+            const uint64_t dv = dv0 + (uint64_t)((t & 1) * (3 * kF32KvPlane >> 4));
 #pragma unroll
-          for (int g = 0; g < 6; ++g)
+            for (int g = 0; g < 6; ++g)
 #pragma unroll
-            for (int kk = 0; kk < kF32BN / 16; ++kk)
-              mma_ts(tm + kF32ColO, tm + (t & 1) * kF32ColBuf + kSplitA[g] * 32 + kk * 8,
-                     dv + (uint64_t)(kSplitB[g] * (kF32KvPlane >> 4) + kk * 128), idesc_pv, g > 0 || kk > 0);
-          tc_commit(&B->v_empty);
-          tc_commit(&B->o_full);
+              for (int kk = 0; kk < kF32BN / 16; ++kk)
+                mma_ts(tm + kF32ColO, tm + (t & 1) * kF32ColBuf + kSplitA[g] * 32 + kk * 8,
+                       dv + (uint64_t)(kSplitB[g] * (kF32KvPlane >> 4) + kk * 128), idesc_pv, g > 0 || kk > 0);
+            tc_commit(&B->v_empty[t & 1]);
+            tc_commit(&B->o_full[i]);
+          }
         }
-      }
-      if (ok) {
-        wait_all(&B->v_empty, (uint32_t)(n_tiles - 1) & 1u);
-        wait_all(&B->o_full, (uint32_t)(n_tiles - 1) & 1u);
-      } else {
-        if (leader) tc_commit(&B->drain);             // let every issued MMA finish before TMEM is freed
-        wait_all(&B->drain, 0);
+        if (ok) {
+          wait_all(&B->o_full[i], (uint32_t)(n_tiles - 1) & 1u);
+        } else {
+          if (leader) tc_commit(&B->drain[i]);          // let every issued MMA finish before TMEM is freed
+          wait_all(&B->drain[i], 0);
+        }
       }
       __syncwarp();
     } else {
       // ------------------------------------------------ K / V splitting
-      // The rows of a tile are requested before the wait for its buffer, so that their latency runs under it.
-      const int ct = (int)threadIdx.x - 160;
+      // A tile's rows are requested as soon as the registers are free, a tile ahead of the buffer they go to.
+      const int ct = (int)threadIdx.x - 320;
       constexpr int kVecs = kF32BN * 8, kPer = (kVecs + kF32Converters - 1) / kF32Converters;
-      auto convert = [&](const float* src, unsigned char* dst, int t, void* empty, void* full) -> bool {
-        float4 x[kPer], y[kPer];
+      struct Rows { float4 x[kPer], y[kPer]; };
+      auto load = [&](const float* src, int t, Rows& w) {
         const int row0 = (t_begin + t) * kF32BN;
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
           const int idx = ct + i * kF32Converters, r = row0 + (idx >> 3);
-          x[i] = y[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          w.x[i] = w.y[i] = make_float4(0.f, 0.f, 0.f, 0.f);
           if (idx < kVecs && r < P.N) {
             const float4* p = reinterpret_cast<const float4*>(src + (size_t)r * C + (size_t)h * kHD + (idx & 7) * 8);
-            x[i] = p[0];
-            y[i] = p[1];
+            w.x[i] = p[0];
+            w.y[i] = p[1];
           }
         }
-        if (t > 0 && !mbar_wait(empty, (uint32_t)(t - 1) & 1u, B, P.status)) return false;
+      };
+      auto convert = [&](const Rows& w, unsigned char* planes, int t, unsigned long long* empty, unsigned long long* full) -> bool {
+        const int s = t & 1;
+        if (t >= kF32Stages && !mbar_wait(&empty[s], (uint32_t)(t / kF32Stages - 1) & 1u, B, P.status)) return false;
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
           const int idx = ct + i * kF32Converters;
-          if (idx < kVecs) store_planes(dst, kF32KvPlane, idx >> 3, idx & 7, x[i], y[i]);
+          if (idx < kVecs) store_planes(planes + s * 3 * kF32KvPlane, kF32KvPlane, idx >> 3, idx & 7, w.x[i], w.y[i]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(full);
+        mbar_arrive(&full[s]);
         return true;
       };
-      for (int t = 0; t < n_tiles; ++t)
-        if (!convert(P.k, sK, t, &B->k_empty, &B->k_full) || !convert(P.v, sV, t, &B->v_empty, &B->v_full)) break;
+      Rows k, v;
+      load(P.k, 0, k);
+      load(P.v, 0, v);
+#pragma unroll 1
+      for (int t = 0; t < n_tiles; ++t) {
+        if (!convert(k, sK, t, B->k_empty, B->k_full)) break;
+        if (t + 1 < n_tiles) load(P.k, t + 1, k);
+        if (!convert(v, sV, t, B->v_empty, B->v_full)) break;
+        if (t + 1 < n_tiles) load(P.v, t + 1, v);
+      }
       __syncwarp();
     }
   } else {
-    // ------------------------------------------------ softmax and accumulation of O (128 threads, one query row each)
+    // ------------------------------------------------ softmax and accumulation of O (128 threads a tile, one query row each)
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kF32RegsSoftmax));
-    const int row = warp * 32 + lane;
-    const uint32_t t_row = tmem + ((uint32_t)(warp * 32) << 16);
+    const int tile = warp >> 2, qt = 2 * (int)blockIdx.x + tile, row = (warp & 3) * 32 + lane;
+    if (tile < tiles) {
+    const uint32_t t_row = tmem + tile * kTmemCols + ((uint32_t)((warp & 3) * 32) << 16);
     const float c = 1.4426950408889634f * 0.125f;     // log2(e) / sqrt(64)
     float mref = -INFINITY, l = 0.0f;
     float acc[kHD];
@@ -277,7 +307,7 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
     bool ok = true;
     // acc += O of tile t (both under the reference that held when its P was made)
     auto take_o = [&](int t) -> bool {
-      if (__all_sync(0xFFFFFFFFu, mbar_wait(&B->o_full, (uint32_t)t & 1u, B, P.status)) == 0) return false;
+      if (__all_sync(0xFFFFFFFFu, mbar_wait(&B->o_full[tile], (uint32_t)t & 1u, B, P.status)) == 0) return false;
       tc_fence_after();
 #pragma unroll
       for (int j = 0; j < kHD; j += 16) {
@@ -291,7 +321,7 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
     };
     for (int t = 0; t < n_tiles; ++t) {
       const uint32_t buf = t_row + (t & 1) * kF32ColBuf;
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->s_full[t & 1], (uint32_t)(t >> 1) & 1u, B, P.status)) != 0;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->s_full[tile][t & 1], (uint32_t)(t >> 1) & 1u, B, P.status)) != 0;
       if (!ok) break;
       tc_fence_after();
       uint32_t s[kF32BN];
@@ -337,7 +367,7 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
       mref = mnew;
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(&B->p_full);
+      mbar_arrive(&B->p_full[tile]);
     }
     if (ok) ok = take_o(n_tiles - 1);
     const int m = qt * kBM + row;
@@ -352,47 +382,51 @@ __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm) k_attn_f32(const __g
       for (int i = 0; i < kHD; i += 4) {
         const float4 x = make_float4(acc[i] * f, acc[i + 1] * f, acc[i + 2] * f, acc[i + 3] * f);
         dst[i / 4] = x;
-        if (!JOIN && whole && !all_finite(x)) B->odd = 1;
+        if (!JOIN && whole && !all_finite(x)) B->odd[tile] = 1;
       }
       if (!whole) P.ml_part[JOIN ? part_row : part_row * P.H + h] = make_float2(mref, l);
       if (whole && P.lse != nullptr) P.lse[(size_t)m * P.H + h] = mref + log2f(l);
     }
-    if constexpr (JOIN)
-      if (join_arrive(J, P.tickets + h * gridDim.x + qt, P.splits, ok)) {
+    if constexpr (JOIN) {
+      const bool last = join_arrive(&J[tile], P.tickets + h * q_tiles + qt, P.splits, ok, tile);
+      if (tiles == 2) asm volatile("bar.sync 3, 256;" ::: "memory");   // (the parts come into planes of both tiles)
+      if (last) {
         const int m0 = qt * kBM;
         const size_t row0 = join_row0(P.M, qt, h, P.splits);
-        join_parts(J, B, smem, reinterpret_cast<float*>(J + 1), P.o_part + row0 * kHD, P.ml_part + row0, min(kBM, P.M - m0),
-                   P.splits, P.out + (size_t)m0 * C + h * kHD, C, P.lse != nullptr ? P.lse + (size_t)m0 * P.H + h : nullptr, P.H,
-                   P.status, &B->odd);
+        join_parts(&J[tile], B, smem + tile * kJoinStages * kPartBytes, reinterpret_cast<float*>(J + 2) + tile * kJoinTable,
+                   P.o_part + row0 * kHD, P.ml_part + row0, min(kBM, P.M - m0), P.splits, P.out + (size_t)m0 * C + h * kHD, C,
+                   P.lse != nullptr ? P.lse + (size_t)m0 * P.H + h : nullptr, P.H, P.status, &B->odd[tile], tile);
       }
-    softmax_warps_sync();
-    if (*(volatile int*)&B->odd) redo_rows(P);
+    }
+    softmax_warps_sync(tile);
+    if (*(volatile int*)&B->odd[tile]) redo_rows(P, qt);
+    }
   }
 
   // ------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
-  if (warp == 4) {
+  if (warp == 8) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * kTmemCols)) : "memory");
   }
   if (!P.wait_first) pdl_wait();
 }
 
 // ---------------------------------------------------------------- host side
 
-// Number of KV splits: waves of CTAs over the 2 x 148 slots, each as long as its tiles plus about two more for the
+// Number of KV splits: waves of CTAs, two query tiles each, over 148 SMs, each as long as its tiles plus about two more for the
 // set-up (query planes, tensor memory); a split costs a merge of about three tiles.  (Also where the parts are joined inside,
 // which is cheaper: a charge of its own there has not been measured, and it would regroup sums.)
 inline int attn_f32_choose_splits(int M, int N, int H) {
-  const int q_tiles = (M + kBM - 1) / kBM, tiles = (N + kF32BN - 1) / kF32BN;
-  const long slots = (long)kCtasPerSm * 148;
+  const int q_pairs = (M + 2 * kBM - 1) / (2 * kBM), tiles = (N + kF32BN - 1) / kF32BN;
+  const long slots = 140;                              // (in a step the selection keeps eight SMs for itself)
   int best = 1;
   long best_cost = -1;
   for (int s = 1; s <= kMaxSplits && s <= tiles; ++s) {
     const int per = (tiles + s - 1) / s;
     if ((tiles + per - 1) / per != s) continue;
-    const long waves = ((long)q_tiles * H * s + slots - 1) / slots;
+    const long waves = ((long)q_pairs * H * s + slots - 1) / slots;
     const long cost = waves * (per + 2) + (s > 1 ? 3 : 0);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
@@ -422,14 +456,14 @@ static inline int attn_f32_launch(const void* q, const void* k, const void* v, i
   P.lse = lse;
   P.status = status;
   P.wait_first = beside_previous ? 0 : 1;
-  const dim3 grid((M + kBM - 1) / kBM, H, P.splits);
-  // (the limit on tiles was measured with bf16 tiles of 192 rows and 1.85 us; one of 64 rows here takes about 1.3 us)
-  const bool join = tickets && P.splits > 1 && attn_join_inside((long)grid.x * grid.y * grid.z, P.tiles_per_split);
+  const dim3 grid((M + 2 * kBM - 1) / (2 * kBM), H, P.splits);
+  // (the limit on tiles was measured with bf16 tiles of 192 rows and 1.85 us; one of 64 rows, for two query tiles, takes about 3 us)
+  const bool join = tickets && P.splits > 1 && attn_join_inside(2L * grid.x * grid.y * grid.z, P.tiles_per_split);
   const auto kernel = join ? k_attn_f32<true> : k_attn_f32<false>;
   static std::atomic<uint64_t> smem_set[2];
   cudaError_t e = allow_smem(kernel, f32_smem_bytes(join), smem_set[join]);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
-  e = launch_dependent(kernel, grid, kAttnThreads, 1, f32_smem_bytes(join), st, true, P);
+  e = launch_dependent(kernel, grid, kF32Threads, 1, f32_smem_bytes(join), st, true, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   const bool merge = P.splits > 1 && !join;
   *launches = merge ? 2 : 1;

@@ -367,7 +367,8 @@ __device__ __forceinline__ void plain_row(const PlainRows& A, int m, int h, floa
 constexpr int kJoinTable = (kMaxSplits + 1) * kBM;      // floats: a weight per part and row, then 1 / denominator per row
 static_assert(kJoinTable * 4 <= kQBytes && kJoinStages * kPartBytes <= 2 * kKVStages * kTileBytes, "the parts do not fit the operand tiles");
 
-__device__ __forceinline__ void softmax_warps_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// (128 softmax threads: those of a CTA's first query tile, or of its second one)
+__device__ __forceinline__ void softmax_warps_sync(int tile = 0) { asm volatile("bar.sync %0, 128;" ::"r"(tile + 1) : "memory"); }
 
 // Where the parts of query tile qt of head h lie: O at [row * 64 + column], (m, l) at [row], part s as many rows after part
 // s - 1 as the tile has, so that one copy fetches a part.
@@ -377,18 +378,19 @@ __device__ __forceinline__ size_t join_row0(int M, int qt, int h, int splits) {
 
 // Called by the 128 softmax threads of every CTA after they have stored their part (ok: the part is complete).  Returns
 // whether this CTA is the last of its tile.
-__device__ __forceinline__ bool join_arrive(PartJoin* J, unsigned* ticket, int splits, bool ok) {
-  if ((threadIdx.x & 31) == 0) J->ok[threadIdx.x >> 5] = ok;
+__device__ __forceinline__ bool join_arrive(PartJoin* J, unsigned* ticket, int splits, bool ok, int tile = 0) {
+  const int tid = threadIdx.x & 127;
+  if ((tid & 31) == 0) J->ok[tid >> 5] = ok;
   __threadfence();
   asm volatile("fence.proxy.async;" ::: "memory");     // (the parts are read by bulk copies)
-  softmax_warps_sync();
-  if (threadIdx.x == 0) {
+  softmax_warps_sync(tile);
+  if (tid == 0) {
     const bool last = atomicInc(ticket, (unsigned)splits - 1u) == (unsigned)splits - 1u;
     J->last = last && J->ok[0] && J->ok[1] && J->ok[2] && J->ok[3];
     __threadfence();
     asm volatile("fence.proxy.async;" ::: "memory");
   }
-  softmax_warps_sync();
+  softmax_warps_sync(tile);
   return J->last != 0;
 }
 
@@ -397,8 +399,8 @@ __device__ __forceinline__ bool join_arrive(PartJoin* J, unsigned* ticket, int s
 template <typename Out, typename Barriers>
 __device__ __forceinline__ void join_parts(PartJoin* J, Barriers* B, unsigned char* stage, float* table, const float* o,
                                            const float2* ml, int rows, int splits, Out* out, int C, float* lse, int H, int* status,
-                                           int* odd) {
-  const int tid = threadIdx.x, c4 = tid & 15, r0 = tid >> 4;
+                                           int* odd, int tile = 0) {
+  const int tid = threadIdx.x & 127, c4 = tid & 15, r0 = tid >> 4;
   const uint32_t bytes = (uint32_t)rows * kHD * 4;
   auto fetch = [&](int s) {
     void* bar = &J->full[s % kJoinStages];
@@ -430,7 +432,7 @@ __device__ __forceinline__ void join_parts(PartJoin* J, Barriers* B, unsigned ch
     table[kMaxSplits * kBM + tid] = 1.0f / den;
     if (lse != nullptr) lse[(size_t)tid * H] = mstar + log2f(den);
   }
-  softmax_warps_sync();
+  softmax_warps_sync(tile);
   float4 acc[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -454,7 +456,7 @@ __device__ __forceinline__ void join_parts(PartJoin* J, Barriers* B, unsigned ch
       }
     }
     if (s + kJoinStages < splits) {
-      softmax_warps_sync();                            // the buffer has been read
+      softmax_warps_sync(tile);                            // the buffer has been read
       if (tid == 0 && ok) {
         fetch(s + kJoinStages);
         fetched = s + kJoinStages + 1;
