@@ -948,11 +948,17 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   if (!P.wait_first) pdl_wait();
 }
 
-// The parts joined by a kernel of its own.  One thread per 4 columns, blockIdx.x = row; all loads of a thread are issued before the arithmetic that needs them.
+// The parts joined by a kernel of its own.  One thread per 4 columns, blockIdx.x = row; all loads of a thread are issued before
+// the arithmetic that needs them.  What bounds it is the trip to L2, where the parts have just been written, times the number
+// of waves its CTAs come in; so up to eight parts there is an instance for each number of them, with registers for no more.
+// Two parts of 1041 x 1024: 3.1 us, 3.8 in the instance for four that they shared before; a step of 1374 + 4096 rows (three
+// parts) 59.9 -> 59.4 us.
+constexpr int kMergeExact = 8;
 template <typename Out, int MAXS>
 __global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ o_part, const float2* __restrict__ ml_part,
-                                                    int M, int H, int splits, Out* __restrict__ out,
+                                                    int M, int H, int n_parts, Out* __restrict__ out,
                                                     float* __restrict__ lse, PlainRows plain) {
+  const int splits = MAXS <= kMergeExact ? MAXS : n_parts;
   pdl_trigger();
   const int C = H * kHD, c4 = (int)(blockIdx.y * blockDim.x + threadIdx.x), m = (int)blockIdx.x, h = (c4 * 4) / kHD;
   // launched with programmatic stream serialisation: its CTAs may become resident while the last attention CTAs
@@ -1117,7 +1123,15 @@ template <typename Out>
 inline int attn_merge_launch(const float* o_part, const float2* ml_part, int M, int H, int splits, Out* out, float* lse,
                              cudaStream_t st, const PlainRows& plain = {}) {
   const int c4 = H * kHD / 4, threads = std::min(256, (c4 + 31) / 32 * 32);
-  const auto kernel = splits <= 4 ? k_attn_merge<Out, 4> : (splits <= 8 ? k_attn_merge<Out, 8> : k_attn_merge<Out, kMaxSplits>);
+  static_assert(kMergeExact == 8, "an instance each");
+  const auto kernel = splits == 2   ? k_attn_merge<Out, 2>
+                      : splits == 3 ? k_attn_merge<Out, 3>
+                      : splits == 4 ? k_attn_merge<Out, 4>
+                      : splits == 5 ? k_attn_merge<Out, 5>
+                      : splits == 6 ? k_attn_merge<Out, 6>
+                      : splits == 7 ? k_attn_merge<Out, 7>
+                      : splits == 8 ? k_attn_merge<Out, 8>
+                                    : k_attn_merge<Out, kMaxSplits>;
   cudaError_t e = launch_dependent(kernel, dim3(M, (c4 + threads - 1) / threads), threads, 1, 0, st, true, o_part,
                                    ml_part, M, H, splits, out, lse, plain);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
