@@ -16,6 +16,9 @@
 // behind its predecessor and prefetches its part of B (weights, as a rule) into L2 while that one drains.
 // Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 9.7 / 6.3 / 14.1 / 17.0 us; the
 // first and the third took 13.9 and 18.1 us with 128 x 128 tiles of three stages and four epilogue warps that stored row by row.
+// A residual is requested while the products run, not after them: 0.65 us a product with one (a frame through 24 + 24 blocks,
+// 96 of them: 5639 -> 5572 us).  A table of GELU, looked up in shared memory instead of two error functions a pair, was slower (the
+// third product 15.1 -> 17.3 us in such a frame).
 // Requirements: K a multiple of 64, N a multiple of 8 (TMA row pitch of 16 bytes), 16-byte aligned bases.  Every
 // barrier wait is bounded (about one second); on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the
 // common teardown, after the MMAs it issued have drained.
@@ -56,8 +59,8 @@ struct GemmArgs {
 // x Phi(x), in the form whose bf16 rounding every bf16 input shares with torch's GELU.
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 
-// Finished bf16 columns [n, n + 8) of row m: where the caller wants them.
-__device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, const uint4& t) {
+// Finished bf16 columns [n, n + 8) of row m: where the caller wants them.  r: those of the residual.
+__device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, const uint4& t, const uint4& r) {
   if (P.out[0] != nullptr) {
     const int i = n / P.part;       // (8 columns lie in one part: its width is a multiple of 8)
     __nv_bfloat16* o = i == 0 ? P.out[0] : (i == 1 ? P.out[1] : P.out[2]);
@@ -65,7 +68,6 @@ __device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, con
   }
   if (P.residual != nullptr) {
     const uint32_t* w = reinterpret_cast<const uint32_t*>(&t);
-    const uint4 r = *reinterpret_cast<const uint4*>(P.residual + (size_t)m * P.N + n);
     const uint32_t* rw = reinterpret_cast<const uint32_t*>(&r);
     uint4 s;
     uint32_t* sw = reinterpret_cast<uint32_t*>(&s);
@@ -123,6 +125,13 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   const uint32_t tmem = *(volatile uint32_t*)&B->tmem_base;
   pdl_wait();
 
+  // The epilogue's 16-byte units: a warp finishes a quarter of the columns of 32 rows, whole lines of a row by neighbouring lanes.
+  constexpr int kCols = BN / 4, kUnits = kCols / 8;        // columns of a warp, their units
+  const int quad = warp & 3, side = warp >> 2;
+  auto unit_row = [&](int i) { return m0 + quad * 32 + (lane + 32 * i) / kUnits; };
+  auto unit_col = [&](int i) { return n0 + side * kCols + (lane + 32 * i) % kUnits * 8; };
+  uint4 residual[kUnits];                                  // requested while the products run
+
   bool ok = aligned;
   if (warp == kProducer) {
     // ------------------------------------------------ TMA producer
@@ -176,12 +185,15 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     }
     __syncwarp();
   } else if (ok) {
+    if (P.residual != nullptr)
+#pragma unroll
+      for (int i = 0; i < kUnits; ++i)
+        if (unit_row(i) < P.M && unit_col(i) < P.N)        // (N is a multiple of 8)
+          residual[i] = *reinterpret_cast<const uint4*>(P.residual + (size_t)unit_row(i) * P.N + unit_col(i));
     ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->acc_full, 0, B, P.status)) != 0;
     tc_fence_after();
   }
   // ------------------------------------------------ epilogue: warps 0-15; the stages are free now
-  constexpr int kCols = BN / 4, kUnits = kCols / 8;        // columns of a warp, their 16-byte units
-  const int quad = warp & 3, side = warp >> 2;
   const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);
   if (side < 4 && ok) {                                    // (the producer and the issuer are past the last side)
     uint4* stage = reinterpret_cast<uint4*>(smem) + warp * 32 * kUnits;
@@ -205,10 +217,11 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       }
     }
     __syncwarp();
-#pragma unroll 4
-    for (int i = lane; i < 32 * kUnits; i += 32) {         // whole lines of a row by neighbouring lanes
-      const int r = i / kUnits, u = i % kUnits, m = m0 + quad * 32 + r, n = n0 + side * kCols + u * 8;
-      if (m < P.M && n < P.N) gemm_store8(P, m, n, stage[r * kUnits + (u ^ (r & (kUnits - 1)))]);   // (N is a multiple of 8)
+#pragma unroll
+    for (int i = 0; i < kUnits; ++i) {
+      const int r = (lane + 32 * i) / kUnits, u = (lane + 32 * i) % kUnits;
+      if (unit_row(i) < P.M && unit_col(i) < P.N)
+        gemm_store8(P, unit_row(i), unit_col(i), stage[r * kUnits + (u ^ (r & (kUnits - 1)))], residual[i]);
     }
   }
 
