@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(256) k_compact(const uint4* __restrict__ k_src
 // |K[row, 64h .. 64h+63]|^2).  A warp holds the row as 16-byte vectors (lane + 32 i); a head is eight consecutive
 // vectors, i.e. eight neighbouring lanes of one i.  Non-negative floats order like their bit patterns, so the maximum
 // is an integer atomicMax, which does not depend on the order of arrival.
-__device__ __forceinline__ void warp_key_norm_max(const uint4* u, int nvec, int lane, float* kmax2) {
+// top: kmax2 of the lane's heads as read some time before (it only grows).
+__device__ __forceinline__ void warp_key_norm_max(const uint4* u, int nvec, int lane, float* kmax2, const float* top) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     float ss = 0.0f;
@@ -58,7 +59,7 @@ __device__ __forceinline__ void warp_key_norm_max(const uint4* u, int nvec, int 
     ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 4);
     if ((lane & 7) == 0 && lane + 32 * i < nvec) {
       const int head = (lane + 32 * i) >> 3;
-      if (ss > kmax2[head]) atomicMax(reinterpret_cast<int*>(kmax2) + head, __float_as_int(ss));
+      if (ss > top[i]) atomicMax(reinterpret_cast<int*>(kmax2) + head, __float_as_int(ss));
     }
   }
 }
@@ -73,7 +74,10 @@ __global__ void __launch_bounds__(256) k_key_norm_max(const uint4* __restrict__ 
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (lane + 32 * i < nvec) u[i] = ld_nc(K + (size_t)r * nvec + lane + 32 * i);
-    warp_key_norm_max(u, nvec, lane, kmax2);
+    float top[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) top[i] = lane + 32 * i < nvec ? kmax2[(lane + 32 * i) >> 3] : 0.0f;
+    warp_key_norm_max(u, nvec, lane, kmax2, top);
   }
 }
 

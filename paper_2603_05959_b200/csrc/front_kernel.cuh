@@ -52,13 +52,36 @@ __device__ __forceinline__ float key_diversity(float dot, float nrm, float kn) {
   return 1.0f - cosv;
 }
 
+// The sums over the warp of four rows' products and squared norms; lane 8 r gets those of row r.  The order of warp_sum, bit for
+// bit, but each step hands half of what is left to the other half of the lanes: 10 shuffles instead of 40, which an SM
+// executes at one a cycle (a step of 1374 + 16384 rows: 154.7 -> 153.5 us).
+__device__ __forceinline__ void warp_sum_rows(const float (&dot)[kFrontRows], const float (&nrm)[kFrontRows], float* dt, float* nr) {
+  static_assert(kFrontRows == 4, "two bits of the lane name the row");
+  const int lane = threadIdx.x & 31;
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  float d[2], n[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    d[j] = (b4 ? dot[j + 2] : dot[j]) + __shfl_xor_sync(0xFFFFFFFFu, b4 ? dot[j] : dot[j + 2], 16);
+    n[j] = (b4 ? nrm[j + 2] : nrm[j]) + __shfl_xor_sync(0xFFFFFFFFu, b4 ? nrm[j] : nrm[j + 2], 16);
+  }
+  const float d1 = (b3 ? d[1] : d[0]) + __shfl_xor_sync(0xFFFFFFFFu, b3 ? d[0] : d[1], 8);
+  const float n1 = (b3 ? n[1] : n[0]) + __shfl_xor_sync(0xFFFFFFFFu, b3 ? n[0] : n[1], 8);
+  float x = (b2 ? n1 : d1) + __shfl_xor_sync(0xFFFFFFFFu, b2 ? d1 : n1, 4);
+  x += __shfl_xor_sync(0xFFFFFFFFu, x, 2);
+  x += __shfl_xor_sync(0xFFFFFFFFu, x, 1);
+  *dt = x;
+  *nr = __shfl_xor_sync(0xFFFFFFFFu, x, 4);
+}
+
 template <int DT>
 __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constant__ FrontArgs A, int nvec) {
   constexpr int VEC = VecOf<DT>::n;
   extern __shared__ __align__(16) float sh_ksum[];
   const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-  const int warps_total = (int)((gridDim.x * (unsigned)blockDim.x) >> 5);
+  // (warp by warp over the CTAs, so that each SM gets its share of the new rows, which take longest: 24 layers of 1374 + 8192 rows
+  // 2694 -> 2683 us, a step of 1374 + 4096 by stored scores 58.0 -> 57.5)
+  const int gw = (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x), warps_total = (int)((gridDim.x * (unsigned)blockDim.x) >> 5);
   const int n_div = A.ksum != nullptr ? front_score_items(A.n) : 0;
   const int n_norm = A.resid != nullptr ? front_score_items(A.M) : 0;
   const int items = A.M + n_div + n_norm;
@@ -69,11 +92,19 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
   if (gridDim.x >= 148) pdl_trigger();
   pdl_wait();
   uint4 u[4][4];
+  // What a new row's append looks up besides its rows, requested with them: two trips to memory after another (the move, then
+  // where it goes) that would otherwise come after the rows are there (a step of 718 + 5003 rows of 12 heads: 36.1 -> 35.6 us).
+  const int n_moves = pending && gw < A.M ? min(*A.n_moves_ptr, A.M) : 0;
+  int move = -1;
+  float top[4];                               // the bounds of the heads whose keys the lane holds
   // the first 128 vectors of an item's rows: the new K and V row and what sits in their slot, or four rows to score
   auto load = [&](int item) {
     if (item < A.M) {
       const int s = A.n + item;
       const bool tail = pending && s >= A.B && s - A.B < A.M;
+      move = tail ? A.tail_move[s - A.B] : -1;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) top[i] = A.kmax2 != nullptr && lane + 32 * i < nvec ? A.kmax2[(lane + 32 * i) >> 3] : 0.0f;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (lane + 32 * i < nvec) {
@@ -98,6 +129,15 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
     }
   };
   if (gw < items) load(gw);
+  int dst = 0, meta = 0;                      // of the move of a new row's slot
+  auto look_up = [&]() {
+    if (move >= n_moves) move = -1;
+    if (move >= 0) {
+      dst = A.move_dst[move];
+      meta = A.move_j[move];
+    }
+  };
+  look_up();
   float kn = 0.0f;                            // |ksum|^2, folded by every warp in the same order
   if (A.ksum != nullptr) {
     const int C = nvec * VEC;
@@ -131,19 +171,18 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
   };
 
   for (int item = gw; item < items; item += warps_total) {
-    if (item != gw) load(item);
+    if (item != gw) {
+      load(item);
+      if (item < A.M) look_up();
+    }
     if (item < A.M) {
       // ---- append row j, after carrying down what a pending move left in its slot
       const int j = item, s = A.n + j;
-      const bool tail = pending && s >= A.B && s - A.B < A.M;
-      int m = tail ? A.tail_move[s - A.B] : -1;
-      const int n_moves = tail ? min(*A.n_moves_ptr, A.M) : 0;
       // (a warp collective, reached by every lane whatever part of the row it holds; rows of up to 128 vectors only,
       //  which is all the bound is kept for)
-      if (A.kmax2 != nullptr) warp_key_norm_max(u[0], nvec, lane, A.kmax2);
-      if (m >= n_moves) m = -1;
-      const int dst = m >= 0 ? A.move_dst[m] : 0;
-      if (m >= 0 && (!index_ok(dst, A.B, A.status) || !index_ok(A.move_j[m], A.B, A.status))) m = -1;
+      if (A.kmax2 != nullptr) warp_key_norm_max(u[0], nvec, lane, A.kmax2, top);
+      int m = move;
+      if (m >= 0 && (!index_ok(dst, A.B, A.status) || !index_ok(meta, A.B, A.status))) m = -1;
       float dot = 0.0f, nrm = 0.0f;
       for (int v0 = lane; v0 < nvec; v0 += 128) {
         if (v0 != lane) {
@@ -180,7 +219,7 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
         if (lane == 0) A.d[dst] = key_diversity(dot, nrm, kn);
       }
       if (lane == 0) {
-        if (m >= 0) A.slot[A.move_j[m]] = dst;
+        if (m >= 0) A.slot[meta] = dst;
         A.ids[s] = A.frame_id * (long long)A.M + j;
         A.flags[s] = OVGGT_FLAG_EVICTABLE;
         A.stored[s] = 0.0f;
@@ -191,8 +230,9 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
       const bool norm = item >= A.M + n_div;
       const int row0 = (norm ? item - A.M - n_div : item - A.M) * kFrontRows, rows = norm ? A.M : A.n;
       const uint4* base = norm ? A.resid : A.k_cache;
-      bool mine = lane < kFrontRows && row0 + lane < rows;   // lane r writes the score of row r
-      if (!norm && pending && mine) mine = A.hole_stamp[row0 + lane] != A.stamp;
+      const int row = row0 + (lane >> 3);
+      bool mine = (lane & 7) == 0 && row < rows;             // lane 8 r writes the score of row r
+      if (!norm && pending && mine) mine = A.hole_stamp[row] != A.stamp;
       float dot[kFrontRows] = {}, nrm[kFrontRows] = {};
       for (int v0 = lane; v0 < nvec; v0 += 128) {
         if (v0 != lane) {
@@ -213,18 +253,11 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
             for (int r = 0; r < kFrontRows; ++r) accumulate(u[r][i], ks, dot[r], nrm[r]);
           }
       }
-      float dt = 0.0f, nr = 0.0f;
-#pragma unroll
-      for (int r = 0; r < kFrontRows; ++r) {
-        const float b = warp_sum(nrm[r]), a = norm ? 0.0f : warp_sum(dot[r]);
-        if (lane == r) {
-          dt = a;
-          nr = b;
-        }
-      }
+      float dt, nr;
+      warp_sum_rows(dot, nrm, &dt, &nr);
       if (mine) {
-        if (norm) A.s_raw[row0 + lane] = __fsqrt_rn(nr);
-        else      A.d[row0 + lane] = key_diversity(dt, nr, kn);
+        if (norm) A.s_raw[row] = __fsqrt_rn(nr);
+        else      A.d[row] = key_diversity(dt, nr, kn);
       }
     }
   }
