@@ -44,7 +44,9 @@ constexpr int kAttnThreads = 256;
 // setmaxnreg only moves registers inside the pool the CTA was launched with (threads x launch registers), and an
 // increase that the pool cannot serve waits for ever: the two warpgroups must fit 256 x 128.
 constexpr int kRegsLaunch = 128;    // what __launch_bounds__(256, 2) gives: 65536 / 512
-constexpr int kRegsSoftmax = 216, kRegsOther = 40;
+// (How the registers are split decides how ptxas lays the softmax loop out: 1374 x 9566 x 16 with 216 + 40 registers 74.8 us, with
+// 208 + 48 73.8, with 200 + 56 74.0; with the key sums 76.4, 75.2 and 75.5.)
+constexpr int kRegsSoftmax = 208, kRegsOther = 48;
 static_assert(128 * kRegsSoftmax + 128 * kRegsOther <= kAttnThreads * kRegsLaunch, "register pool of the CTA exceeded");
 constexpr int kQBytes = kBM * kHD * 2;           // 16 KB
 constexpr int kTileBytes = kBN * kHD * 2;          // 24 KB
@@ -65,6 +67,8 @@ constexpr float kFixedRefMaxGap = 48.0f;           // log2 units between the bou
 constexpr int kPolyNum = OVGGT_ATTN_POLY_NUM, kPolyDen = OVGGT_ATTN_POLY_DEN;
 __host__ __device__ constexpr bool pair_on_fma_pipes(int pair) { return (pair * kPolyNum) % kPolyDen < kPolyNum; }
 constexpr int kMaxSplits = 16;
+constexpr int kOutRow = kHD * 4 + 16;   // bytes between the rows of O in shared memory, an odd number of 16-byte words
+static_assert(kBM * kOutRow <= 2 * kKVStages * kTileBytes, "O does not fit the operand tiles");
 
 // What the warps that join the parts of a split KV range share (see join_parts).
 constexpr int kJoinStages = 3, kPartBytes = kBM * kHD * 4;
@@ -275,11 +279,16 @@ __device__ __forceinline__ bool elect_one() {
 // 2^x for a pair on the FMA pipes, for the share of the exponentials taken off the 16-per-clock special-function
 // unit: x = n + f with n = round(x) (magic-number rounding) and f in [-0.5, 0.5], a cubic for 2^f (Chebyshev nodes,
 // relative error 1e-4, below bf16 rounding), and n added into the exponent field.  x is clamped at -125 so that the
-// exponent field cannot wrap; larger x than the rescale threshold only occurs in a pass whose result is discarded.
+// exponent field cannot wrap (CLAMP; not where the caller knows it to be above); larger x than the rescale threshold only
+// occurs in a pass whose result is discarded.
+constexpr float kPolyLowest = -125.0f;
+template <bool CLAMP>
 __device__ __forceinline__ float2 ex2_poly2(float2 x) {
   const float kMagic = 12582912.0f;                  // 1.5 * 2^23
-  x.x = fmaxf(x.x, -125.0f);
-  x.y = fmaxf(x.y, -125.0f);
+  if constexpr (CLAMP) {
+    x.x = fmaxf(x.x, kPolyLowest);
+    x.y = fmaxf(x.y, kPolyLowest);
+  }
   const float2 t = add2(x, make_float2(kMagic, kMagic));
   const float2 n = add2(t, make_float2(-kMagic, -kMagic));
   const float2 f = fma2(n, make_float2(-1.0f, -1.0f), x);
@@ -381,10 +390,10 @@ __device__ __forceinline__ size_t join_row0(int M, int qt, int h, int splits) {
 __device__ __forceinline__ bool join_arrive(PartJoin* J, unsigned* ticket, int splits, bool ok, int tile = 0) {
   const int tid = threadIdx.x & 127;
   if ((tid & 31) == 0) J->ok[tid >> 5] = ok;
-  __threadfence();
-  asm volatile("fence.proxy.async;" ::: "memory");     // (the parts are read by bulk copies)
   softmax_warps_sync(tile);
   if (tid == 0) {
+    __threadfence();                                   // (of what all 128 have written: the barrier comes before it)
+    asm volatile("fence.proxy.async;" ::: "memory");   // (the parts are read by bulk copies)
     const bool last = atomicInc(ticket, (unsigned)splits - 1u) == (unsigned)splits - 1u;
     J->last = last && J->ok[0] && J->ok[1] && J->ok[2] && J->ok[3];
     __threadfence();
@@ -567,8 +576,9 @@ struct AttnParams {
   KeySums sums;           // wait_first == 0: what that selection leaves to be added up here
 };
 
-// JOIN: the parts of a split KV range are joined here (see join_parts).
-template <bool JOIN>
+// JOIN: the parts of a split KV range are joined here (see join_parts).  SUMS: the key sums are taken here (see take_key_sums); an
+// instance of its own, since the code of the idle warps costs the softmax loop 1 to 2 % (1374 x 9566 x 16: 73.8 and 75.2 us).
+template <bool JOIN, bool SUMS>
 __global__ void __launch_bounds__(kAttnThreads, kCtasPerSm)
 k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const AttnParams P) {
@@ -745,7 +755,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       }
     }
     __syncwarp();
-  } else if (P.sums.ksum_next != nullptr) {
+  } else if (SUMS) {
     pdl_wait();                                      // the selection is complete
     const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     take_key_sums(P.sums, cta * 2 + (warp - 6), (int)(gridDim.x * gridDim.y * gridDim.z) * 2, P.status);
@@ -762,8 +772,9 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // Upper bound of this row's logits in log2 units: |q_row,h| |k|_max log2(e) / 8.  The row's 64 query values are
     // the eight 16-byte chunks of its 128-byte line in the (swizzled) Q tile, in whatever order.
     float bound = 0.0f;
-    bool fixed_ref = false;
+    bool fixed_ref = false, in_range = false;
     if (P.kmax2 != nullptr) {
+      const float kmax2 = __ldcg(P.kmax2 + h);         // (on its way while Q is)
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(&B->q_full, 0, B, P.status)) != 0;
       if (ok) {
         float qn2 = 0.0f;
@@ -778,7 +789,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             qn2 = fmaf(hi, hi, qn2);
           }
         }
-        bound = sqrtf(qn2 * __ldcg(P.kmax2 + h)) * c;
+        bound = sqrtf(qn2 * kmax2) * c;
       }
     }
     for (int idx = 0; idx < 2 * n_tiles && ok; ++idx) {       // idx = 2 * tile + half
@@ -801,8 +812,9 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       };
       // p = 2^(s * c - mref) on pairs, packed to bf16 over the front of s[]; returns the row's sum of p (four
       // independent packed partial sums, folded in a fixed order).  With `track` the raw row maximum is gathered in
-      // the same pass (four chains of 3-input maxima), where it hides behind the exponentials.
-      auto exp_pass = [&](auto track, float& raw_max) -> float {
+      // the same pass (four chains of 3-input maxima), where it hides behind the exponentials; without `clamp` two
+      // instructions in eleven a cubic are saved (1374 x 17758 x 16: 125.0 -> 121.9 us).
+      auto exp_pass = [&](auto track, auto clamp, float& raw_max) -> float {
         const float2 c2 = make_float2(c, c), nm2 = make_float2(-mref, -mref);
         float2 acc[4];
         float m4[4];
@@ -816,7 +828,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const float s0 = __uint_as_float(s[j]), s1 = __uint_as_float(s[j + 1]);
           if constexpr (decltype(track)::value) m4[(j >> 1) & 3] = max3(m4[(j >> 1) & 3], s0, s1);
           const float2 x = fma2(make_float2(s0, s1), c2, nm2);
-          const float2 p = pair_on_fma_pipes(j >> 1) ? ex2_poly2(x) : make_float2(ex2(x.x), ex2(x.y));
+          const float2 p = pair_on_fma_pipes(j >> 1) ? ex2_poly2<decltype(clamp)::value>(x) : make_float2(ex2(x.x), ex2(x.y));
           acc[(j >> 1) & 3] = add2(acc[(j >> 1) & 3], p);
           s[j >> 1] = pack_bf16(p.x, p.y);
         }
@@ -847,15 +859,19 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           // exact power of two, as it is (2^0) when the maximum itself is the reference, so a row that one early key
           // dominates loses nothing to the bf16 rounding of P
           if (fixed_ref) mref += ceilf(bound - mref);
+          // no score is below -bound either: where that leaves every exponent within the cubic's range, the clamp is dead (but
+          // for columns past the last row)
+          in_range = fixed_ref && __all_sync(0xFFFFFFFFu, bound + mref <= -1.0f - kPolyLowest) != 0;
         }
-        add = exp_pass(std::false_type{}, raw);
-      } else if (fixed_ref) {
-        add = exp_pass(std::false_type{}, raw);          // no score can exceed the reference: nothing to track
+        add = exp_pass(std::false_type{}, std::true_type{}, raw);
+      } else if (fixed_ref) {                            // no score can exceed the reference: nothing to track
+        add = in_range && (t_begin + it) * kBN + hf * kHalf + kHalf <= P.N ? exp_pass(std::false_type{}, std::false_type{}, raw)
+                                                                          : exp_pass(std::false_type{}, std::true_type{}, raw);
       } else {
         // Later halves compute p under the reference they inherit while the maximum is gathered, and keep the
         // result unless the maximum outgrew the reference by more than the threshold (rare); then O is rescaled,
         // the scores are read again (P has not been written over them yet) and p is recomputed.
-        add = exp_pass(std::true_type{}, raw);
+        add = exp_pass(std::true_type{}, std::true_type{}, raw);
         const float mx = raw * c;
         const bool grow = mx - mref > kRescaleThreshold;
         if (__any_sync(0xFFFFFFFFu, grow)) {
@@ -881,7 +897,7 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             tmem_st16(t_row + kColO + j * 16, o);
           }
           load_scores();
-          add = exp_pass(std::false_type{}, raw);
+          add = exp_pass(std::false_type{}, std::true_type{}, raw);
         }
       }
       l += add;
@@ -900,31 +916,41 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const float inv = 1.0f / l;
       const size_t part_row = JOIN ? join_row0(P.M, qt, h, P.splits) + (size_t)split * min(kBM, P.M - qt * kBM) + row
                                    : (size_t)split * P.M + m;
-      float* part = JOIN ? P.o_part + part_row * kHD : P.o_part + part_row * C + (size_t)h * kHD;
+      // By way of the operand tiles, which are free now: a thread has a row, but a warp stores whole lines of it (kOutRow keeps
+      // the rows' 16-byte words in different banks).  718 x 5721 x 12 with a row stored by each thread 25.9 us, so 24.0; 1374 x
+      // 17758 x 16 123.9 and 121.8.
+      const bool whole = P.splits == 1;
+      unsigned char* stage = sK + quad * 32 * kOutRow;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         uint32_t o[32];
         tmem_ld32(t_row + kColO + j * 32, o);
         tmem_wait_ld();
-        if (m < P.M) {
-          if (P.splits == 1) {
-            uint4* dst = reinterpret_cast<uint4*>(P.out + (size_t)m * C + (size_t)h * kHD + j * 32);
+        uint4* dst = reinterpret_cast<uint4*>(stage + lane * kOutRow);
+        if (whole) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              uint4 w;
-              w.x = pack_bf16(__uint_as_float(o[8 * e + 0]) * inv, __uint_as_float(o[8 * e + 1]) * inv);
-              w.y = pack_bf16(__uint_as_float(o[8 * e + 2]) * inv, __uint_as_float(o[8 * e + 3]) * inv);
-              w.z = pack_bf16(__uint_as_float(o[8 * e + 4]) * inv, __uint_as_float(o[8 * e + 5]) * inv);
-              w.w = pack_bf16(__uint_as_float(o[8 * e + 6]) * inv, __uint_as_float(o[8 * e + 7]) * inv);
-              dst[e] = w;
-            }
-          } else {
-            uint4* dst = reinterpret_cast<uint4*>(part + j * 32);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) dst[e] = make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+          for (int e = 0; e < 4; ++e) {
+            uint4 w;
+            w.x = pack_bf16(__uint_as_float(o[8 * e + 0]) * inv, __uint_as_float(o[8 * e + 1]) * inv);
+            w.y = pack_bf16(__uint_as_float(o[8 * e + 2]) * inv, __uint_as_float(o[8 * e + 3]) * inv);
+            w.z = pack_bf16(__uint_as_float(o[8 * e + 4]) * inv, __uint_as_float(o[8 * e + 5]) * inv);
+            w.w = pack_bf16(__uint_as_float(o[8 * e + 6]) * inv, __uint_as_float(o[8 * e + 7]) * inv);
+            dst[4 * j + e] = w;
           }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) dst[8 * j + e] = make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
         }
       }
+      __syncwarp();
+      const int lanes = whole ? 8 : 16, sub = lane & (lanes - 1);   // 16-byte words of a row
+      unsigned char* to = whole  ? reinterpret_cast<unsigned char*>(P.out + (size_t)(m - lane) * C + (size_t)h * kHD)
+                          : JOIN ? reinterpret_cast<unsigned char*>(P.o_part + (part_row - lane) * kHD)
+                                 : reinterpret_cast<unsigned char*>(P.o_part + (part_row - lane) * C + (size_t)h * kHD);
+      const size_t pitch = whole ? (size_t)C * 2 : (JOIN ? kHD : (size_t)C) * 4;
+#pragma unroll 8
+      for (int r = lane / lanes; r < 32; r += 32 / lanes)
+        if (m - lane + r < P.M) *reinterpret_cast<uint4*>(to + r * pitch + sub * 16) = *reinterpret_cast<const uint4*>(stage + r * kOutRow + sub * 16);
       if (P.splits > 1 && m < P.M) P.ml_part[JOIN ? part_row : part_row * P.H + h] = make_float2(mref, l);
       if (P.splits == 1 && P.lse != nullptr && m < P.M) P.lse[(size_t)m * P.H + h] = mref + log2f(l);
     }
@@ -1170,9 +1196,11 @@ static inline int attn_tcgen05_launch(const void* q, const void* k, const void* 
   P.sums = sums;
   const dim3 grid((M + kBM - 1) / kBM, H, P.splits);
   const bool join = tickets && P.splits > 1 && attn_join_inside((long)grid.x * grid.y * grid.z, P.tiles_per_split);
-  const auto kernel = join ? k_attn_tcgen05<true> : k_attn_tcgen05<false>;
-  static std::atomic<uint64_t> smem_set[2];
-  cudaError_t e = allow_smem(kernel, kAttnSmemBytes, smem_set[join]);
+  const bool take_sums = sums.ksum_next != nullptr;
+  const auto kernel = join ? (take_sums ? k_attn_tcgen05<true, true> : k_attn_tcgen05<true, false>)
+                           : (take_sums ? k_attn_tcgen05<false, true> : k_attn_tcgen05<false, false>);
+  static std::atomic<uint64_t> smem_set[4];
+  cudaError_t e = allow_smem(kernel, kAttnSmemBytes, smem_set[2 * join + take_sums]);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
   e = launch_dependent(kernel, grid, kAttnThreads, 1, kAttnSmemBytes, st, true, tq, tk, tv, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
