@@ -457,8 +457,10 @@ static inline int attn_f32_launch(const void* q, const void* k, const void* v, i
   P.status = status;
   P.wait_first = beside_previous ? 0 : 1;
   const dim3 grid((M + 2 * kBM - 1) / (2 * kBM), H, P.splits);
-  // (the limit on tiles was measured with bf16 tiles of 192 rows and 1.85 us; one of 64 rows, for two query tiles, takes about 3 us)
-  const bool join = tickets && P.splits > 1 && attn_join_inside(2L * grid.x * grid.y * grid.z, P.tiles_per_split);
+  // Joined inside where a frame is one query tile and a part has one or two KV tiles, over steps of 69 x 325 x 4 to 126 x 726 x 16 as
+  // fast or faster (31.5 -> 28.9 us); with three KV tiles a launch of its own is 2 us faster, with six to eight 7 or 8, and with
+  // two query tiles a CTA always (355 x 1376 x 4: 29.6 -> 25.3).
+  const bool join = tickets && P.splits > 1 && M <= kBM && P.tiles_per_split <= 2 && attn_join_inside(2L * grid.x * grid.y * grid.z, P.tiles_per_split);
   const auto kernel = join ? k_attn_f32<true> : k_attn_f32<false>;
   static std::atomic<uint64_t> smem_set[2];
   cudaError_t e = allow_smem(kernel, f32_smem_bytes(join), smem_set[join]);
