@@ -639,9 +639,10 @@ void close_attend(ovggt_cache* h, LayerState& S, const ovggt_frame_io* io) {
 }
 
 // Whether the layer's attend half is one launch (k_token_attend) and its selection moves the admitted row itself: the camera
-// head's caches, one token a frame, as long as their selection is a single CTA.
+// head's caches, one token a frame, as long as their selection is a single CTA and the centroid fits beside k_token_attend's own
+// shared memory without an opt-in.
 bool takes_token(const ovggt_cache* h, const LayerState& S) {
-  return h->cfg.camera_head && compress_ctas(S.budget + 1, 1) == 1 && h->C * 4 <= 48 * 1024;
+  return h->cfg.camera_head && compress_ctas(S.budget + 1, 1) == 1 && h->C * 4 <= 40 * 1024;
 }
 
 // Column sums of the cached keys afresh, where a step needs them and has none: after an import or the step that filled the

@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("dtype", [B.DTYPE_BF16, B.DTYPE_F32], ids=["bf16", "f32"])
 @pytest.mark.parametrize("compaction", [B.COMPACT_FILL_HOLES, B.COMPACT_STABLE_GATHER], ids=["holes", "stable"])
-@pytest.mark.parametrize("budget,heads", [(4, 1), (15, 3), (31, 16), (32, 5), (255, 2), (256, 16), (511, 3), (1023, 1), (1024, 2)])
+@pytest.mark.parametrize("budget,heads", [(4, 1), (15, 3), (31, 16), (32, 5), (255, 2), (256, 16), (511, 3), (1023, 1), (1024, 2),
+                                          (5, 160), (5, 161), (5, 192)])    # (the most heads of one launch, more)
 def test_token_stream(budget, heads, compaction, dtype):
     cache = B.OvggtCache.camera(n_heads=heads, budget=budget, dtype=dtype, compaction=compaction)
     C, td = heads * 64, B.torch_dtype(dtype)
