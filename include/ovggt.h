@@ -210,7 +210,8 @@ int ovggt_cache_set_overlap(ovggt_cache* cache, int32_t enable);
  * reset; it never shrinks, so it stays a bound when keys are evicted), and |q| |k|_max / sqrt(64) bounds every logit
  * of a query row.  A warp whose 32 rows all find that bound within 2^48 of the true maximum of their first 96 scores
  * uses it for good and skips maximum tracking and rescaling; other warps track the maximum as before.  Results agree
- * within the attention tolerance either way.  On by default; 0 turns it off for the handle. */
+ * within the attention tolerance either way.  A key that is infinite or not a number makes the bound of its head infinite,
+ * so that the head's maximum is tracked from then on, until a reset or an import.  On by default; 0 turns it off for the handle. */
 int ovggt_cache_set_key_bound(ovggt_cache* cache, int32_t enable);
 
 /* The same step with HOST tensors: q, k, v, resid, conf, out are host pointers; score_override must be NULL.
@@ -344,7 +345,8 @@ int ovggt_k_attention(const void* q, const void* k, const void* v, int32_t M, in
 /* The bf16 attention with a fixed softmax reference where it is safe (see ovggt_cache_set_key_bound).
  * ovggt_k_key_norm_bound: kmax2 [n_heads] (device) = max over the rows of K [rows, n_heads * 64] (bf16) of the squared
  * norm of each head's 64 columns; n_heads <= 16.  ovggt_k_attention_bounded: as ovggt_k_attention for bf16, given such
- * a bound for (at least) the N keys it attends over; a bound that is too small voids the result. */
+ * a bound for (at least) the N keys it attends over; a bound that is too small voids the result.  The bound is infinite for a
+ * head with a key that is infinite or not a number. */
 int ovggt_k_key_norm_bound(const void* K, int32_t rows, int32_t n_heads, float* kmax2, void* stream);
 int ovggt_k_attention_bounded(const void* q, const void* k, const void* v, int32_t M, int32_t N, int32_t n_heads,
                               void* out, void* scratch, int32_t* device_status, const float* kmax2, void* stream);

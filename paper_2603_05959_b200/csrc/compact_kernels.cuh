@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(256) k_compact(const uint4* __restrict__ k_src
 // |K[row, 64h .. 64h+63]|^2).  A warp holds the row as 16-byte vectors (lane + 32 i); a head is eight consecutive
 // vectors, i.e. eight neighbouring lanes of one i.  Non-negative floats order like their bit patterns, so the maximum
 // is an integer atomicMax, which does not depend on the order of arrival.
-// top: kmax2 of the lane's heads as read some time before (it only grows).
+// top: kmax2 of the lane's heads as read some time before (it only grows).  A key that is not a number has an infinite norm here:
+// no bound holds for its scores, and the attention's exponentials may leave their range check out only where one does.
 __device__ __forceinline__ void warp_key_norm_max(const uint4* u, int nvec, int lane, float* kmax2, const float* top) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -59,7 +60,7 @@ __device__ __forceinline__ void warp_key_norm_max(const uint4* u, int nvec, int 
     ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 4);
     if ((lane & 7) == 0 && lane + 32 * i < nvec) {
       const int head = (lane + 32 * i) >> 3;
-      if (ss > top[i]) atomicMax(reinterpret_cast<int*>(kmax2) + head, __float_as_int(ss));
+      if (!(ss <= top[i])) atomicMax(reinterpret_cast<int*>(kmax2) + head, __float_as_int(ss == ss ? ss : INFINITY));
     }
   }
 }
