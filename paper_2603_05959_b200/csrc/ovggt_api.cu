@@ -950,10 +950,13 @@ int compress_impl(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaS
   const CompressParams P = select_params(h, S, io, sums_beside);
   const int ncta = compress_ctas(N, M);
   const size_t smem = compress_smem(N, h->Np, M, S.room);
-  const auto kernel = c.dtype == kBF16 ? (ncta == 1 ? k_compress_select<kBF16, true> : k_compress_select<kBF16, false>)
-                                       : (ncta == 1 ? k_compress_select<kF32, true> : k_compress_select<kF32, false>);
-  static std::atomic<uint64_t> smem_set[4];
-  CK(allow_smem(kernel, kSmemLimit, smem_set[(c.dtype == kBF16 ? 2 : 0) + (ncta == 1 ? 1 : 0)]));
+  const bool single = ncta == 1, one = single && N == B + 1;
+  const auto kernel = c.dtype == kBF16 ? (one ? k_compress_select<kBF16, true, true>
+                                          : single ? k_compress_select<kBF16, true, false> : k_compress_select<kBF16, false, false>)
+                                       : (one ? k_compress_select<kF32, true, true>
+                                          : single ? k_compress_select<kF32, true, false> : k_compress_select<kF32, false, false>);
+  static std::atomic<uint64_t> smem_set[6];
+  CK(allow_smem(kernel, kSmemLimit, smem_set[(c.dtype == kBF16 ? 3 : 0) + single + one]));
   {
     ProfScope ps(h, OVGGT_PROF_SELECT, st_sel);
     CK(launch_dependent(kernel, dim3(ncta), kSelectThreads, ncta, smem, st_sel, true, P));

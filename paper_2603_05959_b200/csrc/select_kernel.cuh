@@ -600,7 +600,11 @@ __device__ __noinline__ void fold_key_sums(const CompressParams& P, const int* l
   }
 }
 
-template <int DT, bool SINGLE>
+// ONE: a single CTA and one row more than the budget, as in a cache of one token a frame that is full; two reductions find the row
+// that leaves, and the admitted one is moved here where that is asked for.  An instance of its own, since its code slows the
+// general one down (steps over 300 rows of 5 / 20 / 69 tokens, bf16: 16.3 / 16.8 / 19.0 us beside it, 15.6 / 16.1 / 18.6 without)
+// and the other way round (camera head, 16 heads and 144 rows, fp32: 13.2 and 12.7 us a layer).
+template <int DT, bool SINGLE, bool ONE = false>
 __device__ __forceinline__ void compress_select_body(const CompressParams& P, unsigned char* smem) {
   using G = Peers<SINGLE>;
   const int ncta = G::count(), rank = G::rank();
@@ -623,7 +627,6 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   float* part = sraw;   // over the last three, which are dead by then: [kDeltaCols] this CTA's corrections of the key sums
   int* list = reinterpret_cast<int*>(part + kDeltaCols);          // [M + its share of M] slots of the rows they are made of
   const bool hybrid = P.mode == OVGGT_SCORE_HYBRID, choose = N > P.B;
-  const bool one_leaves = SINGLE && N == P.B + 1;                 // (a cache of one token a frame, at its budget)
   pdl_wait();
   pdl_trigger();   // an attention queued behind this kernel reads nothing of it: it starts as soon as this one runs
   const bool own_rank = P.override_r == nullptr;                  // rank the priorities computed here
@@ -774,7 +777,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
         key = rank_key(v);
         const float steps = linear ? __fmul_rn(v - bin_lo, bin_scale) : (key > bin_key0 ? __fmul_rn((float)(key - bin_key0), bin_scale) : 0.0f);
         bin = (int)fminf((float)(kSelectBins - 2), fmaxf(0.0f, steps));
-        if (choose && !one_leaves) atomicAdd(&sh->hist[bin], 1);
+        if (choose && !ONE) atomicAdd(&sh->hist[bin], 1);
       }
       // The kernel's own priority, also when an override is ranked instead.  Where it can be told from its key it is
       // written with the survivors: a cluster barrier waits for the global stores before it.
@@ -801,10 +804,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   };
   int wlo, whi, kw = 0, uw = 0, dw = 0;                // this warp's positions, and what the block's lower warps hold
   warp_range(cnt, warp, &wlo, &whi);
-  if (!choose) {
-    __syncthreads();
-    kw = wlo;                                          // everything stays
-  } else if (one_leaves) {
+  if constexpr (ONE) {
     // the row that leaves: the lowest key, of equal ones the last
     uint32_t key = 0xFFFFFFFFu;
     int pos = -1;
@@ -836,6 +836,9 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
     warp_totals(wlo, whi, sh, classify, &kw, &uw, &dw);
     up_all = __reduce_add_sync(0xFFFFFFFFu, lane < kSelectWarps ? sh->wtot[lane][1] : 0);
     down_all = __reduce_add_sync(0xFFFFFFFFu, lane < kSelectWarps ? sh->wtot[lane][2] : 0);
+  } else if (!choose) {
+    __syncthreads();
+    kw = wlo;                                          // everything stays
   } else {
     G::sync();
     find_bin<SINGLE>(sh->hist, kSelectBins, P.B, sh);
@@ -1026,14 +1029,14 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       if (fill && up && iu < M) {
         P.move_src[iu] = slot;
         P.move_j[iu] = j;
-        if (SINGLE && P.move_k != nullptr) {
+        if (ONE && P.move_k != nullptr) {
           sh->cnt_bin[0] = slot;
           sh->cnt_bin[1] = j;
         }
       }
       if (fill && down && id < M) {
         P.move_dst[id] = slot;
-        if (SINGLE && P.move_k != nullptr) sh->cnt_bin[2] = slot;
+        if (ONE && P.move_k != nullptr) sh->cnt_bin[2] = slot;
         P.hole_stamp[slot] = P.stamp;
         if (P.sums_list != nullptr) P.sums_list[rank * P.sums_cap + min(M - 1, id - down_before)] = ~slot;
       }
@@ -1045,7 +1048,7 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
       if (fill && slot >= P.B && slot - P.B < M) P.tail_move[slot - P.B] = up && iu < M ? iu : -1;
     }
   }
-  if (SINGLE && P.move_k != nullptr && up_all == 1 && down_all == 1) {
+  if (ONE && P.move_k != nullptr && up_all == 1 && down_all == 1) {
     __syncthreads();
     const int src = sh->cnt_bin[0], dst = sh->cnt_bin[2];
     for (int v = tid; v < P.nvec; v += nthr) {
@@ -1072,10 +1075,10 @@ __device__ __forceinline__ void compress_select_body(const CompressParams& P, un
   G::leave();
 }
 
-template <int DT, bool SINGLE>
+template <int DT, bool SINGLE, bool ONE>
 __global__ void __launch_bounds__(kSelectThreads, 2) k_compress_select(const __grid_constant__ CompressParams P) {
   extern __shared__ __align__(16) unsigned char smem_select[];
-  compress_select_body<DT, SINGLE>(P, smem_select);
+  compress_select_body<DT, SINGLE, ONE>(P, smem_select);
 }
 
 // The same step for several layers in one launch (Sec. 3.2: every layer has its own budget B^(l) and cache): one
