@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
   if (gridDim.x >= 148) pdl_trigger();
   pdl_wait();
   uint4 u[4][4];
-  // What a new row's append looks up besides its rows, requested with them: two trips to memory after another (the move, then
-  // where it goes) that would otherwise come after the rows are there (a step of 718 + 5003 rows of 12 heads: 36.1 -> 35.6 us).
+  // What a new row's append looks up besides its rows is requested with them.  (But for where its slot's move goes, which is known when
+  // the move is: waiting for that before the first item costs small steps 0.1 to 0.4 us and gains none anything.)
   const int n_moves = pending && gw < A.M ? min(*A.n_moves_ptr, A.M) : 0;
   int move = -1;
   float top[4];                               // the bounds of the heads whose keys the lane holds
@@ -129,15 +129,6 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
     }
   };
   if (gw < items) load(gw);
-  int dst = 0, meta = 0;                      // of the move of a new row's slot
-  auto look_up = [&]() {
-    if (move >= n_moves) move = -1;
-    if (move >= 0) {
-      dst = A.move_dst[move];
-      meta = A.move_j[move];
-    }
-  };
-  look_up();
   float kn = 0.0f;                            // |ksum|^2, folded by every warp in the same order
   if (A.ksum != nullptr) {
     const int C = nvec * VEC;
@@ -171,17 +162,15 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
   };
 
   for (int item = gw; item < items; item += warps_total) {
-    if (item != gw) {
-      load(item);
-      if (item < A.M) look_up();
-    }
+    if (item != gw) load(item);
     if (item < A.M) {
       // ---- append row j, after carrying down what a pending move left in its slot
       const int j = item, s = A.n + j;
       // (a warp collective, reached by every lane whatever part of the row it holds; rows of up to 128 vectors only,
       //  which is all the bound is kept for)
       if (A.kmax2 != nullptr) warp_key_norm_max(u[0], nvec, lane, A.kmax2, top);
-      int m = move;
+      int m = move < n_moves ? move : -1;
+      const int dst = m >= 0 ? A.move_dst[m] : 0, meta = m >= 0 ? A.move_j[m] : 0;
       if (m >= 0 && (!index_ok(dst, A.B, A.status) || !index_ok(meta, A.B, A.status))) m = -1;
       float dot = 0.0f, nrm = 0.0f;
       for (int v0 = lane; v0 < nvec; v0 += 128) {
