@@ -195,12 +195,12 @@ int launch_fill_holes(void* kc, void* vc, const int* msrc, const int* mdst, cons
 int launch_attention(const void* q, const void* k, const void* v, int M, int N, int H, int dtype, void* out,
                      void* scratch, int* status, cudaStream_t st, AttnKvMaps* maps = nullptr,
                      const float* kmax2 = nullptr, float* lse = nullptr, bool beside_previous = false,
-                     unsigned* tickets = nullptr, const KeySums& sums = {}) {
+                     unsigned* tickets = nullptr, const KeySums& sums = {}, bool in_step = false) {
   int launches = 0;
   const int rc = dtype == kBF16 ? attn_tcgen05_launch(q, k, v, M, N, H, out, scratch, status, st, maps, kmax2, lse,
                                                       beside_previous, tickets, &launches, sums)
                                 : attn_f32_launch(q, k, v, M, N, H, out, scratch, status, st, lse, beside_previous, tickets,
-                                                  &launches);
+                                                  &launches, in_step);
   g_launches.fetch_add(launches);
   if (rc == OVGGT_ERR_CUDA) cuda_fail((cudaError_t)attn_tcgen05_last_error());
   return rc;
@@ -729,9 +729,9 @@ int enqueue_front(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, bool 
 // The attention over all n + M rows, and the bookkeeping that closes the attend half.  Attention does not care in
 // which order the cached rows lie, so it reads the K/V buffer front to back in either layout.
 // beside_previous: what was enqueued on st just before is the same step's selection, which the attention does not wait for;
-// sums: what that one leaves to be added up beside the attention.
+// sums: what that one leaves to be added up beside the attention.  in_step: the step's selection runs beside it, on whatever stream.
 int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaStream_t st, int N, int kb,
-                      bool beside_previous = false, const KeySums& sums = {}) {
+                      bool beside_previous = false, const KeySums& sums = {}, bool in_step = false) {
   LayerState& S = h->layers[layer];
   int rc;
   {
@@ -739,7 +739,7 @@ int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, c
     rc = launch_attention(io->q, S.kbuf[kb], S.vbuf[kb], h->M, N, h->cfg.n_heads, h->cfg.dtype, io->out,
                           h->attn_scratch, h->status, st, &S.maps[kb], key_norm_bound(h, S),
                           h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous, h->attn_tickets,
-                          sums);
+                          sums, in_step);
   }
   return rc;
 }
@@ -1134,7 +1134,7 @@ extern "C" int ovggt_layer_step(ovggt_cache* h, int32_t layer, const ovggt_frame
   rc = compress_impl(h, layer, io, st, nullptr, sums_beside);
   // (a compress that is refused, as for a frame older than the last anchor decision, leaves the frame attended)
   const int ra = enqueue_attention(h, layer, io, stable ? h->side : st, N, kb, !stable && rc == OVGGT_OK,
-                                   sums_beside && rc == OVGGT_OK ? key_sums(h, S, n) : KeySums{});
+                                   sums_beside && rc == OVGGT_OK ? key_sums(h, S, n) : KeySums{}, true);
   if (sums_beside && rc == OVGGT_OK && ra != OVGGT_OK) S.ksum_valid = false;
   if (rc == OVGGT_OK) rc = ra;
   h->last_stream = st;
