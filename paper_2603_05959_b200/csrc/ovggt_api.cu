@@ -679,7 +679,6 @@ int enqueue_token(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, cudaS
   A.n = S.n; A.H = h->cfg.n_heads;
   A.frame_id = (long long)io->frame_id;
   A.ids = S.ids[b]; A.flags = S.flags[b]; A.stored = S.stored[b]; A.slot = S.slot[b];
-  A.kmax2 = key_norm_bound(h, S);
   if (diversity) { A.ksum = S.ksum[S.kcur]; A.d = S.d; }
   const int scoring = diversity ? std::min(148, (front_score_items(S.n) + kTokenWarps - 1) / kTokenWarps) : 0;
   const auto kernel = h->cfg.dtype == kBF16 ? k_token_attend<kBF16> : k_token_attend<kF32>;

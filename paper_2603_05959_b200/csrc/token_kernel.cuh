@@ -20,7 +20,6 @@ struct TokenArgs {
   int n, H;
   long long frame_id;
   long long* ids; uint8_t* flags; float* stored; int* slot;   // as in FrontArgs
-  float* kmax2;
   const float* ksum; float* d;
 };
 
@@ -143,15 +142,6 @@ __global__ void __launch_bounds__(kTokenThreads) k_token_attend(const __grid_con
       }
     }
     mref = top;
-  }
-  if (DT == kBF16 && A.kmax2 != nullptr && warp == kTokenWarps - 1) {   // the head's running bound, as warp_key_norm_max
-    float f[VEC], ss = 0.0f;
-    unpack<DT>(A.k_new[vec], f);
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) ss = fmaf(f[e], f[e], ss);
-#pragma unroll
-    for (int x = 1; x < kLanes; x <<= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, x);
-    if (lane == 0) atomicMax(reinterpret_cast<int*>(A.kmax2) + h, __float_as_int(ss));
   }
   // the warp's groups, then the warps
 #pragma unroll
