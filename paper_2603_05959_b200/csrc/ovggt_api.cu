@@ -611,9 +611,10 @@ int validate_attend(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io) {
 
 // The bound of the key norms is kept for bf16 caches whose rows the append kernel holds in one round of loads; the
 // attention kernel then takes |q| |k|_max as a fixed softmax reference.  It only grows (evictions do not lower it),
-// which keeps it a bound; ovggt_cache_reset clears it, an import recomputes it.
+// which keeps it a bound; ovggt_cache_reset clears it, an import recomputes it.  It is kept also while the attention is
+// not to take it (ovggt_cache_set_key_bound): it has to hold for what came then when it is taken again.
 float* key_norm_bound(const ovggt_cache* h, const LayerState& S) {
-  return (h->cfg.dtype == kBF16 && h->C * h->elem / 16 <= 128 && h->use_key_bound) ? S.kmax2 : nullptr;
+  return h->cfg.dtype == kBF16 && h->C * h->elem / 16 <= 128 ? S.kmax2 : nullptr;
 }
 
 // Carry out the moves the layer's last compress left, now, with the stand-alone kernel (for whoever reads the K/V
@@ -736,7 +737,7 @@ int enqueue_attention(ovggt_cache* h, int32_t layer, const ovggt_frame_io* io, c
   {
     ProfScope ps(h, OVGGT_PROF_ATTENTION, st);
     rc = launch_attention(io->q, S.kbuf[kb], S.vbuf[kb], h->M, N, h->cfg.n_heads, h->cfg.dtype, io->out,
-                          h->attn_scratch, h->status, st, &S.maps[kb], key_norm_bound(h, S),
+                          h->attn_scratch, h->status, st, &S.maps[kb], h->use_key_bound ? key_norm_bound(h, S) : nullptr,
                           h->cfg.score_mode == OVGGT_SCORE_ATTN ? h->attn_lse : nullptr, beside_previous, h->attn_tickets,
                           sums, in_step);
   }

@@ -1,5 +1,6 @@
-"""bf16 attention with a key that is not a number, in every kind of column of a tile (exponentials of either unit, a tile's halves,
-the first half, which fixes the reference, and the last row): under the key-norm bound the same bits as without it."""
+"""bf16 attention and the key-norm bound.  A key that is not a number, in every kind of column of a tile (exponentials of either unit,
+a tile's halves, the first half, which fixes the reference, and the last row): under the bound the same bits as without it.  The
+bound switched off and on."""
 import pytest
 import torch
 
@@ -42,3 +43,21 @@ def test_step(sign):
     for t in (11, 12, 13):
         assert torch.equal(bits(outs[0][t]), bits(outs[1][t])), t
         assert bool(torch.isfinite(outs[0][t][:, 64:]).all())
+
+
+def test_bound_off_and_on():
+    """Keys that come while the bound is off are under it when it is on again."""
+    H, g = 2, torch.Generator(device="cuda").manual_seed(2)
+    frames = [[_draw(66, H * 64, g) for _ in range(4)] for _ in range(5)]
+    frames[2][1][30:] *= 40                              # scores of some hundreds, behind the first half of a tile
+    outs = []
+    for on in ([True, True, False, True, True], [False] * 5):
+        cache = B.OvggtCache(n_layers=1, n_heads=H, n_special=1, grid_h=5, grid_w=13, budget=1024, anchor_tokens=0, k_max=0)
+        for t, x in enumerate(frames):
+            cache.set_key_bound(on[t])
+            out = cache.layer_step(0, t, *x)
+        outs.append(out.double())
+        cache.stats(0)
+        cache.destroy()
+    # probabilities and outputs are rounded to within 2^-9 of themselves on either side
+    assert (outs[0] - outs[1]).norm() <= 2.0 ** -7 * outs[1].norm()
