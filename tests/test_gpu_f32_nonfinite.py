@@ -41,26 +41,34 @@ KINDS = pytest.mark.parametrize("kind", ["infinite values", "large values", "key
 
 
 @KINDS
-@pytest.mark.parametrize("route", ["one part", "merged", "joined"])
+@pytest.mark.parametrize("route", ["one part", "merged", "joined", "joined, one query tile"])
 def test_nonfinite(kind, route):
     heads, M, n0 = 3, 130, 650                           # 780 rows: 13 tiles of 64, the last one ragged
+    if route == "joined, one query tile":                # (which a CTA of two takes)
+        M = 117
     g = torch.Generator(device="cuda").manual_seed(len(kind))
     q, k, v = (torch.randn((r, heads * 64), generator=g, device="cuda") for r in (M, n0 + M, n0 + M))
     _spoil(kind, q, k, v, 1)
-    if route == "joined":
-        cache = B.OvggtCache(n_layers=1, n_heads=heads, n_special=0, grid_h=10, grid_w=13, budget=n0 + M, anchor_tokens=0, k_max=0,
-                             protect_first_frame=0, dtype=B.DTYPE_F32)
+    before = B.kernel_launches()
+    if route.startswith("joined"):
+        cache = B.OvggtCache(n_layers=1, n_heads=heads, n_special=0, grid_h=M // 13, grid_w=13, budget=n0 + M, anchor_tokens=0, k_max=0,
+                             protect_first_frame=0, dtype=B.DTYPE_F32, score_mode=B.SCORE_RESIDUAL_STORED)
         rows = lambda x: x[:n0].cpu().numpy()
         cache.import_(0, np.arange(n0), np.zeros(n0, np.uint8), np.zeros(n0, np.float32), rows(k), rows(v), n0 // M, 0)
+        before = B.kernel_launches() + 1                 # (of the frame's append)
         got = cache.layer_attend(0, n0 // M, q, k[n0:], v[n0:])
+        launches = B.kernel_launches() - before
         cache.stats(0)
         cache.destroy()
     elif route == "merged":
         got = B.k_attention(q, k, v, heads)
+        launches = B.kernel_launches() - before
     else:
         got = torch.empty_like(q)
         assert B.lib().ovggt_k_attention(q.data_ptr(), k.data_ptr(), v.data_ptr(), M, n0 + M, heads, B.DTYPE_F32, got.data_ptr(), None,
                                          None, torch.cuda.current_stream().cuda_stream) == 0
+        launches = B.kernel_launches() - before
+    assert launches == (2 if route == "merged" else 1)   # a merge is a launch of its own, so is nothing else
     want = _reference(q, k, v, heads)
     assert bool(torch.isfinite(want).all()) == (kind in ("large values", "keys of weight 0"))
     # entries of the size of 1, a few roundings of 2^-24 of up to 6-sigma scores; BIG weighs 1 / 780 and swamps its column

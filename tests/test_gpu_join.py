@@ -1,5 +1,6 @@
 """Parts of a split KV range joined inside the attention: edges of the 128-row query tile, of the KV tiles and of the number of
-parts, and the ticket counters over several launches, against the fp64 oracle."""
+parts, and the ticket counters over several launches, against the fp64 oracle.  (fp32: every shape is joined by "attend", those of one
+query tile also by "step".)"""
 import numpy as np
 import pytest
 import torch
@@ -13,7 +14,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("grid,cached,heads", [((1, 1), 700, 16),      # one row
                                                ((1, 127), 1025, 3),    # a whole tile
                                                ((3, 43), 2049, 2),     # one row more; 11 and 12 parts
-                                       ((3, 43), 2860, 2),     # the largest number of parts, 16, of one KV tile (fp32: of three)
+                                               ((3, 43), 2860, 2),     # the largest number of parts, 16, of one KV tile (fp32: of three)
                                                ((11, 35), 260, 5),     # few parts
                                                ((1, 126), 127, 1)],    # two KV tiles in one part: nothing to join (fp32: 4, then 6 parts)
                          ids=lambda x: str(x).replace(" ", ""))

@@ -13,8 +13,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("compaction", [B.COMPACT_FILL_HOLES, B.COMPACT_STABLE_GATHER], ids=["holes", "stable"])
 @pytest.mark.parametrize("budget,heads", [(4, 1), (15, 3), (31, 16), (32, 5), (255, 2), (256, 16), (511, 3), (1023, 1), (1024, 2),
                                           (5, 160), (5, 161), (5, 192)])    # (the most heads of one launch, more)
-def test_token_stream(budget, heads, compaction, dtype):
-    cache = B.OvggtCache.camera(n_heads=heads, budget=budget, dtype=dtype, compaction=compaction)
+@pytest.mark.parametrize("mode", [B.SCORE_HYBRID, B.SCORE_RESIDUAL_STORED], ids=["hybrid", "stored"])   # (stored: nothing scored beside)
+def test_token_stream(budget, heads, compaction, dtype, mode):
+    cache = B.OvggtCache.camera(n_heads=heads, budget=budget, dtype=dtype, compaction=compaction, score_mode=mode)
     C, td = heads * 64, B.torch_dtype(dtype)
     g = torch.Generator(device="cuda").manual_seed(budget)
     draw = lambda *shape: torch.randn(shape, generator=g, device="cuda").to(td)
@@ -42,7 +43,7 @@ def test_token_stream(budget, heads, compaction, dtype):
         cache.camera_compress(0, t, r, registered, -1)
         flags.append(1 if t == 0 else 2 if registered else 0)
         sel = cache.last_selection(0)
-        if len(ids) > 1 and len(ids) - 1 > flags[:-1].count(1) + flags[:-1].count(2) + 1:
+        if mode == B.SCORE_HYBRID and len(ids) > 1 and len(ids) - 1 > flags[:-1].count(1) + flags[:-1].count(2) + 1:
             c = K[:-1].sum(0)
             d = (1 - K[:-1] @ c / (K[:-1].norm(dim=1) * c.norm())).cpu().numpy()
             free = np.array(flags[:-1]) == 0
