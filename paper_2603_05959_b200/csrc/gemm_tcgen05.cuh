@@ -16,9 +16,10 @@
 // behind its predecessor and prefetches its part of B (weights, as a rule) into L2 while that one drains.
 // Measured, QKV / output / first (GELU) / second MLP product of 1041 rows, width 1024: 9.7 / 6.3 / 14.1 / 17.0 us; the
 // first and the third took 13.9 and 18.1 us with 128 x 128 tiles of three stages and four epilogue warps that stored row by row.
-// A residual is requested while the products run, not after them: 0.65 us a product with one (a frame through 24 + 24 blocks,
-// 96 of them: 5639 -> 5572 us).  A table of GELU in shared memory was slower than the error functions (the third product 15.1 -> 17.3
-// us in such a frame).
+// A residual is requested while the products run, not after them, in instances of their own (RES): output and second MLP product of
+// 1041 rows 7.0 -> 6.5 and 18.5 -> 17.8 us, of 1374 rows 8.7 -> 7.8 and 22.6 -> 21.7; in an instance for both the registers it
+// waits in cost the QKV product 10.7 -> 11.5.  A table of GELU in shared memory was slower than the error functions (the third product
+// 15.1 -> 17.3 us).
 // Requirements: K a multiple of 64, N a multiple of 8 (TMA row pitch of 16 bytes), 16-byte aligned bases.  Every
 // barrier wait is bounded (about one second); on expiry the CTA records OVGGT_ERR_TIMEOUT and leaves through the
 // common teardown, after the MMAs it issued have drained.
@@ -78,13 +79,14 @@ __device__ __forceinline__ uint32_t gelu_pair(uint32_t w) {
 }
 
 // Finished bf16 columns [n, n + 8) of row m: where the caller wants them.  r: those of the residual.
+template <bool RES>
 __device__ __forceinline__ void gemm_store8(const GemmArgs& P, int m, int n, const uint4& t, const uint4& r) {
   if (P.out[0] != nullptr) {
     const int i = n / P.part;       // (8 columns lie in one part: its width is a multiple of 8)
     __nv_bfloat16* o = i == 0 ? P.out[0] : (i == 1 ? P.out[1] : P.out[2]);
     *reinterpret_cast<uint4*>(o + (size_t)m * P.part + (n - i * P.part)) = t;
   }
-  if (P.residual != nullptr) {
+  if constexpr (RES) {
     const uint32_t* w = reinterpret_cast<const uint32_t*>(&t);
     const uint32_t* rw = reinterpret_cast<const uint32_t*>(&r);
     uint4 s;
@@ -101,7 +103,7 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
 
-template <int BN>
+template <int BN, bool RES>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                     const __grid_constant__ GemmArgs P) {
@@ -148,7 +150,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   const int quad = warp & 3, side = warp >> 2;
   auto unit_row = [&](int i) { return m0 + quad * 32 + (lane + 32 * i) / kUnits; };
   auto unit_col = [&](int i) { return n0 + side * kCols + (lane + 32 * i) % kUnits * 8; };
-  uint4 residual[kUnits];                                  // requested while the products run
+  uint4 residual[RES ? kUnits : 1];                        // requested while the products run
 
   bool ok = aligned;
   if (warp == kProducer) {
@@ -203,7 +205,7 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     }
     __syncwarp();
   } else if (ok) {
-    if (P.residual != nullptr)
+    if constexpr (RES)
 #pragma unroll
       for (int i = 0; i < kUnits; ++i)
         if (unit_row(i) < P.M && unit_col(i) < P.N)        // (N is a multiple of 8)
@@ -233,11 +235,11 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       }
     }
     __syncwarp();
-#pragma unroll
+#pragma unroll 4
     for (int i = 0; i < kUnits; ++i) {
       const int r = (lane + 32 * i) / kUnits, u = (lane + 32 * i) % kUnits;
       if (unit_row(i) < P.M && unit_col(i) < P.N)
-        gemm_store8(P, unit_row(i), unit_col(i), stage[r * kUnits + (u ^ (r & (kUnits - 1)))], residual[i]);
+        gemm_store8<RES>(P, unit_row(i), unit_col(i), stage[r * kUnits + (u ^ (r & (kUnits - 1)))], residual[RES ? i : 0]);
     }
   }
 
@@ -268,10 +270,13 @@ static inline int gemm_tcgen05_launch(const void* A, const void* Bm, const GemmA
   rc = make_rows_map(&tb, Bm, P.K, P.N, kGemmBK);          // 64 n-columns x 64 k-rows per box
   if (rc) return rc;
   const int bn = gemm_tile_width(P.M, P.N, P.K);
-  const auto kernel = bn == 256 ? k_gemm_bf16_tcgen05<256> : (bn == 128 ? k_gemm_bf16_tcgen05<128> : k_gemm_bf16_tcgen05<64>);
-  static std::atomic<uint64_t> smem_set[3];
+  const bool res = P.residual != nullptr;
+  const auto kernel = bn == 256   ? (res ? k_gemm_bf16_tcgen05<256, true> : k_gemm_bf16_tcgen05<256, false>)
+                      : bn == 128 ? (res ? k_gemm_bf16_tcgen05<128, true> : k_gemm_bf16_tcgen05<128, false>)
+                                  : (res ? k_gemm_bf16_tcgen05<64, true> : k_gemm_bf16_tcgen05<64, false>);
+  static std::atomic<uint64_t> smem_set[6];
   const size_t smem = gemm_smem_bytes(bn);
-  cudaError_t e = allow_smem(kernel, smem, smem_set[bn == 256 ? 0 : (bn == 128 ? 1 : 2)]);
+  cudaError_t e = allow_smem(kernel, smem, smem_set[(bn == 256 ? 0 : (bn == 128 ? 2 : 4)) + res]);
   if (e == cudaSuccess)
     e = launch_dependent(kernel, dim3((P.N + bn - 1) / bn, (P.M + kGemmBM - 1) / kGemmBM), kGemmThreads, 1, smem, st, true, ta, tb, P);
   if (e != cudaSuccess) { g_attn_last_error = (int)e; return OVGGT_ERR_CUDA; }
