@@ -50,3 +50,14 @@ def test_gelu_over_its_range():
     st = torch.zeros(16, dtype=torch.int32, device="cuda")
     B.k_linear_bf16(a, torch.eye(64, device="cuda").bfloat16(), (out,), gelu=True, status=st)
     assert torch.equal(out, torch.nn.functional.gelu(a))
+
+
+def test_gelu_where_no_value_is_below_its_polynomial():
+    """Every finite bf16 value from -3 on, without the others beside them that send a warp to the error functions."""
+    v = torch.arange(0, 0x7F80, dtype=torch.int16, device="cuda").view(torch.bfloat16)
+    v = torch.cat([v, -v[v <= 3]])
+    a = torch.cat([v, v.new_zeros(-v.numel() % 64)]).view(-1, 64)
+    out = torch.empty_like(a)
+    st = torch.zeros(16, dtype=torch.int32, device="cuda")
+    B.k_linear_bf16(a, torch.eye(64, device="cuda").bfloat16(), (out,), gelu=True, status=st)
+    assert torch.equal(out, torch.nn.functional.gelu(a))
