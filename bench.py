@@ -455,6 +455,8 @@ def run_c2(args) -> None:
                          "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "peak_kind": f"{peak_kind} burst cuBLAS bf16 peak", "traffic": attention_traffic(),
                          "algorithmic_flops": attn_flops, "launch_ms": attn_ms,
+                         "instance": "without the key sums, as the halves of a step launch it one after the other; a "
+                                     "step that overlaps them launches the one that takes the sums too (0.6 % longer)",
                          # the launch is timed right after the K timed steps, at the clocks the step itself ran at;
                          # the same figure against the sustained (power-capped) cuBLAS peak, for long runs
                          "frac_of_sustained_peak": achieved / float(peaks["bf16_tflops_sustained"])},

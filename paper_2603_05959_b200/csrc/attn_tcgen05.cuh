@@ -44,8 +44,8 @@ constexpr int kAttnThreads = 256;
 // setmaxnreg only moves registers inside the pool the CTA was launched with (threads x launch registers), and an
 // increase that the pool cannot serve waits for ever: the two warpgroups must fit 256 x 128.
 constexpr int kRegsLaunch = 128;    // what __launch_bounds__(256, 2) gives: 65536 / 512
-// (How the registers are split decides how ptxas lays the softmax loop out: 1374 x 9566 x 16 with 216 + 40 registers 74.8 us, with
-// 208 + 48 73.8, with 200 + 56 74.0; with the key sums 76.4, 75.2 and 75.5.)
+// (216 + 40 is as fast, within 1 % either way over sizes from 5 x 305 x 4 to 1374 x 34142 x 16.  The instances with the key
+// sums spill a register: 4 bytes stored, 16 loaded.)
 constexpr int kRegsSoftmax = 208, kRegsOther = 48;
 static_assert(128 * kRegsSoftmax + 128 * kRegsOther <= kAttnThreads * kRegsLaunch, "register pool of the CTA exceeded");
 constexpr int kQBytes = kBM * kHD * 2;           // 16 KB
@@ -813,7 +813,8 @@ k_attn_tcgen05(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       // p = 2^(s * c - mref) on pairs, packed to bf16 over the front of s[]; returns the row's sum of p (four
       // independent packed partial sums, folded in a fixed order).  With `track` the raw row maximum is gathered in
       // the same pass (four chains of 3-input maxima), where it hides behind the exponentials; without `clamp` two
-      // instructions in eleven a cubic are saved (1374 x 17758 x 16: 125.0 -> 121.9 us).
+      // instructions in eleven a cubic are saved (1374 x 17758 x 16: 119.9 -> 117.3 us, 1374 x 34142 x 16 216 -> 211.5; ranges of one or
+      // two tiles pay for the second pass's code: 69 x 325 x 4 5.9 -> 6.0 us).
       auto exp_pass = [&](auto track, auto clamp, float& raw_max) -> float {
         const float2 c2 = make_float2(c, c), nm2 = make_float2(-mref, -mref);
         float2 acc[4];

@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(kFrontThreads, 2) k_front(const __grid_constan
   constexpr int VEC = VecOf<DT>::n;
   extern __shared__ __align__(16) float sh_ksum[];
   const int lane = threadIdx.x & 31;
-  // (warp by warp over the CTAs, so that each SM gets its share of the new rows, which take longest: 24 layers of 1374 + 8192 rows
-  // 2694 -> 2683 us, a step of 1374 + 4096 by stored scores 58.0 -> 57.5)
+  // (warp by warp over the CTAs, so that each SM gets its share of the new rows, which take longest: steps of 1374 + 4096 and 69 + 16000
+  // rows are 2 and 3 % faster for it)
   const int gw = (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x), warps_total = (int)((gridDim.x * (unsigned)blockDim.x) >> 5);
   const int n_div = A.ksum != nullptr ? front_score_items(A.n) : 0;
   const int n_norm = A.resid != nullptr ? front_score_items(A.M) : 0;

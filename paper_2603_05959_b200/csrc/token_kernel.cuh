@@ -6,7 +6,7 @@
 // FMA pipes; the others score four rows a warp, as k_front does.  The new row is read where the caller has it and written to the cache
 // on the way; no move is pending, since the selection of such a cache moves its one row itself.  Before, k_front and then the
 // tensor-core attention, 128 query rows for one, were two launches in a row: a frame through four layers of 16 heads and 145
-// rows took 81.4 us and takes 71.4, of which these kernels are 51 and the caller's and the launches' host time bounds the rest.
+// rows took 81.5 us and takes 70.5, of which the kernels are 48 and the caller's and the launches' host time bounds the rest.
 #pragma once
 
 #include "front_kernel.cuh"
