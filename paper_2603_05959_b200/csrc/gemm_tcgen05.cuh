@@ -245,7 +245,8 @@ k_gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tm_a, const __grid_const
         stage[lane * kUnits + ((j / 8 + u) ^ (lane & (kUnits - 1)))] = make_uint4(w[4 * u], w[4 * u + 1], w[4 * u + 2], w[4 * u + 3]);
     }
     __syncwarp();
-#pragma unroll 4
+    constexpr int kAtOnce = RES ? kUnits : 4;              // (a residual's registers have to be named)
+#pragma unroll kAtOnce
     for (int i = 0; i < kUnits; ++i) {
       const int r = (lane + 32 * i) / kUnits, u = (lane + 32 * i) % kUnits;
       if (unit_row(i) < P.M && unit_col(i) < P.N)
